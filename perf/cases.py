@@ -124,8 +124,8 @@ def _near_ties(x, gates, k, gap=1e-3):
     return bad.nonzero()[:, 0]
 
 
-def prepare(case, seed):
-    c = dict(DEFAULTS, **case)
+def _inputs(c, seed):
+    """Weights, biases and batch of one case, in storage type, from the seed alone."""
     g = torch.Generator(device="cuda").manual_seed(int(seed) * 7919 + 17)
     store = torch.float32 if c["dtype"] == "f32" else torch.bfloat16
     H, E, M, D, k = c["heads"], c["experts"], c["d_model"], c["d_head"], c["k"]
@@ -133,12 +133,11 @@ def prepare(case, seed):
     def normal(*shape, fan_in=1):
         return (torch.randn(*shape, generator=g, device="cuda") / math.sqrt(fan_in)).to(store)
 
-    Wq, Wk = normal(H, M, D, fan_in=M), normal(H, M, D, fan_in=M)
-    Wv, Wo = normal(H, E, M, D, fan_in=M), normal(H, E, D, M, fan_in=D)
-    Ws, Wd = normal(H, M, E, fan_in=M), None if c["shared"] else normal(H, M, E, fan_in=M)
-    bias_s = _zipf_bias(c, g) if c["zipf"] else None
-    bias_d = _zipf_bias(c, g) if c["zipf"] and not c["shared"] else None
-    gates = [(Ws, bias_s)] + ([] if Wd is None else [(Wd, bias_d)])
+    w = dict(Wq=normal(H, M, D, fan_in=M), Wk=normal(H, M, D, fan_in=M), Wv=normal(H, E, M, D, fan_in=M), Wo=normal(H, E, D, M, fan_in=D),
+             Ws=normal(H, M, E, fan_in=M), Wd=None if c["shared"] else normal(H, M, E, fan_in=M))
+    w["bias_s"] = _zipf_bias(c, g) if c["zipf"] else None
+    w["bias_d"] = _zipf_bias(c, g) if c["zipf"] and not c["shared"] else None
+    gates = [(w["Ws"], w["bias_s"])] + ([] if c["shared"] else [(w["Wd"], w["bias_d"])])
     n = c["batch"] * (c["cache"] + c["seq"])
     x = normal(n, M)
     # a token whose selection hangs on the last bits of a sum has two right answers: such rows are drawn again
@@ -149,22 +148,97 @@ def prepare(case, seed):
         x[rows] = normal(rows.numel(), M)
         rows = rows[_near_ties(x[rows], gates, k)]
     x = x.view(c["batch"], c["cache"] + c["seq"], M)
+    xl = None
+    if c["positions"]:
+        f32 = lambda *shape, fan_in=1: torch.randn(*shape, generator=g, device="cuda") / math.sqrt(fan_in)
+        xl = (f32(H, M, D, fan_in=M), 0.5 * f32(H, D), 0.5 * f32(H, D))
+    dout = torch.randn(c["batch"], c["seq"], M, generator=g, device="cuda") if c["train"] else None
+    return w, x, xl, dout
 
-    layer = binding.Layer(M, H, D, E, k, shared_selection=c["shared"])
+
+def prepare(case, seed):
+    c = dict(DEFAULTS, **case)
+    w, x, xl, dout = _inputs(c, seed)
+    layer = binding.Layer(c["d_model"], c["heads"], c["d_head"], c["experts"], c["k"], shared_selection=c["shared"])
     layer.sh_configure(binding.SH_F32 if c["dtype"] == "f32" else binding.SH_BF16, c["batch"], c["seq"], cache_len=c["cache"])
-    layer.sh_set_weights(Wq, Wk, Wv, Wo, Ws, Wd, bias_s, bias_d)
+    layer.sh_set_weights(*[w[n] for n in ("Wq", "Wk", "Wv", "Wo", "Ws", "Wd", "bias_s", "bias_d")])
     layer.sh_set_causal(c["causal"])
     if c["rope"]:
         layer.sh_set_rope(10000.0)
     if c["out_f16"]:
         layer.sh_set_output_f16(True)
     if c["positions"]:
-        f32 = lambda *shape, fan_in=1: torch.randn(*shape, generator=g, device="cuda") / math.sqrt(fan_in)
-        layer.sh_set_xl_positions(f32(H, M, D, fan_in=M), 0.5 * f32(H, D), 0.5 * f32(H, D))
+        layer.sh_set_xl_positions(*xl)
     state = dict(layer=layer, x=x)
     if c["train"]:
-        state["dout"] = torch.randn(c["batch"], c["seq"], M, generator=g, device="cuda")
+        state["dout"] = dout
     return state
+
+
+def _select(x, W, bias, k):
+    """Per head the gate values of the k largest logits, zero elsewhere: [n, H, E] (a lower index wins ties)."""
+    z = torch.einsum("nm,hme->nhe", x, W)
+    if bias is not None:
+        z = z + bias
+    order = torch.argsort(z.detach(), dim=2, descending=True, stable=True)[..., :k]
+    return torch.sigmoid(z) * torch.zeros_like(z).scatter(2, order, 1.0)
+
+
+def _layer64(c, w, x, xl):
+    """The layer's equations in the precision of its arguments, plain torch."""
+    B, T, C, M, H, D, E, k = (c[n] for n in ("batch", "seq", "cache", "d_model", "heads", "d_head", "experts", "k"))
+    S = C + T
+    flat = x.reshape(B * S, M)
+    gs = _select(flat, w["Ws"], w["bias_s"], k)
+    gd = gs if c["shared"] else _select(flat, w["Wd"], w["bias_d"], k)
+    rows = torch.arange(B * S, device=x.device).view(B, S)[:, C:].reshape(-1)
+    t = torch.arange(S, device=x.device)
+    seen = t[None, :] <= t[C:, None] if c["causal"] else None
+    y = torch.zeros(B * T, M, dtype=x.dtype, device=x.device)
+    if c["rope"]:
+        ang = t[:, None].double() * 10000.0 ** (-2.0 * torch.arange(D // 2, device=x.device).double() / D)
+        cos, sin = torch.cos(ang), torch.sin(ang)
+    if xl is not None:
+        freq = 10000.0 ** (-2.0 * torch.arange(M // 2, device=x.device).double() / M)
+        emb = torch.cat([torch.sin(t[:, None] * freq), torch.cos(t[:, None] * freq)], dim=1)
+    for h in range(H):
+        q, key = (flat[rows] @ w["Wq"][h]).view(B, T, D), (flat @ w["Wk"][h]).view(B, S, D)
+        if c["rope"]:
+            turn = lambda a: torch.stack([a[..., 0::2] * cos - a[..., 1::2] * sin, a[..., 0::2] * sin + a[..., 1::2] * cos], dim=-1).flatten(-2)
+            q, key = turn(q), turn(key)
+        v = sum(gs[:, h, e, None] * (flat @ w["Wv"][h, e]) for e in range(E)).view(B, S, D)
+        read = []
+        for b in range(B):
+            s = q[b] @ key[b].T
+            if xl is not None:
+                s = (q[b] + xl[1][h]) @ key[b].T
+                r = (q[b] + xl[2][h]) @ (emb @ xl[0][h]).T
+                s = s + r.gather(1, (t[C:, None] - t[None, :]).clamp(min=0))
+            s = s / math.sqrt(D)
+            if seen is not None:
+                s = s.masked_fill(~seen, -math.inf)
+            read.append(torch.softmax(s, dim=1) @ v[b])
+        read = torch.cat(read)
+        for e in range(E):
+            y = y + gd[rows][:, h, e, None] * (read @ w["Wo"][h, e])
+    return y.view(B, T, M)
+
+
+def exact(case, seed):
+    c = dict(DEFAULTS, **case)
+    w, x, xl, dout = _inputs(c, seed)
+    d64 = lambda a: None if a is None else a.double()
+    w, x, xl = {n: d64(a) for n, a in w.items()}, d64(x), None if xl is None else [d64(a) for a in xl]
+    if not c["train"]:
+        with torch.no_grad():
+            return _layer64(c, w, x, xl)
+    names = ("Wq", "Wk", "Wv", "Wo", "Ws", "Wd")
+    wrt = [x] + [w[n] for n in names]
+    for a in wrt:
+        a.requires_grad_(True)
+    out = _layer64(c, w, x, xl)
+    grads = torch.autograd.grad(out, wrt, d64(dout))
+    return dict(zip(["dx"] + ["d" + n for n in names], grads), out=out.detach())
 
 
 def run(state):
