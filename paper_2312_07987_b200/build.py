@@ -12,7 +12,7 @@ LIB_PATH = os.path.join(PKG_DIR, "libswitchhead.so")
 # expert-index use, and launch-structure switches read from the environment).  Tests load it through
 # SWITCHHEAD_LIB; the release library reads nothing from the environment.
 DEBUG_LIB_PATH = os.path.join(PKG_DIR, "libswitchhead_debug.so")
-SOURCES = ["sh_api.cu", "sh_tc.cu", "sh_static.cu"]
+SOURCES = ["sh_api.cu", "sh_tc.cu", "sh_f32.cu", "sh_static.cu"]
 NVCC_FLAGS = ["-std=c++17", "-O3", "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo",
               "-shared", "-Xcompiler", "-fPIC"]
 

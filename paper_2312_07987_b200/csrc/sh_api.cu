@@ -7,8 +7,8 @@
 #include <new>
 
 #include "sh_internal.cuh"
+#include "sh_launch.cuh"
 #include "sh_simt.cuh"
-#include "sh_backward.cuh"
 
 static thread_local char g_err[512] = "";
 
@@ -18,15 +18,6 @@ void sh_set_error(const char* fmt, ...) {
   vsnprintf(g_err, sizeof(g_err), fmt, ap);
   va_end(ap);
 }
-
-#define SH_CUDA_CHECK(expr)                                                          \
-  do {                                                                               \
-    cudaError_t _e = (expr);                                                         \
-    if (_e != cudaSuccess) {                                                         \
-      sh_set_error("%s failed: %s", #expr, cudaGetErrorString(_e));                  \
-      return SH_ERR_CUDA;                                                            \
-    }                                                                                \
-  } while (0)
 
 static size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
@@ -99,8 +90,13 @@ static void layout_workspace(sh_layer* L) {
   // query / key experts (sh_create_moe_qk): [H, E, D, M] like the value experts
   o.wq_e = take(L->moe_q ? HD * d.E * d.M * in : 16);
   o.wk_e = take(L->moe_k ? HD * d.E * d.M * in : 16);      // pair number of every (token, head), source side
-  // fp32 configuration: scratch of the backward pass (dQ, dK, dV, dAhat [N, H, D] and the gate gradients [2, N, H, k])
-  o.bw = take(L->dtype == SH_F32 && !L->dense ? ((size_t)4 * d.N * HD + (size_t)2 * d.N * d.H * d.k) * 4 : 16);
+  // fp32 configuration: scratch of the backward pass (dQ, dK, dV, dAhat [N, H, D] and the gate gradients [2, N, H, k]
+  //  in list order, the gate gradients once more as a matrix [N, G], rowsum(dAhat o Ahat) [N, H]); the gate logits
+  //  [N, G]; per attention row the score maximum and 1 / normaliser)
+  const bool f32 = L->dtype == SH_F32 && !L->dense;
+  o.bw = take(f32 ? ((size_t)4 * d.N * HD + (size_t)2 * d.N * d.H * d.k + (size_t)d.N * (sh_f32_ldz(d) + d.H)) * 4 : 16);
+  o.f32z = take(f32 ? (size_t)d.N * sh_f32_ldz(d) * 4 : 16);
+  o.f32stats = take(f32 ? (size_t)d.N * d.H * 8 : 16);
   o.stamps = take(sizeof(ShStampBlock));
   o.total = off;
 }
@@ -472,6 +468,10 @@ static int forward_simt(sh_layer* L, int stages, const void* x, void* out, cudaS
   return SH_OK;
 }
 
+int sh_simt_attention_f32(sh_layer* L, cudaStream_t st) {
+  return forward_simt<float, float>(L, SH_STAGE_ATTN, nullptr, nullptr, st);
+}
+
 int sh_simt_run_bf16(sh_layer* L, int stages, const void* x, void* out, cudaStream_t st) {
   return forward_simt<__nv_bfloat16, __half>(L, stages, x, out, st);
 }
@@ -572,7 +572,7 @@ extern "C" int sh_forward(sh_layer* L, const void* x, void* out, void* stream) {
   cudaStream_t st = (cudaStream_t)stream;
   L->launches = 0;
   L->fwd_x = x;
-  if (L->dtype == SH_F32) return forward_simt<float, float>(L, SH_STAGE_ALL, x, out, st);
+  if (L->dtype == SH_F32) return L->dense ? forward_simt<float, float>(L, SH_STAGE_ALL, x, out, st) : sh_f32_forward(L, x, out, st);
   return sh_tc_forward(L, x, out, st);
 }
 
@@ -587,37 +587,7 @@ extern "C" int sh_backward(sh_layer* L, const void* x, const float* dout, float*
   }
   if (!x || !dout || !dx || !dWq || !dWk || !dWv || !dWo || !dWs || !dWd) { sh_set_error("sh_backward: NULL argument"); return SH_ERR_INVALID_ARG; }
   if (L->fwd_x != x) { sh_set_error("sh_backward needs the intermediates of sh_forward on the same x: call sh_forward(layer, x, ...) first"); return SH_ERR_NOT_CONFIGURED; }
-  const ShDims& d = L->d;
-  char* ws = L->ws;
-  cudaStream_t st = (cudaStream_t)stream;
-  const size_t nhd = (size_t)d.N * d.H * d.D;
-  ShBwArgs a{};
-  a.d = d; a.x = (const float*)x; a.dy = dout;
-  a.q = (const float*)(ws + L->o.q); a.k = (const float*)(ws + L->o.k); a.v = (const float*)(ws + L->o.v);
-  a.ahat = (const float*)(ws + L->o.ahat);
-  a.idx = (const int*)(ws + L->o.idx); a.gate = (const float*)(ws + L->o.gate);
-  a.wqk = (const float*)(ws + L->o.wqk); a.wv = (const float*)(ws + L->o.wv); a.wo = (const float*)(ws + L->o.wo);
-  a.wgate = (const float*)(ws + L->o.wgate);
-  float* scratch = (float*)(ws + L->o.bw);
-  a.dq = scratch; a.dk = scratch + nhd; a.dv = scratch + 2 * nhd; a.dahat = scratch + 3 * nhd; a.dgate = scratch + 4 * nhd;
-  a.dx = dx; a.dWq = dWq; a.dWk = dWk; a.dWv = dWv; a.dWo = dWo; a.dWs = dWs; a.dWd = dWd;
-  SH_CUDA_CHECK(cudaMemsetAsync(a.dk, 0, 2 * nhd * 4, st));                                   // dK, dV: summed by atomics
-  SH_CUDA_CHECK(cudaMemsetAsync(dx, 0, (size_t)d.N * d.M * 4, st));
-  SH_CUDA_CHECK(cudaMemsetAsync(dWq, 0, (size_t)d.H * d.M * d.Dt * 4, st));
-  SH_CUDA_CHECK(cudaMemsetAsync(dWk, 0, (size_t)d.H * d.M * d.Dt * 4, st));
-  SH_CUDA_CHECK(cudaMemsetAsync(dWv, 0, (size_t)d.H * d.E * d.M * d.Dt * 4, st));
-  SH_CUDA_CHECK(cudaMemsetAsync(dWo, 0, (size_t)d.H * d.E * d.Dt * d.M * 4, st));
-  SH_CUDA_CHECK(cudaMemsetAsync(dWs, 0, (size_t)d.H * d.M * d.E * 4, st));
-  SH_CUDA_CHECK(cudaMemsetAsync(dWd, 0, (size_t)d.H * d.M * d.E * 4, st));
-  sh_bw_o_kernel<<<d.N * d.H, 128, 0, st>>>(a);
-  const long rows = (long)d.B * d.H * d.T;
-  sh_bw_attn_kernel<<<(unsigned)((rows + 3) / 4), 128, 0, st>>>(a);
-  sh_bw_v_kernel<<<d.N * d.H, 128, 0, st>>>(a);
-  sh_bw_qk_kernel<<<d.N, 128, (size_t)2 * d.H * d.D * 4, st>>>(a);
-  sh_bw_gate_kernel<<<d.N, 128, 0, st>>>(a);
-  SH_CUDA_CHECK(cudaGetLastError());
-  L->launches = 5;
-  return SH_OK;
+  return sh_f32_backward(L, x, dout, dx, dWq, dWk, dWv, dWo, dWs, dWd, (cudaStream_t)stream);
 }
 
 extern "C" int sh_forward_timed(sh_layer* L, const void* x, void* out, void* stream, float* stage_ms) {
@@ -740,7 +710,7 @@ extern "C" int sh_gate_topk(sh_layer* L, const void* x, int32_t* idx, float* gat
   if (!x) { sh_set_error("x must not be NULL"); return SH_ERR_INVALID_ARG; }
   cudaStream_t st = (cudaStream_t)stream;
   L->launches = 0;
-  rc = (L->dtype == SH_F32) ? launch_gate_sort<float>(L, x, st) : sh_tc_gate_sort(L, x, st);
+  rc = (L->dtype == SH_F32) ? sh_f32_gate_sort(L, x, st) : sh_tc_gate_sort(L, x, st);
   if (rc != SH_OK) return rc;
   const ShDims& d = L->d;
   // side s of the outputs <- side s of the workspace (with a shared selection both <- the one side)

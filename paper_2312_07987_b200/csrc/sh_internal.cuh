@@ -89,7 +89,7 @@ __device__ __forceinline__ void sh_stamp_end(unsigned long long* s, int k) { if 
 
 struct ShWorkspace {
   size_t status, wqk, wgate, gbias, wv, wo, q, k, v, ahat, idx, gate, blockcnt, blockoff,
-         offsets, lists, lgate, tiles, ntiles, rope, vearly, vearly_cnt, xl_emb, xl_r, xl_uv, xl_r16, xl_vr, xl_uk, xl_bias, wos, gid, wq_e, wk_e, bw, stamps, total;
+         offsets, lists, lgate, tiles, ntiles, rope, vearly, vearly_cnt, xl_emb, xl_r, xl_uv, xl_r16, xl_vr, xl_uk, xl_bias, wos, gid, wq_e, wk_e, bw, f32z, f32stats, stamps, total;
 };
 
 // Words of the 256-byte status block at the start of the workspace.
@@ -186,6 +186,15 @@ enum { SH_STAGE_GATE = 1, SH_STAGE_QK = 2, SH_STAGE_V = 4, SH_STAGE_ATTN = 8, SH
 // CUDA-core stages on bf16 storage with fp16 intermediates (same buffers and layouts as the
 // tensor-core kernels): the on-device reference used while a tensor-core stage is brought up.
 int sh_simt_run_bf16(sh_layer* L, int stages, const void* x, void* out, cudaStream_t st);
+
+// fp32 configuration of the SwitchHead layer (sh_f32.cu).
+inline int sh_f32_ldz(const ShDims& d) { return (d.G + 7) / 8 * 8; }       // row length of the gate-logit / gate-gradient matrix
+int sh_f32_gate_sort(sh_layer* L, const void* x, cudaStream_t st);
+int sh_f32_forward(sh_layer* L, const void* x, void* out, cudaStream_t st);
+int sh_f32_backward(sh_layer* L, const void* x, const float* dout, float* dx, float* dWq, float* dWk, float* dWv,
+                    float* dWo, float* dWs, float* dWd, cudaStream_t st);
+// The CUDA-core attention kernel on fp32 storage (the relative-position term of Transformer-XL).
+int sh_simt_attention_f32(sh_layer* L, cudaStream_t st);
 
 // Tensor-core (tcgen05) path of the bf16 configuration.
 int sh_tc_prepare(sh_layer* L);                 // builds tensor maps after the weights are repacked

@@ -1,0 +1,66 @@
+"""The fp32 configuration's tensor-core GEMMs (split bf16), attention tiles and one-launch selection at the edges of
+their tiles: d_head off the 16-column grid and across 64 / 128 columns, token counts around 32 / 64 / 128, more than one
+selection sweep (1024 tokens), empty experts, split contractions, operands that are only 4-byte aligned."""
+import numpy as np
+import pytest
+import torch
+
+from oracle.switchhead_backward import switchhead_backward
+from oracle.switchhead_oracle import switchhead_forward
+from paper_2312_07987_b200 import binding, inputs
+
+pytestmark = pytest.mark.gpu
+# max-abs error / largest value (an expert nobody selects makes most of a gradient zero, and an RMS over it means
+# nothing).  An fp32 sum of K products differs from the fp64 one by about sqrt(K) 2^-24 of its own size, times 5 for the
+# largest of ~1e5 values: K <= 2100 tokens, 1.4e-5.
+TOL = 1.4e-5
+
+
+def run(B, T, M, H, D, E, k, causal=True, offset=0, zipf=0.0):
+    cfg = inputs.LayerConfig("tiles", inputs.DTYPE_F32, B, T, M, H, D, E, k, seed=77 + T + D, zipf_bias=zipf)
+    inp = inputs.make_inputs(cfg)
+    layer = binding.layer_from_inputs(inp)
+    layer.sh_set_causal(causal)
+    x = binding.to_device(inp.x, cfg.dtype)
+    G = np.random.default_rng(3).standard_normal(inp.x.shape).astype(np.float32)
+    g = torch.empty(G.size + offset, dtype=torch.float32, device="cuda")[offset:].view(G.shape)
+    g.copy_(torch.from_numpy(G))
+    y = layer.sh_forward(x)
+    got = layer.sh_backward(x, g)
+    torch.cuda.synchronize()
+    assert layer.sh_last_status() == 0
+    layer.sh_check_guards()
+    args = (inp.x, inp.Wq, inp.Wk, inp.Wv, inp.Wo, inp.Ws, inp.Wd, cfg.k)
+    want = dict(switchhead_backward(*args, G, inp.bias_s, inp.bias_d, causal=causal))
+    want["y"] = switchhead_forward(*args, inp.bias_s, inp.bias_d, causal=causal, return_stages=False)["y"]
+    got["y"] = y
+    for name in ("y", "dx", "dWq", "dWk", "dWv", "dWo", "dWs", "dWd"):
+        a, r = got[name].cpu().numpy().astype(np.float64).reshape(want[name].shape), want[name]
+        # (one token attends to itself alone: dQ and dK are exactly zero, and what is left of them is the rounding of
+        #  two sums of order one)
+        err = np.abs(a - r).max() / (np.abs(r).max() or 1.0)
+        assert err < TOL, (name, err)
+    layer.close()
+
+
+@pytest.mark.parametrize("B,T,M,H,D,E,k", [
+    (1, 1, 64, 1, 1, 1, 1),          # one of everything
+    (1, 31, 64, 3, 17, 2, 1),        # d_head off the 16-column grid; fewer tokens than a tile
+    (2, 33, 128, 1, 64, 3, 3),       # every expert selected; one token into the second query tile
+    (1, 129, 192, 2, 65, 4, 2),      # one column into the second 64-column tile, one row into the second row tile
+    (1, 127, 64, 1, 128, 2, 2),
+    (1, 65, 448, 2, 129, 5, 2),      # 129: two 128-column tiles, the 256-wide attention kernels
+    (3, 50, 128, 1, 256, 3, 1),
+    (1, 2100, 64, 1, 40, 1, 1),      # three selection sweeps; contractions over tokens in parts
+    (2, 600, 128, 2, 76, 32, 4),     # 32 experts, hardly a full tile among them
+])
+def test_f32_tile_edges(B, T, M, H, D, E, k):
+    run(B, T, M, H, D, E, k)
+
+
+def test_f32_empty_experts_and_no_mask():
+    run(1, 200, 128, 2, 48, 8, 1, causal=False, zipf=4.0)
+
+
+def test_f32_gradient_input_off_its_alignment():
+    run(1, 90, 128, 2, 76, 4, 2, offset=1)
