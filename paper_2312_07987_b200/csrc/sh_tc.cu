@@ -9,6 +9,7 @@
 #include "sh_tc_pgemm.cuh"
 #include "sh_tc_attn2.cuh"
 #include "sh_tc_attn3.cuh"
+#include "sh_tc_attnw.cuh"
 #include "sh_tc_gate.cuh"
 #include "sh_tc_oproj2.cuh"
 #include "sh_tc_qkpair.cuh"
@@ -52,14 +53,14 @@ int sh_tc_encode_2d(CUtensorMap* map, int elem_kind, const void* base, uint64_t 
   return SH_OK;
 }
 
-// 3-D tensor [n2, n1, inner] of fp16 (Q, K, V as [B*H, T, D]); box = 128 rows of 64 elements of
+// 3-D tensor [n2, n1, inner] of fp16 (Q, K, V as [B*H, T, D]); box = 128 (or `rows`) rows of 64 elements of
 // one (batch, head) slice, so rows past the end of a sequence read as zero.
-static int encode_3d_f16(CUtensorMap* map, const void* base, uint64_t inner, uint64_t n1, uint64_t n2) {
+static int encode_3d_f16(CUtensorMap* map, const void* base, uint64_t inner, uint64_t n1, uint64_t n2, uint32_t rows = 128) {
   EncodeTiledFn enc = get_encode();
   if (!enc) { sh_set_error("cuTensorMapEncodeTiled is not available from the driver"); return SH_ERR_CUDA; }
   cuuint64_t dims[3] = {inner, n1, n2};
   cuuint64_t strides[2] = {inner * 2, inner * n1 * 2};
-  cuuint32_t box[3] = {64, 128, 1};
+  cuuint32_t box[3] = {64, rows, 1};
   cuuint32_t estr[3] = {1, 1, 1};
   CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -188,10 +189,6 @@ int sh_tc_prepare(sh_layer* L) {
   S->attn_balanced = !getenv("SH_ATTN_ADJACENT");
   if (const char* env = getenv("SH_SIMT_STAGES")) S->simt_mask = atoi(env);   // bit mask gate=1, qk=2, v=4, attention=8, o=16
 #endif
-  // d_head above 128 (stored as 256: the paper's 132 and 168): S and O of two query tiles no longer fit the 512
-  // tensor-memory columns and the expert kernels are built for 64 / 128 columns, so every stage of such a layer
-  // runs on the CUDA-core kernels (bf16 weights and x, fp16 intermediates, fp32 sums) - correct, not fast
-  if (d.D > 128) S->simt_mask = SH_STAGE_GATE | SH_STAGE_QK | SH_STAGE_V | SH_STAGE_ATTN | SH_STAGE_O;
   // 256-column tiles (CTA pairs, or the persistent single-CTA kernel) need the projection's width to
   // be a multiple of 256; other widths take the one-CTA-per-tile kernel with 128-column tiles
   S->qk_bn = (nproj * HD) % 256 == 0 ? 256 : 128;
@@ -221,12 +218,12 @@ int sh_tc_prepare(sh_layer* L) {
   // (the CUDA-core stages of the debug library read 128-row tiles; with a shared selection its output
   //  projection reads the source side's table)
   const bool simt_tiles = (S->simt_mask & SH_STAGE_V) || (L->d.sides == 1 && (S->simt_mask & SH_STAGE_O));
-  L->d.tile_rows_src = (L->dense || simt_tiles || !big) ? 128 : 256;
+  L->d.tile_rows_src = (L->dense || simt_tiles || !big || d.D > 128) ? 128 : 256;
   int rc;
   if ((rc = sh_tc_encode_2d(&S->map_wqk, 0, ws + L->o.wqk, d.M, (uint64_t)nproj * HD, (uint64_t)d.M * 2, 64, S->qk_bn))) return rc;
   if ((rc = sh_tc_encode_2d(&S->map_wqk128, 0, ws + L->o.wqk, d.M, (uint64_t)nproj * HD, (uint64_t)d.M * 2, 64, 128))) return rc;
   if (!L->dense) {
-    if ((rc = sh_tc_encode_2d(&S->map_wv, 0, ws + L->o.wv, d.M, (uint64_t)d.H * d.E * d.D, (uint64_t)d.M * 2, 64, d.D))) return rc;
+    if ((rc = sh_tc_encode_2d(&S->map_wv, 0, ws + L->o.wv, d.M, (uint64_t)d.H * d.E * d.D, (uint64_t)d.M * 2, 64, d.D > 128 ? (d.Dt + 15) / 16 * 16 : d.D))) return rc;
     if (L->moe_q && (rc = sh_tc_encode_2d(&S->map_wq_e, 0, ws + L->o.wq_e, d.M, (uint64_t)d.H * d.E * d.D, (uint64_t)d.M * 2, 64, d.D))) return rc;
     if (L->moe_k && (rc = sh_tc_encode_2d(&S->map_wk_e, 0, ws + L->o.wk_e, d.M, (uint64_t)d.H * d.E * d.D, (uint64_t)d.M * 2, 64, d.D))) return rc;
     if ((rc = sh_tc_encode_2d(&S->map_wo, 1, ws + L->o.wo, d.D, (uint64_t)d.H * d.E * d.M, (uint64_t)d.D * 2, 64, 128))) return rc;
@@ -242,8 +239,9 @@ int sh_tc_prepare(sh_layer* L) {
     if ((rc = sh_tc_encode_2d(&S->map_wgate_half, 0, ws + L->o.wgate, d.M, d.G, (uint64_t)d.M * 2, 64, S->gate_gp / 2))) return rc;
   }
   if ((rc = encode_3d_f16(&S->map_q, ws + L->o.q, d.D, d.T, (uint64_t)d.B * d.H))) return rc;
-  if ((rc = encode_3d_f16(&S->map_k, ws + L->o.k, d.D, d.T, (uint64_t)d.B * d.H))) return rc;
-  if ((rc = encode_3d_f16(&S->map_v, ws + L->o.v, d.D, d.T, (uint64_t)d.B * d.H))) return rc;
+  // (the attention kernel of d_head above 128 takes 64 keys a step)
+  if ((rc = encode_3d_f16(&S->map_k, ws + L->o.k, d.D, d.T, (uint64_t)d.B * d.H, d.D > 128 ? 64 : 128))) return rc;
+  if ((rc = encode_3d_f16(&S->map_v, ws + L->o.v, d.D, d.T, (uint64_t)d.B * d.H, d.D > 128 ? 64 : 128))) return rc;
   if ((rc = encode_3d_f16_store32(&S->map_q_st, ws + L->o.q, d.D, d.T, (uint64_t)d.B * d.H))) return rc;
   if ((rc = encode_3d_f16_store32(&S->map_k_st, ws + L->o.k, d.D, d.T, (uint64_t)d.B * d.H))) return rc;
   if ((rc = sh_tc_encode_2d(&S->map_ahat, 1, ws + L->o.ahat, HD, d.N, (uint64_t)HD * 2, 64, 128))) return rc;
@@ -732,7 +730,10 @@ static int tc_forward_rest(sh_layer* L, const void* x, void* out, cudaStream_t s
       } else {
         // (128-row tiles of a small workload: the persistent kernel too - one prologue per SM instead of one per tile)
         const unsigned pg = grid.x < (unsigned)L->sm_count ? grid.x : (unsigned)L->sm_count;
-        if (d.D == 128) rc = S->persistent ? launch_pgemm<128, 4, PG_V, 1>(map_x, S->map_wv, g, pg, st, pdl) : launch_gemm<128, 4, GEMM_V, 1, 1>(map_x, S->map_wv, g, grid, st, pdl);
+        if (d.D > 128) {
+          g.ncols = (d.Dt + 15) / 16 * 16;
+          rc = launch_pgemm<256, 4, PG_V, 1>(map_x, S->map_wv, g, pg, st, pdl);
+        } else if (d.D == 128) rc = S->persistent ? launch_pgemm<128, 4, PG_V, 1>(map_x, S->map_wv, g, pg, st, pdl) : launch_gemm<128, 4, GEMM_V, 1, 1>(map_x, S->map_wv, g, grid, st, pdl);
         else rc = S->persistent ? launch_pgemm<64, 4, PG_V, 1>(map_x, S->map_wv, g, pg, st, pdl) : launch_gemm<64, 4, GEMM_V, 1, 1>(map_x, S->map_wv, g, grid, st, pdl);
       }
       if (rc) return rc;
@@ -778,7 +779,11 @@ static int tc_forward_rest(sh_layer* L, const void* x, void* out, cudaStream_t s
     // finer hand-overs shorten the few-step chain of a short sequence); beyond: the whole-S kernel
     // (with halves the issuing thread, eight N = 64 UMMAs per half, bounds a long loop)
     const bool halves = d.T <= 1024;
-    if (d.D == 128) {
+    if (d.D > 128) {
+      const unsigned wgrid = (unsigned)((d.T + 127) / 128 * d.B * d.H);
+      if ((rc = set_smem(sh_tc_attention_wide_kernel, AttnWSmem::TOTAL))) return rc;
+      if ((rc = launch_k(pdl, sh_tc_attention_wide_kernel, dim3(wgrid), dim3(192), AttnWSmem::TOTAL, st, S->map_q, S->map_k, S->map_v, a))) return rc;
+    } else if (d.D == 128) {
       auto kern = halves ? sh_tc_attention3_kernel<128> : sh_tc_attention2_kernel<128>;
       const int smem = halves ? Attn3Smem<128>::TOTAL : Attn2Smem<128>::TOTAL;
       if ((rc = set_smem(kern, smem))) return rc;
@@ -793,8 +798,8 @@ static int tc_forward_rest(sh_layer* L, const void* x, void* out, cudaStream_t s
   }
   sh_mark(L, 4, st);
   // ---- output experts ----------------------------------------------------------------------------
-  if (L->out_f16 && ((simt & SH_STAGE_O) || L->dense)) {
-    sh_set_error("fp16 output is written by the tensor-core output-expert kernels only");
+  if (L->out_f16 && ((simt & SH_STAGE_O) || L->dense || d.D > 128)) {
+    sh_set_error("fp16 output is written by the tensor-core output-expert kernels for d_head up to 128 only");
     return SH_ERR_UNSUPPORTED;
   }
   if (simt & SH_STAGE_O) {
@@ -809,7 +814,8 @@ static int tc_forward_rest(sh_layer* L, const void* x, void* out, cudaStream_t s
     // token's selections in registers).  With more, the single-CTA kernel, which reads the selections
     // from shared memory and multiplies by the gate after the UMMA; a device that cannot hold a two-CTA
     // cluster of the pair kernel's size uses it too.
-    bool pair = S->o_pair && d.k <= OPAIR_KMAX;
+    // (and d_head above 128: its gate-scaled operand would be one more fp16 rounding than such a layer has had)
+    bool pair = S->o_pair && d.k <= OPAIR_KMAX && d.D <= 128;
     const bool sparse = pair && S->o_sparse && sh_o_sparse_ok(L);
     if (sparse) {
       constexpr int psm = OprojSpSmem<128>::TOTAL;
@@ -851,20 +857,26 @@ static int tc_forward_rest(sh_layer* L, const void* x, void* out, cudaStream_t s
     } else {
       a.nwork = ((sh_out_rows(d) + 127) / 128) * ((d.M + 255) / 256);
       const unsigned grid = (unsigned)(a.nwork < L->sm_count ? a.nwork : L->sm_count);
-      int as = 3, smem = 0;
-      for (; as >= 2; --as) {
-        smem = d.D == 128 ? OprojSmem<128>::total(as, d.H, d.k) : OprojSmem<64>::total(as, d.H, d.k);
-        if (smem <= 227 * 1024) break;
-      }
-      if (as < 2) { sh_set_error("output projection: n_heads*k = %d does not fit in shared memory", d.H * d.k); return SH_ERR_UNSUPPORTED; }
-      a.a_slots = as;
-      if (d.D == 128) {
-        if ((rc = set_smem(sh_tc_oproj_kernel<128>, smem))) return rc;
-        if ((rc = launch_k(pdl, sh_tc_oproj_kernel<128>, dim3(grid), dim3(320), smem, st, S->map_ahat, S->map_wo256, a))) return rc;
-      } else {
-        if ((rc = set_smem(sh_tc_oproj_kernel<64>, smem))) return rc;
-        if ((rc = launch_k(pdl, sh_tc_oproj_kernel<64>, dim3(grid), dim3(320), smem, st, S->map_ahat, S->map_wo256, a))) return rc;
-      }
+      auto go = [&](auto kern, int (*total)(int, int, int)) -> int {
+        int as = 3, smem = 0;
+        for (; as >= 2; --as) {
+          smem = total(as, d.H, d.k);
+          if (smem <= 227 * 1024) break;
+        }
+        if (as < 2 && d.D > 128) {                           // (such layers take any n_heads * k)
+          a.sel_global = 1;
+          as = 2; smem = total(2, d.H, 0);
+        }
+        if (as < 2) { sh_set_error("output projection: n_heads*k = %d does not fit in shared memory", d.H * d.k); return SH_ERR_UNSUPPORTED; }
+        a.a_slots = as;
+        if (int r = set_smem(kern, smem)) return r;
+        return launch_k(pdl, kern, dim3(grid), dim3(320), smem, st, S->map_ahat, S->map_wo256, a);
+      };
+      if (d.D == 64) rc = go(sh_tc_oproj_kernel<1, 2>, OprojSmem<1, 2>::total);
+      else if (d.D == 128) rc = go(sh_tc_oproj_kernel<2, 2>, OprojSmem<2, 2>::total);
+      else if (d.Dt <= 192) rc = go(sh_tc_oproj_kernel<3, 2>, OprojSmem<3, 2>::total);
+      else rc = go(sh_tc_oproj_kernel<4, 1>, OprojSmem<4, 1>::total);
+      if (rc) return rc;
     }
     L->launches += 1;
   } else {

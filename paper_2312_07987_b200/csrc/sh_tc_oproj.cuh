@@ -22,7 +22,7 @@
 // Warp roles (320 threads): warp 0 = TMA producer, warp 1 = TMEM owner + UMMA issuer (a second
 // issuing thread for the odd experts was tried: no gain), warps 2..9 = epilogue (thread = one token = TMEM lane, and one half of the 256 features;
 // two warps share a lane quarter).  One expert = one 256-column TMEM buffer (ring of 2); its
-// weights arrive as D/64 stages of 256 features x 64 columns (32 KB, one TMA box each) through
+// weights arrive as DB stages of 256 features x 64 columns (32 KB, one TMA box each) through
 // a ring of 3 (or 2) stages that are released one by one: L2 answers a TMA load after ~0.9 us,
 // so the bytes in flight set the fill rate and a stage handed back early is loading again.
 // All rings run on across work units, so the producer and the issuer work ahead into the
@@ -39,6 +39,7 @@ struct TcOprojArgs {
   float* out;            // [N, M] fp32, or (out_f16) [N, M] fp16 at the same address
   int out_f16;           // 1: the result rows are rounded to fp16 once, on their way out
   int a_slots;           // 32 KB weight stages in the ring: 3 or 2
+  int sel_global;        // single-CTA kernel: selections read from global memory (their copy does not fit shared memory)
   int nwork;             // nblk * ceil(M / 256)
   int* status;
 };
@@ -54,31 +55,32 @@ __device__ __forceinline__ void oproj_put4(float* out, size_t elem, float4 v, in
   }
 }
 
-template <int D>
+// DB: 64-column blocks of d_head; NB: token tiles in the ring (one where two of 256 columns do not fit).
+template <int DB, int NB>
 struct OprojSmem {
   static constexpr int A_BYTES = 256 * 64 * 2;           // one weight stage: 256 features x 64 columns
-  static constexpr int B_BYTES = 128 * D * 2;            // Ahat tile: 128 tokens x D
+  static constexpr int B_BYTES = 128 * DB * 64 * 2;      // Ahat tile: 128 tokens x 64 DB
   static constexpr int STAGING = 8 * 32 * 32 * 4;        // per epilogue warp a 32 x 32 fp32 transpose tile
   static int total(int a_slots, int H, int k) {
-    return a_slots * A_BYTES + 2 * B_BYTES + STAGING + 128 * H * k * 8 + 512 + 1024;
+    return a_slots * A_BYTES + NB * B_BYTES + STAGING + 128 * H * k * 8 + 512 + 1024;
   }
 };
 
-template <int D>
+template <int DB, int NB>
 __global__ void __launch_bounds__(320, 1)
 sh_tc_oproj_kernel(const __grid_constant__ CUtensorMap mapAhat, const __grid_constant__ CUtensorMap mapWo, TcOprojArgs g) {
-  using SM = OprojSmem<D>;
-  constexpr int DB = D / 64;
+  using SM = OprojSmem<DB, NB>;
   constexpr uint32_t TBLK = 128 * 128;                   // one 64-column block of the token tile
   extern __shared__ unsigned char smem_raw[];
   const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
   unsigned char* sgen = smem_raw + (sbase - smem_u32(smem_raw));
   const ShDims& d = g.d;
   const int AS = g.a_slots;                              // 3 or 2
-  const uint32_t a_off = 0, b_off = AS * SM::A_BYTES, stg_off = b_off + 2 * SM::B_BYTES, misc_off = stg_off + SM::STAGING;
+  const uint32_t a_off = 0, b_off = AS * SM::A_BYTES, stg_off = b_off + NB * SM::B_BYTES, misc_off = stg_off + SM::STAGING;
+  const int sel_n = g.sel_global ? 0 : 128 * d.H * d.k;
   int* s_idx = (int*)(sgen + misc_off);                       // [128, H, k] selections of the current tokens
-  float* s_gt = (float*)(s_idx + 128 * d.H * d.k);            // [128, H, k]
-  uint64_t* bars = (uint64_t*)(((uintptr_t)(s_gt + 128 * d.H * d.k) + 15) & ~(uintptr_t)15);
+  float* s_gt = (float*)(s_idx + sel_n);                      // [128, H, k]
+  uint64_t* bars = (uint64_t*)(((uintptr_t)(s_gt + sel_n) + 15) & ~(uintptr_t)15);
   uint64_t* a_full = bars;               // [4]
   uint64_t* a_empty = bars + 4;          // [4]
   uint64_t* b_full = bars + 8;           // [2]
@@ -122,12 +124,12 @@ sh_tc_oproj_kernel(const __grid_constant__ CUtensorMap mapAhat, const __grid_con
         //  chunk length is a multiple of 128, so a tile never straddles two sequences)
         const int row0 = sh_ctx_tok(d, (w / nfc) * 128), fc = w % nfc;
         for (int h = 0; h < d.H && !dead; ++h, ++gh) {
-          const int bs = gh & 1;
-          if (!mbar_wait(&b_empty[bs], ((gh >> 1) & 1) ^ 1, g.status, dead)) break;
+          const int bs = NB == 2 ? gh & 1 : 0;
+          if (!mbar_wait(&b_empty[bs], ((gh / NB) & 1) ^ 1, g.status, dead)) break;
           mbar_expect_tx(&b_full[bs], SM::B_BYTES);
 #pragma unroll
           for (int c = 0; c < DB; ++c)
-            tma_load_2d(sbase + b_off + bs * SM::B_BYTES + c * TBLK, &mapAhat, &b_full[bs], h * D + c * 64, row0);
+            tma_load_2d(sbase + b_off + bs * SM::B_BYTES + c * TBLK, &mapAhat, &b_full[bs], h * d.D + c * 64, row0);
           for (int e = 0; e < d.E && !dead; ++e) {
             // 256 feature rows of expert (h, e), one 64-column stage at a time; a box that runs past
             // the expert's rows (M not a multiple of 256) fetches rows whose columns are never stored
@@ -145,12 +147,13 @@ sh_tc_oproj_kernel(const __grid_constant__ CUtensorMap mapAhat, const __grid_con
     if (lane == 0) {
       constexpr uint32_t idesc = make_idesc_f16(128, 256, 0, 0, 0);
       const uint32_t w_lo0 = desc_lo_k(sbase + a_off), t_lo0 = desc_lo_k(sbase + b_off);
+      const int last_k = (d.Dt - 64 * (DB - 1) + 15) / 16;  // 16-column slices of the last block that d_head reaches
       int gh = 0, ge = 0, s = 0;
       uint32_t apar = 0;                                    // parity of a_full[s] for the current ring pass
       for (int w = blockIdx.x; w < g.nwork && !dead; w += gridDim.x) {
         for (int h = 0; h < d.H && !dead; ++h, ++gh) {
-          const int bs = gh & 1;
-          if (!mbar_wait(&b_full[bs], (gh >> 1) & 1, g.status, dead)) break;
+          const int bs = NB == 2 ? gh & 1 : 0;
+          if (!mbar_wait(&b_full[bs], (gh / NB) & 1, g.status, dead)) break;
           const uint32_t t_lo = t_lo0 + bs * (SM::B_BYTES >> 4);
           for (int e = 0; e < d.E && !dead; ++e, ++ge) {
             const int buf = ge & 1;
@@ -159,9 +162,10 @@ sh_tc_oproj_kernel(const __grid_constant__ CUtensorMap mapAhat, const __grid_con
               if (!mbar_wait(&a_full[s], apar, g.status, dead)) break;
               tc_fence_after();
               const uint32_t w_lo = w_lo0 + s * (SM::A_BYTES >> 4), tc_lo = t_lo + c * (TBLK >> 4);
+              const int kn = c == DB - 1 ? last_k : 4;
 #pragma unroll
               for (int k = 0; k < 4; ++k)
-                umma_f16(tmem + buf * 256, desc_pack(tc_lo + 2 * k), desc_pack(w_lo + 2 * k), idesc, (c | k) != 0);
+                if (k < kn) umma_f16(tmem + buf * 256, desc_pack(tc_lo + 2 * k), desc_pack(w_lo + 2 * k), idesc, (c | k) != 0);
               umma_commit(&a_empty[s]);                     // this stage can load its next box
               if (++s == AS) { s = 0; apar ^= 1; }
             }
@@ -196,23 +200,26 @@ sh_tc_oproj_kernel(const __grid_constant__ CUtensorMap mapAhat, const __grid_con
         const int total = nrows * per_tok;
         const int* gi_ = g.idx + (size_t)tok0 * per_tok;
         const float* gg = g.gate + (size_t)tok0 * per_tok;
-        for (int i = et; i < 128 * per_tok; i += 256) {
+        for (int i = et; i < sel_n; i += 256) {
           s_idx[i] = i < total ? gi_[i] : -1;
           s_gt[i] = i < total ? gg[i] : 0.f;
         }
       }
       mbar_arrive(sel_ready);
       if (!mbar_wait(sel_ready, wpar, g.status, dead)) { ok = false; break; }
+      const size_t own = g.sel_global ? (size_t)(tok0 + min(tok, nrows - 1)) * per_tok : (size_t)tok * per_tok;
+      const int* p_idx = (g.sel_global ? g.idx : s_idx) + own;
+      const float* p_gt = (g.sel_global ? g.gate : s_gt) + own;
       float2 acc2[64];                                     // packed fp32 pairs: one FFMA2 per two features
 #pragma unroll
       for (int f = 0; f < 64; ++f) acc2[f] = make_float2(0.f, 0.f);
       for (int h = 0; h < d.H && ok; ++h) {
-        const int sel = (tok * d.H + h) * d.k;               // this token's selections for head h
+        const int sel = h * d.k;                             // this token's selections for head h
         for (int e = 0; e < d.E; ++e, ++ge) {
           const int buf = ge & 1;
           float gv = 0.f;                                    // gate of expert e for this token (0: not selected)
           for (int j = 0; j < d.k; ++j)
-            if (s_idx[sel + j] == e) gv = s_gt[sel + j];
+            if (p_idx[sel + j] == e) gv = p_gt[sel + j];
           if (!mbar_wait(&d_full[buf], (ge >> 1) & 1, g.status, dead)) { ok = false; break; }
           tc_fence_after();
           const uint32_t ta = tmem + lane_off + buf * 256 + half * 128;

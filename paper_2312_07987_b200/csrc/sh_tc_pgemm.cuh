@@ -13,6 +13,7 @@
 // Warp roles (320 threads): warp 0 = TMA producer, warp 1 = TMEM owner + UMMA issuer,
 // warps 2..5 = epilogue (thread = accumulator row = TMEM lane), warps 6..9 = A-row gatherers
 // (PG_V); in PG_QKV warp 6 is a second TMA producer and warps 7..9 idle.
+// BN = 256 in PG_V: d_head above 128; the tile computes the g.ncols (a multiple of 16) columns there are.
 // Tile = (MT * 128) rows x BN columns, MT * BN <= 256 so that two accumulators fit TMEM.
 #pragma once
 #include "sh_tc_gemm.cuh"
@@ -140,7 +141,7 @@ sh_tc_pgemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_consta
               tma_load_2d(sa + mt * (128 * 64 * 2), &mapA, &full_bar[s], kb * 64, row0 + mt * 128);
           }
           if (do_b) {
-            mbar_expect_tx(&full_bar[s], SM::B_BYTES);
+            mbar_expect_tx(&full_bar[s], GATHER && BN == 256 ? g.ncols * 128 : SM::B_BYTES);
             tma_load_2d(sb, &mapB, &full_bar[s], kb * 64, brow);
           }
           if (++s == STAGES) { s = 0; par ^= 1; }
@@ -152,7 +153,7 @@ sh_tc_pgemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_consta
     // issuing one costs a thread about as long: each half has its own issuing thread (warp 1 / 10),
     // its own accumulator columns and its own commits.
     if (lane == 0) {
-      constexpr uint32_t idesc = make_idesc_f16(128, BN, 1, 1, 0);
+      const uint32_t idesc = make_idesc_f16(128, GATHER && BN == 256 ? g.ncols : BN, 1, 1, 0);
       const int mt = warp == 1 ? 0 : 1;
       const uint32_t a_lo0 = desc_lo_k(sbase) + mt * (128 * 64 * 2 >> 4), b_lo0 = desc_lo_k(sbase + SM::A_BYTES);
       int s = 0, it = 0;
@@ -312,11 +313,12 @@ sh_tc_pgemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_consta
                 float* d32 = g.v_early + (((size_t)bb * d.H + th) * SH_EARLY_ROWS + tt) * d.D + n0;
 #pragma unroll
                 for (int i = 0; i < 8; ++i)
-                  red_add_v4_f32(d32 + 4 * i, __uint_as_float(v[4 * i]) * gt, __uint_as_float(v[4 * i + 1]) * gt,
+                  if (BN != 256 || n0 + 4 * i < g.ncols) red_add_v4_f32(d32 + 4 * i, __uint_as_float(v[4 * i]) * gt, __uint_as_float(v[4 * i + 1]) * gt,
                                  __uint_as_float(v[4 * i + 2]) * gt, __uint_as_float(v[4 * i + 3]) * gt);
               } else {
 #pragma unroll
-                for (int i = 0; i < 4; ++i) red_add_v4_f16x2(dst + 8 * i, p[4 * i], p[4 * i + 1], p[4 * i + 2], p[4 * i + 3]);
+                for (int i = 0; i < 4; ++i)
+                  if (BN != 256 || n0 + 8 * i < g.ncols) red_add_v4_f16x2(dst + 8 * i, p[4 * i], p[4 * i + 1], p[4 * i + 2], p[4 * i + 3]);
               }
             }
           }
