@@ -21,12 +21,15 @@ void sh_set_error(const char* fmt, ...) {
 
 static size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
+// (the fp32 SwitchHead layer keeps its weights split into three bf16 planes)
+static size_t elem_bytes_weight(const sh_layer* L, size_t plain) { return L->dtype == SH_F32 && !L->dense ? 6 : plain; }
 static size_t elem_bytes_in(int dtype) { return dtype == SH_F32 ? 4 : 2; }
 static size_t elem_bytes_mid(int dtype) { return dtype == SH_F32 ? 4 : 2; }
 
 static void layout_workspace(sh_layer* L) {
   const ShDims& d = L->d;
   const size_t in = elem_bytes_in(L->dtype), mid = elem_bytes_mid(L->dtype);
+  const size_t win = elem_bytes_weight(L, in), wmid = elem_bytes_weight(L, mid);
   size_t off = 0;
   // every sub-buffer is followed by a guard of SH_GUARD_BYTES that sh_set_weights fills with a
   // pattern and sh_check_guards verifies: a kernel that writes past the end of its buffer shows there
@@ -42,11 +45,11 @@ static void layout_workspace(sh_layer* L) {
   const size_t HD = (size_t)d.H * d.D;
   const size_t nproj = L->dense ? 3 : 2;
   o.status = take(256);
-  o.wqk = take(nproj * HD * d.M * in);
-  o.wgate = take((size_t)d.G * d.M * in);
+  o.wqk = take(nproj * HD * d.M * win);
+  o.wgate = take((size_t)d.G * d.M * win);
   o.gbias = take((size_t)d.G * 4);
-  o.wv = take(L->dense ? 16 : HD * d.E * d.M * in);
-  o.wo = take(HD * d.E * d.M * mid);
+  o.wv = take(L->dense ? 16 : HD * d.E * d.M * win);
+  o.wo = take(HD * d.E * d.M * wmid);
   o.q = take((size_t)d.N * HD * mid);
   o.k = take((size_t)d.N * HD * mid);
   o.v = take((size_t)d.N * HD * mid);
@@ -88,14 +91,14 @@ static void layout_workspace(sh_layer* L) {
   o.wos = take(sh_o_sparse_ok(L) ? HD * d.E * d.M * mid : 16);
   o.gid = take(vp ? (size_t)2 * d.N * d.H * 4 : 16);  // (both sides: query experts are tiled by the destination side's pairs)
   // query / key experts (sh_create_moe_qk): [H, E, D, M] like the value experts
-  o.wq_e = take(L->moe_q ? HD * d.E * d.M * in : 16);
-  o.wk_e = take(L->moe_k ? HD * d.E * d.M * in : 16);      // pair number of every (token, head), source side
+  o.wq_e = take(L->moe_q ? HD * d.E * d.M * win : 16);
+  o.wk_e = take(L->moe_k ? HD * d.E * d.M * win : 16);      // pair number of every (token, head), source side
   // fp32 configuration: scratch of the backward pass (dQ, dK, dV, dAhat [N, H, D] and the gate gradients [2, N, H, k]
-  //  in list order, the gate gradients once more as a matrix [N, G], rowsum(dAhat o Ahat) [N, H]); the gate logits
-  //  [N, G]; per attention row the score maximum and 1 / normaliser)
+  //  in list order, the gate gradients once more as a matrix [N, G], rowsum(dAhat o Ahat) [N, H]); the gate weights
+  //  once more in fp32; per attention row the score maximum and 1 / normaliser)
   const bool f32 = L->dtype == SH_F32 && !L->dense;
   o.bw = take(f32 ? ((size_t)4 * d.N * HD + (size_t)2 * d.N * d.H * d.k + (size_t)d.N * (sh_f32_ldz(d) + d.H)) * 4 : 16);
-  o.f32z = take(f32 ? (size_t)d.N * sh_f32_ldz(d) * 4 : 16);
+  o.wgate32 = take(f32 ? (size_t)d.G * d.M * 4 : 16);
   o.f32stats = take(f32 ? (size_t)d.N * d.H * 8 : 16);
   o.stamps = take(sizeof(ShStampBlock));
   o.total = off;
@@ -198,6 +201,7 @@ static int configure_common(sh_layer* L, int dtype, int batch, int seq, int cach
   L->d.status = nullptr;
   L->weights_set = false;
   sh_tc_release(L);
+  sh_f32_release(L);
   layout_workspace(L);
   return SH_OK;
 }
@@ -223,6 +227,7 @@ extern "C" int sh_set_workspace(sh_layer* L, void* workspace, size_t bytes) {
   L->ws = (char*)workspace; L->ws_bytes = bytes; L->weights_set = false; L->rope = false; L->xl_positions = false;
   L->d.status = (int*)(L->ws + L->o.status);
   sh_tc_release(L);
+  sh_f32_release(L);
   return SH_OK;
 }
 
@@ -297,6 +302,54 @@ static int set_weights_t(sh_layer* L, const void* Wq, const void* Wk, const void
   return SH_OK;
 }
 
+// The fp32 SwitchHead layer: the same layouts, each weight as three bf16 planes [3, rows, inner].
+static int set_weights_f32(sh_layer* L, const float* Wq, const float* Wk, const float* Wv, const float* Wo,
+                           const float* Ws, const float* Wd, const float* bias_s, const float* bias_d, cudaStream_t st) {
+  const ShDims& d = L->d;
+  char* ws = L->ws;
+  const long HD = (long)d.H * d.D, nqk = 2 * HD * d.M, nexp = HD * d.E * d.M, ngate = (long)d.G * d.M;
+  SH_CUDA_CHECK(cudaMemsetAsync(ws + L->o.status, 0, 256, st));
+  for (int i = 0; i < L->n_guards; ++i) SH_CUDA_CHECK(cudaMemsetAsync(ws + L->guard_off[i], SH_GUARD_BYTE, SH_GUARD_BYTES, st));
+  if (d.D != d.Dt) {
+    SH_CUDA_CHECK(cudaMemsetAsync(ws + L->o.wqk, 0, (size_t)nqk * 6, st));
+    SH_CUDA_CHECK(cudaMemsetAsync(ws + L->o.wv, 0, (size_t)nexp * 6, st));
+    SH_CUDA_CHECK(cudaMemsetAsync(ws + L->o.wo, 0, (size_t)nexp * 6, st));
+    if (L->moe_q) SH_CUDA_CHECK(cudaMemsetAsync(ws + L->o.wq_e, 0, (size_t)nexp * 6, st));
+    if (L->moe_k) SH_CUDA_CHECK(cudaMemsetAsync(ws + L->o.wk_e, 0, (size_t)nexp * 6, st));
+    // (the projections write d_head's columns only: the padding of Q and K is cleared here, once)
+    SH_CUDA_CHECK(cudaMemsetAsync(ws + L->o.q, 0, (size_t)d.N * HD * 4, st));
+    SH_CUDA_CHECK(cudaMemsetAsync(ws + L->o.k, 0, (size_t)d.N * HD * 4, st));
+  }
+  auto split = [&](const float* in, size_t off, long first, int batch, int rows, int cols, long obs, long ors, long oes, long plane) {
+    const long total = (long)batch * rows * cols;
+    long blocks = (total + 255) / 256;
+    blocks = blocks > 65535 * 4 ? 65535 * 4 : blocks;
+    sh_repack_split_kernel<<<(unsigned)blocks, 256, 0, st>>>(in, (__nv_bfloat16*)(ws + off) + first, batch, rows, cols, obs, ors, oes, plane);
+  };
+  const long DM = (long)d.D * d.M;
+  if (L->moe_q) split(Wq, L->o.wq_e, 0, d.H * d.E, d.M, d.Dt, DM, d.M, 1, nexp);
+  else split(Wq, L->o.wqk, 0, d.H, d.M, d.Dt, DM, d.M, 1, nqk);
+  if (L->moe_k) split(Wk, L->o.wk_e, 0, d.H * d.E, d.M, d.Dt, DM, d.M, 1, nexp);
+  else split(Wk, L->o.wqk, HD * d.M, d.H, d.M, d.Dt, DM, d.M, 1, nqk);
+  split(Ws, L->o.wgate, 0, d.H, d.M, d.E, (long)d.E * d.M, d.M, 1, ngate);
+  if (d.sides == 2) split(Wd, L->o.wgate, (long)d.H * d.E * d.M, d.H, d.M, d.E, (long)d.E * d.M, d.M, 1, ngate);
+  // (the logits' kernel reads the gate weights as fp32)
+  float* wg32 = (float*)(ws + L->o.wgate32);
+  repack<float, float>(Ws, wg32, d.H, d.M, d.E, (long)d.E * d.M, d.M, 1, st);
+  if (d.sides == 2) repack<float, float>(Wd, wg32 + (long)d.H * d.E * d.M, d.H, d.M, d.E, (long)d.E * d.M, d.M, 1, st);
+  split(Wv, L->o.wv, 0, d.H * d.E, d.M, d.Dt, DM, d.M, 1, nexp);
+  split(Wo, L->o.wo, 0, d.H * d.E, d.Dt, d.M, DM, d.D, 1, nexp);
+  float* gb = (float*)(ws + L->o.gbias);
+  const size_t hb = (size_t)d.H * d.E * 4;
+  for (int side = 0; side < d.sides; ++side) {
+    const float* bias = side ? bias_d : bias_s;
+    if (bias) SH_CUDA_CHECK(cudaMemcpyAsync((char*)gb + side * hb, bias, hb, cudaMemcpyDeviceToDevice, st));
+    else SH_CUDA_CHECK(cudaMemsetAsync((char*)gb + side * hb, 0, hb, st));
+  }
+  SH_CUDA_CHECK(cudaGetLastError());
+  return sh_f32_prepare(L);
+}
+
 extern "C" int sh_set_weights(sh_layer* L, const void* Wq, const void* Wk, const void* Wv, const void* Wo,
                               const void* Ws, const void* Wd, const float* bias_s, const float* bias_d,
                               void* stream) {
@@ -309,7 +362,9 @@ extern "C" int sh_set_weights(sh_layer* L, const void* Wq, const void* Wk, const
   if (!L->dense && L->d.sides == 1 && (Wd || bias_d)) { sh_set_error("a shared-selection layer has one gate: pass NULL for Wd and bias_d"); return SH_ERR_INVALID_ARG; }
   if (L->dense && (Ws || Wd || bias_s || bias_d)) { sh_set_error("a dense layer has no gates: pass NULL for Ws, Wd and the biases"); return SH_ERR_INVALID_ARG; }
   cudaStream_t st = (cudaStream_t)stream;
-  int rc = (L->dtype == SH_F32)
+  int rc = L->dtype == SH_F32 && !L->dense
+               ? set_weights_f32(L, (const float*)Wq, (const float*)Wk, (const float*)Wv, (const float*)Wo, (const float*)Ws, (const float*)Wd, bias_s, bias_d, st)
+           : L->dtype == SH_F32
                ? set_weights_t<float, float>(L, Wq, Wk, Wv, Wo, Ws, Wd, bias_s, bias_d, st)
                : set_weights_t<__nv_bfloat16, __half>(L, Wq, Wk, Wv, Wo, Ws, Wd, bias_s, bias_d, st);
   if (rc != SH_OK) return rc;
@@ -765,5 +820,6 @@ extern "C" const char* sh_last_error(void) { return g_err; }
 extern "C" void sh_destroy(sh_layer* L) {
   if (!L) return;
   sh_tc_release(L);
+  sh_f32_release(L);
   delete L;
 }

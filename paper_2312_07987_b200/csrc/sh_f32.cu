@@ -7,9 +7,17 @@
 #include "sh_f32_attn.cuh"
 #include "sh_f32_select.cuh"
 
+#include <new>
+
 using namespace shtc;
 
 namespace {
+
+// The split weights as [3 planes, rows, inner]: boxes of 64 rows x 32 positions where a row runs along the
+// contraction (k), of 32 rows x 64 columns where the contraction runs over rows (mn).
+struct PlaneMap { CUtensorMap k, mn; };
+struct F32State { PlaneMap wqk, wgate, wv, wo, wq_e, wk_e; };
+
 
 int sm_count(sh_layer* L) {
   if (L->sm_count == 0) {
@@ -23,30 +31,31 @@ int sm_count(sh_layer* L) {
 // Row tiles of one head in a side's tile table (sh_f32_select_kernel).
 int head_tiles(const ShDims& d) { return (int)(((long long)d.N * d.k + 127ll * d.E) / 128); }
 
-// 64- or 128-column tiles.  A 128-column tile costs about 1.6 times a 64-column one (the row operand is
-// split once either way), so the narrow tile is taken where the wide ones would leave SMs idle.
-bool wide_tile(sh_layer* L, long rows, int cols, int per_head_cols) {
-  const long n128 = rows * cols * ((per_head_cols + 127) / 128), n64 = rows * cols * ((per_head_cols + 63) / 64);
-  const long sms = sm_count(L);
-  const long w128 = (n128 + sms - 1) / sms, w64 = (n64 + sms - 1) / sms;
-  return 8 * w128 <= 5 * w64;
+// One mode's tiles as a part of a launch.
+template <int MODE>
+XPart part(sh_layer* L, const XGemmArgs& g, int gx, int gy, int gz = 1, const PlaneMap* w = nullptr) {
+  const F32State* S = (const F32State*)L->f32;
+  constexpr bool K_MAJOR = MODE == X_QK || MODE == X_V || MODE == X_O;
+  if (!w) w = MODE == X_O || MODE == X_DA ? &S->wo : MODE == X_V || MODE == X_DR ? &S->wv : &S->wqk;
+  XPart p;
+  p.w = K_MAJOR ? w->k : w->mn; p.g = g; p.gx = gx; p.gy = gy; p.n = gx * gy * gz;
+  return p;
 }
 
-template <int MODE>
-int launch_x(XGemmArgs& g, bool wide, dim3 grid, cudaStream_t st) {
-  if (grid.x == 0 || grid.y == 0 || grid.z == 0) return SH_OK;
-  if (wide) {
-    if (int rc = set_smem(sh_f32_gemm_kernel<128, MODE>, XGemmSmem<128>::TOTAL)) return rc;
-    return launch_k(true, sh_f32_gemm_kernel<128, MODE>, grid, dim3(XG_THREADS), XGemmSmem<128>::TOTAL, st, g);
-  }
-  if (int rc = set_smem(sh_f32_gemm_kernel<64, MODE>, XGemmSmem<64>::TOTAL)) return rc;
-  return launch_k(true, sh_f32_gemm_kernel<64, MODE>, grid, dim3(XG_THREADS), XGemmSmem<64>::TOTAL, st, g);
+template <int A, int B = -1, int C = -1>
+int launch_x(sh_layer* L, cudaStream_t st, const XPart& a, const XPart& b = XPart(), const XPart& c = XPart()) {
+  const F32State* S = (const F32State*)L->f32;
+  const int n = a.n + (B >= 0 ? b.n : 0) + (C >= 0 ? c.n : 0);
+  if (n == 0) return SH_OK;
+  auto kern = sh_f32_gemm_kernel<A, B, C>;
+  if (int rc = set_smem(kern, XGemmSmem::TOTAL)) return rc;
+  L->launches += 1;
+  return launch_k(true, kern, dim3((unsigned)n), dim3(XG_THREADS), XGemmSmem::TOTAL, st, S->wgate.mn, a, b, c);
 }
 
 // Column tiles over `cols` columns: how many, and how wide (a multiple of 16).
-void col_tiles(XGemmArgs& g, int cols, bool wide) {
-  const int bn = wide ? 128 : 64;
-  g.nsub = (cols + bn - 1) / bn;
+void col_tiles(XGemmArgs& g, int cols) {
+  g.nsub = (cols + XG_BN - 1) / XG_BN;
   g.sub_cols = ((cols + g.nsub - 1) / g.nsub + 15) / 16 * 16;
 }
 
@@ -57,11 +66,9 @@ XGemmArgs base_args(sh_layer* L, const void* x) {
   g.d = d;
   g.x = (const float*)x;
   g.ahat = (const float*)(ws + L->o.ahat);
-  g.wqk = (const float*)(ws + L->o.wqk); g.wgate = (const float*)(ws + L->o.wgate);
-  g.wv = (const float*)(ws + L->o.wv); g.wo = (const float*)(ws + L->o.wo);
   g.ldz = sh_f32_ldz(d);
   g.ksplit = 1;
-  g.q = (float*)(ws + L->o.q); g.k = (float*)(ws + L->o.k); g.v = (float*)(ws + L->o.v); g.z = (float*)(ws + L->o.f32z);
+  g.q = (float*)(ws + L->o.q); g.k = (float*)(ws + L->o.k); g.v = (float*)(ws + L->o.v);
   g.qscale = 1.4426950408889634f / sqrtf((float)d.Dt);
   g.rope = L->rope ? (const float2*)(ws + L->o.rope) : nullptr;
   g.vec_dy = g.vec_out = 1;
@@ -81,38 +88,40 @@ void use_side(XGemmArgs& g, sh_layer* L, int side) {
   g.tiles = (const ShTile*)(ws + L->o.tiles) + (size_t)side * d.max_tiles;
 }
 
-// x [Wq | Wk | Wgate]: `groups` heads' column groups from `first` on, and the gate columns if asked.
-int launch_qk(sh_layer* L, const void* x, int first, int groups, bool gates, float* zero0, long n0, float* zero1, long n1, cudaStream_t st) {
-  const ShDims& d = L->d;
-  XGemmArgs g = base_args(L, x);
-  g.qk_first = first; g.qk_groups = groups;
-  const bool wide = groups > 0 && wide_tile(L, d.nblk, groups, d.Dt);
-  col_tiles(g, d.Dt, wide);
-  g.zero0 = zero0; g.nzero0 = n0 / 4; g.zero1 = zero1; g.nzero1 = n1 / 4;
-  const int gt = gates ? (d.G + (wide ? 127 : 63)) / (wide ? 128 : 64) : 0;
-  L->launches += 1;
-  return launch_x<X_QK>(g, wide, dim3(d.nblk, groups * g.nsub + gt), st);
-}
-
-int launch_select(sh_layer* L, cudaStream_t st) {
+// Gates, selection and sort; beside them the buffers that later kernels add into are cleared.
+int launch_gate_sort(sh_layer* L, const void* x, float* zero0, long n0, float* zero1, long n1, cudaStream_t st) {
   const ShDims& d = L->d;
   char* ws = L->ws;
-  L->launches += 1;
-  return launch_k(true, sh_f32_select_kernel, dim3(d.sides * d.H), dim3(1024), 0, st, (const float*)(ws + L->o.f32z), sh_f32_ldz(d),
-                  (const float*)(ws + L->o.gbias), (int*)(ws + L->o.idx), (float*)(ws + L->o.gate), (int*)(ws + L->o.offsets),
-                  (int*)(ws + L->o.lists), (float*)(ws + L->o.lgate), (ShTile*)(ws + L->o.tiles), d, head_tiles(d));
+  // eight tokens a block while sixteen would leave SMs with less than two blocks (or their logits do not fit)
+  const bool small = d.N < 32 * sm_count(L) || 16 * (512 + d.G) * 4 > 200 * 1024;
+  const int tok = small ? 8 : 16;
+  const size_t smem = (size_t)tok * (512 + d.G) * 4;
+  auto kern = small ? sh_f32_gate_kernel<8> : sh_f32_gate_kernel<16>;
+  if (int rc = set_smem(kern, (int)smem)) return rc;
+  if (int rc = launch_k(true, kern, dim3((unsigned)((d.N + tok - 1) / tok)), dim3(256), smem, st, (const float*)x, (const float*)(ws + L->o.wgate32),
+                        (const float*)(ws + L->o.gbias), (int*)(ws + L->o.idx), (float*)(ws + L->o.gate), (float4*)zero0, n0 / 4, (float4*)zero1, n1 / 4, d))
+    return rc;
+  L->launches += 2;
+  return launch_k(true, sh_f32_sort_kernel, dim3(d.sides * d.H), dim3(1024), 0, st, (const int*)(ws + L->o.idx), (const float*)(ws + L->o.gate),
+                  (int*)(ws + L->o.offsets), (int*)(ws + L->o.lists), (float*)(ws + L->o.lgate), (ShTile*)(ws + L->o.tiles), d, head_tiles(d));
+}
+
+// x [Wq | Wk]: `groups` heads' column groups from `first` on.
+XPart part_qk(sh_layer* L, const void* x, int first, int groups) {
+  XGemmArgs g = base_args(L, x);
+  g.qk_first = first; g.qk_groups = groups;
+  col_tiles(g, L->d.Dt);
+  return part<X_QK>(L, g, L->d.nblk, groups * g.nsub);
 }
 
 // dst += gate x W^T over a side's expert lists: value experts, and query / key experts where a layer has them.
-int launch_v(sh_layer* L, const void* x, int side, const float* w, float* dst, float scale, cudaStream_t st) {
+XPart part_v(sh_layer* L, const void* x, int side, const PlaneMap& w, float* dst, float scale) {
   const ShDims& d = L->d;
   XGemmArgs g = base_args(L, x);
   use_side(g, L, side);
-  g.wv = w; g.v = dst; g.vscale = scale;
-  const bool wide = wide_tile(L, (long)d.H * head_tiles(d), 1, d.Dt);
-  col_tiles(g, d.Dt, wide);
-  L->launches += 1;
-  return launch_x<X_V>(g, wide, dim3(d.H * head_tiles(d), g.nsub), st);
+  g.v = dst; g.vscale = scale;
+  col_tiles(g, d.Dt);
+  return part<X_V>(L, g, d.H * head_tiles(d), g.nsub, 1, &w);
 }
 
 template <int D>
@@ -165,54 +174,69 @@ int launch_attn_bw_t(sh_layer* L, const BwBuffers& w, cudaStream_t st) {
                   (const float*)(ws + L->o.f32stats), (const float*)w.dsum, w.dq, w.dk, w.dv, d, (int)run);
 }
 
-// Parts of a contraction over tokens: enough blocks for the device, at least four steps each.
+// Parts of a contraction over tokens: enough blocks for the device, at least eight steps each.
 int k_parts(sh_layer* L, long blocks, long steps) {
-  long p = (sm_count(L) + blocks - 1) / blocks;
-  const long most = steps / 4 < 1 ? 1 : steps / 4;
+  long p = (2 * sm_count(L) + blocks - 1) / blocks;
+  const long most = steps / 8 < 1 ? 1 : steps / 8;
   p = p > most ? most : p;
   return p < 1 ? 1 : (int)p;
 }
 
 }  // namespace
 
-int sh_f32_gate_sort(sh_layer* L, const void* x, cudaStream_t st) {
-  if (int rc = launch_qk(L, x, 0, 0, true, nullptr, 0, nullptr, 0, st)) return rc;
-  return launch_select(L, st);
+int sh_f32_prepare(sh_layer* L) {
+  sh_f32_release(L);
+  F32State* S = new (std::nothrow) F32State();
+  if (!S) { sh_set_error("out of host memory"); return SH_ERR_INVALID_ARG; }
+  L->f32 = S;
+  const ShDims& d = L->d;
+  char* ws = L->ws;
+  auto enc = [&](PlaneMap& m, size_t off, uint64_t inner, uint64_t rows) -> int {
+    if (int rc = sh_tc_encode_planes(&m.k, ws + off, inner, rows, XG_BK, XG_BN)) return rc;
+    return sh_tc_encode_planes(&m.mn, ws + off, inner, rows, XG_BN, XG_BK);
+  };
+  const uint64_t HD = (uint64_t)d.H * d.D;
+  int rc;
+  if ((rc = enc(S->wqk, L->o.wqk, d.M, 2 * HD))) return rc;
+  if ((rc = enc(S->wgate, L->o.wgate, d.M, d.G))) return rc;
+  if ((rc = enc(S->wv, L->o.wv, d.M, HD * d.E))) return rc;
+  if ((rc = enc(S->wo, L->o.wo, d.D, (uint64_t)d.H * d.E * d.M))) return rc;
+  if (L->moe_q && (rc = enc(S->wq_e, L->o.wq_e, d.M, HD * d.E))) return rc;
+  if (L->moe_k && (rc = enc(S->wk_e, L->o.wk_e, d.M, HD * d.E))) return rc;
+  return SH_OK;
 }
+
+void sh_f32_release(sh_layer* L) {
+  if (L && L->f32) { delete (F32State*)L->f32; L->f32 = nullptr; }
+}
+
+int sh_f32_gate_sort(sh_layer* L, const void* x, cudaStream_t st) { return launch_gate_sort(L, x, nullptr, 0, nullptr, 0, st); }
 
 int sh_f32_forward(sh_layer* L, const void* x, void* out, cudaStream_t st) {
   const ShDims& d = L->d;
+  const F32State* S = (const F32State*)L->f32;
   char* ws = L->ws;
   const long nhd = (long)d.N * d.H * d.D, nout = (long)sh_out_rows(d) * d.M;
-  const float qscale = 1.4426950408889634f / sqrtf((float)d.Dt);
   float* v = (float*)(ws + L->o.v);
   int rc;
-  // Dense queries and keys (a layer with query / key experts has none of its own), and the gate logits;
-  // a stage-timed pass computes the logits in a launch of their own so that its boundaries mean something.
+  // Dense queries and keys (a layer with query / key experts has none of its own) and the value experts
+  // need nothing of one another: one launch, in a stage-timed pass two.
   const int first = L->moe_q ? d.H : 0, groups = (L->moe_q ? 0 : d.H) + (L->moe_k ? 0 : d.H);
+  const XPart qk = part_qk(L, x, first, groups), pv = part_v(L, x, 0, S->wv, v, 0.f);
   sh_mark(L, 0, st);
-  if (L->ev) {
-    if ((rc = sh_f32_gate_sort(L, x, st))) return rc;
-    sh_mark(L, 1, st);
-    if (groups) { if ((rc = launch_qk(L, x, first, groups, false, v, nhd, (float*)out, nout, st))) return rc; }
-    else {
-      SH_CUDA_CHECK(cudaMemsetAsync(v, 0, (size_t)nhd * 4, st));
-      SH_CUDA_CHECK(cudaMemsetAsync(out, 0, (size_t)nout * 4, st));
-    }
-  } else {
-    if ((rc = launch_qk(L, x, first, groups, true, v, nhd, (float*)out, nout, st))) return rc;
-    if ((rc = launch_select(L, st))) return rc;
-  }
+  if ((rc = launch_gate_sort(L, x, v, nhd, (float*)out, nout, st))) return rc;
+  sh_mark(L, 1, st);
+  if (L->ev && (rc = launch_x<X_QK>(L, st, qk))) return rc;
   if (L->moe_k) {
     SH_CUDA_CHECK(cudaMemsetAsync(ws + L->o.k, 0, (size_t)nhd * 4, st));
-    if ((rc = launch_v(L, x, 0, (const float*)(ws + L->o.wk_e), (float*)(ws + L->o.k), 0.f, st))) return rc;
+    if ((rc = launch_x<X_V>(L, st, part_v(L, x, 0, S->wk_e, (float*)(ws + L->o.k), 0.f)))) return rc;
   }
   if (L->moe_q) {
     SH_CUDA_CHECK(cudaMemsetAsync(ws + L->o.q, 0, (size_t)nhd * 4, st));
-    if ((rc = launch_v(L, x, 1, (const float*)(ws + L->o.wq_e), (float*)(ws + L->o.q), qscale, st))) return rc;
+    if ((rc = launch_x<X_V>(L, st, part_v(L, x, 1, S->wq_e, (float*)(ws + L->o.q), 1.4426950408889634f / sqrtf((float)d.Dt))))) return rc;
   }
   sh_mark(L, 2, st);
-  if ((rc = launch_v(L, x, 0, (const float*)(ws + L->o.wv), v, 0.f, st))) return rc;
+  if ((rc = L->ev ? launch_x<X_V>(L, st, pv) : launch_x<X_QK, X_V>(L, st, qk, pv))) return rc;
   sh_mark(L, 3, st);
   // (the relative-position term of Transformer-XL is in the one-warp-per-query kernel only)
   if ((rc = L->xl_positions ? sh_simt_attention_f32(L, st) : launch_attn(L, st))) return rc;
@@ -220,10 +244,8 @@ int sh_f32_forward(sh_layer* L, const void* x, void* out, cudaStream_t st) {
   XGemmArgs g = base_args(L, x);
   use_side(g, L, 1);
   g.y = (float*)out;
-  const bool wide = wide_tile(L, (long)d.H * head_tiles(d), 1, d.M);
-  col_tiles(g, d.M, wide);
-  if ((rc = launch_x<X_O>(g, wide, dim3(d.H * head_tiles(d), g.nsub), st))) return rc;
-  L->launches += 1;
+  col_tiles(g, d.M);
+  if ((rc = launch_x<X_O>(L, st, part<X_O>(L, g, d.H * head_tiles(d), g.nsub)))) return rc;
   sh_mark(L, 5, st);
   SH_CUDA_CHECK(cudaGetLastError());
   return SH_OK;
@@ -239,19 +261,20 @@ int sh_f32_backward(sh_layer* L, const void* x, const float* dout, float* dx, fl
   L->launches = 0;
   SH_CUDA_CHECK(cudaMemsetAsync(w.dq, 0, w.cleared * 4, st));
   SH_CUDA_CHECK(cudaMemsetAsync(dx, 0, (size_t)d.N * d.M * 4, st));
-  XGemmArgs g = base_args(L, x);
-  g.dy = dout; g.dq = w.dq; g.dk = w.dk; g.dv = w.dv; g.dz = w.dz; g.dahat = w.dahat; g.dx = dx;
-  g.dWq = dWq; g.dWk = dWk; g.dWv = dWv; g.dWo = dWo; g.dWs = dWs; g.dWd = dWd;
+  XGemmArgs src = base_args(L, x);                         // source side; dst: destination side
+  src.dy = dout; src.dq = w.dq; src.dk = w.dk; src.dv = w.dv; src.dz = w.dz; src.dahat = w.dahat; src.dx = dx;
+  src.dWq = dWq; src.dWk = dWk; src.dWv = dWv; src.dWo = dWo; src.dWs = dWs; src.dWd = dWd;
   auto aligned = [](const void* p) { return (uintptr_t)p % 16 == 0; };
-  g.vec_dy = aligned(dout);
-  g.vec_out = aligned(dx) && aligned(dWq) && aligned(dWk) && aligned(dWv) && aligned(dWo);
-  const size_t list_side = (size_t)d.H * d.N * d.k;
+  src.vec_dy = aligned(dout);
+  src.vec_out = aligned(dx) && aligned(dWq) && aligned(dWk) && aligned(dWv) && aligned(dWo);
+  XGemmArgs dst = src;
+  use_side(src, L, 0); use_side(dst, L, 1);
+  src.ds = w.ds; dst.ds = w.ds + (size_t)d.H * d.N * d.k;
+  XGemmArgs g;
   // output experts: dAhat and the destination gates' gradients
-  use_side(g, L, 1);
-  g.ds = w.ds + list_side;
-  bool wide = wide_tile(L, (long)d.H * ht, 1, d.Dt);
-  col_tiles(g, d.Dt, wide);
-  if ((rc = launch_x<X_DA>(g, wide, dim3(d.H * ht, g.nsub), st))) return rc;
+  g = dst;
+  col_tiles(g, d.Dt);
+  if ((rc = launch_x<X_DA>(L, st, part<X_DA>(L, g, d.H * ht, g.nsub)))) return rc;
   // attention
   const int rows = d.N * d.H;
   if ((rc = launch_k(true, sh_f32_rowdot_kernel, dim3((unsigned)((rows + 7) / 8)), dim3(256), 0, st, (const float*)w.dahat,
@@ -259,44 +282,37 @@ int sh_f32_backward(sh_layer* L, const void* x, const float* dout, float* dx, fl
   rc = d.D == 32 ? launch_attn_bw_t<32>(L, w, st) : d.D == 64 ? launch_attn_bw_t<64>(L, w, st)
      : d.D == 128 ? launch_attn_bw_t<128>(L, w, st) : launch_attn_bw_t<256>(L, w, st);
   if (rc) return rc;
-  // value experts: their part of dx, and the source gates' gradients
-  use_side(g, L, 0);
-  g.ds = w.ds;
-  wide = wide_tile(L, (long)d.H * ht, 1, d.M);
-  col_tiles(g, d.M, wide);
-  if ((rc = launch_x<X_DR>(g, wide, dim3(d.H * ht, g.nsub), st))) return rc;
+  // value experts: their part of dx and the source gates' gradients; beside it the expert weights' gradients
+  // (contractions over the experts' lists, in parts where the whole launch would leave block slots idle)
+  g = src;
+  col_tiles(g, d.M);
+  const XPart dr = part<X_DR>(L, g, d.H * ht, g.nsub);
+  const long list_steps = ((long)d.N * d.k / d.E + XG_BK - 1) / XG_BK;
+  XGemmArgs gv = src, go = dst;
+  col_tiles(gv, d.Dt); col_tiles(go, d.M);
+  gv.ksplit = go.ksplit = k_parts(L, (long)d.H * d.E * (mt * gv.nsub + dt * go.nsub), list_steps);
+  if (gv.ksplit > 1) {
+    SH_CUDA_CHECK(cudaMemsetAsync(dWv, 0, (size_t)d.H * d.E * d.M * d.Dt * 4, st));
+    SH_CUDA_CHECK(cudaMemsetAsync(dWo, 0, (size_t)d.H * d.E * d.Dt * d.M * 4, st));
+  }
+  if ((rc = launch_x<X_DWV, X_DWO, X_DR>(L, st, part<X_DWV>(L, gv, d.H * d.E * gv.ksplit, gv.nsub, mt),
+                                         part<X_DWO>(L, go, d.H * d.E * go.ksplit, go.nsub, dt), dr))) return rc;
   if ((rc = launch_k(true, sh_f32_dz_kernel, dim3((unsigned)(((long)d.N * d.k + 255) / 256), 2 * d.H), dim3(256), 0, st, (const float*)w.ds,
-                     (const int*)(ws + L->o.lists), (const float*)(ws + L->o.lgate), (const int*)(ws + L->o.offsets), w.dz, g.ldz, d))) return rc;
-  // queries, keys and gates: the rest of dx, then the weight gradients
-  wide = wide_tile(L, d.nblk, 1, d.M);
-  col_tiles(g, d.M, wide);
-  if ((rc = launch_x<X_DX>(g, wide, dim3(d.nblk, g.nsub), st))) return rc;
-  g.qk_first = 0; g.qk_groups = 2 * d.H;
-  wide = wide_tile(L, mt, 2 * d.H, d.Dt);
-  col_tiles(g, d.Dt, wide);
-  const int ct = g.qk_groups * g.nsub + (d.G + (wide ? 127 : 63)) / (wide ? 128 : 64);
-  g.ksplit = k_parts(L, (long)mt * ct, (d.N + 63) / 64);
-  if (g.ksplit > 1) {
+                     (const int*)(ws + L->o.lists), (const float*)(ws + L->o.lgate), (const int*)(ws + L->o.offsets), w.dz, src.ldz, d))) return rc;
+  // queries, keys and gates: the rest of dx, and the weight gradients
+  XGemmArgs gx = src, gw = src;
+  col_tiles(gx, d.M); col_tiles(gw, d.Dt);
+  gw.qk_first = 0; gw.qk_groups = 2 * d.H;
+  const int ct = gw.qk_groups * gw.nsub + (d.G + XG_BN - 1) / XG_BN;
+  gw.ksplit = k_parts(L, (long)mt * ct + (long)d.nblk * gx.nsub, (d.N + XG_BK - 1) / XG_BK);
+  if (gw.ksplit > 1) {
     SH_CUDA_CHECK(cudaMemsetAsync(dWq, 0, (size_t)d.H * d.M * d.Dt * 4, st));
     SH_CUDA_CHECK(cudaMemsetAsync(dWk, 0, (size_t)d.H * d.M * d.Dt * 4, st));
     SH_CUDA_CHECK(cudaMemsetAsync(dWs, 0, (size_t)d.H * d.M * d.E * 4, st));
     SH_CUDA_CHECK(cudaMemsetAsync(dWd, 0, (size_t)d.H * d.M * d.E * 4, st));
   }
-  if ((rc = launch_x<X_DWQK>(g, wide, dim3(mt, ct, g.ksplit), st))) return rc;
-  // expert weights: contractions over the experts' lists
-  const long list_steps = ((long)d.N * d.k / d.E + 63) / 64;
-  wide = wide_tile(L, (long)d.H * d.E * mt, 1, d.Dt);
-  col_tiles(g, d.Dt, wide);
-  g.ksplit = k_parts(L, (long)d.H * d.E * mt * g.nsub, list_steps);
-  if (g.ksplit > 1) SH_CUDA_CHECK(cudaMemsetAsync(dWv, 0, (size_t)d.H * d.E * d.M * d.Dt * 4, st));
-  if ((rc = launch_x<X_DWV>(g, wide, dim3(d.H * d.E * g.ksplit, g.nsub, mt), st))) return rc;
-  use_side(g, L, 1);
-  wide = wide_tile(L, (long)d.H * d.E * dt, 1, d.M);
-  col_tiles(g, d.M, wide);
-  g.ksplit = k_parts(L, (long)d.H * d.E * dt * g.nsub, list_steps);
-  if (g.ksplit > 1) SH_CUDA_CHECK(cudaMemsetAsync(dWo, 0, (size_t)d.H * d.E * d.Dt * d.M * 4, st));
-  if ((rc = launch_x<X_DWO>(g, wide, dim3(d.H * d.E * g.ksplit, g.nsub, dt), st))) return rc;
+  if ((rc = launch_x<X_DX, X_DWQK>(L, st, part<X_DX>(L, gx, d.nblk, gx.nsub), part<X_DWQK>(L, gw, mt, ct, gw.ksplit)))) return rc;
   SH_CUDA_CHECK(cudaGetLastError());
-  L->launches = 9;
+  L->launches += 3;
   return SH_OK;
 }

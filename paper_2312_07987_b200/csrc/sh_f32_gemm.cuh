@@ -3,29 +3,40 @@
 //
 // An fp32 value is the exact sum of three bf16 values, x = h + m + l (8 + 8 + 8 mantissa bits: h is x
 // rounded, m the rest rounded, l what is left), so a product of two is
-//   hh' + (hm' + mh' + mm' + hl' + lh') + terms below 2^-25 of it,
-// six bf16 UMMAs.  The tensor core adds into fp32 but drops the bits below the accumulator's last one
-// instead of rounding, so a long chain of additions drifts towards zero: the hh' products, which carry
-// the size of the result, go to an accumulator of their own that is read back and added in fp32
-// registers every 128 contraction positions (8 additions); the five correction products, 2^-8 of it
-// and smaller, share a second accumulator over the whole contraction.
+//   hh' + (hm' + mh') + (hl' + mm' + lh') + terms below 2^-25 of it,
+// six bf16 products.  The tensor core adds into fp32 but drops the bits below the accumulator's last one
+// instead of rounding, so a long chain of additions drifts towards zero: the accumulators are read back
+// and added in fp32 registers every 128 contraction positions (8 additions of hh', which carries the
+// size of the result).
 //
-// Why not FFMA: the CUDA cores' 74 TFLOP/s fp32 peak against 2.25 PFLOP/s / 6 = 375; what bounds this
-// kernel is shared memory (a 128 x 128 x 16 UMMA reads 8 KB in 64 cycles, all an SM's shared memory
-// delivers; the operand planes are written through it too).
+// Three UMMAs per 16 positions do the six products: the planes of B lie one behind the other, so that
+// they are one operand of 192 columns, and with accumulator blocks P0 P1 P2 of 64 columns
+//   h x [h' m' l'] -> P0 P1 P2,   m x [h' m'] -> P1 P2,   l x h' -> P2.
+// (As six UMMAs of 64 columns the loop was bound by their issue, ~57 cycles each against 32 of tensor
+// time: 2800 cycles a step of 64 positions.)
 //
-// Tile: 128 rows x BN columns (64 or 128), contraction steps of 64.  512 worker threads read the fp32
-// operands of step i + 1 into registers while the UMMAs of step i run, split them and store three
-// 128-byte-swizzled planes per operand (two stages); one thread issues the UMMAs; the workers read
-// the accumulators and write the result.  Operands are addressed row by row (a gathered token list, a
-// head's slice of a row), either as rows of the contraction (K-major) or as rows of the other index
-// (MN-major: the weight gradients contract over tokens), so no transposed or gathered copy is made.
+// Why not FFMA: the CUDA cores' 74 TFLOP/s fp32 peak against 2.25 PFLOP/s / 6 = 375.  What bounds a tile
+// is latency: gather list -> rows -> split -> shared memory -> UMMA -> read-back, and a tile's set-up and
+// result, 6 to 8 us of which little is work.  So a block is half an SM: 128 rows x 64 columns, contraction
+// steps of 32, three stages of 36 KB, 256 worker threads; two blocks share an SM and fill each other's
+// waits.  (One block per SM with 512 workers and steps of 64 ran each kernel 1.5 to 2 times as long.)
+//
+// Weights are split once, when they are set, and come as planes by TMA (one box of all three planes); an
+// activation is read as fp32 by the workers - the pieces of step i + 1 in registers while step i is
+// multiplied -, split and stored into the swizzled planes.  One thread issues the UMMAs; the workers read
+// the accumulators and write the result.
+// Operands are addressed row by row (a gathered token list, a head's slice of a row), either as rows of
+// the contraction (K-major) or as rows of the other index (MN-major: the weight gradients contract over
+// tokens), so no transposed or gathered copy is made.  Results that are added to, and rows handed on
+// whole, go through a padded copy in shared memory and leave as one bulk operation per row: as vector
+// reductions from the accumulator layout (a lane per row, 16 bytes each) they were a third of the
+// short contractions' time.
 #pragma once
 #include "sh_tc_prims.cuh"
 
 namespace shtc {
 
-enum { X_QK = 0,    // z | q, k = x [Wgate | Wq | Wk]        rows: tokens
+enum { X_QK = 0,    // q, k = x [Wq | Wk]                     rows: tokens
        X_V = 1,     // v += g x Wv                           rows: a value expert's list
        X_O = 2,     // y += g ahat Wo                        rows: an output expert's list
        X_DA = 3,    // dahat += g dy Wo^T, ds = ahat . that  rows: an output expert's list
@@ -40,66 +51,67 @@ struct XGemmArgs {
   const float *x, *dy;                   // [N, M]; dy [N, M]
   const float *ahat, *dahat_in;          // [N, H, D]
   const float *dq, *dk, *dv, *dz;        // [N, H, D]; dz [N, ldz] (columns (side*H + h)*E + e)
-  const float *wqk, *wgate, *wv, *wo;    // repacked weights: [(which*H + h)*D + dd][m], [g][m], [(h*E + e)*D + dd][m], [(h*E + e)*M + m][dd]
   int ldz;
   const int* lists; const float* lgate; const int* offsets; const ShTile* tiles;   // of the side the mode works on
   int nsub, sub_cols;                    // column tiles per head (or of M), and columns per tile (a multiple of 16)
   int qk_first, qk_groups;               // X_QK: first group ((which*H + h)) and how many
   int ksplit;                            // X_DW*: parts of the contraction (more than one: the results are added)
-  float *q, *k, *v, *z;                  // X_QK: q, k [B, H, T, D], logits z [N, ldz]; X_V: v
+  float *q, *k, *v;                      // X_QK: q, k [B, H, T, D]; X_V: v
   float *y;                              // X_O [rows of out, M]
   float *dahat, *ds, *dx;                // ds: gate gradients in list order
   float *dWq, *dWk, *dWv, *dWo, *dWs, *dWd;
-  float *zero0, *zero1; long nzero0, nzero1;   // X_QK: buffers that later kernels add into (16-byte pieces), cleared beside the products
   float qscale, vscale;
   const float2* rope;
   int vec_dy, vec_out;                   // dy / the written gradients are 16-byte aligned
   int* status;
 };
 
-template <int BN>
+constexpr int XG_BN = 64, XG_BK = 32, XG_STAGES = 3;
 struct XGemmSmem {
-  static constexpr int A_PLANE = 128 * 128, B_PLANE = BN * 128;
+  static constexpr int A_PLANE = 128 * XG_BK * 2, B_PLANE = XG_BN * XG_BK * 2;
   static constexpr int STAGE = 3 * (A_PLANE + B_PLANE);
-  static constexpr int BAR_OFF = 2 * STAGE;
+  static constexpr int BAR_OFF = XG_STAGES * STAGE;
   static constexpr int TOTAL = BAR_OFF + 128 + 1024;
 };
 
-constexpr int XG_WORKERS = 512, XG_THREADS = XG_WORKERS + 32;
-constexpr int XG_CHUNK = 2;              // steps per promotion of the main accumulator
+constexpr int XG_WORKERS = 256, XG_THREADS = XG_WORKERS + 64;   // + a warp that issues UMMAs, + one that loads weights
+constexpr int XG_CHUNK = 128 / XG_BK;    // steps per promotion of the accumulators
 
-template <int N>
-__device__ __forceinline__ void tmem_ld_n(uint32_t taddr, float (&r)[N]);
-template <>
-__device__ __forceinline__ void tmem_ld_n<32>(uint32_t taddr, float (&r)[32]) {
-  uint32_t u[32];
-  tmem_ld32(taddr, u);
-  tmem_ld_wait();
-#pragma unroll
-  for (int i = 0; i < 32; ++i) r[i] = __uint_as_float(u[i]);
+// K-major planes: rows of 32 values (64 bytes), 64-byte swizzle, 8-row groups 512 bytes apart.
+constexpr uint32_t DESC_HI_SW64 = (512u >> 4) | (1u << 14) | (4u << 29);
+__device__ __forceinline__ uint64_t xg_desc(uint32_t lo, bool mn_major) {
+  return ((uint64_t)(mn_major ? DESC_HI_SW128 : DESC_HI_SW64) << 32) | lo;
 }
-template <>
-__device__ __forceinline__ void tmem_ld_n<16>(uint32_t taddr, float (&r)[16]) {
-  uint32_t u[16];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-      : "=r"(u[0]), "=r"(u[1]), "=r"(u[2]), "=r"(u[3]), "=r"(u[4]), "=r"(u[5]), "=r"(u[6]), "=r"(u[7]),
-        "=r"(u[8]), "=r"(u[9]), "=r"(u[10]), "=r"(u[11]), "=r"(u[12]), "=r"(u[13]), "=r"(u[14]), "=r"(u[15])
-      : "r"(taddr)
-      : "memory");
-  tmem_ld_wait();
+
+// acc += 16 tensor-memory columns at a time (more in flight than that costs registers the operands need).
+template <int N>
+__device__ __forceinline__ void tmem_add(uint32_t taddr, float (&acc)[N]) {
 #pragma unroll
-  for (int i = 0; i < 16; ++i) r[i] = __uint_as_float(u[i]);
+  for (int c = 0; c < N; c += 16) {
+    uint32_t u[16];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+        : "=r"(u[0]), "=r"(u[1]), "=r"(u[2]), "=r"(u[3]), "=r"(u[4]), "=r"(u[5]), "=r"(u[6]), "=r"(u[7]),
+          "=r"(u[8]), "=r"(u[9]), "=r"(u[10]), "=r"(u[11]), "=r"(u[12]), "=r"(u[13]), "=r"(u[14]), "=r"(u[15])
+        : "r"(taddr + c)
+        : "memory");
+    tmem_ld_wait();
+#pragma unroll
+    for (int i = 0; i < 16; ++i) acc[c + i] += __uint_as_float(u[i]);
+  }
 }
 
 // Two fp32 values as three packed bf16 pairs whose sum they are.
+__device__ __forceinline__ float2 sub_bf16x2(float2 x, uint32_t p) {
+  return __ffma2_rn(make_float2(__uint_as_float(p << 16), __uint_as_float(p & 0xFFFF0000u)), make_float2(-1.f, -1.f), x);
+}
 __device__ __forceinline__ void split_bf16x3(float a, float b, uint32_t& h, uint32_t& m, uint32_t& l) {
   asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(h) : "f"(b), "f"(a));
-  a -= __uint_as_float(h << 16); b -= __uint_as_float(h & 0xFFFF0000u);
-  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(m) : "f"(b), "f"(a));
-  a -= __uint_as_float(m << 16); b -= __uint_as_float(m & 0xFFFF0000u);
-  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(l) : "f"(b), "f"(a));
+  float2 r = sub_bf16x2(make_float2(a, b), h);
+  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(m) : "f"(r.y), "f"(r.x));
+  r = sub_bf16x2(r, m);
+  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(l) : "f"(r.y), "f"(r.x));
 }
 
 // Eight values into the three planes at byte offset `off` of the operand's tile.
@@ -112,20 +124,15 @@ __device__ __forceinline__ void store_planes(unsigned char* tile, uint32_t off, 
   *reinterpret_cast<uint4*>(tile + off + 2 * plane) = make_uint4(l[0], l[1], l[2], l[3]);
 }
 
-// Eight consecutive values of a row; those at or past `valid` (and all of a null row) are zero.
-__device__ __forceinline__ void load8(float (&v)[8], const float* p, int valid, bool vec) {
-  if (p == nullptr || valid <= 0) {
-#pragma unroll
-    for (int i = 0; i < 8; ++i) v[i] = 0.f;
-    return;
-  }
-  if (vec && valid >= 8) {
+// Eight consecutive values of a row (16-byte aligned, or not).
+__device__ __forceinline__ void load8(float (&v)[8], const float* p, bool vec) {
+  if (vec) {
     const float4 a = __ldg(reinterpret_cast<const float4*>(p)), b = __ldg(reinterpret_cast<const float4*>(p) + 1);
     v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
-    return;
-  }
+  } else {
 #pragma unroll
-  for (int i = 0; i < 8; ++i) v[i] = i < valid ? __ldg(p + i) : 0.f;
+    for (int i = 0; i < 8; ++i) v[i] = __ldg(p + i);
+  }
 }
 
 // acc += the row's gate times a value: four adjacent floats at a time when the row is 16-byte aligned.
@@ -152,24 +159,29 @@ __device__ __forceinline__ void store_row(float* dst, const float (&v)[N], int v
   }
 }
 
-template <int BN, int MODE>
-__global__ void __launch_bounds__(XG_THREADS, 1)
-sh_f32_gemm_kernel(const __grid_constant__ XGemmArgs g) {
-  using SM = XGemmSmem<BN>;
+struct XTile { int x, y, z; };           // which tile of its mode a block works on
+
+// One tile.  mapW: planes of the mode's weights, rows [(which*H + h)*D + dd][m] (Q, K), [(h*E + e)*D + dd][m] (V),
+// [(h*E + e)*M + m][dd] (O); mapG: of the gates' weights, rows [(side*H + h)*E + e][m].
+template <int MODE>
+__device__ __forceinline__ void xg_tile(const CUtensorMap& mapW, const CUtensorMap& mapG, const XGemmArgs& g, XTile blk) {
+  using SM = XGemmSmem;
+  constexpr int BN = XG_BN;
   constexpr bool A_MN = MODE == X_DWO || MODE == X_DWV || MODE == X_DWQK;
   constexpr bool B_MN = MODE >= X_DA;
   constexpr bool LIST_ROWS = MODE == X_V || MODE == X_O || MODE == X_DA || MODE == X_DR;
   constexpr bool LIST_K = MODE == X_DWO || MODE == X_DWV;
-  constexpr int COLS = BN / 4;                             // columns of a worker thread
-  constexpr int NB = BN / 64;                              // operand pieces (8 values) per thread: two of A, NB of B
+  constexpr bool B_TMA = MODE <= X_DR && MODE != X_DWO || MODE == X_DX;
+  constexpr bool BULK = LIST_ROWS || MODE == X_QK;         // results that leave as one bulk operation per row
+  constexpr int COLS = BN / 2;                             // columns of a worker thread
   extern __shared__ unsigned char smem_raw[];
   const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
   unsigned char* sgen = smem_raw + (sbase - smem_u32(smem_raw));
-  uint64_t* full_bar = (uint64_t*)(sgen + SM::BAR_OFF);    // [2]
-  uint64_t* empty_bar = full_bar + 2;                      // [2]
-  uint64_t* acc_full = empty_bar + 2;                      // [2]
-  uint64_t* acc_empty = acc_full + 2;                      // [2]
-  uint32_t* tmem_slot = (uint32_t*)(acc_empty + 2);
+  uint64_t* full_bar = (uint64_t*)(sgen + SM::BAR_OFF);    // [XG_STAGES]
+  uint64_t* empty_bar = full_bar + XG_STAGES;              // [XG_STAGES]
+  uint64_t* acc_full = empty_bar + XG_STAGES;
+  uint64_t* acc_empty = acc_full + 1;
+  uint32_t* tmem_slot = (uint32_t*)(acc_empty + 1);
   const ShDims& d = g.d;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int HD = d.H * d.D;
@@ -177,40 +189,41 @@ sh_f32_gemm_kernel(const __grid_constant__ XGemmArgs g) {
 
   pdl_trigger();
   if (tid == 0) {
-    for (int s = 0; s < 2; ++s) { mbar_init(&full_bar[s], 16); mbar_init(&empty_bar[s], 1); mbar_init(&acc_full[s], 1); mbar_init(&acc_empty[s], 16); }
+    for (int s = 0; s < XG_STAGES; ++s) { mbar_init(&full_bar[s], B_TMA ? 9 : 8); mbar_init(&empty_bar[s], 1); }
+    mbar_init(acc_full, 1); mbar_init(acc_empty, 8);
     fence_barrier_init();
   }
   pdl_wait();
   // ---- which tile ------------------------------------------------------------------------------
   int h = 0, e = 0, which = 0, row0 = 0, nrows = 0, n0 = 0, ncols = 0, m0 = 0, steps = 0;
   int kbeg = 0, kend = 0;                                  // LIST_K, X_DWQK: positions of the contraction
-  bool gates = false;                                      // X_QK / X_DWQK: the tile of the gate columns
-  const int sps = (d.Dt + 63) / 64;                        // steps over one head's d_head
+  bool gates = false;                                      // X_DWQK: the tile of the gate columns
+  const int sps = (d.Dt + XG_BK - 1) / XG_BK;                        // steps over one head's d_head
   if (LIST_ROWS) {
-    const ShTile tl = g.tiles[blockIdx.x];
+    const ShTile tl = g.tiles[blk.x];
     if (tl.nrows == 0) return;                             // (before any allocation)
     h = tl.h; e = tl.e; row0 = tl.row0; nrows = tl.nrows;
-    n0 = blockIdx.y * g.sub_cols;
+    n0 = blk.y * g.sub_cols;
     ncols = min(g.sub_cols, ((MODE == X_O || MODE == X_DR) ? d.M : d.Dt) - n0);
-    steps = (MODE == X_V || MODE == X_DA) ? d.M / 64 : sps;
+    steps = (MODE == X_V || MODE == X_DA) ? d.M / XG_BK : sps;
   } else if (LIST_K) {
-    const int grp = blockIdx.x / g.ksplit, part = blockIdx.x % g.ksplit;
+    const int grp = blk.x / g.ksplit, part = blk.x % g.ksplit;
     h = grp / d.E; e = grp % d.E;
     const int o0 = g.offsets[h * (d.E + 1) + e], o1 = g.offsets[h * (d.E + 1) + e + 1];
-    const int per = (((o1 - o0 + 63) / 64 + g.ksplit - 1) / g.ksplit) * 64;
+    const int per = (((o1 - o0 + XG_BK - 1) / XG_BK + g.ksplit - 1) / g.ksplit) * XG_BK;
     kbeg = min(o1, o0 + part * per); kend = min(o1, kbeg + per);
     if (g.ksplit > 1 && kbeg >= kend) return;              // (the results are added to zeros)
-    steps = (kend - kbeg + 63) / 64;
-    n0 = blockIdx.y * g.sub_cols; m0 = blockIdx.z * 128;
+    steps = (kend - kbeg + XG_BK - 1) / XG_BK;
+    n0 = blk.y * g.sub_cols; m0 = blk.z * 128;
     ncols = min(g.sub_cols, (MODE == X_DWO ? d.M : d.Dt) - n0);
     nrows = min(128, (MODE == X_DWO ? d.Dt : d.M) - m0);
   } else if (MODE == X_DX) {
-    row0 = blockIdx.x * 128; nrows = min(128, d.N - row0);
-    n0 = blockIdx.y * g.sub_cols; ncols = min(g.sub_cols, d.M - n0);
-    steps = 2 * d.H * sps + (d.G + 63) / 64;
+    row0 = blk.x * 128; nrows = min(128, d.N - row0);
+    n0 = blk.y * g.sub_cols; ncols = min(g.sub_cols, d.M - n0);
+    steps = 2 * d.H * sps + (d.G + XG_BK - 1) / XG_BK;
   } else {
     // X_QK, X_DWQK: column tiles 0 .. qk_groups*nsub - 1 are the heads' columns, the rest the gate columns
-    const int ct = blockIdx.y;
+    const int ct = blk.y;
     if (ct < g.qk_groups * g.nsub) {
       const int grp = g.qk_first + ct / g.nsub;
       which = grp / d.H; h = grp % d.H;
@@ -220,211 +233,215 @@ sh_f32_gemm_kernel(const __grid_constant__ XGemmArgs g) {
       n0 = (ct - g.qk_groups * g.nsub) * BN; ncols = min(BN, d.G - n0);
     }
     if (MODE == X_QK) {
-      row0 = blockIdx.x * 128; nrows = min(128, d.N - row0);
-      steps = d.M / 64;
+      row0 = blk.x * 128; nrows = min(128, d.N - row0);
+      steps = d.M / XG_BK;
     } else {
-      m0 = blockIdx.x * 128; nrows = min(128, d.M - m0);
-      const int per = (((d.N + 63) / 64 + g.ksplit - 1) / g.ksplit) * 64;
-      kbeg = min(d.N, (int)blockIdx.z * per); kend = min(d.N, kbeg + per);
+      m0 = blk.x * 128; nrows = min(128, d.M - m0);
+      const int per = (((d.N + XG_BK - 1) / XG_BK + g.ksplit - 1) / g.ksplit) * XG_BK;
+      kbeg = min(d.N, blk.z * per); kend = min(d.N, kbeg + per);
       if (g.ksplit > 1 && kbeg >= kend) return;
-      steps = (kend - kbeg + 63) / 64;
+      steps = (kend - kbeg + XG_BK - 1) / XG_BK;
     }
   }
-  if (warp == 16) { tmem_alloc(tmem_slot, BN == 128 ? 512 : 256); tmem_relinquish(); }
+  if (warp == 8) { tmem_alloc(tmem_slot, 256); tmem_relinquish(); }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   // contraction positions of step i that exist (the rest of the operand rows is zero)
   auto kvalid = [&](int i) -> int {
-    if (MODE == X_O || MODE == X_DR) return min(64, d.Dt - 64 * i);
-    if (A_MN) return min(64, kend - kbeg - 64 * i);
+    if (MODE == X_O || MODE == X_DR) return min(XG_BK, d.Dt - XG_BK * i);
+    if (A_MN) return min(XG_BK, kend - kbeg - XG_BK * i);
     if (MODE == X_DX) {
       const int seg = i / sps;
-      return seg < 2 * d.H ? min(64, d.Dt - (i - seg * sps) * 64) : min(64, d.G - (i - 2 * d.H * sps) * 64);
+      return seg < 2 * d.H ? min(XG_BK, d.Dt - (i - seg * sps) * XG_BK) : min(XG_BK, d.G - (i - 2 * d.H * sps) * XG_BK);
     }
-    return 64;
+    return XG_BK;
   };
-  const uint32_t tmem = *tmem_slot;
-  const uint32_t corr = tmem + 2 * BN;                     // columns: main 0, main 1, corrections
-  const int chunks = (steps + XG_CHUNK - 1) / XG_CHUNK;
-  const int nmma = (ncols + 15) & ~15;
+  const uint32_t tmem = *tmem_slot;                        // accumulator blocks P0 P1 P2
 
-  if (warp == 16) {
+  if (warp == 8) {
     if (lane == 0) {
-      const uint32_t idesc = make_idesc_f16(128, nmma, 1, 1, B_MN ? 1 : 0) | (A_MN ? 1u << 15 : 0u);
+      constexpr uint32_t maj = (B_MN ? 1u << 16 : 0u) | (A_MN ? 1u << 15 : 0u);
+      constexpr uint32_t id3 = make_idesc_f16(128, 192, 1, 1, 0) | maj, id2 = make_idesc_f16(128, 128, 1, 1, 0) | maj,
+                         id1 = make_idesc_f16(128, 64, 1, 1, 0) | maj;
+      const uint32_t a0 = A_MN ? desc_lo_mn(sbase, 64 * XG_BK * 2) : desc_lo_k(sbase);
+      const uint32_t b0 = B_MN ? desc_lo_mn(sbase + 3 * SM::A_PLANE, SM::B_PLANE) : desc_lo_k(sbase + 3 * SM::A_PLANE);
+      constexpr uint32_t AK = A_MN ? 128 : 2, BK = B_MN ? 128 : 2, AP = SM::A_PLANE >> 4;
+      int s = 0;
+      uint32_t par = 0;
       for (int i = 0; i < steps && !dead; ++i) {
-        const int s = i & 1, c = i / XG_CHUNK, b = c & 1;
-        if (i % XG_CHUNK == 0 && c >= 2 && !mbar_wait(&acc_empty[b], ((c >> 1) & 1) ^ 1, g.status, dead)) break;
-        if (!mbar_wait(&full_bar[s], (i >> 1) & 1, g.status, dead)) break;
+        if (i % XG_CHUNK == 0 && i > 0 && !mbar_wait(acc_empty, ((i / XG_CHUNK) & 1) ^ 1, g.status, dead)) break;
+        if (!mbar_wait(&full_bar[s], par, g.status, dead)) break;
         tc_fence_after();
-        const uint32_t abase = sbase + s * SM::STAGE, bbase = abase + 3 * SM::A_PLANE;
-        const uint32_t alo = A_MN ? desc_lo_mn(abase, 8192) : desc_lo_k(abase);
-        const uint32_t blo = B_MN ? desc_lo_mn(bbase, 8192) : desc_lo_k(bbase);
-        constexpr uint32_t AK = A_MN ? 128 : 2, BK = B_MN ? 128 : 2;
-        constexpr uint32_t AP = SM::A_PLANE >> 4, BP = SM::B_PLANE >> 4;
+        const uint32_t alo = a0 + s * (SM::STAGE >> 4), blo = b0 + s * (SM::STAGE >> 4);
         const int kn = (kvalid(i) + 15) / 16;
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
+        for (int k = 0; k < XG_BK / 16; ++k) {
           if (k >= kn) break;
-          const uint32_t a = alo + AK * k, bb = blo + BK * k;
-          umma_f16(tmem + b * BN, desc_pack(a), desc_pack(bb), idesc, (i % XG_CHUNK | k) != 0);
-          umma_f16(corr, desc_pack(a + 2 * AP), desc_pack(bb), idesc, (i | k) != 0);
-          umma_f16(corr, desc_pack(a), desc_pack(bb + 2 * BP), idesc, 1);
-          umma_f16(corr, desc_pack(a + AP), desc_pack(bb + BP), idesc, 1);
-          umma_f16(corr, desc_pack(a + AP), desc_pack(bb), idesc, 1);
-          umma_f16(corr, desc_pack(a), desc_pack(bb + BP), idesc, 1);
+          const uint32_t a = alo + AK * k;
+          const uint64_t bb = xg_desc(blo + BK * k, B_MN);
+          umma_f16(tmem, xg_desc(a, A_MN), bb, id3, (i % XG_CHUNK | k) != 0);
+          umma_f16(tmem + 64, xg_desc(a + AP, A_MN), bb, id2, 1);
+          umma_f16(tmem + 128, xg_desc(a + 2 * AP, A_MN), bb, id1, 1);
         }
         umma_commit(&empty_bar[s]);
-        if (i % XG_CHUNK == XG_CHUNK - 1 || i == steps - 1) umma_commit(&acc_full[b]);
+        if (i % XG_CHUNK == XG_CHUNK - 1 || i == steps - 1) umma_commit(acc_full);
+        if (++s == XG_STAGES) { s = 0; par ^= 1; }
+      }
+    }
+    __syncwarp();
+  } else if (warp == 9) {
+    if (B_TMA && lane == 0) {
+      int s = 0;
+      uint32_t par = 1;
+      for (int i = 0; i < steps && !dead; ++i) {
+        if (!mbar_wait(&empty_bar[s], par, g.status, dead)) break;
+        mbar_expect_tx(&full_bar[s], 3 * SM::B_PLANE);
+        int x = i * XG_BK, y = 0;
+        bool gm = false;
+        if (MODE == X_QK) y = (which * d.H + h) * d.D + n0;
+        if (MODE == X_V) y = (h * d.E + e) * d.D + n0;
+        if (MODE == X_O) y = (h * d.E + e) * d.M + n0;
+        if (MODE == X_DA) { x = n0; y = (h * d.E + e) * d.M + i * XG_BK; }
+        if (MODE == X_DR) { x = n0; y = (h * d.E + e) * d.D + i * XG_BK; }
+        if (MODE == X_DX) {
+          const int seg = i / sps;
+          x = n0;
+          gm = seg >= 2 * d.H;
+          y = gm ? (i - 2 * d.H * sps) * XG_BK : seg * d.D + (i - seg * sps) * XG_BK;
+        }
+        tma_load_3d(sbase + s * SM::STAGE + 3 * SM::A_PLANE, gm ? &mapG : &mapW, &full_bar[s], x, y, 0);
+        if (++s == XG_STAGES) { s = 0; par ^= 1; }
       }
     }
     __syncwarp();
   } else {
     // ---- workers: operands, promotions, result -----------------------------------------------------
-    // K-major pieces: 8 values of a row's 64 contraction positions; MN-major: 8 values of the row of
+    // K-major pieces: 8 values of a row's 32 contraction positions; MN-major: 8 values of the row of
     // one contraction position
-    const int ac = A_MN ? tid & 15 : tid & 7, ar = A_MN ? tid >> 4 : tid >> 3;    // + 32 j / + 64 j
-    const int bc = B_MN && BN == 128 ? tid & 15 : tid & 7, br = B_MN && BN == 128 ? tid >> 4 : tid >> 3;
-    constexpr int AR = A_MN ? 32 : 64, BR = B_MN && BN == 128 ? 32 : 64;
-    uint32_t aoff[2], boff[NB];
+    const int ac = A_MN ? tid & 15 : tid & 3, ar = A_MN ? tid >> 4 : tid >> 2;    // + 16 j / + 64 j
+    const int bc = tid & 7, br = tid >> 3;                 // (a B that is split here is MN-major: 32 rows, one piece per thread)
+    constexpr int AR = A_MN ? 16 : 64;
+    uint32_t aoff[2];
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
       const int r = ar + AR * j;
-      aoff[j] = A_MN ? (uint32_t)((ac >> 3) * 8192 + r * 128 + (((ac & 7) ^ (r & 7)) << 4)) : (uint32_t)(r * 128 + ((ac ^ (r & 7)) << 4));
+      aoff[j] = A_MN ? (uint32_t)((ac >> 3) * (64 * XG_BK * 2) + r * 128 + (((ac & 7) ^ (r & 7)) << 4))
+                     : (uint32_t)(r * 64 + ((ac ^ ((r >> 1) & 3)) << 4));
     }
-#pragma unroll
-    for (int j = 0; j < NB; ++j) {
-      const int r = br + BR * j;
-      boff[j] = B_MN ? (uint32_t)((bc >> 3) * 8192 + r * 128 + (((bc & 7) ^ (r & 7)) << 4)) : (uint32_t)(r * 128 + ((bc ^ (r & 7)) << 4));
-    }
-    // rows that stay the same over the contraction
+    const uint32_t boff = (uint32_t)(br * 128 + ((bc ^ (br & 7)) << 4));
     const size_t lbase = (size_t)h * d.N * d.k;
-    const float* arow[2] = {nullptr, nullptr};
-    const float* brow[NB];
-    int atok[2] = {0, 0};
+    const bool vdy = (MODE != X_DA && MODE != X_DWO) || g.vec_dy != 0;
+    // What lies past the tile never needs masking, only an address inside the operand: rows past a K-major A's
+    // last one and columns past an MN-major operand's width end in accumulators nobody reads, and positions
+    // past d_head (or the gate columns) are zeros in memory - a step of 32 never leaves the stored d_head.
+    // Only the positions past the end of a contraction over tokens are zeroed here.
+    const float* arow[2];
     if (!A_MN) {
 #pragma unroll
       for (int j = 0; j < 2; ++j) {
-        const int r = ar + AR * j;
-        if (r < nrows) {
-          const int t = LIST_ROWS ? g.lists[lbase + row0 + r] : row0 + r;
-          atok[j] = t;
-          arow[j] = MODE == X_QK || MODE == X_V ? g.x + (size_t)t * d.M
-                  : MODE == X_O ? g.ahat + (size_t)t * HD + h * d.D
-                  : MODE == X_DA ? g.dy + (size_t)t * d.M
-                  : MODE == X_DR ? g.dv + (size_t)t * HD + h * d.D : g.dq;
-        }
+        const int r = row0 + min(ar + AR * j, nrows - 1);
+        const size_t t = LIST_ROWS ? g.lists[lbase + r] : r;
+        arow[j] = (MODE == X_QK || MODE == X_V ? g.x + t * d.M
+                 : MODE == X_O ? g.ahat + t * HD + h * d.D
+                 : MODE == X_DA ? g.dy + t * d.M
+                 : MODE == X_DR ? g.dv + t * HD + h * d.D : g.dq + t * HD) + ac * 8;
       }
     }
+    const int acol = A_MN ? min(m0 + ac * 8, (MODE == X_DWO ? d.D : d.M) - 8) : 0;
+    const int bcol = !B_TMA ? min(n0 + bc * 8, (MODE == X_DWO ? d.M : MODE == X_DWQK && gates ? g.ldz : d.D) - 8) : 0;
+    const float* bsrc = MODE == X_DWO ? g.dy + bcol : MODE == X_DWV ? g.dv + h * d.D + bcol
+                      : MODE == X_DWQK ? (gates ? g.dz + bcol : (which ? g.dk : g.dq) + h * d.D + bcol) : nullptr;
+    const size_t bld = MODE == X_DWO ? d.M : MODE == X_DWQK && gates ? g.ldz : HD;
+    // lists: the entries of a step are fetched one step ahead of its rows
+    int ta[2] = {0, 0}, tb = 0;
+    float ga[2] = {0.f, 0.f};
+    auto fetch = [&](int i) {
+      if (LIST_K) {
 #pragma unroll
-    for (int j = 0; j < NB; ++j) {
-      const int r = br + BR * j;
-      brow[j] = nullptr;
-      if (!B_MN && r < ncols)
-        brow[j] = MODE == X_QK ? (gates ? g.wgate + (size_t)(n0 + r) * d.M : g.wqk + ((size_t)(which * d.H + h) * d.D + n0 + r) * d.M)
-                : MODE == X_V ? g.wv + ((size_t)(h * d.E + e) * d.D + n0 + r) * d.M
-                : g.wo + ((size_t)(h * d.E + e) * d.M + n0 + r) * d.D;
-    }
-    float ra[2][8], rb[NB][8], rg[2] = {1.f, 1.f};
+        for (int j = 0; j < 2; ++j) {
+          const int pos = kbeg + i * XG_BK + ar + AR * j;
+          if (pos < kend) { ta[j] = __ldg(g.lists + lbase + pos); ga[j] = __ldg(g.lgate + lbase + pos); }
+        }
+        const int pos = kbeg + i * XG_BK + br;
+        if (pos < kend) tb = __ldg(g.lists + lbase + pos);
+      }
+    };
+    int xseg = 0, xoff = 0;                                // X_DX: the step's head (of dq, then dk), and where in it
+    float ra[2][8], rb[8], rg[2];                          // the next step's pieces
     auto load = [&](int i) {
-      // A
       if (!A_MN) {
-        const int kv = kvalid(i);
-        int seg = 0, off = i * 64;
+        const float *p0, *p1;
         if (MODE == X_DX) {
-          seg = i / sps;
-          off = seg < 2 * d.H ? (i - seg * sps) * 64 : (i - 2 * d.H * sps) * 64;
-        }
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-          const float* p = arow[j];
-          if (MODE == X_DX && p) {
-            p = seg < d.H ? g.dq + (size_t)atok[j] * HD + seg * d.D
-              : seg < 2 * d.H ? g.dk + (size_t)atok[j] * HD + (seg - d.H) * d.D : g.dz + (size_t)atok[j] * g.ldz;
+          const long o = xseg < 2 * d.H ? (xseg >= d.H ? (long)(g.dk - g.dq) + (long)(xseg - d.H) * d.D : (long)xseg * d.D) + xoff : 0;
+          p0 = arow[0] + o; p1 = arow[1] + o;
+          if (xseg == 2 * d.H) {
+            p0 = g.dz + (size_t)(row0 + min(ar, nrows - 1)) * g.ldz + xoff + ac * 8;
+            p1 = g.dz + (size_t)(row0 + min(ar + AR, nrows - 1)) * g.ldz + xoff + ac * 8;
           }
-          load8(ra[j], p ? p + off + ac * 8 : nullptr, kv - ac * 8, MODE == X_DA ? g.vec_dy != 0 : true);
+          xoff += XG_BK;
+          if (xseg < 2 * d.H && xoff >= d.Dt) { xoff = 0; ++xseg; }
+        } else {
+          p0 = arow[0] + i * XG_BK; p1 = arow[1] + i * XG_BK;
         }
+        load8(ra[0], p0, vdy);
+        load8(ra[1], p1, vdy);
       } else {
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
-          const int pos = kbeg + i * 64 + ar + 32 * j;
-          const float* p = nullptr;
-          rg[j] = 1.f;
+          const int pos = kbeg + i * XG_BK + ar + AR * j;
+          rg[j] = ga[j];
           if (pos < kend) {
-            const int t = LIST_K ? g.lists[lbase + pos] : pos;
-            if (LIST_K) rg[j] = g.lgate[lbase + pos];
-            p = MODE == X_DWO ? g.ahat + (size_t)t * HD + h * d.D + m0 : g.x + (size_t)t * d.M + m0;
+            const size_t t = LIST_K ? ta[j] : pos;
+            load8(ra[j], (MODE == X_DWO ? g.ahat + t * HD + h * d.D : g.x + t * d.M) + acol, true);
+          } else {
+#pragma unroll
+            for (int x = 0; x < 8; ++x) ra[j][x] = 0.f;
           }
-          load8(ra[j], p ? p + ac * 8 : nullptr, nrows - ac * 8, true);
         }
       }
-      // B
-      if (!B_MN) {
-        const int kv = kvalid(i);
+      if (!B_TMA) {
+        const int pos = kbeg + i * XG_BK + br;
+        if (pos < kend) load8(rb, bsrc + (size_t)(LIST_K ? tb : pos) * bld, vdy);
+        else {
 #pragma unroll
-        for (int j = 0; j < NB; ++j) load8(rb[j], brow[j] ? brow[j] + i * 64 + bc * 8 : nullptr, kv - bc * 8, true);
-      } else {
-#pragma unroll
-        for (int j = 0; j < NB; ++j) {
-          const int kr = br + BR * j;
-          const float* p = nullptr;
-          if (MODE == X_DA) p = g.wo + ((size_t)(h * d.E + e) * d.M + i * 64 + kr) * d.D + n0;
-          if (MODE == X_DR && i * 64 + kr < d.Dt) p = g.wv + ((size_t)(h * d.E + e) * d.D + i * 64 + kr) * d.M + n0;
-          if (MODE == X_DX) {
-            const int seg = i / sps;
-            if (seg < 2 * d.H) {
-              const int dd = (i - seg * sps) * 64 + kr;
-              if (dd < d.Dt) p = g.wqk + ((size_t)seg * d.D + dd) * d.M + n0;
-            } else {
-              const int gc = (i - 2 * d.H * sps) * 64 + kr;
-              if (gc < d.G) p = g.wgate + (size_t)gc * d.M + n0;
-            }
-          }
-          if (LIST_K || MODE == X_DWQK) {
-            const int pos = kbeg + i * 64 + kr;
-            if (pos < kend) {
-              const int t = LIST_K ? g.lists[lbase + pos] : pos;
-              p = MODE == X_DWO ? g.dy + (size_t)t * d.M + n0
-                : MODE == X_DWV ? g.dv + (size_t)t * HD + h * d.D + n0
-                : gates ? g.dz + (size_t)t * g.ldz + n0
-                : (which ? g.dk : g.dq) + (size_t)t * HD + h * d.D + n0;
-            }
-          }
-          load8(rb[j], p ? p + bc * 8 : nullptr, ncols - bc * 8, MODE == X_DWO ? g.vec_dy != 0 : true);
+          for (int x = 0; x < 8; ++x) rb[x] = 0.f;
         }
       }
+      if (i + 1 < steps) fetch(i + 1);
     };
     const int q = warp & 3, cb = warp >> 2;
     const uint32_t tlane = ((uint32_t)(q * 32) << 16) + cb * COLS;
     float acc[COLS];
 #pragma unroll
     for (int i = 0; i < COLS; ++i) acc[i] = 0.f;
-    const bool mine = cb * COLS < nmma;                    // (whole warps: columns past the tile's are not computed)
+    const bool mine = cb * COLS < ncols;                   // (whole warps)
     auto promote = [&](int c) {
-      const int b = c & 1;
-      if (!mbar_wait(&acc_full[b], (c >> 1) & 1, g.status, dead)) return;
+      if (!mbar_wait(acc_full, c & 1, g.status, dead)) return;
       tc_fence_after();
       if (mine) {
-        float t[COLS];
-        tmem_ld_n<COLS>(tmem + b * BN + tlane, t);
 #pragma unroll
-        for (int i = 0; i < COLS; ++i) acc[i] += t[i];
+        for (int c0 = 0; c0 < COLS; c0 += 16) {
+          float t[16];
+#pragma unroll
+          for (int i = 0; i < 16; ++i) t[i] = 0.f;
+          tmem_add<16>(tmem + 128 + tlane + c0, t);          // (smallest first)
+          tmem_add<16>(tmem + 64 + tlane + c0, t);
+          tmem_add<16>(tmem + tlane + c0, t);
+#pragma unroll
+          for (int i = 0; i < 16; ++i) acc[c0 + i] += t[i];
+        }
       }
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(&acc_empty[b]);
+      if (lane == 0) mbar_arrive(acc_empty);
     };
-    if (steps > 0) load(0);
-    if (MODE == X_QK) {
-      const long n = (long)gridDim.x * gridDim.y * XG_WORKERS, i0 = ((long)blockIdx.y * gridDim.x + blockIdx.x) * XG_WORKERS + tid;
-      for (long i = i0; i < g.nzero0; i += n) reinterpret_cast<float4*>(g.zero0)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-      for (long i = i0; i < g.nzero1; i += n) reinterpret_cast<float4*>(g.zero1)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-    for (int i = 0; i < steps; ++i) {
-      const int s = i & 1;
-      if (i >= 2 && !mbar_wait(&empty_bar[s], ((i >> 1) & 1) ^ 1, g.status, dead)) break;
+    if (steps > 0) { fetch(0); load(0); }
+    int s = 0, done = 0;                                   // done: chunks promoted
+    uint32_t par = 1;
+    for (int i = 0; i < steps && !dead; ++i) {
+      if (!mbar_wait(&empty_bar[s], par, g.status, dead)) break;
       unsigned char* at = sgen + s * SM::STAGE;
-      unsigned char* bt = at + 3 * SM::A_PLANE;
 #pragma unroll
       for (int j = 0; j < 2; ++j) {
         if (LIST_K) {
@@ -433,25 +450,16 @@ sh_f32_gemm_kernel(const __grid_constant__ XGemmArgs g) {
         }
         store_planes(at, aoff[j], SM::A_PLANE, ra[j]);
       }
-#pragma unroll
-      for (int j = 0; j < NB; ++j) store_planes(bt, boff[j], SM::B_PLANE, rb[j]);
+      if (!B_TMA) store_planes(at + 3 * SM::A_PLANE, boff, SM::B_PLANE, rb);
       fence_proxy_async_smem();
       __syncwarp();
       if (lane == 0) mbar_arrive(&full_bar[s]);
+      if (++s == XG_STAGES) { s = 0; par ^= 1; }
       if (i + 1 < steps) load(i + 1);
-      if (i % XG_CHUNK == XG_CHUNK - 1 && i / XG_CHUNK >= 1) promote(i / XG_CHUNK - 1);
+      // a chunk is read once two steps of the next one are in shared memory
+      if (i % XG_CHUNK == 1 && i > XG_CHUNK) promote(done++);
     }
-    // chunks not read yet: the last one, and the one before it when the last is a short one
-    if (steps > 0) {
-      const int done = steps / XG_CHUNK >= 1 ? steps / XG_CHUNK - 1 : 0;      // chunks promoted in the loop
-      for (int c = done; c < chunks; ++c) promote(c);
-      if (mine && !dead) {
-        float t[COLS];
-        tmem_ld_n<COLS>(corr + tlane, t);                  // (complete: the last chunk's commit came behind its UMMAs)
-#pragma unroll
-        for (int i = 0; i < COLS; ++i) acc[i] += t[i];
-      }
-    }
+    for (; done < (steps + XG_CHUNK - 1) / XG_CHUNK && !dead; ++done) promote(done);
     // ---- result: thread = row q*32 + lane, columns cb*COLS ... ------------------------------------
     const int r = q * 32 + lane, c0 = cb * COLS;
     const int valid = min(COLS, ncols - c0);
@@ -479,17 +487,6 @@ sh_f32_gemm_kernel(const __grid_constant__ XGemmArgs g) {
         const float f = MODE == X_V && g.vscale != 0.f ? gt * g.vscale : gt;
 #pragma unroll
         for (int i = 0; i < COLS; ++i) acc[i] *= f;
-        if (MODE == X_V) {
-          const int b = t / d.T, tt = t % d.T;
-          red_row(g.v + (((size_t)b * d.H + h) * d.T + tt) * d.D + n0 + c0, acc, valid, true);
-        } else if (MODE == X_O) {
-          const int orow = sh_out_row(d, t);               // (cache tokens have no output row)
-          if (orow >= 0) red_row(g.y + (size_t)orow * d.M + n0 + c0, acc, valid, true);
-        } else if (MODE == X_DA) {
-          red_row(g.dahat + (size_t)t * HD + h * d.D + n0 + c0, acc, valid, true);
-        } else {
-          red_row(g.dx + (size_t)t * d.M + n0 + c0, acc, valid, g.vec_out != 0);
-        }
       } else if (LIST_K) {
         // dWo [(h*E + e)*Dt + dd][m]; dWv [(h*E + e)*M + m][dd < Dt]
         float* o = MODE == X_DWO ? g.dWo + ((size_t)(h * d.E + e) * d.Dt + m0 + r) * d.M + n0 + c0
@@ -529,43 +526,88 @@ sh_f32_gemm_kernel(const __grid_constant__ XGemmArgs g) {
         }
       } else {                                             // X_QK
         const int tok = row0 + r;
-        if (gates) {
-          store_row(g.z + (size_t)tok * g.ldz + n0 + c0, acc, valid, true);
-        } else {
-          const int b = tok / d.T, t = tok % d.T;
-          if (g.rope) {
-            const float2* cs = g.rope + (size_t)((n0 + c0) >> 1) * d.T + t;
+        if (g.rope) {
+          const float2* cs = g.rope + (size_t)((n0 + c0) >> 1) * d.T + tok % d.T;
 #pragma unroll
-            for (int i = 0; i < COLS; i += 2)
-              if (i < valid) {
-                const float2 w = cs[(size_t)(i >> 1) * d.T];
-                const float a0 = acc[i], a1 = acc[i + 1];
-                acc[i] = a0 * w.x - a1 * w.y;
-                acc[i + 1] = a0 * w.y + a1 * w.x;
-              }
-          }
-          if (which == 0) {
+          for (int i = 0; i < COLS; i += 2)
+            if (i < valid) {
+              const float2 w = cs[(size_t)(i >> 1) * d.T];
+              const float a0 = acc[i], a1 = acc[i + 1];
+              acc[i] = a0 * w.x - a1 * w.y;
+              acc[i + 1] = a0 * w.y + a1 * w.x;
+            }
+        }
+        if (which == 0) {
 #pragma unroll
-            for (int i = 0; i < COLS; ++i) acc[i] *= g.qscale;
-          }
-          // (columns between d_head and its stored width: zero, as the padded weight rows would give)
-          float* o = (which ? g.k : g.q) + (((size_t)b * d.H + h) * d.T + t) * d.D + n0 + c0;
-          store_row(o, acc, valid, true);
+          for (int i = 0; i < COLS; ++i) acc[i] *= g.qscale;
         }
       }
     }
-    if (MODE == X_QK && !gates && n0 + ncols >= d.Dt && d.D > d.Dt && !dead && cb == 0 && r < nrows) {
-      const int tok = row0 + r, b = tok / d.T, t = tok % d.T;
-      float* o = (which ? g.k : g.q) + (((size_t)b * d.H + h) * d.T + t) * d.D;
-      for (int i = d.Dt; i < d.D; ++i) o[i] = 0.f;
+    if (BULK) {
+      // rows through shared memory (the operand stages are free: every UMMA has been waited for), 16 bytes of
+      // padding a row so that eight lanes' 16-byte stores meet different banks
+      constexpr int LD = BN + 4;
+      float* stg = reinterpret_cast<float*>(sgen);
+      if (r < nrows && valid > 0 && !dead) {
+#pragma unroll
+        for (int i = 0; i < COLS; i += 4)
+          *reinterpret_cast<float4*>(stg + r * LD + c0 + i) = make_float4(acc[i], acc[i + 1], acc[i + 2], acc[i + 3]);
+      }
+      fence_proxy_async_smem();
+      asm volatile("bar.sync 1, 256;" ::: "memory");
+      if (tid < nrows && !dead) {
+        // (whole 16-byte pieces: the columns that pad the last one of a head are zero columns of its stored width)
+        const int n = (ncols + 3) & ~3;
+        float* o = nullptr;
+        if (LIST_ROWS) {
+          const int t = g.lists[lbase + row0 + tid];
+          if (MODE == X_V) o = g.v + (((size_t)(t / d.T) * d.H + h) * d.T + t % d.T) * d.D + n0;
+          if (MODE == X_O) { const int orow = sh_out_row(d, t); if (orow >= 0) o = g.y + (size_t)orow * d.M + n0; }   // (cache tokens have no output row)
+          if (MODE == X_DA) o = g.dahat + (size_t)t * HD + h * d.D + n0;
+          if (MODE == X_DR) o = g.dx + (size_t)t * d.M + n0;
+        } else {
+          const int tok = row0 + tid;
+          o = (which ? g.k : g.q) + (((size_t)(tok / d.T) * d.H + h) * d.T + tok % d.T) * d.D + n0;
+        }
+        if (o) {
+          const uint32_t src = smem_u32(stg + tid * LD);
+          if (MODE == X_QK) bulk_store(o, src, n * 4);
+          else if (MODE != X_DR || g.vec_out) bulk_reduce_add_f32(o, src, n * 4);
+          else
+            for (int i = 0; i < n; ++i) atomicAdd(o + i, stg[tid * LD + i]);
+        }
+        bulk_commit();
+        bulk_wait_all();
+      }
     }
   }
   tc_fence_before();
   __syncthreads();
-  if (warp == 16) {
+  if (warp == 8) {
     tc_fence_after();
-    tmem_dealloc(tmem, BN == 128 ? 512 : 256);
+    tmem_dealloc(tmem, 256);
   }
+}
+
+// Block number i of a mode's gx x gy x gz tiles.
+__device__ __forceinline__ XTile xg_unpack(int i, int gx, int gy) { return {i % gx, i / gx % gy, i / (gx * gy)}; }
+
+// A launch of up to three modes whose tiles do not depend on one another: the first n0 blocks work on
+// tiles of mode A, the next n1 on mode B, the rest on mode C.  (One launch each leaves half of the block
+// slots idle in its last round, and pays its set-up and drain by itself.)
+struct XPart { CUtensorMap w; XGemmArgs g; int gx, gy, n; };
+template <int A, int B, int C>
+__global__ void __launch_bounds__(XG_THREADS, 2)
+sh_f32_gemm_kernel(const __grid_constant__ CUtensorMap mapG, const __grid_constant__ XPart pa, const __grid_constant__ XPart pb,
+                   const __grid_constant__ XPart pc) {
+  int i = blockIdx.x;
+  if (i < pa.n) { xg_tile<A>(pa.w, mapG, pa.g, xg_unpack(i, pa.gx, pa.gy)); return; }
+  i -= pa.n;
+  if (B >= 0) {
+    if (i < pb.n) { xg_tile<(B >= 0 ? B : A)>(pb.w, mapG, pb.g, xg_unpack(i, pb.gx, pb.gy)); return; }
+    i -= pb.n;
+  }
+  if (C >= 0) xg_tile<(C >= 0 ? C : A)>(pc.w, mapG, pc.g, xg_unpack(i, pc.gx, pc.gy));
 }
 
 }  // namespace shtc

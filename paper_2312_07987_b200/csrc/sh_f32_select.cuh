@@ -1,18 +1,112 @@
-// Selection and bucket sort of the fp32 configuration, one launch.
-//
-// Block = (side, head): top-k of every token's logits (a larger logit first, the lower index on a
-// tie), sigmoid of the chosen ones, and the stable counting sort of the tokens by chosen expert, in two
-// sweeps of 1024 tokens at a time (totals, then placement).  No block needs another's counts: every
-// head owns a fixed range of the row-tile table (mt = (N k + 127 E) / 128 entries, the unused ones
-// empty).  What bounds it is latency (two sweeps of a few dependent loads): a block per 128 tokens
-// with a histogram exchange between two kernels took 490 + 13 us on 1024 tokens of 32 gate columns,
-// this one and the gate columns of the projection GEMM a few us.
+// Gates, selection and bucket sort of the fp32 configuration.
 #pragma once
 #include "sh_internal.cuh"
 
+// Logits, top-k (a larger logit first, the lower index on a tie) and sigmoid of the chosen ones, on the
+// CUDA cores: TOK tokens per block with their rows in shared memory (512 columns at a time), a warp per
+// gate column, lanes along d_model.  The block also clears its share of the buffers that later kernels
+// add into.  What bounds it is the latency of its few loads, so blocks are small: 1024 tokens of 32 gate
+// columns took 490 us in blocks of 128 tokens with a warp per token.
+template <int TOK>
+static __global__ void __launch_bounds__(256)
+sh_f32_gate_kernel(const float* __restrict__ x, const float* __restrict__ wgate, const float* __restrict__ gbias, int* __restrict__ idx,
+                   float* __restrict__ gate, float4* __restrict__ zero0, long nzero0, float4* __restrict__ zero1, long nzero1, ShDims d) {
+  extern __shared__ __align__(16) float gsm[];             // [TOK][512] of x, then [TOK][G] logits
+  float* s_z = gsm + TOK * 512;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int t0 = blockIdx.x * TOK;
+  const long nthr = (long)gridDim.x * 256, me = (long)blockIdx.x * 256 + tid;
+  for (int m0 = 0; m0 < d.M; m0 += 512) {
+    const int mw = min(512, d.M - m0);                     // a multiple of 64
+    __syncthreads();
+    for (int i = tid; i < TOK * 128; i += 256) {
+      const int r = i >> 7, c = (i & 127) * 4;
+      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (c < mw && t0 + r < d.N) v = __ldg(reinterpret_cast<const float4*>(x + (size_t)(t0 + r) * d.M + m0 + c));
+      *reinterpret_cast<float4*>(gsm + r * 512 + c) = v;
+    }
+    if (m0 == 0) {
+      for (long i = me; i < nzero0; i += nthr) zero0[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+      for (long i = me; i < nzero1; i += nthr) zero1[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    __syncthreads();
+    for (int g = warp; g < d.G; g += 16) {                  // two columns at a time: eight 16-byte loads in flight per lane
+      const bool two = g + 8 < d.G;
+      const float* w0 = wgate + (size_t)g * d.M + m0;
+      const float* w1 = w0 + (two ? (size_t)8 * d.M : 0);
+      float4 wv[2][4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int c = u * 128 + lane * 4;
+        wv[0][u] = wv[1][u] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (c < mw) { wv[0][u] = __ldg(reinterpret_cast<const float4*>(w0 + c)); wv[1][u] = __ldg(reinterpret_cast<const float4*>(w1 + c)); }
+      }
+      float acc[2][TOK];
+#pragma unroll
+      for (int r = 0; r < TOK; ++r) {
+        acc[0][r] = acc[1][r] = 0.f;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const float4 xv = *reinterpret_cast<const float4*>(gsm + r * 512 + u * 128 + lane * 4);
+#pragma unroll
+          for (int q = 0; q < 2; ++q)
+            acc[q][r] = fmaf(xv.x, wv[q][u].x, fmaf(xv.y, wv[q][u].y, fmaf(xv.z, wv[q][u].z, fmaf(xv.w, wv[q][u].w, acc[q][r]))));
+        }
+      }
+      // lane sums of TOK tokens: at each step a lane keeps half of its tokens and hands the others over
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        int tokn = 0;
+#pragma unroll
+        for (int n = TOK / 2, o = 16; n >= 1; n >>= 1, o >>= 1) {
+          const bool up = (lane & o) != 0;
+#pragma unroll
+          for (int r = 0; r < n; ++r) {
+            const float give = up ? acc[q][r] : acc[q][r + n], keep = up ? acc[q][r + n] : acc[q][r];
+            acc[q][r] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+          }
+          tokn += up ? n : 0;
+        }
+#pragma unroll
+        for (int o = 32 / TOK / 2; o > 0; o >>= 1) acc[q][0] += __shfl_xor_sync(0xffffffffu, acc[q][0], o);
+        if (lane % (32 / TOK) == 0 && (q == 0 || two)) {
+          float* z = s_z + tokn * d.G + g + 8 * q;
+          *z = (m0 == 0 ? 0.f : *z) + acc[q][0];
+        }
+      }
+    }
+  }
+  __syncthreads();
+  const int groups = d.sides * d.H;
+  for (int i = tid; i < TOK * groups; i += 256) {
+    const int r = i / groups, grp = i % groups, side = grp / d.H, h = grp % d.H, t = t0 + r;
+    if (t >= d.N) continue;
+    float* z = s_z + r * d.G + grp * d.E;
+    for (int e = 0; e < d.E; ++e) z[e] += gbias[grp * d.E + e];
+    const size_t o = (((size_t)side * d.N + t) * d.H + h) * d.k;
+    unsigned sel = 0;
+    for (int j = 0; j < d.k; ++j) {
+      float best = 0.f;
+      int pick = -1;
+      for (int e = 0; e < d.E; ++e) {
+        const float v = z[e];
+        if (!((sel >> e) & 1u) && (pick < 0 || v > best)) { best = v; pick = e; }
+      }
+      sel |= 1u << pick;
+      idx[o + j] = pick;
+      gate[o + j] = 1.f / (1.f + expf(-best));
+    }
+  }
+}
+
+// Bucket sort, one block per (side, head): the stable counting sort of the tokens by chosen expert, in
+// two sweeps of 1024 tokens at a time (totals, then placement).  No block needs another's counts: every
+// head owns a fixed range of the row-tile table (mt = (N k + 127 E) / 128 entries, the unused ones empty).
 static __global__ void __launch_bounds__(1024)
-sh_f32_select_kernel(const float* __restrict__ z, int ldz, const float* __restrict__ gbias, int* __restrict__ idx, float* __restrict__ gate,
-                     int* __restrict__ offsets, int* __restrict__ lists, float* __restrict__ lgate, ShTile* __restrict__ tiles, ShDims d, int mt) {
+sh_f32_sort_kernel(const int* __restrict__ idx, const float* __restrict__ gate, int* __restrict__ offsets, int* __restrict__ lists,
+                   float* __restrict__ lgate, ShTile* __restrict__ tiles, ShDims d, int mt) {
   __shared__ int s_tot[32], s_off[33], s_run[32];
   __shared__ int s_w[32][33];                              // [warp][expert]
   __shared__ int s_tile[33];
@@ -20,27 +114,16 @@ sh_f32_select_kernel(const float* __restrict__ z, int ldz, const float* __restri
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int grp = blockIdx.x, side = grp / d.H, h = grp % d.H;
-  const float bias = lane < d.E ? gbias[grp * d.E + lane] : 0.f;
   if (tid < 32) s_tot[tid] = 0;
   __syncthreads();
   int mine = 0;                                            // lane e: selections of expert e by this warp's tokens
   for (int t0 = 0; t0 < d.N; t0 += 1024) {
     const int t = t0 + tid;
     unsigned sel = 0;
-    const bool live = t < d.N;
-    const float* zr = z + (size_t)(live ? t : 0) * ldz + grp * d.E;
-    const size_t o = (((size_t)side * d.N + t) * d.H + h) * d.k;
-    for (int j = 0; j < d.k; ++j) {
-      float best = 0.f;
-      int pick = -1;
-      for (int e = 0; e < d.E; ++e) {
-        const float v = zr[e] + __shfl_sync(0xffffffffu, bias, e);
-        if (!((sel >> e) & 1u) && (pick < 0 || v > best)) { best = v; pick = e; }
-      }
-      sel |= 1u << pick;
-      if (live) { idx[o + j] = pick; gate[o + j] = 1.f / (1.f + expf(-best)); }
+    if (t < d.N) {
+      const size_t o = (((size_t)side * d.N + t) * d.H + h) * d.k;
+      for (int j = 0; j < d.k; ++j) sel |= 1u << idx[o + j];
     }
-    if (!live) sel = 0;
     for (int e = 0; e < d.E; ++e) {
       const unsigned bal = __ballot_sync(0xffffffffu, (sel >> e) & 1u);
       if (lane == e) mine += __popc(bal);
@@ -80,7 +163,7 @@ sh_f32_select_kernel(const float* __restrict__ z, int ldz, const float* __restri
     const size_t o = (((size_t)side * d.N + t) * d.H + h) * d.k;
     unsigned sel = 0;
     if (live)
-      for (int j = 0; j < d.k; ++j) sel |= 1u << idx[o + j];           // (this thread's own entries)
+      for (int j = 0; j < d.k; ++j) sel |= 1u << idx[o + j];
     for (int e = 0; e < d.E; ++e) {
       const unsigned bal = __ballot_sync(0xffffffffu, (sel >> e) & 1u);
       if (lane == e) s_w[warp][e] = __popc(bal);

@@ -89,7 +89,7 @@ __device__ __forceinline__ void sh_stamp_end(unsigned long long* s, int k) { if 
 
 struct ShWorkspace {
   size_t status, wqk, wgate, gbias, wv, wo, q, k, v, ahat, idx, gate, blockcnt, blockoff,
-         offsets, lists, lgate, tiles, ntiles, rope, vearly, vearly_cnt, xl_emb, xl_r, xl_uv, xl_r16, xl_vr, xl_uk, xl_bias, wos, gid, wq_e, wk_e, bw, f32z, f32stats, stamps, total;
+         offsets, lists, lgate, tiles, ntiles, rope, vearly, vearly_cnt, xl_emb, xl_r, xl_uv, xl_r16, xl_vr, xl_uk, xl_bias, wos, gid, wq_e, wk_e, bw, wgate32, f32stats, stamps, total;
 };
 
 // Words of the 256-byte status block at the start of the workspace.
@@ -123,6 +123,7 @@ struct sh_layer {
   int launches = 0;
   int sm_count = 0;
   void* tc = nullptr;      // tensor-core path state (tensor maps), owned by the layer
+  void* f32 = nullptr;     // fp32 configuration: tensor maps of the split weights, owned by the layer
   cudaEvent_t* ev = nullptr;  // when set (sh_forward_timed): 6 events recorded at the stage boundaries
   size_t guard_off[SH_MAX_GUARDS] = {};   // byte offsets of the guards behind the workspace sub-buffers
   int n_guards = 0;
@@ -188,7 +189,9 @@ enum { SH_STAGE_GATE = 1, SH_STAGE_QK = 2, SH_STAGE_V = 4, SH_STAGE_ATTN = 8, SH
 int sh_simt_run_bf16(sh_layer* L, int stages, const void* x, void* out, cudaStream_t st);
 
 // fp32 configuration of the SwitchHead layer (sh_f32.cu).
-inline int sh_f32_ldz(const ShDims& d) { return (d.G + 7) / 8 * 8; }       // row length of the gate-logit / gate-gradient matrix
+inline int sh_f32_ldz(const ShDims& d) { return (d.G + 31) / 32 * 32; }       // row length of the gate-gradient matrix
+int sh_f32_prepare(sh_layer* L);                // tensor maps, after the weights are split
+void sh_f32_release(sh_layer* L);
 int sh_f32_gate_sort(sh_layer* L, const void* x, cudaStream_t st);
 int sh_f32_forward(sh_layer* L, const void* x, void* out, cudaStream_t st);
 int sh_f32_backward(sh_layer* L, const void* x, const float* dout, float* dx, float* dWq, float* dWk, float* dWv,

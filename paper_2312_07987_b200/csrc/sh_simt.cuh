@@ -21,6 +21,25 @@ __global__ void sh_repack_kernel(const TI* __restrict__ in, TO* __restrict__ out
   }
 }
 
+// The same into three bf16 planes, `plane` elements apart, whose sum is the fp32 value (fp32 configuration).
+static __global__ void sh_repack_split_kernel(const float* __restrict__ in, __nv_bfloat16* __restrict__ out, int batch, int rows,
+                                              int cols, long obs, long ors, long oes, long plane) {
+  const long total = (long)batch * rows * cols;
+  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < total; i += (long)gridDim.x * blockDim.x) {
+    const int r = (int)(i % rows);
+    const long t = i / rows;
+    const int c = (int)(t % cols), b = (int)(t / cols);
+    float v = in[((long)b * rows + r) * cols + c];
+    __nv_bfloat16* o = out + b * obs + c * ors + r * oes;
+#pragma unroll
+    for (int p = 0; p < 3; ++p) {
+      const __nv_bfloat16 w = __float2bfloat16_rn(v);
+      o[p * plane] = w;
+      v -= __bfloat162float(w);
+    }
+  }
+}
+
 // ---------------------------------------------------------------------------------------
 // Gate: z = x W (+ b) per (side, head), sigmoid, top-k with lower-index-wins, per-block
 // histogram of the selections (Sec. 2.2: s = sigmoid(x W_S), E = arg top-k).

@@ -53,6 +53,22 @@ int sh_tc_encode_2d(CUtensorMap* map, int elem_kind, const void* base, uint64_t 
   return SH_OK;
 }
 
+// Three bf16 planes [3, rows, inner] of an fp32 matrix, box = box_rows rows of box_inner
+// (32: 64-byte swizzle, 64: 128-byte swizzle) elements of all three.
+int sh_tc_encode_planes(CUtensorMap* map, const void* base, uint64_t inner, uint64_t rows, uint32_t box_inner, uint32_t box_rows) {
+  EncodeTiledFn enc = get_encode();
+  if (!enc) { sh_set_error("cuTensorMapEncodeTiled is not available from the driver"); return SH_ERR_CUDA; }
+  cuuint64_t dims[3] = {inner, rows, 3};
+  cuuint64_t strides[2] = {inner * 2, inner * rows * 2};
+  cuuint32_t box[3] = {box_inner, box_rows, 3};
+  cuuint32_t estr[3] = {1, 1, 1};
+  CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
+                   CU_TENSOR_MAP_INTERLEAVE_NONE, box_inner == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r != CUDA_SUCCESS) { sh_set_error("cuTensorMapEncodeTiled (planes) failed with CUresult %d", (int)r); return SH_ERR_CUDA; }
+  return SH_OK;
+}
+
 // 3-D tensor [n2, n1, inner] of fp16 (Q, K, V as [B*H, T, D]); box = 128 (or `rows`) rows of 64 elements of
 // one (batch, head) slice, so rows past the end of a sequence read as zero.
 static int encode_3d_f16(CUtensorMap* map, const void* base, uint64_t inner, uint64_t n1, uint64_t n2, uint32_t rows = 128) {

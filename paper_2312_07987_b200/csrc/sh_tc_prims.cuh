@@ -105,6 +105,10 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map
 __device__ __forceinline__ void bulk_reduce_add_f32(float* gdst, uint32_t ssrc, uint32_t bytes) {
   asm volatile("cp.reduce.async.bulk.global.shared::cta.bulk_group.add.f32 [%0], [%1], %2;" ::"l"(gdst), "r"(ssrc), "r"(bytes) : "memory");
 }
+// Copy of a contiguous run from shared to global memory (the same alignment rules).
+__device__ __forceinline__ void bulk_store(float* gdst, uint32_t ssrc, uint32_t bytes) {
+  asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(gdst), "r"(ssrc), "r"(bytes) : "memory");
+}
 // Tile store from this CTA's shared memory (bulk async-group completion: bulk_commit / bulk_wait_*).
 __device__ __forceinline__ void tma_store_3d(const CUtensorMap* map, uint32_t src, int x, int y, int z) {
   asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%2, %3, %4}], [%1];"
@@ -370,3 +374,4 @@ __device__ __forceinline__ void red_add_v4_f16x2(__half* dst, uint32_t a, uint32
 // Host: tensor-map encoding through the driver entry point (no link-time libcuda dependency).
 int sh_tc_encode_2d(CUtensorMap* map, int elem_kind /*0 = bf16, 1 = f16*/, const void* base, uint64_t inner,
                     uint64_t outer, uint64_t outer_stride_bytes, uint32_t box_inner, uint32_t box_outer);
+int sh_tc_encode_planes(CUtensorMap* map, const void* base, uint64_t inner, uint64_t rows, uint32_t box_inner, uint32_t box_rows);
