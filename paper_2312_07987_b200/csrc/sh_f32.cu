@@ -4,6 +4,7 @@
 #include "sh_internal.cuh"
 #include "sh_launch.cuh"
 #include "sh_f32_gemm.cuh"
+#include "sh_f32_wgrad.cuh"
 #include "sh_f32_attn.cuh"
 #include "sh_f32_select.cuh"
 
@@ -42,15 +43,15 @@ XPart part(sh_layer* L, const XGemmArgs& g, int gx, int gy, int gz = 1, const Pl
   return p;
 }
 
-template <int A, int B = -1, int C = -1>
-int launch_x(sh_layer* L, cudaStream_t st, const XPart& a, const XPart& b = XPart(), const XPart& c = XPart()) {
+template <int A, int B = -1>
+int launch_x(sh_layer* L, cudaStream_t st, const XPart& a, const XPart& b = XPart()) {
   const F32State* S = (const F32State*)L->f32;
-  const int n = a.n + (B >= 0 ? b.n : 0) + (C >= 0 ? c.n : 0);
+  const int n = a.n + (B >= 0 ? b.n : 0);
   if (n == 0) return SH_OK;
-  auto kern = sh_f32_gemm_kernel<A, B, C>;
+  auto kern = sh_f32_gemm_kernel<A, B>;
   if (int rc = set_smem(kern, XGemmSmem::TOTAL)) return rc;
   L->launches += 1;
-  return launch_k(true, kern, dim3((unsigned)n), dim3(XG_THREADS), XGemmSmem::TOTAL, st, S->wgate.mn, a, b, c);
+  return launch_k(true, kern, dim3((unsigned)n), dim3(XG_THREADS), XGemmSmem::TOTAL, st, S->wgate.mn, a, b);
 }
 
 // Column tiles over `cols` columns: how many, and how wide (a multiple of 16).
@@ -176,7 +177,7 @@ int launch_attn_bw_t(sh_layer* L, const BwBuffers& w, cudaStream_t st) {
 
 // Parts of a contraction over tokens: enough blocks for the device, at least eight steps each.
 int k_parts(sh_layer* L, long blocks, long steps) {
-  long p = (2 * sm_count(L) + blocks - 1) / blocks;
+  long p = (sm_count(L) + blocks - 1) / blocks;
   const long most = steps / 8 < 1 ? 1 : steps / 8;
   p = p > most ? most : p;
   return p < 1 ? 1 : (int)p;
@@ -282,37 +283,39 @@ int sh_f32_backward(sh_layer* L, const void* x, const float* dout, float* dx, fl
   rc = d.D == 32 ? launch_attn_bw_t<32>(L, w, st) : d.D == 64 ? launch_attn_bw_t<64>(L, w, st)
      : d.D == 128 ? launch_attn_bw_t<128>(L, w, st) : launch_attn_bw_t<256>(L, w, st);
   if (rc) return rc;
-  // value experts: their part of dx and the source gates' gradients; beside it the expert weights' gradients
-  // (contractions over the experts' lists, in parts where the whole launch would leave block slots idle)
+  // value experts: their part of dx, and the source gates' gradients
   g = src;
   col_tiles(g, d.M);
-  const XPart dr = part<X_DR>(L, g, d.H * ht, g.nsub);
-  const long list_steps = ((long)d.N * d.k / d.E + XG_BK - 1) / XG_BK;
-  XGemmArgs gv = src, go = dst;
-  col_tiles(gv, d.Dt); col_tiles(go, d.M);
-  gv.ksplit = go.ksplit = k_parts(L, (long)d.H * d.E * (mt * gv.nsub + dt * go.nsub), list_steps);
-  if (gv.ksplit > 1) {
-    SH_CUDA_CHECK(cudaMemsetAsync(dWv, 0, (size_t)d.H * d.E * d.M * d.Dt * 4, st));
-    SH_CUDA_CHECK(cudaMemsetAsync(dWo, 0, (size_t)d.H * d.E * d.Dt * d.M * 4, st));
-  }
-  if ((rc = launch_x<X_DWV, X_DWO, X_DR>(L, st, part<X_DWV>(L, gv, d.H * d.E * gv.ksplit, gv.nsub, mt),
-                                         part<X_DWO>(L, go, d.H * d.E * go.ksplit, go.nsub, dt), dr))) return rc;
+  if ((rc = launch_x<X_DR>(L, st, part<X_DR>(L, g, d.H * ht, g.nsub)))) return rc;
   if ((rc = launch_k(true, sh_f32_dz_kernel, dim3((unsigned)(((long)d.N * d.k + 255) / 256), 2 * d.H), dim3(256), 0, st, (const float*)w.ds,
                      (const int*)(ws + L->o.lists), (const float*)(ws + L->o.lgate), (const int*)(ws + L->o.offsets), w.dz, src.ldz, d))) return rc;
-  // queries, keys and gates: the rest of dx, and the weight gradients
-  XGemmArgs gx = src, gw = src;
-  col_tiles(gx, d.M); col_tiles(gw, d.Dt);
-  gw.qk_first = 0; gw.qk_groups = 2 * d.H;
-  const int ct = gw.qk_groups * gw.nsub + (d.G + XG_BN - 1) / XG_BN;
-  gw.ksplit = k_parts(L, (long)mt * ct + (long)d.nblk * gx.nsub, (d.N + XG_BK - 1) / XG_BK);
-  if (gw.ksplit > 1) {
+  // queries, keys and gates: the rest of dx
+  g = src;
+  col_tiles(g, d.M);
+  if ((rc = launch_x<X_DX>(L, st, part<X_DX>(L, g, d.nblk, g.nsub)))) return rc;
+  // weight gradients, one launch; contractions in parts where whole ones would leave SMs without a tile
+  auto wpart = [](const XGemmArgs& a, int gx, int gy, int gz) { XWPart p; p.g = a; p.gx = gx; p.gy = gy; p.n = gx * gy * gz; return p; };
+  XGemmArgs gq = src, gv = src, go = dst;
+  col_tiles(gq, d.Dt); col_tiles(gv, d.Dt); col_tiles(go, d.M);
+  gq.qk_groups = 2 * d.H;
+  const int ct = gq.qk_groups * gq.nsub + (d.G + XG_BN - 1) / XG_BN;
+  const long blocks = (long)mt * ct + (long)d.H * d.E * (mt * gv.nsub + dt * go.nsub);
+  gq.ksplit = k_parts(L, blocks, (d.N + XG_BK - 1) / XG_BK);
+  gv.ksplit = go.ksplit = k_parts(L, blocks, ((long)d.N * d.k / d.E + XG_BK - 1) / XG_BK);
+  if (gq.ksplit > 1) {
     SH_CUDA_CHECK(cudaMemsetAsync(dWq, 0, (size_t)d.H * d.M * d.Dt * 4, st));
     SH_CUDA_CHECK(cudaMemsetAsync(dWk, 0, (size_t)d.H * d.M * d.Dt * 4, st));
     SH_CUDA_CHECK(cudaMemsetAsync(dWs, 0, (size_t)d.H * d.M * d.E * 4, st));
     SH_CUDA_CHECK(cudaMemsetAsync(dWd, 0, (size_t)d.H * d.M * d.E * 4, st));
   }
-  if ((rc = launch_x<X_DX, X_DWQK>(L, st, part<X_DX>(L, gx, d.nblk, gx.nsub), part<X_DWQK>(L, gw, mt, ct, gw.ksplit)))) return rc;
+  if (gv.ksplit > 1) {
+    SH_CUDA_CHECK(cudaMemsetAsync(dWv, 0, (size_t)d.H * d.E * d.M * d.Dt * 4, st));
+    SH_CUDA_CHECK(cudaMemsetAsync(dWo, 0, (size_t)d.H * d.E * d.Dt * d.M * 4, st));
+  }
+  const XWPart pq = wpart(gq, mt, ct, gq.ksplit), pv = wpart(gv, d.H * d.E * gv.ksplit, gv.nsub, mt), po = wpart(go, d.H * d.E * go.ksplit, go.nsub, dt);
+  if ((rc = set_smem(sh_f32_wgrad_kernel, XWgradSmem::TOTAL))) return rc;
+  if ((rc = launch_k(true, sh_f32_wgrad_kernel, dim3((unsigned)(pq.n + pv.n + po.n)), dim3(XW_THREADS), XWgradSmem::TOTAL, st, pq, pv, po))) return rc;
   SH_CUDA_CHECK(cudaGetLastError());
-  L->launches += 3;
+  L->launches += 4;
   return SH_OK;
 }

@@ -18,13 +18,14 @@
 // Why not FFMA: the CUDA cores' 74 TFLOP/s fp32 peak against 2.25 PFLOP/s / 6 = 375.  What bounds a tile
 // is latency: gather list -> rows -> split -> shared memory -> UMMA -> read-back, and a tile's set-up and
 // result, 6 to 8 us of which little is work.  So a block is half an SM: 128 rows x 64 columns, contraction
-// steps of 32, three stages of 36 KB, 256 worker threads; two blocks share an SM and fill each other's
-// waits.  (One block per SM with 512 workers and steps of 64 ran each kernel 1.5 to 2 times as long.)
+// steps of 32, two stages of 36 KB, 256 worker threads; two blocks share an SM and fill each other's
+// waits.  (One block per SM with 512 workers and steps of 64 ran the short contractions 1.5 times as long.)
 //
-// Weights are split once, when they are set, and come as planes by TMA (one box of all three planes); an
-// activation is read as fp32 by the workers - the pieces of step i + 1 in registers while step i is
-// multiplied -, split and stored into the swizzled planes.  One thread issues the UMMAs; the workers read
-// the accumulators and write the result.
+// Weights are split once, when they are set, and come as planes by TMA (one box of all three planes).  An
+// activation is read as fp32 by the workers, two steps ahead, by asynchronous copies into shared memory
+// that only the copying warp uses (a prefetch that costs no registers and no block-wide barrier), split and
+// stored into the swizzled planes.  One thread issues the UMMAs; the workers read the accumulators and
+// write the result.  The weight gradients, whose operands are both activations, are in sh_f32_wgrad.cuh.
 // Operands are addressed row by row (a gathered token list, a head's slice of a row), either as rows of
 // the contraction (K-major) or as rows of the other index (MN-major: the weight gradients contract over
 // tokens), so no transposed or gathered copy is made.  Results that are added to, and rows handed on
@@ -66,11 +67,12 @@ struct XGemmArgs {
   int* status;
 };
 
-constexpr int XG_BN = 64, XG_BK = 32, XG_STAGES = 3;
+constexpr int XG_BN = 64, XG_BK = 32, XG_STAGES = 2;
 struct XGemmSmem {
   static constexpr int A_PLANE = 128 * XG_BK * 2, B_PLANE = XG_BN * XG_BK * 2;
   static constexpr int STAGE = 3 * (A_PLANE + B_PLANE);
-  static constexpr int BAR_OFF = XG_STAGES * STAGE;
+  static constexpr int RAW_OFF = XG_STAGES * STAGE, RAW = 128 * XG_BK * 4;     // fp32 pieces of a step, two steps
+  static constexpr int BAR_OFF = RAW_OFF + 2 * RAW;
   static constexpr int TOTAL = BAR_OFF + 128 + 1024;
 };
 
@@ -124,15 +126,22 @@ __device__ __forceinline__ void store_planes(unsigned char* tile, uint32_t off, 
   *reinterpret_cast<uint4*>(tile + off + 2 * plane) = make_uint4(l[0], l[1], l[2], l[3]);
 }
 
-// Eight consecutive values of a row (16-byte aligned, or not).
-__device__ __forceinline__ void load8(float (&v)[8], const float* p, bool vec) {
-  if (vec) {
-    const float4 a = __ldg(reinterpret_cast<const float4*>(p)), b = __ldg(reinterpret_cast<const float4*>(p) + 1);
-    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
-  } else {
+// A warp's fp32 pieces of a step pass through 1 KB (64 chunks of 16 bytes) of shared memory that only this
+// warp uses: copied chunk by chunk in the order of the rows, so that an instruction covers whole 128-byte
+// lines, read as two neighbouring chunks (8 values of a row) by each lane.  Chunk c sits at c ^ (c >> 3 & 1):
+// the eight lanes of a read phase then meet eight different 16-byte banks.
+__device__ __forceinline__ uint32_t raw_chunk(int c) { return (uint32_t)((c ^ ((c >> 3) & 1)) << 4); }
+__device__ __forceinline__ void fetch4(uint32_t dst, const float* p, bool vec, bool live = true) {
+  if (vec) cp_async_16(dst, p, live ? 16 : 0);             // (a dead piece is zeros; its address is still a valid one)
+  else {
 #pragma unroll
-    for (int i = 0; i < 8; ++i) v[i] = __ldg(p + i);
+    for (int i = 0; i < 4; ++i)
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst + i * 4), "l"(p + i), "r"(live ? 4 : 0) : "memory");
   }
+}
+__device__ __forceinline__ void read8(float (&v)[8], const unsigned char* kb, int c) {
+  const float4 a = *reinterpret_cast<const float4*>(kb + raw_chunk(c)), b = *reinterpret_cast<const float4*>(kb + raw_chunk(c + 1));
+  v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
 }
 
 // acc += the row's gate times a value: four adjacent floats at a time when the row is 16-byte aligned.
@@ -167,11 +176,8 @@ template <int MODE>
 __device__ __forceinline__ void xg_tile(const CUtensorMap& mapW, const CUtensorMap& mapG, const XGemmArgs& g, XTile blk) {
   using SM = XGemmSmem;
   constexpr int BN = XG_BN;
-  constexpr bool A_MN = MODE == X_DWO || MODE == X_DWV || MODE == X_DWQK;
   constexpr bool B_MN = MODE >= X_DA;
   constexpr bool LIST_ROWS = MODE == X_V || MODE == X_O || MODE == X_DA || MODE == X_DR;
-  constexpr bool LIST_K = MODE == X_DWO || MODE == X_DWV;
-  constexpr bool B_TMA = MODE <= X_DR && MODE != X_DWO || MODE == X_DX;
   constexpr bool BULK = LIST_ROWS || MODE == X_QK;         // results that leave as one bulk operation per row
   constexpr int COLS = BN / 2;                             // columns of a worker thread
   extern __shared__ unsigned char smem_raw[];
@@ -189,15 +195,13 @@ __device__ __forceinline__ void xg_tile(const CUtensorMap& mapW, const CUtensorM
 
   pdl_trigger();
   if (tid == 0) {
-    for (int s = 0; s < XG_STAGES; ++s) { mbar_init(&full_bar[s], B_TMA ? 9 : 8); mbar_init(&empty_bar[s], 1); }
+    for (int s = 0; s < XG_STAGES; ++s) { mbar_init(&full_bar[s], 9); mbar_init(&empty_bar[s], 1); }
     mbar_init(acc_full, 1); mbar_init(acc_empty, 8);
     fence_barrier_init();
   }
   pdl_wait();
   // ---- which tile ------------------------------------------------------------------------------
-  int h = 0, e = 0, which = 0, row0 = 0, nrows = 0, n0 = 0, ncols = 0, m0 = 0, steps = 0;
-  int kbeg = 0, kend = 0;                                  // LIST_K, X_DWQK: positions of the contraction
-  bool gates = false;                                      // X_DWQK: the tile of the gate columns
+  int h = 0, e = 0, which = 0, row0 = 0, nrows = 0, n0 = 0, ncols = 0, steps = 0;
   const int sps = (d.Dt + XG_BK - 1) / XG_BK;                        // steps over one head's d_head
   if (LIST_ROWS) {
     const ShTile tl = g.tiles[blk.x];
@@ -206,42 +210,16 @@ __device__ __forceinline__ void xg_tile(const CUtensorMap& mapW, const CUtensorM
     n0 = blk.y * g.sub_cols;
     ncols = min(g.sub_cols, ((MODE == X_O || MODE == X_DR) ? d.M : d.Dt) - n0);
     steps = (MODE == X_V || MODE == X_DA) ? d.M / XG_BK : sps;
-  } else if (LIST_K) {
-    const int grp = blk.x / g.ksplit, part = blk.x % g.ksplit;
-    h = grp / d.E; e = grp % d.E;
-    const int o0 = g.offsets[h * (d.E + 1) + e], o1 = g.offsets[h * (d.E + 1) + e + 1];
-    const int per = (((o1 - o0 + XG_BK - 1) / XG_BK + g.ksplit - 1) / g.ksplit) * XG_BK;
-    kbeg = min(o1, o0 + part * per); kend = min(o1, kbeg + per);
-    if (g.ksplit > 1 && kbeg >= kend) return;              // (the results are added to zeros)
-    steps = (kend - kbeg + XG_BK - 1) / XG_BK;
-    n0 = blk.y * g.sub_cols; m0 = blk.z * 128;
-    ncols = min(g.sub_cols, (MODE == X_DWO ? d.M : d.Dt) - n0);
-    nrows = min(128, (MODE == X_DWO ? d.Dt : d.M) - m0);
   } else if (MODE == X_DX) {
     row0 = blk.x * 128; nrows = min(128, d.N - row0);
     n0 = blk.y * g.sub_cols; ncols = min(g.sub_cols, d.M - n0);
     steps = 2 * d.H * sps + (d.G + XG_BK - 1) / XG_BK;
   } else {
-    // X_QK, X_DWQK: column tiles 0 .. qk_groups*nsub - 1 are the heads' columns, the rest the gate columns
-    const int ct = blk.y;
-    if (ct < g.qk_groups * g.nsub) {
-      const int grp = g.qk_first + ct / g.nsub;
-      which = grp / d.H; h = grp % d.H;
-      n0 = (ct % g.nsub) * g.sub_cols; ncols = min(g.sub_cols, d.Dt - n0);
-    } else {
-      gates = true;
-      n0 = (ct - g.qk_groups * g.nsub) * BN; ncols = min(BN, d.G - n0);
-    }
-    if (MODE == X_QK) {
-      row0 = blk.x * 128; nrows = min(128, d.N - row0);
-      steps = d.M / XG_BK;
-    } else {
-      m0 = blk.x * 128; nrows = min(128, d.M - m0);
-      const int per = (((d.N + XG_BK - 1) / XG_BK + g.ksplit - 1) / g.ksplit) * XG_BK;
-      kbeg = min(d.N, blk.z * per); kend = min(d.N, kbeg + per);
-      if (g.ksplit > 1 && kbeg >= kend) return;
-      steps = (kend - kbeg + XG_BK - 1) / XG_BK;
-    }
+    const int grp = g.qk_first + blk.y / g.nsub;
+    which = grp / d.H; h = grp % d.H;
+    n0 = (blk.y % g.nsub) * g.sub_cols; ncols = min(g.sub_cols, d.Dt - n0);
+    row0 = blk.x * 128; nrows = min(128, d.N - row0);
+    steps = d.M / XG_BK;
   }
   if (warp == 8) { tmem_alloc(tmem_slot, 256); tmem_relinquish(); }
   tc_fence_before();
@@ -250,7 +228,6 @@ __device__ __forceinline__ void xg_tile(const CUtensorMap& mapW, const CUtensorM
   // contraction positions of step i that exist (the rest of the operand rows is zero)
   auto kvalid = [&](int i) -> int {
     if (MODE == X_O || MODE == X_DR) return min(XG_BK, d.Dt - XG_BK * i);
-    if (A_MN) return min(XG_BK, kend - kbeg - XG_BK * i);
     if (MODE == X_DX) {
       const int seg = i / sps;
       return seg < 2 * d.H ? min(XG_BK, d.Dt - (i - seg * sps) * XG_BK) : min(XG_BK, d.G - (i - 2 * d.H * sps) * XG_BK);
@@ -261,12 +238,12 @@ __device__ __forceinline__ void xg_tile(const CUtensorMap& mapW, const CUtensorM
 
   if (warp == 8) {
     if (lane == 0) {
-      constexpr uint32_t maj = (B_MN ? 1u << 16 : 0u) | (A_MN ? 1u << 15 : 0u);
+      constexpr uint32_t maj = B_MN ? 1u << 16 : 0u;
       constexpr uint32_t id3 = make_idesc_f16(128, 192, 1, 1, 0) | maj, id2 = make_idesc_f16(128, 128, 1, 1, 0) | maj,
                          id1 = make_idesc_f16(128, 64, 1, 1, 0) | maj;
-      const uint32_t a0 = A_MN ? desc_lo_mn(sbase, 64 * XG_BK * 2) : desc_lo_k(sbase);
+      const uint32_t a0 = desc_lo_k(sbase);
       const uint32_t b0 = B_MN ? desc_lo_mn(sbase + 3 * SM::A_PLANE, SM::B_PLANE) : desc_lo_k(sbase + 3 * SM::A_PLANE);
-      constexpr uint32_t AK = A_MN ? 128 : 2, BK = B_MN ? 128 : 2, AP = SM::A_PLANE >> 4;
+      constexpr uint32_t BK = B_MN ? 128 : 2, AP = SM::A_PLANE >> 4;
       int s = 0;
       uint32_t par = 0;
       for (int i = 0; i < steps && !dead; ++i) {
@@ -278,11 +255,11 @@ __device__ __forceinline__ void xg_tile(const CUtensorMap& mapW, const CUtensorM
 #pragma unroll
         for (int k = 0; k < XG_BK / 16; ++k) {
           if (k >= kn) break;
-          const uint32_t a = alo + AK * k;
+          const uint32_t a = alo + 2 * k;
           const uint64_t bb = xg_desc(blo + BK * k, B_MN);
-          umma_f16(tmem, xg_desc(a, A_MN), bb, id3, (i % XG_CHUNK | k) != 0);
-          umma_f16(tmem + 64, xg_desc(a + AP, A_MN), bb, id2, 1);
-          umma_f16(tmem + 128, xg_desc(a + 2 * AP, A_MN), bb, id1, 1);
+          umma_f16(tmem, xg_desc(a, false), bb, id3, (i % XG_CHUNK | k) != 0);
+          umma_f16(tmem + 64, xg_desc(a + AP, false), bb, id2, 1);
+          umma_f16(tmem + 128, xg_desc(a + 2 * AP, false), bb, id1, 1);
         }
         umma_commit(&empty_bar[s]);
         if (i % XG_CHUNK == XG_CHUNK - 1 || i == steps - 1) umma_commit(acc_full);
@@ -291,7 +268,7 @@ __device__ __forceinline__ void xg_tile(const CUtensorMap& mapW, const CUtensorM
     }
     __syncwarp();
   } else if (warp == 9) {
-    if (B_TMA && lane == 0) {
+    if (lane == 0) {
       int s = 0;
       uint32_t par = 1;
       for (int i = 0; i < steps && !dead; ++i) {
@@ -317,98 +294,50 @@ __device__ __forceinline__ void xg_tile(const CUtensorMap& mapW, const CUtensorM
     __syncwarp();
   } else {
     // ---- workers: operands, promotions, result -----------------------------------------------------
-    // K-major pieces: 8 values of a row's 32 contraction positions; MN-major: 8 values of the row of
-    // one contraction position
-    const int ac = A_MN ? tid & 15 : tid & 3, ar = A_MN ? tid >> 4 : tid >> 2;    // + 16 j / + 64 j
-    const int bc = tid & 7, br = tid >> 3;                 // (a B that is split here is MN-major: 32 rows, one piece per thread)
-    constexpr int AR = A_MN ? 16 : 64;
+    // a thread's two pieces of a step: 8 values of rows ar and ar + 64
+    const int ac = tid & 3, ar = tid >> 2;
     uint32_t aoff[2];
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
-      const int r = ar + AR * j;
-      aoff[j] = A_MN ? (uint32_t)((ac >> 3) * (64 * XG_BK * 2) + r * 128 + (((ac & 7) ^ (r & 7)) << 4))
-                     : (uint32_t)(r * 64 + ((ac ^ ((r >> 1) & 3)) << 4));
+      const int r = ar + 64 * j;
+      aoff[j] = (uint32_t)(r * 64 + ((ac ^ ((r >> 1) & 3)) << 4));
     }
-    const uint32_t boff = (uint32_t)(br * 128 + ((bc ^ (br & 7)) << 4));
     const size_t lbase = (size_t)h * d.N * d.k;
-    const bool vdy = (MODE != X_DA && MODE != X_DWO) || g.vec_dy != 0;
-    // What lies past the tile never needs masking, only an address inside the operand: rows past a K-major A's
-    // last one and columns past an MN-major operand's width end in accumulators nobody reads, and positions
-    // past d_head (or the gate columns) are zeros in memory - a step of 32 never leaves the stored d_head.
-    // Only the positions past the end of a contraction over tokens are zeroed here.
-    const float* arow[2];
-    if (!A_MN) {
+    const bool vdy = MODE != X_DA || g.vec_dy != 0;
+    // What lies past the tile never needs masking, only an address inside the operand: rows past the last one
+    // end in accumulators nobody reads, and positions past d_head (or the gate columns) are zeros in memory -
+    // a step of 32 never leaves the stored d_head.
+    // (copies: lane -> chunk lane & 7 of rows 8 warp + (lane >> 3) + 4 u + 64 j; a row's 32 positions are 8 chunks)
+    const float* arow[2][2];
 #pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        const int r = row0 + min(ar + AR * j, nrows - 1);
+    for (int j = 0; j < 2; ++j)
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int r = row0 + min(8 * warp + (lane >> 3) + 4 * u + 64 * j, nrows - 1);
         const size_t t = LIST_ROWS ? g.lists[lbase + r] : r;
-        arow[j] = (MODE == X_QK || MODE == X_V ? g.x + t * d.M
-                 : MODE == X_O ? g.ahat + t * HD + h * d.D
-                 : MODE == X_DA ? g.dy + t * d.M
-                 : MODE == X_DR ? g.dv + t * HD + h * d.D : g.dq + t * HD) + ac * 8;
+        arow[j][u] = (MODE == X_QK || MODE == X_V ? g.x + t * d.M
+                    : MODE == X_O ? g.ahat + t * HD + h * d.D
+                    : MODE == X_DA ? g.dy + t * d.M
+                    : MODE == X_DR ? g.dv + t * HD + h * d.D : g.dq + t * HD) + (lane & 7) * 4;
       }
-    }
-    const int acol = A_MN ? min(m0 + ac * 8, (MODE == X_DWO ? d.D : d.M) - 8) : 0;
-    const int bcol = !B_TMA ? min(n0 + bc * 8, (MODE == X_DWO ? d.M : MODE == X_DWQK && gates ? g.ldz : d.D) - 8) : 0;
-    const float* bsrc = MODE == X_DWO ? g.dy + bcol : MODE == X_DWV ? g.dv + h * d.D + bcol
-                      : MODE == X_DWQK ? (gates ? g.dz + bcol : (which ? g.dk : g.dq) + h * d.D + bcol) : nullptr;
-    const size_t bld = MODE == X_DWO ? d.M : MODE == X_DWQK && gates ? g.ldz : HD;
-    // lists: the entries of a step are fetched one step ahead of its rows
-    int ta[2] = {0, 0}, tb = 0;
-    float ga[2] = {0.f, 0.f};
-    auto fetch = [&](int i) {
-      if (LIST_K) {
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-          const int pos = kbeg + i * XG_BK + ar + AR * j;
-          if (pos < kend) { ta[j] = __ldg(g.lists + lbase + pos); ga[j] = __ldg(g.lgate + lbase + pos); }
-        }
-        const int pos = kbeg + i * XG_BK + br;
-        if (pos < kend) tb = __ldg(g.lists + lbase + pos);
-      }
-    };
     int xseg = 0, xoff = 0;                                // X_DX: the step's head (of dq, then dk), and where in it
-    float ra[2][8], rb[8], rg[2];                          // the next step's pieces
-    auto load = [&](int i) {
-      if (!A_MN) {
-        const float *p0, *p1;
-        if (MODE == X_DX) {
-          const long o = xseg < 2 * d.H ? (xseg >= d.H ? (long)(g.dk - g.dq) + (long)(xseg - d.H) * d.D : (long)xseg * d.D) + xoff : 0;
-          p0 = arow[0] + o; p1 = arow[1] + o;
-          if (xseg == 2 * d.H) {
-            p0 = g.dz + (size_t)(row0 + min(ar, nrows - 1)) * g.ldz + xoff + ac * 8;
-            p1 = g.dz + (size_t)(row0 + min(ar + AR, nrows - 1)) * g.ldz + xoff + ac * 8;
-          }
-          xoff += XG_BK;
-          if (xseg < 2 * d.H && xoff >= d.Dt) { xoff = 0; ++xseg; }
-        } else {
-          p0 = arow[0] + i * XG_BK; p1 = arow[1] + i * XG_BK;
-        }
-        load8(ra[0], p0, vdy);
-        load8(ra[1], p1, vdy);
-      } else {
+    const uint32_t rbase = sbase + SM::RAW_OFF + warp * 2048;
+    auto load = [&](int i) {                               // step i on its way
+      long o = (long)i * XG_BK;
+      if (MODE == X_DX) o = (xseg >= d.H ? (long)(g.dk - g.dq) + (long)(xseg - d.H) * d.D : (long)xseg * d.D) + xoff;
 #pragma unroll
-        for (int j = 0; j < 2; ++j) {
-          const int pos = kbeg + i * XG_BK + ar + AR * j;
-          rg[j] = ga[j];
-          if (pos < kend) {
-            const size_t t = LIST_K ? ta[j] : pos;
-            load8(ra[j], (MODE == X_DWO ? g.ahat + t * HD + h * d.D : g.x + t * d.M) + acol, true);
-          } else {
+      for (int j = 0; j < 2; ++j)
 #pragma unroll
-            for (int x = 0; x < 8; ++x) ra[j][x] = 0.f;
-          }
+        for (int u = 0; u < 2; ++u) {
+          const float* p = arow[j][u] + o;
+          if (MODE == X_DX && xseg == 2 * d.H)
+            p = g.dz + (size_t)(row0 + min(8 * warp + (lane >> 3) + 4 * u + 64 * j, nrows - 1)) * g.ldz + xoff + (lane & 7) * 4;
+          fetch4(rbase + (i & 1) * SM::RAW + j * 1024 + raw_chunk(lane + 32 * u), p, vdy);
         }
+      if (MODE == X_DX) {
+        xoff += XG_BK;
+        if (xseg < 2 * d.H && xoff >= d.Dt) { xoff = 0; ++xseg; }
       }
-      if (!B_TMA) {
-        const int pos = kbeg + i * XG_BK + br;
-        if (pos < kend) load8(rb, bsrc + (size_t)(LIST_K ? tb : pos) * bld, vdy);
-        else {
-#pragma unroll
-          for (int x = 0; x < 8; ++x) rb[x] = 0.f;
-        }
-      }
-      if (i + 1 < steps) fetch(i + 1);
     };
     const int q = warp & 3, cb = warp >> 2;
     const uint32_t tlane = ((uint32_t)(q * 32) << 16) + cb * COLS;
@@ -436,29 +365,34 @@ __device__ __forceinline__ void xg_tile(const CUtensorMap& mapW, const CUtensorM
       __syncwarp();
       if (lane == 0) mbar_arrive(acc_empty);
     };
-    if (steps > 0) { fetch(0); load(0); }
+    load(0);
+    cp_async_commit();
+    if (steps > 1) load(1);
+    cp_async_commit();
     int s = 0, done = 0;                                   // done: chunks promoted
     uint32_t par = 1;
     for (int i = 0; i < steps && !dead; ++i) {
+      cp_async_wait<1>();                                  // this warp's pieces of step i are there
+      __syncwarp();
       if (!mbar_wait(&empty_bar[s], par, g.status, dead)) break;
       unsigned char* at = sgen + s * SM::STAGE;
+      const unsigned char* raw = sgen + SM::RAW_OFF + (i & 1) * SM::RAW + warp * 2048;
 #pragma unroll
       for (int j = 0; j < 2; ++j) {
-        if (LIST_K) {
-#pragma unroll
-          for (int x = 0; x < 8; ++x) ra[j][x] *= rg[j];
-        }
-        store_planes(at, aoff[j], SM::A_PLANE, ra[j]);
+        float v[8];
+        read8(v, raw + j * 1024, 2 * lane);
+        store_planes(at, aoff[j], SM::A_PLANE, v);
       }
-      if (!B_TMA) store_planes(at + 3 * SM::A_PLANE, boff, SM::B_PLANE, rb);
       fence_proxy_async_smem();
       __syncwarp();
       if (lane == 0) mbar_arrive(&full_bar[s]);
       if (++s == XG_STAGES) { s = 0; par ^= 1; }
-      if (i + 1 < steps) load(i + 1);
+      if (i + 2 < steps) load(i + 2);
+      cp_async_commit();
       // a chunk is read once two steps of the next one are in shared memory
       if (i % XG_CHUNK == 1 && i > XG_CHUNK) promote(done++);
     }
+    cp_async_wait<0>();
     for (; done < (steps + XG_CHUNK - 1) / XG_CHUNK && !dead; ++done) promote(done);
     // ---- result: thread = row q*32 + lane, columns cb*COLS ... ------------------------------------
     const int r = q * 32 + lane, c0 = cb * COLS;
@@ -487,13 +421,6 @@ __device__ __forceinline__ void xg_tile(const CUtensorMap& mapW, const CUtensorM
         const float f = MODE == X_V && g.vscale != 0.f ? gt * g.vscale : gt;
 #pragma unroll
         for (int i = 0; i < COLS; ++i) acc[i] *= f;
-      } else if (LIST_K) {
-        // dWo [(h*E + e)*Dt + dd][m]; dWv [(h*E + e)*M + m][dd < Dt]
-        float* o = MODE == X_DWO ? g.dWo + ((size_t)(h * d.E + e) * d.Dt + m0 + r) * d.M + n0 + c0
-                                 : g.dWv + ((size_t)(h * d.E + e) * d.M + m0 + r) * d.Dt + n0 + c0;
-        const bool vec = g.vec_out != 0 && (MODE == X_DWO || d.Dt % 4 == 0);
-        if (g.ksplit > 1) red_row(o, acc, valid, vec);
-        else store_row(o, acc, valid, vec);
       } else if (MODE == X_DX) {
         float* o = g.dx + (size_t)(row0 + r) * d.M + n0 + c0;
 #pragma unroll
@@ -506,23 +433,6 @@ __device__ __forceinline__ void xg_tile(const CUtensorMap& mapW, const CUtensorM
 #pragma unroll
             for (int j = 0; j < 4; ++j) if (i + j < valid) o[i + j] += acc[i + j];
           }
-        }
-      } else if (MODE == X_DWQK) {
-        const int m = m0 + r;
-        if (!gates) {
-          float* o = (which ? g.dWk : g.dWq) + ((size_t)h * d.M + m) * d.Dt + n0 + c0;
-          const bool vec = g.vec_out != 0 && d.Dt % 4 == 0;
-          if (g.ksplit > 1) red_row(o, acc, valid, vec);
-          else store_row(o, acc, valid, vec);
-        } else {
-#pragma unroll
-          for (int i = 0; i < COLS; ++i)
-            if (i < valid) {
-              const int gc = n0 + c0 + i, side = gc / (d.H * d.E), hh = (gc / d.E) % d.H, ee = gc % d.E;
-              float* o = (side ? g.dWd : g.dWs) + ((size_t)hh * d.M + m) * d.E + ee;
-              if (g.ksplit > 1) atomicAdd(o, acc[i]);
-              else *o = acc[i];
-            }
         }
       } else {                                             // X_QK
         const int tok = row0 + r;
@@ -592,22 +502,16 @@ __device__ __forceinline__ void xg_tile(const CUtensorMap& mapW, const CUtensorM
 // Block number i of a mode's gx x gy x gz tiles.
 __device__ __forceinline__ XTile xg_unpack(int i, int gx, int gy) { return {i % gx, i / gx % gy, i / (gx * gy)}; }
 
-// A launch of up to three modes whose tiles do not depend on one another: the first n0 blocks work on
-// tiles of mode A, the next n1 on mode B, the rest on mode C.  (One launch each leaves half of the block
-// slots idle in its last round, and pays its set-up and drain by itself.)
+// A launch of one or two modes whose tiles do not depend on one another: the first blocks work on tiles
+// of mode A, the rest on mode B.  (One launch each leaves half of the block slots idle in its last round,
+// and pays its set-up and drain by itself.)
 struct XPart { CUtensorMap w; XGemmArgs g; int gx, gy, n; };
-template <int A, int B, int C>
+template <int A, int B>
 __global__ void __launch_bounds__(XG_THREADS, 2)
-sh_f32_gemm_kernel(const __grid_constant__ CUtensorMap mapG, const __grid_constant__ XPart pa, const __grid_constant__ XPart pb,
-                   const __grid_constant__ XPart pc) {
-  int i = blockIdx.x;
-  if (i < pa.n) { xg_tile<A>(pa.w, mapG, pa.g, xg_unpack(i, pa.gx, pa.gy)); return; }
-  i -= pa.n;
-  if (B >= 0) {
-    if (i < pb.n) { xg_tile<(B >= 0 ? B : A)>(pb.w, mapG, pb.g, xg_unpack(i, pb.gx, pb.gy)); return; }
-    i -= pb.n;
-  }
-  if (C >= 0) xg_tile<(C >= 0 ? C : A)>(pc.w, mapG, pc.g, xg_unpack(i, pc.gx, pc.gy));
+sh_f32_gemm_kernel(const __grid_constant__ CUtensorMap mapG, const __grid_constant__ XPart pa, const __grid_constant__ XPart pb) {
+  const int i = blockIdx.x;
+  if (B < 0 || i < pa.n) xg_tile<A>(pa.w, mapG, pa.g, xg_unpack(i, pa.gx, pa.gy));
+  else xg_tile<(B >= 0 ? B : A)>(pb.w, mapG, pb.g, xg_unpack(i - pa.n, pb.gx, pb.gy));
 }
 
 }  // namespace shtc
