@@ -94,12 +94,14 @@ int launch_gate_sort(sh_layer* L, const void* x, float* zero0, long n0, float* z
   const ShDims& d = L->d;
   char* ws = L->ws;
   // eight tokens a block while sixteen would leave SMs with less than two blocks (or their logits do not fit)
-  const bool small = d.N < 32 * sm_count(L) || 16 * (512 + d.G) * 4 > 200 * 1024;
+  const int ch = d.M <= 512 ? 512 : 1024;
+  const bool small = d.N < 32 * sm_count(L) || 16 * (ch + d.G) * 4 > 200 * 1024;
   const int tok = small ? 8 : 16;
-  const size_t smem = (size_t)tok * (512 + d.G) * 4;
-  auto kern = small ? sh_f32_gate_kernel<8> : sh_f32_gate_kernel<16>;
+  const size_t smem = (size_t)tok * (ch + d.G) * 4;
+  auto kern = small ? (ch == 512 ? sh_f32_gate_kernel<8, 512> : sh_f32_gate_kernel<8, 1024>)
+                    : (ch == 512 ? sh_f32_gate_kernel<16, 512> : sh_f32_gate_kernel<16, 1024>);
   if (int rc = set_smem(kern, (int)smem)) return rc;
-  if (int rc = launch_k(true, kern, dim3((unsigned)((d.N + tok - 1) / tok)), dim3(256), smem, st, (const float*)x, (const float*)(ws + L->o.wgate32),
+  if (int rc = launch_k(true, kern, dim3((unsigned)((d.N + tok - 1) / tok)), dim3(512), smem, st, (const float*)x, (const float*)(ws + L->o.wgate32),
                         (const float*)(ws + L->o.gbias), (int*)(ws + L->o.idx), (float*)(ws + L->o.gate), (float4*)zero0, n0 / 4, (float4*)zero1, n1 / 4, d))
     return rc;
   L->launches += 2;

@@ -3,56 +3,56 @@
 #include "sh_internal.cuh"
 
 // Logits, top-k (a larger logit first, the lower index on a tie) and sigmoid of the chosen ones, on the
-// CUDA cores: TOK tokens per block with their rows in shared memory (512 columns at a time), a warp per
-// gate column, lanes along d_model.  The block also clears its share of the buffers that later kernels
+// CUDA cores: TOK tokens per block with their rows in shared memory (CH columns at a time: 512, or 1024 where d_model is larger), a warp per
+// two gate columns, lanes along d_model.  The block also clears its share of the buffers that later kernels
 // add into.  What bounds it is the latency of its few loads, so blocks are small: 1024 tokens of 32 gate
 // columns took 490 us in blocks of 128 tokens with a warp per token.
-template <int TOK>
-static __global__ void __launch_bounds__(256)
+template <int TOK, int CH>
+static __global__ void __launch_bounds__(512, 1)
 sh_f32_gate_kernel(const float* __restrict__ x, const float* __restrict__ wgate, const float* __restrict__ gbias, int* __restrict__ idx,
                    float* __restrict__ gate, float4* __restrict__ zero0, long nzero0, float4* __restrict__ zero1, long nzero1, ShDims d) {
-  extern __shared__ __align__(16) float gsm[];             // [TOK][512] of x, then [TOK][G] logits
-  float* s_z = gsm + TOK * 512;
+  extern __shared__ __align__(16) float gsm[];             // [TOK][CH] of x, then [TOK][G] logits
+  float* s_z = gsm + TOK * CH;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
+  constexpr int U = CH / 32;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int t0 = blockIdx.x * TOK;
-  const long nthr = (long)gridDim.x * 256, me = (long)blockIdx.x * 256 + tid;
-  for (int m0 = 0; m0 < d.M; m0 += 512) {
-    const int mw = min(512, d.M - m0);                     // a multiple of 64
+  const long nthr = (long)gridDim.x * 512, me = (long)blockIdx.x * 512 + tid;
+  for (int m0 = 0; m0 < d.M; m0 += CH) {
+    const int mw = min(CH, d.M - m0);           // a multiple of 64
     __syncthreads();
-    for (int i = tid; i < TOK * 128; i += 256) {
-      const int r = i >> 7, c = (i & 127) * 4;
+    for (int i = tid; i < TOK * (CH / 4); i += 512) {
+      const int r = i / (CH / 4), c = (i % (CH / 4)) * 4;
       float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
       if (c < mw && t0 + r < d.N) v = __ldg(reinterpret_cast<const float4*>(x + (size_t)(t0 + r) * d.M + m0 + c));
-      *reinterpret_cast<float4*>(gsm + r * 512 + c) = v;
+      *reinterpret_cast<float4*>(gsm + r * CH + c) = v;
     }
-    if (m0 == 0) {
-      for (long i = me; i < nzero0; i += nthr) zero0[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-      for (long i = me; i < nzero1; i += nthr) zero1[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-    __syncthreads();
-    for (int g = warp; g < d.G; g += 16) {                  // two columns at a time: eight 16-byte loads in flight per lane
-      const bool two = g + 8 < d.G;
+    for (int g = warp; g < d.G; g += 32) {                  // two columns at a time, all of their loads in flight
+      const bool two = g + 16 < d.G;
       const float* w0 = wgate + (size_t)g * d.M + m0;
-      const float* w1 = w0 + (two ? (size_t)8 * d.M : 0);
-      float4 wv[2][4];
+      const float* w1 = w0 + (two ? (size_t)16 * d.M : 0);
+      // (lane l sums the columns l, l + 32, ... in order and the lanes are added as a butterfly: the order of
+      //  sh_gate_topk_kernel, so that the allocation-free entry point gives the same bits up to CH columns)
+      float wv[2][U];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int c = u * 128 + lane * 4;
-        wv[0][u] = wv[1][u] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (c < mw) { wv[0][u] = __ldg(reinterpret_cast<const float4*>(w0 + c)); wv[1][u] = __ldg(reinterpret_cast<const float4*>(w1 + c)); }
+      for (int u = 0; u < U; ++u) {
+        const int c = u * 32 + lane;
+        wv[0][u] = c < mw ? __ldg(w0 + c) : 0.f;
+        wv[1][u] = c < mw ? __ldg(w1 + c) : 0.f;
       }
+      if (g == warp) __syncthreads();                       // (every warp's first round, or the one behind the loop)
       float acc[2][TOK];
 #pragma unroll
-      for (int r = 0; r < TOK; ++r) {
-        acc[0][r] = acc[1][r] = 0.f;
+      for (int r = 0; r < TOK; ++r) acc[0][r] = acc[1][r] = 0.f;
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const float4 xv = *reinterpret_cast<const float4*>(gsm + r * 512 + u * 128 + lane * 4);
+      for (int u = 0; u < U; ++u) {
+        if (u * 32 >= mw) break;
 #pragma unroll
-          for (int q = 0; q < 2; ++q)
-            acc[q][r] = fmaf(xv.x, wv[q][u].x, fmaf(xv.y, wv[q][u].y, fmaf(xv.z, wv[q][u].z, fmaf(xv.w, wv[q][u].w, acc[q][r]))));
+        for (int r = 0; r < TOK; ++r) {
+          const float xv = gsm[r * CH + u * 32 + lane];
+          acc[0][r] = fmaf(xv, wv[0][u], acc[0][r]);
+          acc[1][r] = fmaf(xv, wv[1][u], acc[1][r]);
         }
       }
       // lane sums of TOK tokens: at each step a lane keeps half of its tokens and hands the others over
@@ -72,15 +72,20 @@ sh_f32_gate_kernel(const float* __restrict__ x, const float* __restrict__ wgate,
 #pragma unroll
         for (int o = 32 / TOK / 2; o > 0; o >>= 1) acc[q][0] += __shfl_xor_sync(0xffffffffu, acc[q][0], o);
         if (lane % (32 / TOK) == 0 && (q == 0 || two)) {
-          float* z = s_z + tokn * d.G + g + 8 * q;
+          float* z = s_z + tokn * d.G + g + 16 * q;
           *z = (m0 == 0 ? 0.f : *z) + acc[q][0];
         }
       }
     }
+    if (warp >= d.G) __syncthreads();                      // (a warp without a column meets the barrier of the others' first round here)
+    if (m0 == 0) {
+      for (long i = me; i < nzero0; i += nthr) zero0[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+      for (long i = me; i < nzero1; i += nthr) zero1[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
   }
   __syncthreads();
   const int groups = d.sides * d.H;
-  for (int i = tid; i < TOK * groups; i += 256) {
+  for (int i = tid; i < TOK * groups; i += 512) {
     const int r = i / groups, grp = i % groups, side = grp / d.H, h = grp % d.H, t = t0 + r;
     if (t >= d.N) continue;
     float* z = s_z + r * d.G + grp * d.E;
@@ -131,16 +136,17 @@ sh_f32_sort_kernel(const int* __restrict__ idx, const float* __restrict__ gate, 
   }
   if (lane < d.E && mine) atomicAdd(&s_tot[lane], mine);
   __syncthreads();
-  if (tid == 0) {
-    int run = 0, tiles_before = 0;
-    for (int e = 0; e < d.E; ++e) {
-      s_off[e] = run; s_run[e] = run; s_tile[e] = tiles_before;
-      offsets[(size_t)grp * (d.E + 1) + e] = run;
-      run += s_tot[e];
-      tiles_before += (s_tot[e] + SH_TILE_ROWS - 1) / SH_TILE_ROWS;
+  if (warp == 0) {                                         // lane e: exclusive sums over the experts
+    const int tot = lane < d.E ? s_tot[lane] : 0, nt = (tot + SH_TILE_ROWS - 1) / SH_TILE_ROWS;
+    int run = tot, tl = nt;
+#pragma unroll
+    for (int s = 1; s < 32; s <<= 1) {
+      const int u = __shfl_up_sync(0xffffffffu, run, s), w = __shfl_up_sync(0xffffffffu, tl, s);
+      if (lane >= s) { run += u; tl += w; }
     }
-    s_off[d.E] = run; s_tile[d.E] = tiles_before;
-    offsets[(size_t)grp * (d.E + 1) + d.E] = run;
+    s_run[lane] = s_off[lane] = run - tot; s_tile[lane] = tl - nt;
+    if (lane < d.E) offsets[(size_t)grp * (d.E + 1) + lane] = run - tot;
+    if (lane == d.E - 1) { s_off[d.E] = run; s_tile[d.E] = tl; offsets[(size_t)grp * (d.E + 1) + d.E] = run; }
   }
   __syncthreads();
   ShTile* tp = tiles + (size_t)side * d.max_tiles + (size_t)h * mt;
@@ -164,9 +170,10 @@ sh_f32_sort_kernel(const int* __restrict__ idx, const float* __restrict__ gate, 
     unsigned sel = 0;
     if (live)
       for (int j = 0; j < d.k; ++j) sel |= 1u << idx[o + j];
+    unsigned mybal = 0;                                    // lane e: which lanes chose expert e
     for (int e = 0; e < d.E; ++e) {
       const unsigned bal = __ballot_sync(0xffffffffu, (sel >> e) & 1u);
-      if (lane == e) s_w[warp][e] = __popc(bal);
+      if (lane == e) { s_w[warp][e] = __popc(bal); mybal = bal; }
     }
     __syncthreads();
     if (warp < d.E) {                                      // warp e: where each warp's tokens of expert e start
@@ -182,15 +189,13 @@ sh_f32_sort_kernel(const int* __restrict__ idx, const float* __restrict__ gate, 
       if (lane == 31) s_run[warp] = base + inc;
     }
     __syncthreads();
-    for (int e = 0; e < d.E; ++e) {
-      const unsigned bal = __ballot_sync(0xffffffffu, (sel >> e) & 1u);
-      if ((sel >> e) & 1u) {
+    for (int j = 0; j < d.k; ++j) {
+      const int e = live ? idx[o + j] : 0;
+      const unsigned bal = __shfl_sync(0xffffffffu, mybal, e);
+      if (live) {
         const int pos = s_w[warp][e] + __popc(bal & ((1u << lane) - 1u));
-        float gv = 0.f;
-        for (int j = 0; j < d.k; ++j)
-          if (idx[o + j] == e) gv = gate[o + j];
         ls[pos] = t;
-        lg[pos] = gv;
+        lg[pos] = gate[o + j];
       }
     }
     __syncthreads();
