@@ -37,7 +37,7 @@ static EncodeTiledFn get_encode() {
 }
 
 // 2-D row-major tensor [outer, inner] of 16-bit elements, 128-byte swizzle, box = box_outer
-// rows of box_inner (= 64) elements.
+// rows of box_inner (64; 32 or 16: 64- / 32-byte swizzle) elements.
 int sh_tc_encode_2d(CUtensorMap* map, int elem_kind, const void* base, uint64_t inner, uint64_t outer,
                     uint64_t outer_stride_bytes, uint32_t box_inner, uint32_t box_outer) {
   EncodeTiledFn enc = get_encode();
@@ -48,7 +48,7 @@ int sh_tc_encode_2d(CUtensorMap* map, int elem_kind, const void* base, uint64_t 
   cuuint32_t estr[2] = {1, 1};
   CUresult r = enc(map, elem_kind == 0 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2,
                    const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                   CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+                   box_inner == 16 ? CU_TENSOR_MAP_SWIZZLE_32B : box_inner == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) { sh_set_error("cuTensorMapEncodeTiled failed with CUresult %d", (int)r); return SH_ERR_CUDA; }
   return SH_OK;
 }
@@ -104,7 +104,7 @@ static int encode_3d_f16_store32(CUtensorMap* map, const void* base, uint64_t in
 struct TcState {
   CUtensorMap map_q, map_k, map_v;
   CUtensorMap map_q_st, map_k_st;   // Q and K as the one-grid front's epilogue stores them
-  CUtensorMap map_wqk, map_wqk128, map_wv, map_wq_e, map_wk_e, map_wo, map_wo256, map_wos, map_ahat, map_wgate;
+  CUtensorMap map_wqk, map_wqk128, map_wv, map_wq_e, map_wk_e, map_wo, map_wo256, map_wo_tail, map_ahat_tail, map_wos, map_ahat, map_wgate;
   CUtensorMap map_q2d, map_r16;  // score-bias GEMM of the Transformer-XL position term: Q as [B*H*T, D], R16 as [H*T, D]
   CUtensorMap map_x;             // tensor map of the last x pointer seen (x_cached)
   CUtensorMap map_x64;           // the same tensor in 64-token boxes (gate tile of the one-grid front, 64 tokens per CTA)
@@ -112,6 +112,7 @@ struct TcState {
   const void* x_cached = nullptr;
   int gate_gp;          // gate columns padded to a multiple of 16; 0 = CUDA-core gate kernel (more than 256 gate columns)
   int qk_bn;            // column tile of the dense projection: 256 (CTA pairs / persistent) when 2*H*D allows, else 128
+  int o_tail;           // d_head above 128: columns the single-CTA output projection loads of the last 64-column block
   int o_pairs_max;      // clusters of the CTA-pair output projection the device holds at once (0: not asked yet, -1: none)
   int qk_pairs_max;     // the same for the dense Q/K projection
   int gate_coop;        // 1: the gate kernel can be launched cooperatively (fused sort), -1: it cannot
@@ -261,6 +262,11 @@ int sh_tc_prepare(sh_layer* L) {
   if ((rc = encode_3d_f16_store32(&S->map_q_st, ws + L->o.q, d.D, d.T, (uint64_t)d.B * d.H))) return rc;
   if ((rc = encode_3d_f16_store32(&S->map_k_st, ws + L->o.k, d.D, d.T, (uint64_t)d.B * d.H))) return rc;
   if ((rc = sh_tc_encode_2d(&S->map_ahat, 1, ws + L->o.ahat, HD, d.N, (uint64_t)HD * 2, 64, 128))) return rc;
+  S->o_tail = d.D > 128 ? ((d.Dt - 1) % 64 < 16 ? 16 : (d.Dt - 1) % 64 < 32 ? 32 : 64) : 64;
+  if (!L->dense) {
+    if ((rc = sh_tc_encode_2d(&S->map_wo_tail, 1, ws + L->o.wo, d.D, (uint64_t)d.H * d.E * d.M, (uint64_t)d.D * 2, S->o_tail, 256))) return rc;
+    if ((rc = sh_tc_encode_2d(&S->map_ahat_tail, 1, ws + L->o.ahat, HD, d.N, (uint64_t)HD * 2, S->o_tail, 128))) return rc;
+  }
   if (!L->dense && d.Tc > 0) {
     if ((rc = sh_tc_encode_2d(&S->map_q2d, 1, ws + L->o.q, d.D, (uint64_t)d.B * d.H * d.T, (uint64_t)d.D * 2, 64, 128))) return rc;
     if ((rc = sh_tc_encode_2d(&S->map_r16, 1, ws + L->o.xl_r16, d.D, (uint64_t)d.H * d.T, (uint64_t)d.D * 2, 64, 64))) return rc;
@@ -873,20 +879,20 @@ static int tc_forward_rest(sh_layer* L, const void* x, void* out, cudaStream_t s
     } else {
       a.nwork = ((sh_out_rows(d) + 127) / 128) * ((d.M + 255) / 256);
       const unsigned grid = (unsigned)(a.nwork < L->sm_count ? a.nwork : L->sm_count);
-      auto go = [&](auto kern, int (*total)(int, int, int)) -> int {
+      auto go = [&](auto kern, int (*total)(int, int, int, int)) -> int {
         int as = 3, smem = 0;
         for (; as >= 2; --as) {
-          smem = total(as, d.H, d.k);
+          smem = total(as, d.H, d.k, S->o_tail);
           if (smem <= 227 * 1024) break;
         }
         if (as < 2 && d.D > 128) {                           // (such layers take any n_heads * k)
           a.sel_global = 1;
-          as = 2; smem = total(2, d.H, 0);
+          as = 2; smem = total(2, d.H, 0, S->o_tail);
         }
         if (as < 2) { sh_set_error("output projection: n_heads*k = %d does not fit in shared memory", d.H * d.k); return SH_ERR_UNSUPPORTED; }
-        a.a_slots = as;
+        a.a_slots = as; a.tail = S->o_tail;
         if (int r = set_smem(kern, smem)) return r;
-        return launch_k(pdl, kern, dim3(grid), dim3(320), smem, st, S->map_ahat, S->map_wo256, a);
+        return launch_k(pdl, kern, dim3(grid), dim3(320), smem, st, S->map_ahat, S->map_wo256, S->map_ahat_tail, S->map_wo_tail, a);
       };
       if (d.D == 64) rc = go(sh_tc_oproj_kernel<1, 2>, OprojSmem<1, 2>::total);
       else if (d.D == 128) rc = go(sh_tc_oproj_kernel<2, 2>, OprojSmem<2, 2>::total);

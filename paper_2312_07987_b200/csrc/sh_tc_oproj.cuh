@@ -39,6 +39,7 @@ struct TcOprojArgs {
   float* out;            // [N, M] fp32, or (out_f16) [N, M] fp16 at the same address
   int out_f16;           // 1: the result rows are rounded to fp16 once, on their way out
   int a_slots;           // 32 KB weight stages in the ring: 3 or 2
+  int tail;              // single-CTA kernel: columns loaded of d_head's last 64-column block (64, 32 or 16)
   int sel_global;        // single-CTA kernel: selections read from global memory (their copy does not fit shared memory)
   int nwork;             // nblk * ceil(M / 256)
   int* status;
@@ -55,20 +56,24 @@ __device__ __forceinline__ void oproj_put4(float* out, size_t elem, float4 v, in
   }
 }
 
-// DB: 64-column blocks of d_head; NB: token tiles in the ring (one where two of 256 columns do not fit).
+// DB: 64-column blocks of d_head; NB: token tiles in the ring (one where two of 256 columns do not fit).  With
+// d_head above 128 the last block is loaded 16 or 32 columns wide (32- / 64-byte swizzle) where d_head
+// reaches no further into it: for 132 that is a quarter less weight traffic, and room for a third stage.
 template <int DB, int NB>
 struct OprojSmem {
   static constexpr int A_BYTES = 256 * 64 * 2;           // one weight stage: 256 features x 64 columns
   static constexpr int B_BYTES = 128 * DB * 64 * 2;      // Ahat tile: 128 tokens x 64 DB
   static constexpr int STAGING = 8 * 32 * 32 * 4;        // per epilogue warp a 32 x 32 fp32 transpose tile
-  static int total(int a_slots, int H, int k) {
-    return a_slots * A_BYTES + NB * B_BYTES + STAGING + 128 * H * k * 8 + 512 + 1024;
+  __host__ __device__ static int b_bytes(int tail) { return (DB - 1) * 128 * 128 + 128 * tail * 2; }   // tail: columns loaded of the last block
+  static int total(int a_slots, int H, int k, int tail) {
+    return a_slots * A_BYTES + NB * b_bytes(tail) + STAGING + 128 * H * k * 8 + 512 + 1024;
   }
 };
 
 template <int DB, int NB>
 __global__ void __launch_bounds__(320, 1)
-sh_tc_oproj_kernel(const __grid_constant__ CUtensorMap mapAhat, const __grid_constant__ CUtensorMap mapWo, TcOprojArgs g) {
+sh_tc_oproj_kernel(const __grid_constant__ CUtensorMap mapAhat, const __grid_constant__ CUtensorMap mapWo,
+                   const __grid_constant__ CUtensorMap mapAhatTail, const __grid_constant__ CUtensorMap mapWoTail, TcOprojArgs g) {
   using SM = OprojSmem<DB, NB>;
   constexpr uint32_t TBLK = 128 * 128;                   // one 64-column block of the token tile
   extern __shared__ unsigned char smem_raw[];
@@ -76,7 +81,8 @@ sh_tc_oproj_kernel(const __grid_constant__ CUtensorMap mapAhat, const __grid_con
   unsigned char* sgen = smem_raw + (sbase - smem_u32(smem_raw));
   const ShDims& d = g.d;
   const int AS = g.a_slots;                              // 3 or 2
-  const uint32_t a_off = 0, b_off = AS * SM::A_BYTES, stg_off = b_off + NB * SM::B_BYTES, misc_off = stg_off + SM::STAGING;
+  const uint32_t b_slot = SM::b_bytes(g.tail);
+  const uint32_t a_off = 0, b_off = AS * SM::A_BYTES, stg_off = b_off + NB * b_slot, misc_off = stg_off + SM::STAGING;
   const int sel_n = g.sel_global ? 0 : 128 * d.H * d.k;
   int* s_idx = (int*)(sgen + misc_off);                       // [128, H, k] selections of the current tokens
   float* s_gt = (float*)(s_idx + sel_n);                      // [128, H, k]
@@ -126,17 +132,17 @@ sh_tc_oproj_kernel(const __grid_constant__ CUtensorMap mapAhat, const __grid_con
         for (int h = 0; h < d.H && !dead; ++h, ++gh) {
           const int bs = NB == 2 ? gh & 1 : 0;
           if (!mbar_wait(&b_empty[bs], ((gh / NB) & 1) ^ 1, g.status, dead)) break;
-          mbar_expect_tx(&b_full[bs], SM::B_BYTES);
+          mbar_expect_tx(&b_full[bs], b_slot);
 #pragma unroll
           for (int c = 0; c < DB; ++c)
-            tma_load_2d(sbase + b_off + bs * SM::B_BYTES + c * TBLK, &mapAhat, &b_full[bs], h * d.D + c * 64, row0);
+            tma_load_2d(sbase + b_off + bs * b_slot + c * TBLK, c == DB - 1 ? &mapAhatTail : &mapAhat, &b_full[bs], h * d.D + c * 64, row0);
           for (int e = 0; e < d.E && !dead; ++e) {
             // 256 feature rows of expert (h, e), one 64-column stage at a time; a box that runs past
             // the expert's rows (M not a multiple of 256) fetches rows whose columns are never stored
             for (int c = 0; c < DB; ++c) {
               if (!mbar_wait(&a_empty[s], apar, g.status, dead)) break;
-              mbar_expect_tx(&a_full[s], SM::A_BYTES);
-              tma_load_2d(sbase + a_off + s * SM::A_BYTES, &mapWo, &a_full[s], c * 64, (h * d.E + e) * d.M + fc * 256);
+              mbar_expect_tx(&a_full[s], c == DB - 1 ? 256 * g.tail * 2 : SM::A_BYTES);
+              tma_load_2d(sbase + a_off + s * SM::A_BYTES, c == DB - 1 ? &mapWoTail : &mapWo, &a_full[s], c * 64, (h * d.E + e) * d.M + fc * 256);
               if (++s == AS) { s = 0; apar ^= 1; }
             }
           }
@@ -148,13 +154,15 @@ sh_tc_oproj_kernel(const __grid_constant__ CUtensorMap mapAhat, const __grid_con
       constexpr uint32_t idesc = make_idesc_f16(128, 256, 0, 0, 0);
       const uint32_t w_lo0 = desc_lo_k(sbase + a_off), t_lo0 = desc_lo_k(sbase + b_off);
       const int last_k = (d.Dt - 64 * (DB - 1) + 15) / 16;  // 16-column slices of the last block that d_head reaches
+      // (rows of 32 or 64 bytes: the swizzle spans that much, and 8-row groups are 256 or 512 bytes apart)
+      const uint32_t tail_hi = g.tail == 16 ? ((256u >> 4) | (1u << 14) | (6u << 29)) : g.tail == 32 ? ((512u >> 4) | (1u << 14) | (4u << 29)) : DESC_HI_SW128;
       int gh = 0, ge = 0, s = 0;
       uint32_t apar = 0;                                    // parity of a_full[s] for the current ring pass
       for (int w = blockIdx.x; w < g.nwork && !dead; w += gridDim.x) {
         for (int h = 0; h < d.H && !dead; ++h, ++gh) {
           const int bs = NB == 2 ? gh & 1 : 0;
           if (!mbar_wait(&b_full[bs], (gh / NB) & 1, g.status, dead)) break;
-          const uint32_t t_lo = t_lo0 + bs * (SM::B_BYTES >> 4);
+          const uint32_t t_lo = t_lo0 + bs * (b_slot >> 4);
           for (int e = 0; e < d.E && !dead; ++e, ++ge) {
             const int buf = ge & 1;
             if (!mbar_wait(&d_empty[buf], ((ge >> 1) & 1) ^ 1, g.status, dead)) break;
@@ -163,9 +171,10 @@ sh_tc_oproj_kernel(const __grid_constant__ CUtensorMap mapAhat, const __grid_con
               tc_fence_after();
               const uint32_t w_lo = w_lo0 + s * (SM::A_BYTES >> 4), tc_lo = t_lo + c * (TBLK >> 4);
               const int kn = c == DB - 1 ? last_k : 4;
+              const uint64_t hi = (uint64_t)(c == DB - 1 ? tail_hi : DESC_HI_SW128) << 32;
 #pragma unroll
               for (int k = 0; k < 4; ++k)
-                if (k < kn) umma_f16(tmem + buf * 256, desc_pack(tc_lo + 2 * k), desc_pack(w_lo + 2 * k), idesc, (c | k) != 0);
+                if (k < kn) umma_f16(tmem + buf * 256, hi | (tc_lo + 2 * k), hi | (w_lo + 2 * k), idesc, (c | k) != 0);
               umma_commit(&a_empty[s]);                     // this stage can load its next box
               if (++s == AS) { s = 0; apar ^= 1; }
             }
