@@ -118,13 +118,14 @@ XPart part_qk(sh_layer* L, const void* x, int first, int groups) {
 }
 
 // dst += gate x W^T over a side's expert lists: value experts, and query / key experts where a layer has them.
-XPart part_v(sh_layer* L, const void* x, int side, const PlaneMap& w, float* dst, float scale) {
+XPart part_v(sh_layer* L, const void* x, int side, const PlaneMap& w, float* dst, float scale, int ksplit = 1) {
   const ShDims& d = L->d;
   XGemmArgs g = base_args(L, x);
   use_side(g, L, side);
   g.v = dst; g.vscale = scale;
   col_tiles(g, d.Dt);
-  return part<X_V>(L, g, d.H * head_tiles(d), g.nsub, 1, &w);
+  g.ksplit = ksplit;
+  return part<X_V>(L, g, d.H * head_tiles(d), g.nsub, ksplit, &w);
 }
 
 template <int D>
@@ -183,6 +184,16 @@ int k_parts(sh_layer* L, long blocks, long steps) {
   const long most = steps / 8 < 1 ? 1 : steps / 8;
   p = p > most ? most : p;
   return p < 1 ? 1 : (int)p;
+}
+
+// Parts of a contraction on the half-SM blocks, where its result is added anyway: enough blocks for both
+// places of every SM, at least eight steps each (a block works off about one step a us whether it has the SM
+// to itself or shares it).
+int half_blocks(sh_layer* L, long blocks, long steps) {
+  long p = 2l * sm_count(L) / (blocks < 1 ? 1 : blocks);
+  const long most = steps / 8;
+  p = p > most ? most : p;
+  return p < 1 ? 1 : p > 8 ? 8 : (int)p;
 }
 
 }  // namespace
@@ -277,7 +288,9 @@ int sh_f32_backward(sh_layer* L, const void* x, const float* dout, float* dx, fl
   // output experts: dAhat and the destination gates' gradients
   g = dst;
   col_tiles(g, d.Dt);
-  if ((rc = launch_x<X_DA>(L, st, part<X_DA>(L, g, d.H * ht, g.nsub)))) return rc;
+  // (about half of the experts' last tiles are worth counting; the rest of the table is empty)
+  g.ksplit = half_blocks(L, ((long)d.H * d.N * d.k / 128 + d.H * d.E / 2) * g.nsub, d.M / XG_BK);
+  if ((rc = launch_x<X_DA>(L, st, part<X_DA>(L, g, d.H * ht, g.nsub, g.ksplit)))) return rc;
   // attention
   const int rows = d.N * d.H;
   if ((rc = launch_k(true, sh_f32_rowdot_kernel, dim3((unsigned)((rows + 7) / 8)), dim3(256), 0, st, (const float*)w.dahat,
@@ -294,7 +307,8 @@ int sh_f32_backward(sh_layer* L, const void* x, const float* dout, float* dx, fl
   // queries, keys and gates: the rest of dx
   g = src;
   col_tiles(g, d.M);
-  if ((rc = launch_x<X_DX>(L, st, part<X_DX>(L, g, d.nblk, g.nsub)))) return rc;
+  g.ksplit = half_blocks(L, (long)d.nblk * g.nsub, 2 * d.H * ((d.Dt + XG_BK - 1) / XG_BK));
+  if ((rc = launch_x<X_DX>(L, st, part<X_DX>(L, g, d.nblk, g.nsub, g.ksplit)))) return rc;
   // weight gradients, one launch; contractions in parts where whole ones would leave SMs without a tile
   auto wpart = [](const XGemmArgs& a, int gx, int gy, int gz) { XWPart p; p.g = a; p.gx = gx; p.gy = gy; p.n = gx * gy * gz; return p; };
   XGemmArgs gq = src, gv = src, go = dst;

@@ -56,7 +56,7 @@ struct XGemmArgs {
   const int* lists; const float* lgate; const int* offsets; const ShTile* tiles;   // of the side the mode works on
   int nsub, sub_cols;                    // column tiles per head (or of M), and columns per tile (a multiple of 16)
   int qk_first, qk_groups;               // X_QK: first group ((which*H + h)) and how many
-  int ksplit;                            // X_DW*: parts of the contraction (more than one: the results are added)
+  int ksplit;                            // parts of the contraction (weight gradients: with more than one the results are added)
   float *q, *k, *v;                      // X_QK: q, k [B, H, T, D]; X_V: v
   float *y;                              // X_O [rows of out, M]
   float *dahat, *ds, *dx;                // ds: gate gradients in list order
@@ -178,7 +178,7 @@ __device__ __forceinline__ void xg_tile(const CUtensorMap& mapW, const CUtensorM
   constexpr int BN = XG_BN;
   constexpr bool B_MN = MODE >= X_DA;
   constexpr bool LIST_ROWS = MODE == X_V || MODE == X_O || MODE == X_DA || MODE == X_DR;
-  constexpr bool BULK = LIST_ROWS || MODE == X_QK;         // results that leave as one bulk operation per row
+  constexpr bool ADDED = MODE != X_QK;                     // results that are added to (as one bulk operation per row; stored by X_QK)
   constexpr int COLS = BN / 2;                             // columns of a worker thread
   extern __shared__ unsigned char smem_raw[];
   const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -221,12 +221,21 @@ __device__ __forceinline__ void xg_tile(const CUtensorMap& mapW, const CUtensorM
     row0 = blk.x * 128; nrows = min(128, d.N - row0);
     steps = d.M / XG_BK;
   }
+  // a part of the contraction (modes whose results are added): steps s0 ...
+  int s0 = 0;
+  if (ADDED && g.ksplit > 1) {
+    const int per = (steps + g.ksplit - 1) / g.ksplit;
+    s0 = blk.z * per;
+    steps = min(per, steps - s0);
+    if (steps <= 0) return;
+  }
   if (warp == 8) { tmem_alloc(tmem_slot, 256); tmem_relinquish(); }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   // contraction positions of step i that exist (the rest of the operand rows is zero)
   auto kvalid = [&](int i) -> int {
+    i += s0;
     if (MODE == X_O || MODE == X_DR) return min(XG_BK, d.Dt - XG_BK * i);
     if (MODE == X_DX) {
       const int seg = i / sps;
@@ -274,18 +283,19 @@ __device__ __forceinline__ void xg_tile(const CUtensorMap& mapW, const CUtensorM
       for (int i = 0; i < steps && !dead; ++i) {
         if (!mbar_wait(&empty_bar[s], par, g.status, dead)) break;
         mbar_expect_tx(&full_bar[s], 3 * SM::B_PLANE);
-        int x = i * XG_BK, y = 0;
+        const int ii = s0 + i;
+        int x = ii * XG_BK, y = 0;
         bool gm = false;
         if (MODE == X_QK) y = (which * d.H + h) * d.D + n0;
         if (MODE == X_V) y = (h * d.E + e) * d.D + n0;
         if (MODE == X_O) y = (h * d.E + e) * d.M + n0;
-        if (MODE == X_DA) { x = n0; y = (h * d.E + e) * d.M + i * XG_BK; }
-        if (MODE == X_DR) { x = n0; y = (h * d.E + e) * d.D + i * XG_BK; }
+        if (MODE == X_DA) { x = n0; y = (h * d.E + e) * d.M + ii * XG_BK; }
+        if (MODE == X_DR) { x = n0; y = (h * d.E + e) * d.D + ii * XG_BK; }
         if (MODE == X_DX) {
-          const int seg = i / sps;
+          const int seg = ii / sps;
           x = n0;
           gm = seg >= 2 * d.H;
-          y = gm ? (i - 2 * d.H * sps) * XG_BK : seg * d.D + (i - seg * sps) * XG_BK;
+          y = gm ? (ii - 2 * d.H * sps) * XG_BK : seg * d.D + (ii - seg * sps) * XG_BK;
         }
         tma_load_3d(sbase + s * SM::STAGE + 3 * SM::A_PLANE, gm ? &mapG : &mapW, &full_bar[s], x, y, 0);
         if (++s == XG_STAGES) { s = 0; par ^= 1; }
@@ -320,10 +330,10 @@ __device__ __forceinline__ void xg_tile(const CUtensorMap& mapW, const CUtensorM
                     : MODE == X_DA ? g.dy + t * d.M
                     : MODE == X_DR ? g.dv + t * HD + h * d.D : g.dq + t * HD) + (lane & 7) * 4;
       }
-    int xseg = 0, xoff = 0;                                // X_DX: the step's head (of dq, then dk), and where in it
+    int xseg = min(s0 / sps, 2 * d.H), xoff = (s0 - xseg * sps) * XG_BK;   // X_DX: the step's head (of dq, then dk), and where in it
     const uint32_t rbase = sbase + SM::RAW_OFF + warp * 2048;
     auto load = [&](int i) {                               // step i on its way
-      long o = (long)i * XG_BK;
+      long o = (long)(s0 + i) * XG_BK;
       if (MODE == X_DX) o = (xseg >= d.H ? (long)(g.dk - g.dq) + (long)(xseg - d.H) * d.D : (long)xseg * d.D) + xoff;
 #pragma unroll
       for (int j = 0; j < 2; ++j)
@@ -421,20 +431,7 @@ __device__ __forceinline__ void xg_tile(const CUtensorMap& mapW, const CUtensorM
         const float f = MODE == X_V && g.vscale != 0.f ? gt * g.vscale : gt;
 #pragma unroll
         for (int i = 0; i < COLS; ++i) acc[i] *= f;
-      } else if (MODE == X_DX) {
-        float* o = g.dx + (size_t)(row0 + r) * d.M + n0 + c0;
-#pragma unroll
-        for (int i = 0; i < COLS; i += 4) {
-          if (i + 4 <= valid && g.vec_out) {
-            float4 p = *reinterpret_cast<const float4*>(o + i);
-            p.x += acc[i]; p.y += acc[i + 1]; p.z += acc[i + 2]; p.w += acc[i + 3];
-            *reinterpret_cast<float4*>(o + i) = p;
-          } else {
-#pragma unroll
-            for (int j = 0; j < 4; ++j) if (i + j < valid) o[i + j] += acc[i + j];
-          }
-        }
-      } else {                                             // X_QK
+      } else if (MODE == X_QK) {
         const int tok = row0 + r;
         if (g.rope) {
           const float2* cs = g.rope + (size_t)((n0 + c0) >> 1) * d.T + tok % d.T;
@@ -453,7 +450,7 @@ __device__ __forceinline__ void xg_tile(const CUtensorMap& mapW, const CUtensorM
         }
       }
     }
-    if (BULK) {
+    {
       // rows through shared memory (the operand stages are free: every UMMA has been waited for), 16 bytes of
       // padding a row so that eight lanes' 16-byte stores meet different banks
       constexpr int LD = BN + 4;
@@ -475,6 +472,8 @@ __device__ __forceinline__ void xg_tile(const CUtensorMap& mapW, const CUtensorM
           if (MODE == X_O) { const int orow = sh_out_row(d, t); if (orow >= 0) o = g.y + (size_t)orow * d.M + n0; }   // (cache tokens have no output row)
           if (MODE == X_DA) o = g.dahat + (size_t)t * HD + h * d.D + n0;
           if (MODE == X_DR) o = g.dx + (size_t)t * d.M + n0;
+        } else if (MODE == X_DX) {
+          o = g.dx + (size_t)(row0 + tid) * d.M + n0;
         } else {
           const int tok = row0 + tid;
           o = (which ? g.k : g.q) + (((size_t)(tok / d.T) * d.H + h) * d.T + tok % d.T) * d.D + n0;
@@ -482,7 +481,7 @@ __device__ __forceinline__ void xg_tile(const CUtensorMap& mapW, const CUtensorM
         if (o) {
           const uint32_t src = smem_u32(stg + tid * LD);
           if (MODE == X_QK) bulk_store(o, src, n * 4);
-          else if (MODE != X_DR || g.vec_out) bulk_reduce_add_f32(o, src, n * 4);
+          else if ((MODE != X_DR && MODE != X_DX) || g.vec_out) bulk_reduce_add_f32(o, src, n * 4);
           else
             for (int i = 0; i < n; ++i) atomicAdd(o + i, stg[tid * LD + i]);
         }
