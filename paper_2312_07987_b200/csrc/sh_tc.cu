@@ -104,7 +104,7 @@ static int encode_3d_f16_store32(CUtensorMap* map, const void* base, uint64_t in
 struct TcState {
   CUtensorMap map_q, map_k, map_v;
   CUtensorMap map_q_st, map_k_st;   // Q and K as the one-grid front's epilogue stores them
-  CUtensorMap map_wqk, map_wqk128, map_wv, map_wq_e, map_wk_e, map_wo, map_wo256, map_wo_tail, map_ahat_tail, map_wos, map_ahat, map_wgate;
+  CUtensorMap map_wqk, map_wqk128, map_wv, map_wq_e, map_wk_e, map_wo, map_wo256, map_wo_tail, map_ahat_tail, map_wos, map_wo_n[2], map_wos_n[2], map_ahat, map_wgate;
   CUtensorMap map_q2d, map_r16;  // score-bias GEMM of the Transformer-XL position term: Q as [B*H*T, D], R16 as [H*T, D]
   CUtensorMap map_x;             // tensor map of the last x pointer seen (x_cached)
   CUtensorMap map_x64;           // the same tensor in 64-token boxes (gate tile of the one-grid front, 64 tokens per CTA)
@@ -245,6 +245,11 @@ int sh_tc_prepare(sh_layer* L) {
     if (L->moe_k && (rc = sh_tc_encode_2d(&S->map_wk_e, 0, ws + L->o.wk_e, d.M, (uint64_t)d.H * d.E * d.D, (uint64_t)d.M * 2, 64, d.D))) return rc;
     if ((rc = sh_tc_encode_2d(&S->map_wo, 1, ws + L->o.wo, d.D, (uint64_t)d.H * d.E * d.M, (uint64_t)d.D * 2, 64, 128))) return rc;
     if ((rc = sh_tc_encode_2d(&S->map_wo256, 1, ws + L->o.wo, d.D, (uint64_t)d.H * d.E * d.M, (uint64_t)d.D * 2, 64, 256))) return rc;
+    // (the pair kernels' narrower units: 64 or 32 rows per CTA)
+    for (int i = 0; i < 2; ++i) {
+      if ((rc = sh_tc_encode_2d(&S->map_wo_n[i], 1, ws + L->o.wo, d.D, (uint64_t)d.H * d.E * d.M, (uint64_t)d.D * 2, 64, 64 >> i))) return rc;
+      if (sh_o_sparse_ok(L) && (rc = sh_tc_encode_2d(&S->map_wos_n[i], 1, ws + L->o.wos, (uint64_t)d.D * d.E, (uint64_t)d.H * d.M, (uint64_t)d.D * d.E * 2, 64, 64 >> i))) return rc;
+    }
     if (sh_o_sparse_ok(L) && (rc = sh_tc_encode_2d(&S->map_wos, 1, ws + L->o.wos, (uint64_t)d.D * d.E, (uint64_t)d.H * d.M, (uint64_t)d.D * d.E * 2, 64, 128))) return rc;
   } else {
     if ((rc = sh_tc_encode_2d(&S->map_wo, 1, ws + L->o.wo, HD, d.M, (uint64_t)HD * 2, 64, 128))) return rc;
@@ -543,6 +548,24 @@ static int qk_pairs_max(TcState* S) {
   return S->qk_pairs_max;
 }
 
+// Clusters of a CTA-pair output projection the device holds at once (-1: none).
+template <typename K>
+static int o_pairs(K kern, int smem) {
+  if (set_smem(kern, smem) != SH_OK) return -1;
+  const int n = max_pairs(kern, 480, smem);
+  return n > 0 ? n : -1;
+}
+
+// Output features per work unit of those kernels.  A unit works off all experts of its tokens whatever its width -
+// the pipe's part of it shrinks with the width, the builders' does not -, so narrower units pay exactly as long as
+// the wide ones leave pairs without a unit.
+static int oproj_features(const TcState* S, const ShDims& d) {
+  const int rows = (sh_out_rows(d) + 255) / 256;
+  int fn = 256;
+  while (fn > 64 && rows * ((d.M + fn / 2 - 1) / (fn / 2)) <= S->o_pairs_max) fn /= 2;
+  return fn;
+}
+
 // The launches of one forward pass after grid A of a split Q/K projection is out (see sh_tc_forward).
 static int tc_forward_rest(sh_layer* L, const void* x, void* out, cudaStream_t st, const CUtensorMap& map_x, bool overlap,
                            int qkA, int qkB, TcGemmArgs& qg, bool front);
@@ -839,42 +862,40 @@ static int tc_forward_rest(sh_layer* L, const void* x, void* out, cudaStream_t s
     // (and d_head above 128: its gate-scaled operand would be one more fp16 rounding than such a layer has had)
     bool pair = S->o_pair && d.k <= OPAIR_KMAX && d.D <= 128;
     const bool sparse = pair && S->o_sparse && sh_o_sparse_ok(L);
-    if (sparse) {
-      constexpr int psm = OprojSpSmem<128>::TOTAL;
-      if (d.E == 4) { if ((rc = set_smem(sh_tc_oproj_sp_kernel<128, 1>, psm))) return rc; }
-      else if ((rc = set_smem(sh_tc_oproj_sp_kernel<128, 2>, psm))) return rc;
-      if (S->o_pairs_max == 0) {
-        S->o_pairs_max = d.E == 4 ? max_pairs(sh_tc_oproj_sp_kernel<128, 1>, 480, psm) : max_pairs(sh_tc_oproj_sp_kernel<128, 2>, 480, psm);
-        if (S->o_pairs_max <= 0) S->o_pairs_max = -1;
-      }
-      if (S->o_pairs_max < 0) pair = false;
-    } else if (pair) {
-      const int psm = d.D == 128 ? OprojPairSmem<128>::TOTAL : OprojPairSmem<64>::TOTAL;
-      if (d.D == 128) { if ((rc = set_smem(sh_tc_oproj_pair_kernel<128>, psm))) return rc; }
-      else if ((rc = set_smem(sh_tc_oproj_pair_kernel<64>, psm))) return rc;
-      if (S->o_pairs_max == 0) {
-        S->o_pairs_max = d.D == 128 ? max_pairs(sh_tc_oproj_pair_kernel<128>, 480, psm) : max_pairs(sh_tc_oproj_pair_kernel<64>, 480, psm);
-        if (S->o_pairs_max <= 0) S->o_pairs_max = -1;
-      }
-      if (S->o_pairs_max < 0) pair = false;
+    if (pair && S->o_pairs_max == 0) {
+      S->o_pairs_max = sparse ? (d.E == 4 ? o_pairs(sh_tc_oproj_sp_kernel<128, 1, 256>, OprojSpSmem<128, 256>::TOTAL)
+                                          : o_pairs(sh_tc_oproj_sp_kernel<128, 2, 256>, OprojSpSmem<128, 256>::TOTAL))
+                     : d.D == 128 ? o_pairs(sh_tc_oproj_pair_kernel<128, 256>, OprojPairSmem<128, 256>::TOTAL)
+                                  : o_pairs(sh_tc_oproj_pair_kernel<64, 256>, OprojPairSmem<64, 256>::TOTAL);
     }
-    if (pair && sparse) {
-      // 256 tokens x 256 features per unit, the selection as 2:4 sparsity of the gate-scaled A operand
-      constexpr int psm = OprojSpSmem<128>::TOTAL;
-      a.nwork = ((sh_out_rows(d) + 255) / 256) * ((d.M + 255) / 256);
-      const unsigned pgrid = 2u * (unsigned)(a.nwork < S->o_pairs_max ? a.nwork : S->o_pairs_max);
+    if (pair && S->o_pairs_max < 0) pair = false;
+    if (pair) {
+      // 256 tokens x 256 (128, 64) features per unit; the gates are folded into the A operand, the selection - where
+      // at most two of four neighbouring experts are chosen - is its 2:4 sparsity
       const __half* ahat = (const __half*)(ws + L->o.ahat);
-      if (d.E == 4) rc = launch_k_pairs(pdl, sh_tc_oproj_sp_kernel<128, 1>, dim3(pgrid), dim3(480), psm, st, S->map_wos, a, ahat);
-      else rc = launch_k_pairs(pdl, sh_tc_oproj_sp_kernel<128, 2>, dim3(pgrid), dim3(480), psm, st, S->map_wos, a, ahat);
-      if (rc) return rc;
-    } else if (pair) {
-      // 256 tokens x 256 features per unit, gates folded into the A operand
-      const int psm = d.D == 128 ? OprojPairSmem<128>::TOTAL : OprojPairSmem<64>::TOTAL;
-      a.nwork = ((sh_out_rows(d) + 255) / 256) * ((d.M + 255) / 256);
-      const unsigned pgrid = 2u * (unsigned)(a.nwork < S->o_pairs_max ? a.nwork : S->o_pairs_max);
-      const __half* ahat = (const __half*)(ws + L->o.ahat);
-      if (d.D == 128) rc = launch_k_pairs(pdl, sh_tc_oproj_pair_kernel<128>, dim3(pgrid), dim3(480), psm, st, S->map_wo, a, ahat);
-      else rc = launch_k_pairs(pdl, sh_tc_oproj_pair_kernel<64>, dim3(pgrid), dim3(480), psm, st, S->map_wo, a, ahat);
+      const int fn = oproj_features(S, d);
+      auto go = [&](auto kern, int psm, const CUtensorMap& map) -> int {
+        a.nwork = ((sh_out_rows(d) + 255) / 256) * ((d.M + fn - 1) / fn);
+        const unsigned pgrid = 2u * (unsigned)(a.nwork < S->o_pairs_max ? a.nwork : S->o_pairs_max);
+        if (int r = set_smem(kern, psm)) return r;
+        return launch_k_pairs(pdl, kern, dim3(pgrid), dim3(480), psm, st, map, a, ahat);
+      };
+      if (fn == 256) {
+        if (sparse) rc = d.E == 4 ? go(sh_tc_oproj_sp_kernel<128, 1, 256>, OprojSpSmem<128, 256>::TOTAL, S->map_wos)
+                                  : go(sh_tc_oproj_sp_kernel<128, 2, 256>, OprojSpSmem<128, 256>::TOTAL, S->map_wos);
+        else rc = d.D == 128 ? go(sh_tc_oproj_pair_kernel<128, 256>, OprojPairSmem<128, 256>::TOTAL, S->map_wo)
+                             : go(sh_tc_oproj_pair_kernel<64, 256>, OprojPairSmem<64, 256>::TOTAL, S->map_wo);
+      } else if (fn == 128) {
+        if (sparse) rc = d.E == 4 ? go(sh_tc_oproj_sp_kernel<128, 1, 128>, OprojSpSmem<128, 128>::TOTAL, S->map_wos_n[0])
+                                  : go(sh_tc_oproj_sp_kernel<128, 2, 128>, OprojSpSmem<128, 128>::TOTAL, S->map_wos_n[0]);
+        else rc = d.D == 128 ? go(sh_tc_oproj_pair_kernel<128, 128>, OprojPairSmem<128, 128>::TOTAL, S->map_wo_n[0])
+                             : go(sh_tc_oproj_pair_kernel<64, 128>, OprojPairSmem<64, 128>::TOTAL, S->map_wo_n[0]);
+      } else {
+        if (sparse) rc = d.E == 4 ? go(sh_tc_oproj_sp_kernel<128, 1, 64>, OprojSpSmem<128, 64>::TOTAL, S->map_wos_n[1])
+                                  : go(sh_tc_oproj_sp_kernel<128, 2, 64>, OprojSpSmem<128, 64>::TOTAL, S->map_wos_n[1]);
+        else rc = d.D == 128 ? go(sh_tc_oproj_pair_kernel<128, 64>, OprojPairSmem<128, 64>::TOTAL, S->map_wo_n[1])
+                             : go(sh_tc_oproj_pair_kernel<64, 64>, OprojPairSmem<64, 64>::TOTAL, S->map_wo_n[1]);
+      }
       if (rc) return rc;
     } else {
       a.nwork = ((sh_out_rows(d) + 127) / 128) * ((d.M + 255) / 256);

@@ -39,9 +39,10 @@ namespace shtc {
 
 constexpr int OPAIR_KMAX = 4;                            // selections per (token, head) a builder keeps in registers (the kernel serves k <= 4)
 
-template <int D>
+// FN: output features of a work unit (256, or 128 / 64 where units of 256 would leave pairs without work).
+template <int D, int FN>
 struct OprojPairSmem {
-  static constexpr int W_BYTES = 128 * 64 * 2;           // one 64-column block of this CTA's 128 feature rows of an expert
+  static constexpr int W_BYTES = FN / 2 * 64 * 2;        // one 64-column block of this CTA's half of an expert's feature rows
   static constexpr int P_BYTES = 128 * D * 2;            // scaled token tile: this CTA's 128 tokens x D
   static constexpr int WST = 5, PST = 4;                 // ring depths
   static constexpr int STAGING = 4 * 32 * 32 * 4;        // per epilogue warp a 32 x 32 fp32 transpose tile
@@ -70,10 +71,10 @@ __device__ __forceinline__ void oproj_store_chunk(uint32_t taddr, int c, float* 
   }
 }
 
-template <int D>
+template <int D, int FN>
 __global__ void __launch_bounds__(480, 1)
 sh_tc_oproj_pair_kernel(const __grid_constant__ CUtensorMap mapWo, TcOprojArgs g, const __half* __restrict__ ahat) {
-  using SM = OprojPairSmem<D>;
+  using SM = OprojPairSmem<D, FN>;
   constexpr int DB = D / 64;                             // 64-column (128-byte) blocks per row
   constexpr int WST = SM::WST, PST = SM::PST;
   static_assert(WST <= 8 && PST <= 4, "barrier slots");
@@ -97,7 +98,7 @@ sh_tc_oproj_pair_kernel(const __grid_constant__ CUtensorMap mapWo, TcOprojArgs g
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();               // 0 = leader
   const int pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
-  const int nfc = (d.M + 255) / 256;
+  const int nfc = (d.M + FN - 1) / FN;
   const int HD = d.H * D;
   const int nout = sh_out_rows(d);                       // rows of out (= tokens, unless a cache sits in front of every sequence)
   bool dead = false;
@@ -127,13 +128,13 @@ sh_tc_oproj_pair_kernel(const __grid_constant__ CUtensorMap mapWo, TcOprojArgs g
       for (int w = pair; w < g.nwork && !dead; w += npairs) {
         const int fc = w % nfc;
         for (int he = 0; he < d.H * d.E && !dead; ++he) {
-          // this CTA's 128 of the 256 feature rows of expert he = h * E + e, one 64-column block at a
+          // this CTA's half of the unit's feature rows of expert he = h * E + e, one 64-column block at a
           // time; a box that runs past the expert's rows (M not a multiple of 256) fetches rows whose
           // columns are never stored
           for (int c = 0; c < DB; ++c) {
             if (!mbar_wait(&w_empty[s], wpar, g.status, dead)) break;
             if (rank == 0) mbar_expect_tx(&w_full[s], 2 * SM::W_BYTES);
-            tma_load_2d_pair(sbase + w_off + s * SM::W_BYTES, &mapWo, &w_full[s], c * 64, he * d.M + fc * 256 + (int)rank * 128);
+            tma_load_2d_pair(sbase + w_off + s * SM::W_BYTES, &mapWo, &w_full[s], c * 64, he * d.M + fc * FN + (int)rank * (FN / 2));
             if (++s == WST) { s = 0; wpar ^= 1; }
           }
         }
@@ -149,7 +150,7 @@ sh_tc_oproj_pair_kernel(const __grid_constant__ CUtensorMap mapWo, TcOprojArgs g
       // only while it holds the token: every earlier phase of those barriers is then complete, so a
       // barrier it has not watched for a while cannot answer with a stale parity.
       const int me = warp == 1 ? 0 : 1;
-      constexpr uint32_t idesc = make_idesc_f16(256, 256, 0, 0, 0);
+      constexpr uint32_t idesc = make_idesc_f16(256, FN, 0, 0, 0);
       const uint32_t w_lo0 = desc_lo_k(sbase + w_off), p_lo0 = desc_lo_k(sbase + p_off);
       int un = 0, s = 0, ps = 0, ge = 0;
       uint32_t wpar = 0, ppar = 0;                          // parities to wait for on w_full[s], p_full[ps]
@@ -269,7 +270,7 @@ sh_tc_oproj_pair_kernel(const __grid_constant__ CUtensorMap mapWo, TcOprojArgs g
       }
     }
   } else if (warp < 14) {
-    // ---- epilogue: warp = 32 tokens (TMEM lane quarter warp & 3), all 256 features of the unit ----
+    // ---- epilogue: warp = 32 tokens (TMEM lane quarter warp & 3), all features of the unit ----
     const int q = warp & 3;
     const uint32_t lane_off = (uint32_t)(q * 32) << 16;
     float* stg = reinterpret_cast<float*>(sgen + stg_off) + (warp - 10) * 1024;
@@ -280,11 +281,11 @@ sh_tc_oproj_pair_kernel(const __grid_constant__ CUtensorMap mapWo, TcOprojArgs g
       const int rows_here = min(32, nout - row0 - q * 32); // <= 0: these rows are past the end
       if (!mbar_wait(&d_full[buf], (un >> 1) & 1, g.status, dead)) break;
       tc_fence_after();
-      const size_t obase = (size_t)(row0 + q * 32) * d.M + fc * 256;
+      const size_t obase = (size_t)(row0 + q * 32) * d.M + fc * FN;
 #pragma unroll 1
-      for (int c = 0; c < 8; ++c) {
-        oproj_store_chunk(tmem + lane_off + buf * 256, c, stg, g.out, obase, g.out_f16, d.M, rows_here, fc * 256 + c * 32 < d.M, lane);
-        if (c == 7) {                                      // everything has been read: hand the accumulator back
+      for (int c = 0; c < FN / 32; ++c) {
+        oproj_store_chunk(tmem + lane_off + buf * 256, c, stg, g.out, obase, g.out_f16, d.M, rows_here, fc * FN + c * 32 < d.M, lane);
+        if (c == FN / 32 - 1) {                                      // everything has been read: hand the accumulator back
           tc_fence_before();
           __syncwarp();
           if (lane == 0) mbar_arrive_leader(&d_empty[buf]);

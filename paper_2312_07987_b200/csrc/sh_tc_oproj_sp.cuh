@@ -40,9 +40,11 @@ namespace shtc {
 
 constexpr int OSP_MAXH = 4;                              // heads whose position codes the epilogue keeps in registers
 
-template <int D>
+// FN: output features of a work unit (256, or 128 / 64 where units of 256 would leave pairs without work: see
+// oproj_features in sh_tc.cu).  Every output element is the same sum in the same order with any of them.
+template <int D, int FN>
 struct OprojSpSmem {
-  static constexpr int W_BYTES = 128 * 64 * 2;           // 64 logical K positions of this CTA's 128 feature rows
+  static constexpr int W_BYTES = FN / 2 * 64 * 2;        // 64 logical K positions of this CTA's half of the feature rows
   static constexpr int P_BYTES = 128 * 128 * 2;          // 128 compressed columns of this CTA's 128 tokens
   static constexpr int WST = 7, PST = 3;                 // ring depths
   static constexpr int STAGING = 4 * 32 * 32 * 4;
@@ -86,11 +88,11 @@ __device__ __forceinline__ __half2 osp_scale(__half a, __half2 g_hi, __half2 g_l
 }
 
 // SPT = E / 4: stages a builder thread fills per head (and groups per d).
-template <int D, int SPT>
+template <int D, int SPT, int FN>
 __global__ void __launch_bounds__(480, 1)
 sh_tc_oproj_sp_kernel(const __grid_constant__ CUtensorMap mapWos, TcOprojArgs g, const __half* __restrict__ ahat) {
   static_assert(D == 128 && (SPT == 1 || SPT == 2), "served shapes");
-  using SM = OprojSpSmem<D>;
+  using SM = OprojSpSmem<D, FN>;
   constexpr int WST = SM::WST, PST = SM::PST;
   constexpr int SPH = 2 * SPT;                           // ring stages per head
   constexpr int WPH = 8 * SPT;                           // weight blocks per head (E * D / 64)
@@ -119,7 +121,7 @@ sh_tc_oproj_sp_kernel(const __grid_constant__ CUtensorMap mapWos, TcOprojArgs g,
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();               // 0 = leader
   const int pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
-  const int nfc = (d.M + 255) / 256;
+  const int nfc = (d.M + FN - 1) / FN;
   const int HD = d.H * D;
   const int nout = sh_out_rows(d);
   bool dead = false;
@@ -152,12 +154,12 @@ sh_tc_oproj_sp_kernel(const __grid_constant__ CUtensorMap mapWos, TcOprojArgs g,
       for (int w = pair; w < g.nwork && !dead; w += npairs) {
         const int fc = w % nfc;
         for (int h = 0; h < d.H && !dead; ++h) {
-          // this CTA's 128 of the unit's 256 feature rows of W_cat^h, 64 K positions at a time; a box that
+          // this CTA's half of the unit's feature rows of W_cat^h, 64 K positions at a time; a box that
           // runs past the head's rows (M not a multiple of 256) fetches rows whose columns are never stored
           for (int c = 0; c < WPH; ++c) {
             if (!mbar_wait(&w_empty[s], wpar, g.status, dead)) break;
             if (rank == 0) mbar_expect_tx(&w_full[s], 2 * SM::W_BYTES);
-            tma_load_2d_pair(sbase + w_off + s * SM::W_BYTES, &mapWos, &w_full[s], c * 64, h * d.M + fc * 256 + (int)rank * 128);
+            tma_load_2d_pair(sbase + w_off + s * SM::W_BYTES, &mapWos, &w_full[s], c * 64, h * d.M + fc * FN + (int)rank * (FN / 2));
             if (++s == WST) { s = 0; wpar ^= 1; }
           }
         }
@@ -167,7 +169,7 @@ sh_tc_oproj_sp_kernel(const __grid_constant__ CUtensorMap mapWos, TcOprojArgs g,
     if (lane == 0 && rank == 0) {
       // two issuing threads take the ring stages in turn and pass a token (see sh_tc_oproj_pair_kernel)
       const int me = warp == 1 ? 0 : 1;
-      constexpr uint32_t idesc = make_idesc_f16(256, 256, 0, 0, 0) | (1u << 2);     // sparse A
+      constexpr uint32_t idesc = make_idesc_f16(256, FN, 0, 0, 0) | (1u << 2);     // sparse A
       const uint32_t w_lo0 = desc_lo_k(sbase + w_off), p_lo0 = desc_lo_k(sbase + p_off);
       int un = 0, s = 0, ps = 0, ge = 0;
       uint32_t wpar = 0, ppar = 0;
@@ -295,7 +297,7 @@ sh_tc_oproj_sp_kernel(const __grid_constant__ CUtensorMap mapWos, TcOprojArgs g,
       }
     }
   } else if (warp < 14) {
-    // ---- epilogue: warp = 32 tokens (TMEM lane quarter warp & 3), all 256 features of the unit ----
+    // ---- epilogue: warp = 32 tokens (TMEM lane quarter warp & 3), all features of the unit ----
     const int q = warp & 3;
     const uint32_t lane_off = (uint32_t)(q * 32) << 16;
     float* stg = reinterpret_cast<float*>(sgen + stg_off) + (warp - 10) * 1024;
@@ -343,10 +345,10 @@ sh_tc_oproj_sp_kernel(const __grid_constant__ CUtensorMap mapWos, TcOprojArgs g,
       if (more) codes_of(w + npairs);                      // (fetched before the wait: an L2 round trip)
       if (!mbar_wait(&d_full[buf], (un >> 1) & 1, g.status, dead)) break;
       tc_fence_after();
-      const size_t obase = (size_t)(row0 + q * 32) * d.M + fc * 256;
+      const size_t obase = (size_t)(row0 + q * 32) * d.M + fc * FN;
       const uint32_t taddr = tmem + lane_off + buf * 256;
 #pragma unroll 1
-      for (int c = 0; c < 8; ++c) {
+      for (int c = 0; c < FN / 32; ++c) {
         uint32_t v[32];
         tmem_ld32(taddr + c * 32, v);
         tmem_ld_wait();
@@ -356,7 +358,7 @@ sh_tc_oproj_sp_kernel(const __grid_constant__ CUtensorMap mapWos, TcOprojArgs g,
         for (int ch = 0; ch < 8; ++ch)
           *reinterpret_cast<uint4*>(stg + lane * 32 + ((ch ^ (lane & 7)) << 2)) = make_uint4(v[4 * ch], v[4 * ch + 1], v[4 * ch + 2], v[4 * ch + 3]);
         __syncwarp();
-        if (fc * 256 + c * 32 < d.M) {
+        if (fc * FN + c * 32 < d.M) {
 #pragma unroll
           for (int r4 = 0; r4 < 32; r4 += 4) {
             const int r = r4 + (lane >> 3), ch = lane & 7;
@@ -364,7 +366,7 @@ sh_tc_oproj_sp_kernel(const __grid_constant__ CUtensorMap mapWos, TcOprojArgs g,
               oproj_put4(g.out, obase + (size_t)r * d.M + c * 32 + 4 * ch, *reinterpret_cast<const float4*>(stg + r * 32 + ((ch ^ (r & 7)) << 2)), g.out_f16);
           }
         }
-        if (c == 7) {
+        if (c == FN / 32 - 1) {
           tc_fence_before();
           __syncwarp();
           if (lane == 0) mbar_arrive_leader(&d_empty[buf]);
