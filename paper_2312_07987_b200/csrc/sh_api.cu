@@ -231,14 +231,12 @@ extern "C" int sh_set_workspace(sh_layer* L, void* workspace, size_t bytes) {
   return SH_OK;
 }
 
-template <typename TI, typename TO>
+template <typename TI, typename TO, int PLANES = 1>
 static void repack(const void* in, void* out, int batch, int rows, int cols, long obs, long ors, long oes,
-                   cudaStream_t st) {
-  long total = (long)batch * rows * cols;
-  int blocks = (int)((total + 255) / 256);
-  if (blocks > 65535 * 4) blocks = 65535 * 4;
-  if (blocks < 1) blocks = 1;
-  sh_repack_kernel<TI, TO><<<blocks, 256, 0, st>>>((const TI*)in, (TO*)out, batch, rows, cols, obs, ors, oes);
+                   cudaStream_t st, long plane = 0) {
+  const unsigned gy = (unsigned)((rows + 31) / 32), gz = (unsigned)batch;
+  dim3 grid((unsigned)((cols + 31) / 32), gy < 65535 ? gy : 65535, gz < 65535 ? gz : 65535);
+  sh_repack_kernel<TI, TO, PLANES><<<grid, 256, 0, st>>>((const TI*)in, (TO*)out, batch, rows, cols, obs, ors, oes, plane);
 }
 
 template <typename TI, typename TM>
@@ -321,10 +319,7 @@ static int set_weights_f32(sh_layer* L, const float* Wq, const float* Wk, const 
     SH_CUDA_CHECK(cudaMemsetAsync(ws + L->o.k, 0, (size_t)d.N * HD * 4, st));
   }
   auto split = [&](const float* in, size_t off, long first, int batch, int rows, int cols, long obs, long ors, long oes, long plane) {
-    const long total = (long)batch * rows * cols;
-    long blocks = (total + 255) / 256;
-    blocks = blocks > 65535 * 4 ? 65535 * 4 : blocks;
-    sh_repack_split_kernel<<<(unsigned)blocks, 256, 0, st>>>(in, (__nv_bfloat16*)(ws + off) + first, batch, rows, cols, obs, ors, oes, plane);
+    repack<float, __nv_bfloat16, 3>(in, (__nv_bfloat16*)(ws + off) + first, batch, rows, cols, obs, ors, oes, st, plane);
   };
   const long DM = (long)d.D * d.M;
   if (L->moe_q) split(Wq, L->o.wq_e, 0, d.H * d.E, d.M, d.Dt, DM, d.M, 1, nexp);

@@ -4,40 +4,39 @@
 #include "sh_internal.cuh"
 
 // ---------------------------------------------------------------------------------------
-// Weight repack: out[b*obs + c*ors + r*oes] = in[b*rows*cols + r*cols + c]  (a batched
-// transpose with free output strides), with type conversion.
+// Weight repack: out[b*obs + c*ors + r*oes] = in[b*rows*cols + r*cols + c]  (a batched transpose with free
+// output strides), with type conversion; PLANES = 3: into three bf16 planes, `plane` elements apart, whose
+// sum is the fp32 value (fp32 configuration).  32 x 32 tiles through shared memory, so that reads run along
+// c and writes along r (a thread per element in output order read a column of `in` at a time, a 32-byte
+// sector for every value).
 // ---------------------------------------------------------------------------------------
-template <typename TI, typename TO>
-__global__ void sh_repack_kernel(const TI* __restrict__ in, TO* __restrict__ out, int batch, int rows,
-                                 int cols, long obs, long ors, long oes) {
-  long total = (long)batch * rows * cols;
-  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < total; i += (long)gridDim.x * blockDim.x) {
-    int r = (int)(i % rows);
-    long t = i / rows;
-    int c = (int)(t % cols);
-    int b = (int)(t / cols);
-    float v = sh_to_float<TI>(in[((long)b * rows + r) * cols + c]);
-    out[b * obs + c * ors + r * oes] = sh_from_float<TO>(v);
-  }
-}
-
-// The same into three bf16 planes, `plane` elements apart, whose sum is the fp32 value (fp32 configuration).
-static __global__ void sh_repack_split_kernel(const float* __restrict__ in, __nv_bfloat16* __restrict__ out, int batch, int rows,
-                                              int cols, long obs, long ors, long oes, long plane) {
-  const long total = (long)batch * rows * cols;
-  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < total; i += (long)gridDim.x * blockDim.x) {
-    const int r = (int)(i % rows);
-    const long t = i / rows;
-    const int c = (int)(t % cols), b = (int)(t / cols);
-    float v = in[((long)b * rows + r) * cols + c];
-    __nv_bfloat16* o = out + b * obs + c * ors + r * oes;
+template <typename TI, typename TO, int PLANES = 1>
+__global__ void __launch_bounds__(256)
+sh_repack_kernel(const TI* __restrict__ in, TO* __restrict__ out, int batch, int rows, int cols, long obs, long ors, long oes, long plane) {
+  __shared__ float tile[32][33];
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const int c0 = blockIdx.x * 32;
+  for (int b = blockIdx.z; b < batch; b += gridDim.z)
+    for (int r0 = blockIdx.y * 32; r0 < rows; r0 += gridDim.y * 32) {
+      __syncthreads();
 #pragma unroll
-    for (int p = 0; p < 3; ++p) {
-      const __nv_bfloat16 w = __float2bfloat16_rn(v);
-      o[p * plane] = w;
-      v -= __bfloat162float(w);
+      for (int i = 0; i < 32; i += 8)
+        if (r0 + ty + i < rows && c0 + tx < cols) tile[ty + i][tx] = sh_to_float<TI>(in[((long)b * rows + r0 + ty + i) * cols + c0 + tx]);
+      __syncthreads();
+#pragma unroll
+      for (int i = 0; i < 32; i += 8) {
+        const int r = r0 + tx, c = c0 + ty + i;
+        if (r >= rows || c >= cols) continue;
+        float v = tile[tx][ty + i];
+        TO* o = out + b * obs + c * ors + r * oes;
+#pragma unroll
+        for (int p = 0; p < PLANES; ++p) {
+          const TO w = sh_from_float<TO>(v);
+          o[p * plane] = w;
+          v -= sh_to_float<TO>(w);
+        }
+      }
     }
-  }
 }
 
 // ---------------------------------------------------------------------------------------
