@@ -69,8 +69,8 @@ enum {
 
 /* Create a layer description.  Host-only, no CUDA call.
  * Requires 1 <= k <= n_experts <= 32, n_heads >= 1, 1 <= d_head <= 256, d_model a positive multiple of 64.
- * (bf16 storage with d_head above 128 - the paper's 132 and 168 - runs every stage on the CUDA-core
- * kernels: correct and slow, the plain layer only; the tensor-core kernels serve d_head <= 128.)
+ * (bf16 storage with d_head above 128 - the paper's 132 and 168 - serves the plain layer only: no cache,
+ * no query / key experts, fp32 output.)
  * d_head is stored padded with zero columns to 64, 128 or 256 (bf16 storage) or to 32, 64, 128 or 256 (fp32): the padding changes no result (the scale stays 1/sqrt(d_head)),
  * it costs the time of the padded size, and the Q, K, V, Ahat debug buffers have the padded
  * width.  Returns NULL on error (see sh_last_error). */
@@ -106,8 +106,9 @@ sh_layer* sh_create_moe_qk(int d_model, int n_heads, int d_head, int n_experts, 
  * and Ws = Wd = NULL.  Returns NULL on error. */
 sh_layer* sh_create_dense(int d_model, int n_heads, int d_head);
 
-/* Fix the storage type and the problem size.  dtype SH_F32: x and weights fp32, all
- * arithmetic fp32 on CUDA cores.  dtype SH_BF16: x and weights bf16, tensor-core products
+/* Fix the storage type and the problem size.  dtype SH_F32: x and weights fp32;
+ * projections on the tensor cores with every fp32 operand as the sum of three bf16 values (six products,
+ * fp32 accumulation: fp32 accuracy), gates and attention in fp32 on the CUDA cores.  dtype SH_BF16: x and weights bf16, tensor-core products
  * with fp32 accumulation, fp16 intermediates (Q, K, V, P, A^h V^h); requires d_model a
  * multiple of 128.  `out` is fp32 in both cases.
  * batch*seq*n_heads*k must be below 2^31.  Invalidates workspace and weights. */
@@ -205,8 +206,7 @@ enum {
  * (%globaltimer, nanoseconds): `resident` = its first CTA running, `start` = its first CTA past
  * the wait for the kernel it depends on, `end` = its last CTA done.  Waits for `stream`, then
  * fills the HOST array stamps[3][SH_STAMP_COUNT] = {resident[], start[], end[]}.  A kernel that
- * did not run in this pass (and every kernel of the fp32 configuration, whose CUDA-core kernels
- * carry no stamps) leaves resident = start = UINT64_MAX and end = 0.  The spans of kernels that
+ * did not run in this pass (and every kernel of the fp32 configuration, which carry no stamps) leaves resident = start = UINT64_MAX and end = 0.  The spans of kernels that
  * overlap in time may be subtracted from one another: they share one clock. */
 int sh_forward_stamped(sh_layer* layer, const void* x, void* out, void* stream, uint64_t* stamps);
 
@@ -265,7 +265,7 @@ int sh_noalloc_gate_topk(int dtype, int n_tokens, int d_model, int n_heads, int 
  * left in the workspace; otherwise SH_ERR_NOT_CONFIGURED).  dout [batch, seq, d_model] fp32 = dL/dout.
  * Every result is a device buffer of the caller, fp32, OVERWRITTEN: dx [batch, seq, d_model]; dWq, dWk
  * [H, d_model, d_head]; dWv [H, E, d_model, d_head]; dWo [H, E, d_head, d_model]; dWs, dWd [H, d_model, E]
- * (the layouts sh_set_weights takes).  CUDA-core kernels with fp32 atomics: sums over tokens arrive in
+ * (the layouts sh_set_weights takes).  Several contributions to a value are added by fp32 reductions in
  * any order, so two calls agree to rounding, not bit for bit.  Work enqueued on `stream`. */
 int sh_backward(sh_layer* layer, const void* x, const float* dout, float* dx, float* dWq, float* dWk,
                 float* dWv, float* dWo, float* dWs, float* dWd, void* stream);

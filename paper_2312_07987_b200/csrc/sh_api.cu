@@ -156,8 +156,8 @@ static int configure_common(sh_layer* L, int dtype, int batch, int seq, int cach
     return SH_ERR_UNSUPPORTED;
   }
   if (dtype == SH_BF16 && d0.Dt > 128 && (L->dense || cache_len > 0)) {
-    // (the tensor-core attention kernel keeps S and O of two query tiles in the 512 TMEM columns: d_head <= 128;
-    //  above that a bf16 layer runs on the CUDA-core kernels - see sh_tc_prepare - which this build keeps to the plain layer)
+    // (above 128 columns S and O of two query tiles no longer fit the 512 TMEM columns: an attention kernel of its own,
+    //  without a cache or a score bias - sh_tc_attention_wide_kernel)
     sh_set_error("bf16 storage with d_head above 128 (got %d): the plain layer without a cache only; the fp32 configuration takes every form", d0.Dt);
     return SH_ERR_UNSUPPORTED;
   }

@@ -1,4 +1,5 @@
-// CUDA-core (FFMA) kernels: the whole fp32 configuration runs on these; the gate, top-k and
+// CUDA-core (FFMA) kernels: the dense comparator in fp32, attention with the relative-position term in fp32,
+// cross-check stages of the debug library; the gate, top-k and
 // bucket-sort kernels also serve the bf16 configuration.
 #pragma once
 #include "sh_internal.cuh"

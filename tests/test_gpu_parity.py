@@ -266,7 +266,7 @@ def test_d_head_above_128_in_the_fp32_configuration(D, T):
 
 @pytest.mark.parametrize("D,T,k", [(132, 300, 2), (168, 140, 3), (256, 65, 2)])
 def test_d_head_above_128_with_bf16_storage(D, T, k):
-    # stored as 256 columns: every stage on the CUDA-core kernels (bf16 weights and x, fp16 intermediates); the
+    # stored as 256 columns (bf16 weights and x, fp16 intermediates); the
     # plain layer only - a cache or the dense comparator is refused
     cfg = inputs.LayerConfig("dbig_bf16", inputs.DTYPE_BF16, 2, T, 256, 2, D, 5, k, seed=90 + D)
     full_check(inputs.make_inputs(cfg))
