@@ -55,8 +55,8 @@ int launch_x(sh_layer* L, cudaStream_t st, const XPart& a, const XPart& b = XPar
 }
 
 // Column tiles over `cols` columns: how many, and how wide (a multiple of 16).
-void col_tiles(XGemmArgs& g, int cols) {
-  g.nsub = (cols + XG_BN - 1) / XG_BN;
+void col_tiles(XGemmArgs& g, int cols, int bn = XG_BN) {
+  g.nsub = (cols + bn - 1) / bn;
   g.sub_cols = ((cols + g.nsub - 1) / g.nsub + 15) / 16 * 16;
 }
 
@@ -176,14 +176,6 @@ int launch_attn_bw_t(sh_layer* L, const BwBuffers& w, cudaStream_t st) {
   return launch_k(true, sh_f32_attn_bw_kernel<D>, dim3((unsigned)kt * d.B * d.H, (unsigned)((qt + run - 1) / run)), dim3(256), FBwSmem<D>::TOTAL, st,
                   (const float*)(ws + L->o.q), (const float*)(ws + L->o.k), (const float*)(ws + L->o.v), (const float*)w.dahat,
                   (const float*)(ws + L->o.f32stats), (const float*)w.dsum, w.dq, w.dk, w.dv, d, (int)run);
-}
-
-// Parts of a contraction over tokens: enough blocks for the device, at least eight steps each.
-int k_parts(sh_layer* L, long blocks, long steps) {
-  long p = (sm_count(L) + blocks - 1) / blocks;
-  const long most = steps / 8 < 1 ? 1 : steps / 8;
-  p = p > most ? most : p;
-  return p < 1 ? 1 : (int)p;
 }
 
 // Parts of a contraction on the half-SM blocks, where its result is added anyway: enough blocks for both
@@ -309,15 +301,21 @@ int sh_f32_backward(sh_layer* L, const void* x, const float* dout, float* dx, fl
   col_tiles(g, d.M);
   g.ksplit = half_blocks(L, (long)d.nblk * g.nsub, 2 * d.H * ((d.Dt + XG_BK - 1) / XG_BK));
   if ((rc = launch_x<X_DX>(L, st, part<X_DX>(L, g, d.nblk, g.nsub, g.ksplit)))) return rc;
-  // weight gradients, one launch; contractions in parts where whole ones would leave SMs without a tile
+  // weight gradients, one launch
   auto wpart = [](const XGemmArgs& a, int gx, int gy, int gz) { XWPart p; p.g = a; p.gx = gx; p.gy = gy; p.n = gx * gy * gz; return p; };
   XGemmArgs gq = src, gv = src, go = dst;
-  col_tiles(gq, d.Dt); col_tiles(gv, d.Dt); col_tiles(go, d.M);
+  col_tiles(gq, d.Dt, XW_BN); col_tiles(gv, d.Dt, XW_BN); col_tiles(go, d.M, XW_BN);
   gq.qk_groups = 2 * d.H;
-  const int ct = gq.qk_groups * gq.nsub + (d.G + XG_BN - 1) / XG_BN;
-  const long blocks = (long)mt * ct + (long)d.H * d.E * (mt * gv.nsub + dt * go.nsub);
-  gq.ksplit = k_parts(L, blocks, (d.N + XG_BK - 1) / XG_BK);
-  gv.ksplit = go.ksplit = k_parts(L, blocks, ((long)d.N * d.k / d.E + XG_BK - 1) / XG_BK);
+  const int ct = gq.qk_groups * gq.nsub + (d.G + XW_BN - 1) / XW_BN;
+  // parts: the shortest ones (of eight steps at least) that still fit the SMs in one round; one part each where
+  // whole contractions already need more rounds
+  const long nq = (long)mt * ct, nl = (long)d.H * d.E * (mt * gv.nsub + dt * go.nsub);
+  const long sq = (d.N + XG_BK - 1) / XG_BK, sl = ((long)d.N * d.k / d.E + XG_BK - 1) / XG_BK;
+  long len = sq > sl ? sq : sl;
+  for (long l = 8; l < len; ++l)
+    if (nq * ((sq + l - 1) / l) + nl * ((sl + l - 1) / l) <= sm_count(L)) { len = l; break; }
+  gq.ksplit = (int)((sq + len - 1) / len);
+  gv.ksplit = go.ksplit = (int)((sl + len - 1) / len);
   if (gq.ksplit > 1) {
     SH_CUDA_CHECK(cudaMemsetAsync(dWq, 0, (size_t)d.H * d.M * d.Dt * 4, st));
     SH_CUDA_CHECK(cudaMemsetAsync(dWk, 0, (size_t)d.H * d.M * d.Dt * 4, st));

@@ -4,41 +4,42 @@
 //   X_DWQK dWq[h], dWk[h], dWs, dWd = sum over all tokens: x[t]^T [dq dk dz][t]
 //
 // The split products, accumulators and promotion are those of sh_f32_gemm.cuh; both operands are
-// MN-major (a row of shared memory is 64 columns of one token).  Tile 128 x 64, steps of 32 tokens.  Both
-// operands pass through the worker threads, so what bounds a step is shared memory (132 KB of traffic,
-// about 1000 cycles) - if the gathered rows are there in time: list entry -> row is two dependent trips to
-// L2.  One block per SM with 512 workers, the rows of the next four steps on their way by asynchronous
-// copies into warp-private memory and the list entries of a fifth in registers; accumulators doubled, so
-// that the UMMAs run on while a set is read.  (As modes of the half-SM kernel, with the next step's pieces
-// in registers, a step took 3100 cycles.)
+// MN-major (a row of shared memory is 64 columns of one token).  Tile 128 x 128 (B as two halves of 64
+// columns, each with its three accumulator blocks), steps of 32 tokens.  Both operands pass through the
+// worker threads, so what bounds a step is shared memory (208 KB of traffic, about 1600 cycles) - if the
+// gathered rows are there in time: list entry -> row is two dependent trips to L2.  One block per SM with
+// 512 workers, the rows of the next three steps on their way by asynchronous copies into warp-private memory
+// and the list entries of one more in registers.  (262M-scale step, 2 x 512 tokens: 328 tiles in 96 us;
+// 648 tiles of 64 columns took 108, of which a third was their set-up and drain; as modes of the half-SM
+// kernel 150.)
 #pragma once
 #include "sh_f32_gemm.cuh"
 
 namespace shtc {
 
 struct XWgradSmem {
-  static constexpr int A_PLANE = 128 * XG_BK * 2, B_PLANE = XG_BN * XG_BK * 2;
-  static constexpr int STAGES = 3, STAGE = 3 * (A_PLANE + B_PLANE);
-  static constexpr int NRAW = 4, RAW_A = 128 * XG_BK * 4, RAW_B = XG_BN * XG_BK * 4, RAW = RAW_A + RAW_B;
+  static constexpr int A_PLANE = 128 * XG_BK * 2, B_PLANE = 64 * XG_BK * 2, B_HALF = 3 * B_PLANE;
+  static constexpr int STAGES = 2, STAGE = 3 * A_PLANE + 2 * B_HALF;
+  static constexpr int NRAW = 3, RAW_A = 128 * XG_BK * 4, RAW = 2 * RAW_A;
   static constexpr int RAW_OFF = STAGES * STAGE;
   static constexpr int BAR_OFF = RAW_OFF + NRAW * RAW;
   static constexpr int TOTAL = BAR_OFF + 128 + 1024;
 };
-constexpr int XW_WORKERS = 512, XW_THREADS = XW_WORKERS + 32;
+constexpr int XW_WORKERS = 512, XW_THREADS = XW_WORKERS + 32, XW_BN = 128;
 
 template <int MODE>
 __device__ __forceinline__ void xw_tile(const XGemmArgs& g, XTile blk) {
   using SM = XWgradSmem;
   constexpr bool LIST = MODE != X_DWQK;
-  constexpr int COLS = XG_BN / 4;
+  constexpr int COLS = XW_BN / 4;
   extern __shared__ unsigned char smem_raw[];
   const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
   unsigned char* sgen = smem_raw + (sbase - smem_u32(smem_raw));
   uint64_t* full_bar = (uint64_t*)(sgen + SM::BAR_OFF);    // [STAGES]
   uint64_t* empty_bar = full_bar + SM::STAGES;             // [STAGES]
-  uint64_t* acc_full = empty_bar + SM::STAGES;             // [2]
-  uint64_t* acc_empty = acc_full + 2;                      // [2]
-  uint32_t* tmem_slot = (uint32_t*)(acc_empty + 2);
+  uint64_t* acc_full = empty_bar + SM::STAGES;
+  uint64_t* acc_empty = acc_full + 1;
+  uint32_t* tmem_slot = (uint32_t*)(acc_empty + 1);
   const ShDims& d = g.d;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int HD = d.H * d.D;
@@ -47,7 +48,7 @@ __device__ __forceinline__ void xw_tile(const XGemmArgs& g, XTile blk) {
   pdl_trigger();
   if (tid == 0) {
     for (int s = 0; s < SM::STAGES; ++s) { mbar_init(&full_bar[s], 16); mbar_init(&empty_bar[s], 1); }
-    for (int b = 0; b < 2; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], 16); }
+    mbar_init(acc_full, 1); mbar_init(acc_empty, 16);
     fence_barrier_init();
   }
   pdl_wait();
@@ -70,7 +71,7 @@ __device__ __forceinline__ void xw_tile(const XGemmArgs& g, XTile blk) {
       n0 = (blk.y % g.nsub) * g.sub_cols; ncols = min(g.sub_cols, d.Dt - n0);
     } else {
       gates = true;
-      n0 = (blk.y - g.qk_groups * g.nsub) * XG_BN; ncols = min(XG_BN, d.G - n0);
+      n0 = (blk.y - g.qk_groups * g.nsub) * XW_BN; ncols = min(XW_BN, d.G - n0);
     }
     m0 = blk.x * 128; nrows = min(128, d.M - m0);
     const int per = (((d.N + XG_BK - 1) / XG_BK + g.ksplit - 1) / g.ksplit) * XG_BK;
@@ -82,7 +83,7 @@ __device__ __forceinline__ void xw_tile(const XGemmArgs& g, XTile blk) {
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *tmem_slot;                        // two sets of accumulator blocks, 256 columns apart
+  const uint32_t tmem = *tmem_slot;                        // accumulator blocks P0 P1 P2 of the two halves, 192 columns apart
 
   if (warp == 16) {
     if (lane == 0) {
@@ -91,59 +92,57 @@ __device__ __forceinline__ void xw_tile(const XGemmArgs& g, XTile blk) {
                          id1 = make_idesc_f16(128, 64, 1, 1, 0) | maj;
       const uint32_t a0 = desc_lo_mn(sbase, 64 * XG_BK * 2), b0 = desc_lo_mn(sbase + 3 * SM::A_PLANE, SM::B_PLANE);
       constexpr uint32_t AP = SM::A_PLANE >> 4;
+      const int halves = ncols > 64 ? 2 : 1;
       int s = 0;
       uint32_t par = 0;
       for (int i = 0; i < steps && !dead; ++i) {
-        const int c = i / XG_CHUNK, b = c & 1;
-        if (i % XG_CHUNK == 0 && c >= 2 && !mbar_wait(&acc_empty[b], ((c >> 1) & 1) ^ 1, g.status, dead)) break;
+        if (i % XG_CHUNK == 0 && i > 0 && !mbar_wait(acc_empty, ((i / XG_CHUNK) & 1) ^ 1, g.status, dead)) break;
         if (!mbar_wait(&full_bar[s], par, g.status, dead)) break;
         tc_fence_after();
-        const uint32_t alo = a0 + s * (SM::STAGE >> 4), blo = b0 + s * (SM::STAGE >> 4), td = tmem + b * 256;
+        const uint32_t alo = a0 + s * (SM::STAGE >> 4), blo = b0 + s * (SM::STAGE >> 4);
         const int kn = (min(XG_BK, kend - kbeg - XG_BK * i) + 15) / 16;
 #pragma unroll
         for (int k = 0; k < XG_BK / 16; ++k) {
           if (k >= kn) break;
           const uint32_t a = alo + 128 * k;
-          const uint64_t bb = xg_desc(blo + 128 * k, true);
-          umma_f16(td, xg_desc(a, true), bb, id3, (i % XG_CHUNK | k) != 0);
-          umma_f16(td + 64, xg_desc(a + AP, true), bb, id2, 1);
-          umma_f16(td + 128, xg_desc(a + 2 * AP, true), bb, id1, 1);
+          for (int hf = 0; hf < halves; ++hf) {
+            const uint32_t td = tmem + hf * 192;
+            const uint64_t bb = xg_desc(blo + hf * (SM::B_HALF >> 4) + 128 * k, true);
+            umma_f16(td, xg_desc(a, true), bb, id3, (i % XG_CHUNK | k) != 0);
+            umma_f16(td + 64, xg_desc(a + AP, true), bb, id2, 1);
+            umma_f16(td + 128, xg_desc(a + 2 * AP, true), bb, id1, 1);
+          }
         }
         umma_commit(&empty_bar[s]);
-        if (i % XG_CHUNK == XG_CHUNK - 1 || i == steps - 1) umma_commit(&acc_full[b]);
+        if (i % XG_CHUNK == XG_CHUNK - 1 || i == steps - 1) umma_commit(acc_full);
         if (++s == SM::STAGES) { s = 0; par ^= 1; }
       }
     }
     __syncwarp();
   } else {
-    // a thread's pieces of a step: 8 columns (ac) of token row ar of A; threads 0..255 also of row br of B
-    const int ac = tid & 15, ar = tid >> 4, bc = tid & 7, br = (tid >> 3) & 31;
-    const bool has_b = tid < 256;
-    const uint32_t aoff = (uint32_t)((ac >> 3) * (64 * XG_BK * 2) + ar * 128 + (((ac & 7) ^ (ar & 7)) << 4));
-    const uint32_t boff = (uint32_t)(br * 128 + ((bc ^ (br & 7)) << 4));
+    // a thread's pieces of a step: 8 columns (ac) of token row ar, of A and of B
+    const int ac = tid & 15, ar = tid >> 4;
+    const uint32_t poff = (uint32_t)(ar * 128 + (((ac & 7) ^ (ar & 7)) << 4));
+    const uint32_t aoff = (ac >> 3) * (64 * XG_BK * 2) + poff, boff = (ac >> 3) * SM::B_HALF + poff;
     const size_t lbase = (size_t)h * d.N * d.k;
     const bool vdy = MODE != X_DWO || g.vec_dy != 0;
     // (columns past the operands' widths end in accumulators nobody reads: any address inside the row will do)
     const int acol = min(m0 + lane * 4, (MODE == X_DWO ? d.D : d.M) - 4);
-    const int bcol = min(n0 + (lane & 15) * 4, (MODE == X_DWO ? d.M : gates ? g.ldz : d.D) - 4);
+    const int bcol = min(n0 + lane * 4, (MODE == X_DWO ? d.M : gates ? g.ldz : d.D) - 4);
     const float* asrc = (MODE == X_DWO ? g.ahat + h * d.D : g.x) + acol;
     const size_t ald = MODE == X_DWO ? HD : d.M;
     const float* bsrc = (MODE == X_DWO ? g.dy : MODE == X_DWV ? g.dv + h * d.D : gates ? g.dz : (which ? g.dk : g.dq) + h * d.D) + bcol;
     const size_t bld = MODE == X_DWO ? d.M : gates ? g.ldz : HD;
-    // copies: a warp's two token rows of A are two instructions; of B (warps 0..7) four rows are
-    int ta[2] = {0, 0}, tb[2] = {0, 0};                    // the next step's tokens
+    // copies: a warp's two token rows are two instructions, of A and of B
+    int ta[2] = {0, 0};                                    // the next step's tokens
     float gnext = 0.f;
     auto entries = [&](int i) {
       const int p0 = kbeg + i * XG_BK;
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
-        const int pa = p0 + 2 * warp + u, pb = p0 + 4 * (warp & 7) + (lane >> 4) + 2 * u;
-        if (LIST) {
-          if (pa < kend) ta[u] = __ldg(g.lists + lbase + pa);
-          if (has_b && pb < kend) tb[u] = __ldg(g.lists + lbase + pb);
-        } else {
-          ta[u] = min(pa, d.N - 1); tb[u] = min(pb, d.N - 1);
-        }
+        const int pa = p0 + 2 * warp + u;
+        if (!LIST) ta[u] = min(pa, d.N - 1);
+        else if (pa < kend) ta[u] = __ldg(g.lists + lbase + pa);
       }
       if (LIST && p0 + ar < kend) gnext = __ldg(g.lgate + lbase + p0 + ar);
     };
@@ -153,34 +152,36 @@ __device__ __forceinline__ void xw_tile(const XGemmArgs& g, XTile blk) {
       const int p0 = kbeg + i * XG_BK;
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
-        fetch4(raw + raw_chunk(lane + 32 * u), asrc + (size_t)ta[u] * ald, true, p0 + 2 * warp + u < kend);
-        if (has_b)
-          fetch4(raw + SM::RAW_A + raw_chunk(lane + 32 * u), bsrc + (size_t)tb[u] * bld, vdy, p0 + 4 * warp + (lane >> 4) + 2 * u < kend);
+        const bool live = p0 + 2 * warp + u < kend;
+        fetch4(raw + raw_chunk(lane + 32 * u), asrc + (size_t)ta[u] * ald, true, live);
+        fetch4(raw + SM::RAW_A + raw_chunk(lane + 32 * u), bsrc + (size_t)ta[u] * bld, vdy, live);
       }
     };
     const int q = warp & 3, cb = warp >> 2;
-    const uint32_t tlane = ((uint32_t)(q * 32) << 16) + cb * COLS;
     float acc[COLS];
 #pragma unroll
     for (int i = 0; i < COLS; ++i) acc[i] = 0.f;
     const bool mine = cb * COLS < ncols;                   // (whole warps)
     auto promote = [&](int c) {
-      const int b = c & 1;
-      if (!mbar_wait(&acc_full[b], (c >> 1) & 1, g.status, dead)) return;
+      if (!mbar_wait(acc_full, c & 1, g.status, dead)) return;
       tc_fence_after();
       if (mine) {
-        float t[COLS];
+        const uint32_t tb = tmem + (cb >> 1) * 192 + ((uint32_t)(q * 32) << 16) + (cb & 1) * 32;
 #pragma unroll
-        for (int i = 0; i < COLS; ++i) t[i] = 0.f;
-        tmem_add<COLS>(tmem + b * 256 + 128 + tlane, t);     // (smallest first)
-        tmem_add<COLS>(tmem + b * 256 + 64 + tlane, t);
-        tmem_add<COLS>(tmem + b * 256 + tlane, t);
+        for (int c0 = 0; c0 < COLS; c0 += 16) {
+          float t[16];
 #pragma unroll
-        for (int i = 0; i < COLS; ++i) acc[i] += t[i];
+          for (int i = 0; i < 16; ++i) t[i] = 0.f;
+          tmem_add<16>(tb + 128 + c0, t);                    // (smallest first)
+          tmem_add<16>(tb + 64 + c0, t);
+          tmem_add<16>(tb + c0, t);
+#pragma unroll
+          for (int i = 0; i < 16; ++i) acc[c0 + i] += t[i];
+        }
       }
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(&acc_empty[b]);
+      if (lane == 0) mbar_arrive(acc_empty);
     };
     if (steps > 0) entries(0);
 #pragma unroll
@@ -208,10 +209,8 @@ __device__ __forceinline__ void xw_tile(const XGemmArgs& g, XTile blk) {
           for (int x = 0; x < 8; ++x) v[x] *= gring[u];
         }
         store_planes(at, aoff, SM::A_PLANE, v);
-        if (has_b) {
-          read8(v, raw + SM::RAW_A, 2 * lane);
-          store_planes(at + 3 * SM::A_PLANE, boff, SM::B_PLANE, v);
-        }
+        read8(v, raw + SM::RAW_A, 2 * lane);
+        store_planes(at + 3 * SM::A_PLANE, boff, SM::B_PLANE, v);
         fence_proxy_async_smem();
         __syncwarp();
         if (lane == 0) mbar_arrive(&full_bar[s]);
