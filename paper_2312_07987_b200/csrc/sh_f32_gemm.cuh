@@ -6,8 +6,8 @@
 //   hh' + (hm' + mh') + (hl' + mm' + lh') + terms below 2^-25 of it,
 // six bf16 products.  The tensor core adds into fp32 but drops the bits below the accumulator's last one
 // instead of rounding, so a long chain of additions drifts towards zero: the accumulators are read back
-// and added in fp32 registers every 128 contraction positions (8 additions of hh', which carries the
-// size of the result).
+// and added in fp32 registers every 128 (64) contraction positions: 8 additions of hh', which carries the
+// size of the result.
 //
 // Three UMMAs per 16 positions do the six products: the planes of B lie one behind the other, so that
 // they are one operand of 192 columns, and with accumulator blocks P0 P1 P2 of 64 columns
@@ -77,7 +77,9 @@ struct XGemmSmem {
 };
 
 constexpr int XG_WORKERS = 256, XG_THREADS = XG_WORKERS + 64;   // + a warp that issues UMMAs, + one that loads weights
-constexpr int XG_CHUNK = 128 / XG_BK;    // steps per promotion of the accumulators
+// Steps per promotion of the accumulators: 128 positions; 64 in contractions of up to 256, where an FFMA chain
+// is short too and its error is the smaller one to stay below (64 everywhere: a quarter less error, 7 % more time).
+__device__ __forceinline__ int xg_chunk(int steps) { return steps <= 8 ? 2 : 4; }
 
 // K-major planes: rows of 32 values (64 bytes), 64-byte swizzle, 8-row groups 512 bytes apart.
 constexpr uint32_t DESC_HI_SW64 = (512u >> 4) | (1u << 14) | (4u << 29);
@@ -229,6 +231,7 @@ __device__ __forceinline__ void xg_tile(const CUtensorMap& mapW, const CUtensorM
     steps = min(per, steps - s0);
     if (steps <= 0) return;
   }
+  const int chunk = xg_chunk(steps);
   if (warp == 8) { tmem_alloc(tmem_slot, 256); tmem_relinquish(); }
   tc_fence_before();
   __syncthreads();
@@ -256,7 +259,7 @@ __device__ __forceinline__ void xg_tile(const CUtensorMap& mapW, const CUtensorM
       int s = 0;
       uint32_t par = 0;
       for (int i = 0; i < steps && !dead; ++i) {
-        if (i % XG_CHUNK == 0 && i > 0 && !mbar_wait(acc_empty, ((i / XG_CHUNK) & 1) ^ 1, g.status, dead)) break;
+        if ((i & (chunk - 1)) == 0 && i > 0 && !mbar_wait(acc_empty, ((i / chunk) & 1) ^ 1, g.status, dead)) break;
         if (!mbar_wait(&full_bar[s], par, g.status, dead)) break;
         tc_fence_after();
         const uint32_t alo = a0 + s * (SM::STAGE >> 4), blo = b0 + s * (SM::STAGE >> 4);
@@ -266,12 +269,12 @@ __device__ __forceinline__ void xg_tile(const CUtensorMap& mapW, const CUtensorM
           if (k >= kn) break;
           const uint32_t a = alo + 2 * k;
           const uint64_t bb = xg_desc(blo + BK * k, B_MN);
-          umma_f16(tmem, xg_desc(a, false), bb, id3, (i % XG_CHUNK | k) != 0);
+          umma_f16(tmem, xg_desc(a, false), bb, id3, ((i & (chunk - 1)) | k) != 0);
           umma_f16(tmem + 64, xg_desc(a + AP, false), bb, id2, 1);
           umma_f16(tmem + 128, xg_desc(a + 2 * AP, false), bb, id1, 1);
         }
         umma_commit(&empty_bar[s]);
-        if (i % XG_CHUNK == XG_CHUNK - 1 || i == steps - 1) umma_commit(acc_full);
+        if ((i & (chunk - 1)) == chunk - 1 || i == steps - 1) umma_commit(acc_full);
         if (++s == XG_STAGES) { s = 0; par ^= 1; }
       }
     }
@@ -400,10 +403,10 @@ __device__ __forceinline__ void xg_tile(const CUtensorMap& mapW, const CUtensorM
       if (i + 2 < steps) load(i + 2);
       cp_async_commit();
       // a chunk is read once two steps of the next one are in shared memory
-      if (i % XG_CHUNK == 1 && i > XG_CHUNK) promote(done++);
+      if ((i & (chunk - 1)) == 1 && i > chunk) promote(done++);
     }
     cp_async_wait<0>();
-    for (; done < (steps + XG_CHUNK - 1) / XG_CHUNK && !dead; ++done) promote(done);
+    for (; done < (steps + chunk - 1) / chunk && !dead; ++done) promote(done);
     // ---- result: thread = row q*32 + lane, columns cb*COLS ... ------------------------------------
     const int r = q * 32 + lane, c0 = cb * COLS;
     const int valid = min(COLS, ncols - c0);

@@ -79,6 +79,7 @@ __device__ __forceinline__ void xw_tile(const XGemmArgs& g, XTile blk) {
   }
   if (g.ksplit > 1 && kbeg >= kend) return;                // (the results are added to zeros)
   const int steps = (kend - kbeg + XG_BK - 1) / XG_BK;
+  const int chunk = xg_chunk(steps);
   if (warp == 16) { tmem_alloc(tmem_slot, 512); tmem_relinquish(); }
   tc_fence_before();
   __syncthreads();
@@ -96,7 +97,7 @@ __device__ __forceinline__ void xw_tile(const XGemmArgs& g, XTile blk) {
       int s = 0;
       uint32_t par = 0;
       for (int i = 0; i < steps && !dead; ++i) {
-        if (i % XG_CHUNK == 0 && i > 0 && !mbar_wait(acc_empty, ((i / XG_CHUNK) & 1) ^ 1, g.status, dead)) break;
+        if ((i & (chunk - 1)) == 0 && i > 0 && !mbar_wait(acc_empty, ((i / chunk) & 1) ^ 1, g.status, dead)) break;
         if (!mbar_wait(&full_bar[s], par, g.status, dead)) break;
         tc_fence_after();
         const uint32_t alo = a0 + s * (SM::STAGE >> 4), blo = b0 + s * (SM::STAGE >> 4);
@@ -108,13 +109,13 @@ __device__ __forceinline__ void xw_tile(const XGemmArgs& g, XTile blk) {
           for (int hf = 0; hf < halves; ++hf) {
             const uint32_t td = tmem + hf * 192;
             const uint64_t bb = xg_desc(blo + hf * (SM::B_HALF >> 4) + 128 * k, true);
-            umma_f16(td, xg_desc(a, true), bb, id3, (i % XG_CHUNK | k) != 0);
+            umma_f16(td, xg_desc(a, true), bb, id3, ((i & (chunk - 1)) | k) != 0);
             umma_f16(td + 64, xg_desc(a + AP, true), bb, id2, 1);
             umma_f16(td + 128, xg_desc(a + 2 * AP, true), bb, id1, 1);
           }
         }
         umma_commit(&empty_bar[s]);
-        if (i % XG_CHUNK == XG_CHUNK - 1 || i == steps - 1) umma_commit(acc_full);
+        if ((i & (chunk - 1)) == chunk - 1 || i == steps - 1) umma_commit(acc_full);
         if (++s == SM::STAGES) { s = 0; par ^= 1; }
       }
     }
@@ -221,11 +222,11 @@ __device__ __forceinline__ void xw_tile(const XGemmArgs& g, XTile blk) {
           if (i + SM::NRAW + 1 < steps) entries(i + SM::NRAW + 1);
         }
         cp_async_commit();
-        if (i % XG_CHUNK == 1 && i > XG_CHUNK) promote(done++);
+        if ((i & (chunk - 1)) == 1 && i > chunk) promote(done++);
       }
     }
     cp_async_wait<0>();
-    for (; done < (steps + XG_CHUNK - 1) / XG_CHUNK && !dead; ++done) promote(done);
+    for (; done < (steps + chunk - 1) / chunk && !dead; ++done) promote(done);
     const int r = q * 32 + lane, c0 = cb * COLS;
     const int valid = min(COLS, ncols - c0);
     if (r < nrows && valid > 0 && !dead) {
