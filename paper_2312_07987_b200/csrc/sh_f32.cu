@@ -102,7 +102,7 @@ int launch_gate_sort(sh_layer* L, const void* x, float* zero0, long n0, float* z
                     : (ch == 512 ? sh_f32_gate_kernel<16, 512> : sh_f32_gate_kernel<16, 1024>);
   if (int rc = set_smem(kern, (int)smem)) return rc;
   if (int rc = launch_k(true, kern, dim3((unsigned)((d.N + tok - 1) / tok)), dim3(512), smem, st, (const float*)x, (const float*)(ws + L->o.wgate32),
-                        (const float*)(ws + L->o.gbias), (int*)(ws + L->o.idx), (float*)(ws + L->o.gate), (float4*)zero0, n0 / 4, (float4*)zero1, n1 / 4, d))
+                        (const float*)(ws + L->o.gbias), (int*)(ws + L->o.idx), (float*)(ws + L->o.gate), (float4*)zero0, n0 / 4, (float4*)zero1, n1 / 4, d, (int)((uintptr_t)x % 16 == 0)))
     return rc;
   L->launches += 2;
   return launch_k(true, sh_f32_sort_kernel, dim3(d.sides * d.H), dim3(1024), 0, st, (const int*)(ws + L->o.idx), (const float*)(ws + L->o.gate),

@@ -10,7 +10,7 @@
 template <int TOK, int CH>
 static __global__ void __launch_bounds__(512, 1)
 sh_f32_gate_kernel(const float* __restrict__ x, const float* __restrict__ wgate, const float* __restrict__ gbias, int* __restrict__ idx,
-                   float* __restrict__ gate, float4* __restrict__ zero0, long nzero0, float4* __restrict__ zero1, long nzero1, ShDims d) {
+                   float* __restrict__ gate, float4* __restrict__ zero0, long nzero0, float4* __restrict__ zero1, long nzero1, ShDims d, int vec) {
   extern __shared__ __align__(16) float gsm[];             // [TOK][CH] of x, then [TOK][G] logits
   float* s_z = gsm + TOK * CH;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -25,7 +25,10 @@ sh_f32_gate_kernel(const float* __restrict__ x, const float* __restrict__ wgate,
     for (int i = tid; i < TOK * (CH / 4); i += 512) {
       const int r = i / (CH / 4), c = (i % (CH / 4)) * 4;
       float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (c < mw && t0 + r < d.N) v = __ldg(reinterpret_cast<const float4*>(x + (size_t)(t0 + r) * d.M + m0 + c));
+      if (c < mw && t0 + r < d.N) {
+        const float* p = x + (size_t)(t0 + r) * d.M + m0 + c;
+        v = vec ? __ldg(reinterpret_cast<const float4*>(p)) : make_float4(__ldg(p), __ldg(p + 1), __ldg(p + 2), __ldg(p + 3));   // (x off its alignment: sh_gate_topk takes it)
+      }
       *reinterpret_cast<float4*>(gsm + r * CH + c) = v;
     }
     for (int g = warp; g < d.G; g += 32) {                  // two columns at a time, all of their loads in flight

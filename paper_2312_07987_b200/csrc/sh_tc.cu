@@ -324,8 +324,9 @@ static int tc_gate_sort(sh_layer* L, const void* x, void* out, bool zero_for_for
   const ShDims& d = L->d;
   char* ws = L->ws;
   int rc;
-  if (!S->gate_gp || (S->simt_mask & SH_STAGE_GATE)) {
-    // more than 256 gate columns (or the debug library's switch): the CUDA-core gate kernel
+  if (!S->gate_gp || (S->simt_mask & SH_STAGE_GATE) || (d.D > 128 && (uintptr_t)x % 16 != 0)) {
+    // more than 256 gate columns (or the debug library's switch): the CUDA-core gate kernel; also an x that no
+    // tensor map can describe, which sh_gate_topk has taken for such layers (sh_forward wants x aligned)
     if ((rc = sh_simt_run_bf16(L, SH_STAGE_GATE, x, nullptr, st))) return rc;
     if (zero_for_forward) {
       SH_CUDA_CHECK(cudaMemsetAsync(ws + L->o.v, 0, (size_t)d.N * d.H * d.D * 2, st));

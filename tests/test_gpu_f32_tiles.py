@@ -64,3 +64,15 @@ def test_f32_empty_experts_and_no_mask():
 
 def test_f32_gradient_input_off_its_alignment():
     run(1, 90, 128, 2, 76, 4, 2, offset=1)
+
+
+def test_f32_selection_of_an_input_off_its_alignment():
+    cfg = inputs.LayerConfig("tiles", inputs.DTYPE_F32, 1, 70, 128, 2, 32, 4, 2, seed=5)
+    inp = inputs.make_inputs(cfg)
+    layer = binding.layer_from_inputs(inp)
+    x = binding.to_device(inp.x, cfg.dtype)
+    shifted = torch.empty(x.numel() + 1, dtype=torch.float32, device="cuda")[1:].view(x.shape)
+    shifted.copy_(x)
+    for a, b in zip(layer.sh_gate_topk(x), layer.sh_gate_topk(shifted)):
+        assert torch.equal(a, b)
+    layer.close()

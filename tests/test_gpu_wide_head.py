@@ -54,3 +54,16 @@ def test_half_precision_output_stays_refused():
     with pytest.raises(binding.SwitchHeadError):
         layer.sh_forward(binding.to_device(inp.x, inp.cfg.dtype))
     layer.close()
+
+
+def test_selection_of_an_input_off_its_alignment():
+    inp = inputs.make_inputs(config(1, 70, 128, 2, 132, 4, 2))
+    layer = binding.layer_from_inputs(inp)
+    x = binding.to_device(inp.x, inp.cfg.dtype)
+    shifted = torch.empty(x.numel() + 1, dtype=x.dtype, device="cuda")[1:].view(x.shape)
+    shifted.copy_(x)
+    idx, gate, off, lists = (t.cpu().numpy() for t in layer.sh_gate_topk(shifted))
+    ref = pu.oracle_selection(inp)
+    pu.check_selection(idx, gate, ref, 70, 2e-5)
+    pu.check_lists(off, lists, ref)
+    layer.close()
