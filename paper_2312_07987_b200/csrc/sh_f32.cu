@@ -89,8 +89,8 @@ void use_side(XGemmArgs& g, sh_layer* L, int side) {
   g.tiles = (const ShTile*)(ws + L->o.tiles) + (size_t)side * d.max_tiles;
 }
 
-// Gates, selection and sort; beside them the buffers that later kernels add into are cleared.
-int launch_gate_sort(sh_layer* L, const void* x, float* zero0, long n0, float* zero1, long n1, cudaStream_t st) {
+// Gates, selection and sort; beside them `zero` (n values), which a later kernel adds into, is cleared.
+int launch_gate_sort(sh_layer* L, const void* x, float* zero, long n, cudaStream_t st) {
   const ShDims& d = L->d;
   char* ws = L->ws;
   // eight tokens a block while sixteen would leave SMs with less than two blocks (or their logits do not fit)
@@ -102,7 +102,7 @@ int launch_gate_sort(sh_layer* L, const void* x, float* zero0, long n0, float* z
                     : (ch == 512 ? sh_f32_gate_kernel<16, 512> : sh_f32_gate_kernel<16, 1024>);
   if (int rc = set_smem(kern, (int)smem)) return rc;
   if (int rc = launch_k(true, kern, dim3((unsigned)((d.N + tok - 1) / tok)), dim3(512), smem, st, (const float*)x, (const float*)(ws + L->o.wgate32),
-                        (const float*)(ws + L->o.gbias), (int*)(ws + L->o.idx), (float*)(ws + L->o.gate), (float4*)zero0, n0 / 4, (float4*)zero1, n1 / 4, d, (int)((uintptr_t)x % 16 == 0)))
+                        (const float*)(ws + L->o.gbias), (int*)(ws + L->o.idx), (float*)(ws + L->o.gate), (float4*)zero, n / 4, d, (int)((uintptr_t)x % 16 == 0)))
     return rc;
   L->launches += 2;
   return launch_k(true, sh_f32_sort_kernel, dim3(d.sides * d.H), dim3(1024), 0, st, (const int*)(ws + L->o.idx), (const float*)(ws + L->o.gate),
@@ -129,23 +129,24 @@ XPart part_v(sh_layer* L, const void* x, int side, const PlaneMap& w, float* dst
 }
 
 template <int D>
-int launch_attn_t(sh_layer* L, cudaStream_t st) {
+int launch_attn_t(sh_layer* L, float* zero, long n, cudaStream_t st) {
   const ShDims& d = L->d;
   char* ws = L->ws;
   if (int rc = set_smem(sh_f32_attn_kernel<D>, FAttnSmem<D>::TOTAL)) return rc;
   const int nq = (d.T - d.Tc + 31) / 32;
   return launch_k(true, sh_f32_attn_kernel<D>, dim3((unsigned)nq * d.B * d.H), dim3(256), FAttnSmem<D>::TOTAL, st,
                   (const float*)(ws + L->o.q), (const float*)(ws + L->o.k), (const float*)(ws + L->o.v), (float*)(ws + L->o.ahat),
-                  (float*)(ws + L->o.f32stats), d);
+                  (float*)(ws + L->o.f32stats), (float4*)zero, n / 4, d);
 }
 
-int launch_attn(sh_layer* L, cudaStream_t st) {
+// Attention; beside it `zero` (n values), which the output projection adds into, is cleared.
+int launch_attn(sh_layer* L, float* zero, long n, cudaStream_t st) {
   L->launches += 1;
   switch (L->d.D) {
-    case 32: return launch_attn_t<32>(L, st);
-    case 64: return launch_attn_t<64>(L, st);
-    case 128: return launch_attn_t<128>(L, st);
-    default: return launch_attn_t<256>(L, st);
+    case 32: return launch_attn_t<32>(L, zero, n, st);
+    case 64: return launch_attn_t<64>(L, zero, n, st);
+    case 128: return launch_attn_t<128>(L, zero, n, st);
+    default: return launch_attn_t<256>(L, zero, n, st);
   }
 }
 
@@ -216,7 +217,7 @@ void sh_f32_release(sh_layer* L) {
   if (L && L->f32) { delete (F32State*)L->f32; L->f32 = nullptr; }
 }
 
-int sh_f32_gate_sort(sh_layer* L, const void* x, cudaStream_t st) { return launch_gate_sort(L, x, nullptr, 0, nullptr, 0, st); }
+int sh_f32_gate_sort(sh_layer* L, const void* x, cudaStream_t st) { return launch_gate_sort(L, x, nullptr, 0, st); }
 
 int sh_f32_forward(sh_layer* L, const void* x, void* out, cudaStream_t st) {
   const ShDims& d = L->d;
@@ -230,7 +231,7 @@ int sh_f32_forward(sh_layer* L, const void* x, void* out, cudaStream_t st) {
   const int first = L->moe_q ? d.H : 0, groups = (L->moe_q ? 0 : d.H) + (L->moe_k ? 0 : d.H);
   const XPart qk = part_qk(L, x, first, groups), pv = part_v(L, x, 0, S->wv, v, 0.f);
   sh_mark(L, 0, st);
-  if ((rc = launch_gate_sort(L, x, v, nhd, (float*)out, nout, st))) return rc;
+  if ((rc = launch_gate_sort(L, x, v, nhd, st))) return rc;
   sh_mark(L, 1, st);
   if (L->ev && (rc = launch_x<X_QK>(L, st, qk))) return rc;
   if (L->moe_k) {
@@ -244,8 +245,10 @@ int sh_f32_forward(sh_layer* L, const void* x, void* out, cudaStream_t st) {
   sh_mark(L, 2, st);
   if ((rc = L->ev ? launch_x<X_V>(L, st, pv) : launch_x<X_QK, X_V>(L, st, qk, pv))) return rc;
   sh_mark(L, 3, st);
-  // (the relative-position term of Transformer-XL is in the one-warp-per-query kernel only)
-  if ((rc = L->xl_positions ? sh_simt_attention_f32(L, st) : launch_attn(L, st))) return rc;
+  // (the relative-position term of Transformer-XL is in the one-warp-per-query kernel only; `out` is cleared
+  //  behind the last read of x either way: the two may be the same buffer)
+  if ((rc = L->xl_positions ? sh_simt_attention_f32(L, st) : launch_attn(L, (float*)out, nout, st))) return rc;
+  if (L->xl_positions) SH_CUDA_CHECK(cudaMemsetAsync(out, 0, (size_t)nout * 4, st));
   sh_mark(L, 4, st);
   XGemmArgs g = base_args(L, x);
   use_side(g, L, 1);

@@ -38,6 +38,8 @@ __device__ __forceinline__ float dot4(float4 a, float4 b, float s) {
 // ty + 8 i and columns 4 tx + 64 c.  K of the next tile is fetched under the P V product, V under the
 // scores.  Rows are D + 4 floats apart: the eight 16-byte loads of a phase fall into different banks.
 // stats [B, H, T, 2]: the row's score maximum (base 2) and 1 / normaliser, for the backward pass.
+// The blocks also clear the layer's output, which the next kernel adds into: this is the first kernel behind
+// the last read of x, and a caller may pass x itself as the output.
 template <int D>
 struct FAttnSmem {
   static constexpr int LD = D + 4, KT = D == 256 ? 32 : 64, PLD = KT + 4;
@@ -48,7 +50,7 @@ struct FAttnSmem {
 template <int D>
 __global__ void __launch_bounds__(256)
 sh_f32_attn_kernel(const float* __restrict__ Q, const float* __restrict__ K, const float* __restrict__ V, float* __restrict__ Ahat,
-                   float* __restrict__ stats, ShDims d) {
+                   float* __restrict__ stats, float4* __restrict__ zero, long nzero, ShDims d) {
   using SM = FAttnSmem<D>;
   constexpr int LD = SM::LD, KT = SM::KT, PLD = SM::PLD, KJ = KT / 16;
   constexpr int NC = D >= 64 ? D / 64 : 1;
@@ -75,6 +77,7 @@ sh_f32_attn_kernel(const float* __restrict__ Q, const float* __restrict__ K, con
   fa_commit();
   if (kt < ntile) fa_tile<D>(sV, Vb + (size_t)kt * KT * D, KT, d.T - kt * KT, D, t);
   fa_commit();
+  for (long i = (long)blockIdx.x * 256 + tid; i < nzero; i += (long)gridDim.x * 256) zero[i] = make_float4(0.f, 0.f, 0.f, 0.f);
   fa_wait<1>();
   __syncthreads();
   float o[4][4 * NC], m[4], l[4];

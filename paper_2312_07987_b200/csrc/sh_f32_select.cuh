@@ -4,13 +4,13 @@
 
 // Logits, top-k (a larger logit first, the lower index on a tie) and sigmoid of the chosen ones, on the
 // CUDA cores: TOK tokens per block with their rows in shared memory (CH columns at a time: 512, or 1024 where d_model is larger), a warp per
-// two gate columns, lanes along d_model.  The block also clears its share of the buffers that later kernels
-// add into.  What bounds it is the latency of its few loads, so blocks are small: 1024 tokens of 32 gate
+// two gate columns, lanes along d_model.  The block also clears its share of the value rows, which a later kernel
+// adds into.  What bounds it is the latency of its few loads, so blocks are small: 1024 tokens of 32 gate
 // columns took 490 us in blocks of 128 tokens with a warp per token.
 template <int TOK, int CH>
 static __global__ void __launch_bounds__(512, 1)
 sh_f32_gate_kernel(const float* __restrict__ x, const float* __restrict__ wgate, const float* __restrict__ gbias, int* __restrict__ idx,
-                   float* __restrict__ gate, float4* __restrict__ zero0, long nzero0, float4* __restrict__ zero1, long nzero1, ShDims d, int vec) {
+                   float* __restrict__ gate, float4* __restrict__ zero, long nzero, ShDims d, int vec) {
   extern __shared__ __align__(16) float gsm[];             // [TOK][CH] of x, then [TOK][G] logits
   float* s_z = gsm + TOK * CH;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -82,8 +82,7 @@ sh_f32_gate_kernel(const float* __restrict__ x, const float* __restrict__ wgate,
     }
     if (warp >= d.G) __syncthreads();                      // (a warp without a column meets the barrier of the others' first round here)
     if (m0 == 0) {
-      for (long i = me; i < nzero0; i += nthr) zero0[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-      for (long i = me; i < nzero1; i += nthr) zero1[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+      for (long i = me; i < nzero; i += nthr) zero[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
   }
   __syncthreads();

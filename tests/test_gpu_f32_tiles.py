@@ -76,3 +76,20 @@ def test_f32_selection_of_an_input_off_its_alignment():
     for a, b in zip(layer.sh_gate_topk(x), layer.sh_gate_topk(shifted)):
         assert torch.equal(a, b)
     layer.close()
+
+
+@pytest.mark.parametrize("cache,shared,positions", [(0, False, False), (0, True, False), (64, False, True)])
+def test_f32_output_in_place_of_the_input(cache, shared, positions):
+    # the first rows of a larger x hold the output (with a cache there are fewer of them than tokens)
+    cfg = inputs.LayerConfig("tiles", inputs.DTYPE_F32, 2, 300 + cache, 448, 2, 76, 5, 3, seed=17)
+    inp = inputs.make_inputs(cfg)
+    layer = binding.layer_from_inputs(inp, shared_selection=shared, cache_len=cache)
+    if positions:
+        g = torch.Generator(device="cuda").manual_seed(1)
+        layer.sh_set_xl_positions(torch.randn(2, 448, 76, generator=g, device="cuda") / 21, None, None)
+    x = binding.to_device(inp.x, cfg.dtype)
+    want = layer.sh_forward(x)
+    out = x.view(-1)[:want.numel()].view(want.shape)
+    layer.sh_forward(x, out=out)
+    assert float((out - want).abs().max() / want.abs().max()) < TOL
+    layer.close()
