@@ -169,7 +169,7 @@ int sh_set_weights(sh_layer* layer, const void* Wq, const void* Wk, const void* 
 /* Attention mask.  causal != 0 (the default): the language-model setting, key s is visible to
  * query t iff s <= t.  causal == 0: every key of the sequence is visible (the paper's ListOps
  * classifier uses SwitchHead without autoregressive masking).  Host-only; takes effect with
- * the next sh_forward. */
+ * the next sh_forward (sh_backward differentiates the pass that was made, with its mask). */
 int sh_set_causal(sh_layer* layer, int causal);
 
 /* Rotary position embeddings on the queries and keys (the paper's appendix "RoPE Positional

@@ -621,7 +621,7 @@ extern "C" int sh_forward(sh_layer* L, const void* x, void* out, void* stream) {
   if ((uintptr_t)x % 16 != 0 || (uintptr_t)out % 16 != 0) { sh_set_error("x and out must be 16-byte aligned"); return SH_ERR_INVALID_ARG; }
   cudaStream_t st = (cudaStream_t)stream;
   L->launches = 0;
-  L->fwd_x = x;
+  L->fwd_x = x; L->fwd_causal = L->d.causal;
   if (L->dtype == SH_F32) return L->dense ? forward_simt<float, float>(L, SH_STAGE_ALL, x, out, st) : sh_f32_forward(L, x, out, st);
   return sh_tc_forward(L, x, out, st);
 }

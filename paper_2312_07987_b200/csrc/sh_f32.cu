@@ -165,7 +165,8 @@ BwBuffers bw_buffers(sh_layer* L) {
 
 template <int D>
 int launch_attn_bw_t(sh_layer* L, const BwBuffers& w, cudaStream_t st) {
-  const ShDims& d = L->d;
+  ShDims d = L->d;
+  d.causal = L->fwd_causal;
   char* ws = L->ws;
   if (int rc = set_smem(sh_f32_attn_bw_kernel<D>, FBwSmem<D>::TOTAL)) return rc;
   // A block's run of query tiles: short enough that the blocks fill the device about four times over,

@@ -12,7 +12,7 @@ pytestmark = pytest.mark.gpu
 TOL = 2e-4          # max-abs error / RMS of the gradient: fp32 products, sums and atomics against fp64
 
 
-def check(cfg, causal=True, batch=None):
+def check(cfg, causal=True, batch=None, causal_after=None):
     inp = inputs.make_inputs(cfg, batch=batch)
     layer = binding.layer_from_inputs(inp)
     if not causal:
@@ -21,6 +21,8 @@ def check(cfg, causal=True, batch=None):
     rg = np.random.default_rng(cfg.seed + 1)
     G = rg.standard_normal(inp.x.shape).astype(np.float32)
     layer.sh_forward(x)
+    if causal_after is not None:
+        layer.sh_set_causal(causal_after)
     got = layer.sh_backward(x, torch.from_numpy(G).cuda())
     torch.cuda.synchronize()
     assert layer.sh_last_status() == 0
@@ -40,6 +42,12 @@ def test_backward_tiny_f32():
 @pytest.mark.parametrize("T,B,M,H,D,E,k,causal", [(70, 2, 128, 2, 40, 5, 3, True), (33, 3, 64, 3, 64, 4, 1, False), (150, 1, 192, 1, 132, 6, 2, True)])
 def test_backward_shapes(T, B, M, H, D, E, k, causal):
     check(inputs.LayerConfig("bw", inputs.DTYPE_F32, B, T, M, H, D, E, k, seed=900 + T, zipf_bias=1.2 if E == 5 else 0.0), causal=causal)
+
+
+@pytest.mark.parametrize("causal", [True, False])
+def test_backward_takes_the_mask_of_the_forward_pass(causal):
+    # (sh_set_causal takes effect with the next forward pass)
+    check(inputs.CONFIGS["tiny_f32"], causal=causal, causal_after=not causal)
 
 
 def test_backward_argument_checks():
