@@ -262,7 +262,8 @@ int sh_noalloc_gate_topk(int dtype, int n_tokens, int d_model, int n_heads, int 
  * backward formulas - its training differentiates the forward equations of Sec. 2.2 automatically -
  * so this is the chain rule for those equations with the expert selection held fixed.  Call it after
  * sh_forward(layer, x, ...) on the SAME x (it reads the Q, K, V, Ahat, selections and gates that pass
- * left in the workspace; otherwise SH_ERR_NOT_CONFIGURED).  dout [batch, seq, d_model] fp32 = dL/dout.
+ * left in the workspace; otherwise - also after an sh_configure, sh_set_workspace or sh_gate_topk on another
+ * input in between, or a pass with a positional term - SH_ERR_NOT_CONFIGURED).  dout [batch, seq, d_model] fp32 = dL/dout.
  * Every result is a device buffer of the caller, fp32, OVERWRITTEN: dx [batch, seq, d_model]; dWq, dWk
  * [H, d_model, d_head]; dWv [H, E, d_model, d_head]; dWo [H, E, d_head, d_model]; dWs, dWd [H, d_model, E]
  * (the layouts sh_set_weights takes).  Several contributions to a value are added by fp32 reductions in

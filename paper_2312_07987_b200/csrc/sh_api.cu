@@ -198,6 +198,7 @@ static int configure_common(sh_layer* L, int dtype, int batch, int seq, int cach
   //  unaveraged, summed in fp32 they stay within 4e-3)
   L->d.early_rows = (dtype == SH_BF16 && (T >= SH_EARLY_MIN_SEQ || d0.k >= 3)) ? SH_EARLY_ROWS : 0;
   L->ws = nullptr; L->ws_bytes = 0; L->rope = false; L->xl_positions = false;
+  L->fwd_x = nullptr;
   L->d.status = nullptr;
   L->weights_set = false;
   sh_tc_release(L);
@@ -225,6 +226,7 @@ extern "C" int sh_set_workspace(sh_layer* L, void* workspace, size_t bytes) {
   if ((uintptr_t)workspace % 256 != 0) { sh_set_error("workspace must be 256-byte aligned"); return SH_ERR_WORKSPACE; }
   if (bytes < L->o.total) { sh_set_error("workspace too small: %zu bytes given, %zu needed", bytes, L->o.total); return SH_ERR_WORKSPACE; }
   L->ws = (char*)workspace; L->ws_bytes = bytes; L->weights_set = false; L->rope = false; L->xl_positions = false;
+  L->fwd_x = nullptr;
   L->d.status = (int*)(L->ws + L->o.status);
   sh_tc_release(L);
   sh_f32_release(L);
@@ -621,9 +623,12 @@ extern "C" int sh_forward(sh_layer* L, const void* x, void* out, void* stream) {
   if ((uintptr_t)x % 16 != 0 || (uintptr_t)out % 16 != 0) { sh_set_error("x and out must be 16-byte aligned"); return SH_ERR_INVALID_ARG; }
   cudaStream_t st = (cudaStream_t)stream;
   L->launches = 0;
-  L->fwd_x = x; L->fwd_causal = L->d.causal;
-  if (L->dtype == SH_F32) return L->dense ? forward_simt<float, float>(L, SH_STAGE_ALL, x, out, st) : sh_f32_forward(L, x, out, st);
-  return sh_tc_forward(L, x, out, st);
+  L->fwd_x = nullptr; L->fwd_causal = L->d.causal;
+  if (L->dtype == SH_BF16) return sh_tc_forward(L, x, out, st);
+  rc = L->dense ? forward_simt<float, float>(L, SH_STAGE_ALL, x, out, st) : sh_f32_forward(L, x, out, st);
+  // (a pass with a positional term leaves rotated Q and K, or no row maxima: not what sh_backward differentiates)
+  if (rc == SH_OK && !L->rope && !L->xl_positions) L->fwd_x = x;
+  return rc;
 }
 
 extern "C" int sh_backward(sh_layer* L, const void* x, const float* dout, float* dx, float* dWq, float* dWk, float* dWv,
@@ -636,7 +641,7 @@ extern "C" int sh_backward(sh_layer* L, const void* x, const float* dout, float*
     return SH_ERR_UNSUPPORTED;
   }
   if (!x || !dout || !dx || !dWq || !dWk || !dWv || !dWo || !dWs || !dWd) { sh_set_error("sh_backward: NULL argument"); return SH_ERR_INVALID_ARG; }
-  if (L->fwd_x != x) { sh_set_error("sh_backward needs the intermediates of sh_forward on the same x: call sh_forward(layer, x, ...) first"); return SH_ERR_NOT_CONFIGURED; }
+  if (L->fwd_x != x) { sh_set_error("sh_backward needs the intermediates of a plain sh_forward on the same x: call sh_forward(layer, x, ...) first"); return SH_ERR_NOT_CONFIGURED; }
   return sh_f32_backward(L, x, dout, dx, dWq, dWk, dWv, dWo, dWs, dWd, (cudaStream_t)stream);
 }
 
@@ -760,6 +765,7 @@ extern "C" int sh_gate_topk(sh_layer* L, const void* x, int32_t* idx, float* gat
   if (!x) { sh_set_error("x must not be NULL"); return SH_ERR_INVALID_ARG; }
   cudaStream_t st = (cudaStream_t)stream;
   L->launches = 0;
+  if (x != L->fwd_x) L->fwd_x = nullptr;                   // (the workspace then holds this input's selections)
   rc = (L->dtype == SH_F32) ? sh_f32_gate_sort(L, x, st) : sh_tc_gate_sort(L, x, st);
   if (rc != SH_OK) return rc;
   const ShDims& d = L->d;

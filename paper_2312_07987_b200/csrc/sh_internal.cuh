@@ -117,7 +117,7 @@ struct sh_layer {
   size_t ws_bytes = 0;
   ShWorkspace o{};
   bool weights_set = false;
-  const void* fwd_x = nullptr;   // input of the last forward pass (sh_backward wants the same one)
+  const void* fwd_x = nullptr;   // input of the forward pass whose intermediates the workspace holds (sh_backward wants the same one); nullptr: none
   int fwd_causal = 1;            // that pass's mask (its row maxima and normalisers belong to it)
   bool rope = false;       // rotary position embeddings on Q, K (table in the workspace)
   bool xl_positions = false;   // Transformer-XL relative-position term (fp32 configuration; tables in the workspace)

@@ -50,6 +50,43 @@ def test_backward_takes_the_mask_of_the_forward_pass(causal):
     check(inputs.CONFIGS["tiny_f32"], causal=causal, causal_after=not causal)
 
 
+def test_backward_wants_the_intermediates_of_a_plain_pass_on_this_input():
+    inp = inputs.make_inputs(inputs.CONFIGS["tiny_f32"])
+    cfg = inp.cfg
+    layer = binding.layer_from_inputs(inp)
+    x = binding.to_device(inp.x, cfg.dtype)
+    G = torch.ones(inp.x.shape, dtype=torch.float32, device="cuda")
+
+    def refused():
+        with pytest.raises(binding.SwitchHeadError, match="NOT_CONFIGURED"):
+            layer.sh_backward(x, G)
+
+    layer.sh_forward(x)
+    layer.sh_gate_topk(x)                                  # the same selections once more
+    layer.sh_set_rope(10000.0)                             # (for the next forward pass)
+    layer.sh_set_rope(0.0)
+    layer.sh_backward(x, G)
+    other = x + 1
+    layer.sh_gate_topk(other)                              # another input's selections
+    refused()
+    for positional in (True, False):
+        layer.sh_set_rope(10000.0 if positional else 0.0)
+        layer.sh_forward(x)
+        layer.sh_set_rope(0.0)
+        if positional:
+            refused()
+    layer.sh_backward(x, G)
+    layer.sh_set_xl_positions(torch.zeros(cfg.n_heads, cfg.d_model, cfg.d_head, device="cuda"))
+    layer.sh_forward(x)
+    layer.sh_set_xl_positions(None)
+    refused()
+    layer.sh_forward(x)
+    layer.sh_configure(cfg.dtype, *inp.x.shape[:2])        # a workspace without any pass's intermediates
+    layer.sh_set_weights(*[binding.to_device(a, cfg.dtype) for a in (inp.Wq, inp.Wk, inp.Wv, inp.Wo, inp.Ws, inp.Wd)])
+    refused()
+    layer.close()
+
+
 def test_backward_argument_checks():
     inp = inputs.make_inputs(inputs.CONFIGS["tiny_f32"])
     layer = binding.layer_from_inputs(inp)
