@@ -316,9 +316,10 @@ static int set_weights_f32(sh_layer* L, const float* Wq, const float* Wk, const 
     SH_CUDA_CHECK(cudaMemsetAsync(ws + L->o.wo, 0, (size_t)nexp * 6, st));
     if (L->moe_q) SH_CUDA_CHECK(cudaMemsetAsync(ws + L->o.wq_e, 0, (size_t)nexp * 6, st));
     if (L->moe_k) SH_CUDA_CHECK(cudaMemsetAsync(ws + L->o.wk_e, 0, (size_t)nexp * 6, st));
-    // (the projections write d_head's columns only: the padding of Q and K is cleared here, once)
-    SH_CUDA_CHECK(cudaMemsetAsync(ws + L->o.q, 0, (size_t)d.N * HD * 4, st));
-    SH_CUDA_CHECK(cudaMemsetAsync(ws + L->o.k, 0, (size_t)d.N * HD * 4, st));
+    // (the projections write d_head's columns only: the padding of Q and K is cleared here, once - and nothing
+    //  else of them, a backward pass may still want the rest)
+    for (size_t off : {L->o.q, L->o.k})
+      SH_CUDA_CHECK(cudaMemset2DAsync(ws + off + (size_t)d.Dt * 4, (size_t)d.D * 4, 0, (size_t)(d.D - d.Dt) * 4, (size_t)d.N * d.H, st));
   }
   auto split = [&](const float* in, size_t off, long first, int batch, int rows, int cols, long obs, long ors, long oes, long plane) {
     repack<float, __nv_bfloat16, 3>(in, (__nv_bfloat16*)(ws + off) + first, batch, rows, cols, obs, ors, oes, st, plane);

@@ -50,6 +50,21 @@ def test_backward_takes_the_mask_of_the_forward_pass(causal):
     check(inputs.CONFIGS["tiny_f32"], causal=causal, causal_after=not causal)
 
 
+def test_weights_loaded_again_keep_the_intermediates():
+    # d_head 40 is stored as 64 columns
+    inp = inputs.make_inputs(inputs.LayerConfig("bw", inputs.DTYPE_F32, 2, 70, 128, 2, 40, 5, 3, seed=970))
+    layer = binding.layer_from_inputs(inp)
+    x = binding.to_device(inp.x, inp.cfg.dtype)
+    G = torch.ones(inp.x.shape, dtype=torch.float32, device="cuda")
+    layer.sh_forward(x)
+    want = layer.sh_backward(x, G)
+    layer.sh_set_weights(*[binding.to_device(a, inp.cfg.dtype) for a in (inp.Wq, inp.Wk, inp.Wv, inp.Wo, inp.Ws, inp.Wd)])
+    got = layer.sh_backward(x, G)
+    for name, w in want.items():
+        assert float((got[name] - w).abs().max() / w.abs().max()) < 1e-5, name      # (sums in another order)
+    layer.close()
+
+
 def test_backward_wants_the_intermediates_of_a_plain_pass_on_this_input():
     inp = inputs.make_inputs(inputs.CONFIGS["tiny_f32"])
     cfg = inp.cfg
