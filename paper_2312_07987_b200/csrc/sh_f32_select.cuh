@@ -19,45 +19,55 @@ sh_f32_gate_kernel(const float* __restrict__ x, const float* __restrict__ wgate,
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int t0 = blockIdx.x * TOK;
   const long nthr = (long)gridDim.x * 512, me = (long)blockIdx.x * 512 + tid;
-  for (int m0 = 0; m0 < d.M; m0 += CH) {
-    const int mw = min(CH, d.M - m0);           // a multiple of 64
-    __syncthreads();
-    for (int i = tid; i < TOK * (CH / 4); i += 512) {
-      const int r = i / (CH / 4), c = (i % (CH / 4)) * 4;
-      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (c < mw && t0 + r < d.N) {
-        const float* p = x + (size_t)(t0 + r) * d.M + m0 + c;
-        v = vec ? __ldg(reinterpret_cast<const float4*>(p)) : make_float4(__ldg(p), __ldg(p + 1), __ldg(p + 2), __ldg(p + 3));   // (x off its alignment: sh_gate_topk takes it)
-      }
-      *reinterpret_cast<float4*>(gsm + r * CH + c) = v;
-    }
-    for (int g = warp; g < d.G; g += 32) {                  // two columns at a time, all of their loads in flight
-      const bool two = g + 16 < d.G;
-      const float* w0 = wgate + (size_t)g * d.M + m0;
-      const float* w1 = w0 + (two ? (size_t)16 * d.M : 0);
-      // (lane l sums the columns l, l + 32, ... in order and the lanes are added as a butterfly: the order of
-      //  sh_gate_topk_kernel, so that the allocation-free entry point gives the same bits up to CH columns)
-      float wv[2][U];
+  for (int g0 = 0; g0 < d.G; g0 += 32) {                    // a warp's two columns at a time, all of their loads in flight
+    const int g = g0 + warp;
+    const bool one = g < d.G, two = g + 16 < d.G;
+    // (lane l sums the columns l, l + 32, ... of the whole row in order and the lanes are added as a butterfly: the
+    //  order of sh_gate_topk_kernel, so that the allocation-free entry point gives the same bits)
+    float acc[2][TOK];
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int c = u * 32 + lane;
-        wv[0][u] = c < mw ? __ldg(w0 + c) : 0.f;
-        wv[1][u] = c < mw ? __ldg(w1 + c) : 0.f;
-      }
-      if (g == warp) __syncthreads();                       // (every warp's first round, or the one behind the loop)
-      float acc[2][TOK];
-#pragma unroll
-      for (int r = 0; r < TOK; ++r) acc[0][r] = acc[1][r] = 0.f;
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        if (u * 32 >= mw) break;
-#pragma unroll
-        for (int r = 0; r < TOK; ++r) {
-          const float xv = gsm[r * CH + u * 32 + lane];
-          acc[0][r] = fmaf(xv, wv[0][u], acc[0][r]);
-          acc[1][r] = fmaf(xv, wv[1][u], acc[1][r]);
+    for (int r = 0; r < TOK; ++r) acc[0][r] = acc[1][r] = 0.f;
+    for (int m0 = 0; m0 < d.M; m0 += CH) {
+      const int mw = min(CH, d.M - m0);         // a multiple of 64
+      const bool fresh = g0 == 0 || d.M > CH;   // (a row that fits is read once)
+      if (fresh) {
+        __syncthreads();
+        for (int i = tid; i < TOK * (CH / 4); i += 512) {
+          const int r = i / (CH / 4), c = (i % (CH / 4)) * 4;
+          float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (c < mw && t0 + r < d.N) {
+            const float* p = x + (size_t)(t0 + r) * d.M + m0 + c;
+            v = vec ? __ldg(reinterpret_cast<const float4*>(p)) : make_float4(__ldg(p), __ldg(p + 1), __ldg(p + 2), __ldg(p + 3));   // (x off its alignment: sh_gate_topk takes it)
+          }
+          *reinterpret_cast<float4*>(gsm + r * CH + c) = v;
         }
       }
+      float wv[2][U];
+      if (one) {
+        const float* w0 = wgate + (size_t)g * d.M + m0;
+        const float* w1 = w0 + (two ? (size_t)16 * d.M : 0);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int c = u * 32 + lane;
+          wv[0][u] = c < mw ? __ldg(w0 + c) : 0.f;
+          wv[1][u] = c < mw ? __ldg(w1 + c) : 0.f;
+        }
+      }
+      if (fresh) __syncthreads();
+      if (one) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          if (u * 32 >= mw) break;
+#pragma unroll
+          for (int r = 0; r < TOK; ++r) {
+            const float xv = gsm[r * CH + u * 32 + lane];
+            acc[0][r] = fmaf(xv, wv[0][u], acc[0][r]);
+            acc[1][r] = fmaf(xv, wv[1][u], acc[1][r]);
+          }
+        }
+      }
+    }
+    if (one) {
       // lane sums of TOK tokens: at each step a lane keeps half of its tokens and hands the others over
 #pragma unroll
       for (int q = 0; q < 2; ++q) {
@@ -74,17 +84,11 @@ sh_f32_gate_kernel(const float* __restrict__ x, const float* __restrict__ wgate,
         }
 #pragma unroll
         for (int o = 32 / TOK / 2; o > 0; o >>= 1) acc[q][0] += __shfl_xor_sync(0xffffffffu, acc[q][0], o);
-        if (lane % (32 / TOK) == 0 && (q == 0 || two)) {
-          float* z = s_z + tokn * d.G + g + 16 * q;
-          *z = (m0 == 0 ? 0.f : *z) + acc[q][0];
-        }
+        if (lane % (32 / TOK) == 0 && (q == 0 || two)) s_z[tokn * d.G + g + 16 * q] = acc[q][0];
       }
     }
-    if (warp >= d.G) __syncthreads();                      // (a warp without a column meets the barrier of the others' first round here)
-    if (m0 == 0) {
-      for (long i = me; i < nzero; i += nthr) zero[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
   }
+  for (long i = me; i < nzero; i += nthr) zero[i] = make_float4(0.f, 0.f, 0.f, 0.f);
   __syncthreads();
   const int groups = d.sides * d.H;
   for (int i = tid; i < TOK * groups; i += 512) {

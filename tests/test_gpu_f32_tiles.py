@@ -93,3 +93,30 @@ def test_f32_output_in_place_of_the_input(cache, shared, positions):
     layer.sh_forward(x, out=out)
     assert float((out - want).abs().max() / want.abs().max()) < TOL
     layer.close()
+
+
+@pytest.mark.parametrize("blocks", ["8 tokens", "16 tokens"])
+@pytest.mark.parametrize("M,H,E,k", [
+    (64, 1, 2, 1),                   # fewer gate columns than warps
+    (512, 3, 16, 4),                 # 96: three rounds of 32
+    (576, 2, 9, 3),                  # rows staged in 1024 columns, 36 gate columns
+    (1088, 2, 4, 2),                 # one piece of 64 behind the first 1024
+    (2112, 1, 17, 2),                # three pieces, two rounds
+])
+def test_f32_gate_kernel_sums_as_the_allocation_free_one(M, H, E, k, blocks):
+    # blocks of 16 tokens from 32 tokens per SM on; every output bit for bit: both sum a logit in the same order
+    N = 69 if blocks == "8 tokens" else 32 * torch.cuda.get_device_properties(0).multi_processor_count + 5
+    g = torch.Generator(device="cuda").manual_seed(M + N)
+    normal = lambda *shape: torch.randn(*shape, generator=g, device="cuda")
+    W = [normal(H, M, E) / M ** 0.5 for _ in range(2)]
+    bias = [normal(H, E) for _ in range(2)]
+    layer = binding.Layer(M, H, 16, E, k)
+    layer.sh_configure(binding.SH_F32, 1, N)
+    layer.sh_set_weights(normal(H, M, 16), normal(H, M, 16), normal(H, E, M, 16), normal(H, E, 16, M), *W, *bias)
+    x = normal(1, N, M)
+    got = layer.sh_gate_topk(x)
+    want = binding.sh_noalloc_gate_topk(binding.SH_F32, x[0], torch.cat([w.transpose(1, 2).reshape(H * E, M) for w in W]).contiguous(),
+                                        torch.cat([b.reshape(-1) for b in bias]), H, E, k)
+    for a, b in zip(got, want):
+        assert torch.equal(a, b)
+    layer.close()
