@@ -106,12 +106,13 @@ __device__ __forceinline__ void tmem_add(uint32_t taddr, float (&acc)[N]) {
   }
 }
 
-// Two fp32 values as three packed bf16 pairs whose sum they are.
+// Two fp32 values as three packed bf16 pairs whose sum they are.  (The leading part saturates: fp32 reaches half a
+// bf16 step past the largest bf16 value, and an infinity there would leave a rest of minus infinity.)
 __device__ __forceinline__ float2 sub_bf16x2(float2 x, uint32_t p) {
   return __ffma2_rn(make_float2(__uint_as_float(p << 16), __uint_as_float(p & 0xFFFF0000u)), make_float2(-1.f, -1.f), x);
 }
 __device__ __forceinline__ void split_bf16x3(float a, float b, uint32_t& h, uint32_t& m, uint32_t& l) {
-  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(h) : "f"(b), "f"(a));
+  asm("cvt.rn.satfinite.bf16x2.f32 %0, %1, %2;" : "=r"(h) : "f"(b), "f"(a));
   float2 r = sub_bf16x2(make_float2(a, b), h);
   asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(m) : "f"(r.y), "f"(r.x));
   r = sub_bf16x2(r, m);

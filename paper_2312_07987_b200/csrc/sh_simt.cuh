@@ -32,7 +32,8 @@ sh_repack_kernel(const TI* __restrict__ in, TO* __restrict__ out, int batch, int
         TO* o = out + b * obs + c * ors + r * oes;
 #pragma unroll
         for (int p = 0; p < PLANES; ++p) {
-          const TO w = sh_from_float<TO>(v);
+          // (the leading one of three saturates: see split_bf16x3)
+          const TO w = sh_from_float<TO>(PLANES == 3 && p == 0 ? fminf(fmaxf(v, -3.3895313892515355e38f), 3.3895313892515355e38f) : v);
           o[p * plane] = w;
           v -= sh_to_float<TO>(w);
         }

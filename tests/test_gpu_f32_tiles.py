@@ -16,13 +16,15 @@ pytestmark = pytest.mark.gpu
 TOL = 1.4e-5
 
 
-def run(B, T, M, H, D, E, k, causal=True, offset=0, zipf=0.0):
+def run(B, T, M, H, D, E, k, causal=True, offset=0, zipf=0.0, change=None):
     cfg = inputs.LayerConfig("tiles", inputs.DTYPE_F32, B, T, M, H, D, E, k, seed=77 + T + D, zipf_bias=zipf)
     inp = inputs.make_inputs(cfg)
+    G = np.random.default_rng(3).standard_normal(inp.x.shape).astype(np.float32)
+    if change:
+        change(inp, G)
     layer = binding.layer_from_inputs(inp)
     layer.sh_set_causal(causal)
     x = binding.to_device(inp.x, cfg.dtype)
-    G = np.random.default_rng(3).standard_normal(inp.x.shape).astype(np.float32)
     g = torch.empty(G.size + offset, dtype=torch.float32, device="cuda")[offset:].view(G.shape)
     g.copy_(torch.from_numpy(G))
     y = layer.sh_forward(x)
@@ -64,6 +66,22 @@ def test_f32_empty_experts_and_no_mask():
 
 def test_f32_gradient_input_off_its_alignment():
     run(1, 90, 128, 2, 76, 4, 2, offset=1)
+
+
+def large_weight(inp, G):
+    inp.Wo[0, 0, 0, 0] = 3.4e38
+    G *= 1e-3
+
+
+def large_gradient(inp, G):
+    G[0, 0, 0] = -3.4e38
+    inp.Wo *= 1e-3                   # (no partial sum overflows)
+
+
+@pytest.mark.parametrize("change", [large_weight, large_gradient])
+def test_f32_values_past_the_largest_bf16(change):
+    # (half a bf16 step past 3.3895e38; results and gradients stay finite)
+    run(1, 90, 128, 2, 76, 4, 2, causal=False, change=change)
 
 
 def test_f32_selection_of_an_input_off_its_alignment():
