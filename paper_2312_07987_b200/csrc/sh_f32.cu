@@ -32,6 +32,9 @@ int sm_count(sh_layer* L) {
 // Row tiles of one head in a side's tile table (sh_f32_select_kernel).
 int head_tiles(const ShDims& d) { return (int)(((long long)d.N * d.k + 127ll * d.E) / 128); }
 
+// Kernels are chained by programmatic dependent launch, except in a stage-timed pass.
+bool chained(const sh_layer* L) { return !L->ev; }
+
 // One mode's tiles as a part of a launch.
 template <int MODE>
 XPart part(sh_layer* L, const XGemmArgs& g, int gx, int gy, int gz = 1, const PlaneMap* w = nullptr) {
@@ -51,7 +54,7 @@ int launch_x(sh_layer* L, cudaStream_t st, const XPart& a, const XPart& b = XPar
   auto kern = sh_f32_gemm_kernel<A, B>;
   if (int rc = set_smem(kern, XGemmSmem::TOTAL)) return rc;
   L->launches += 1;
-  return launch_k(true, kern, dim3((unsigned)n), dim3(XG_THREADS), XGemmSmem::TOTAL, st, S->wgate.mn, a, b);
+  return launch_k(chained(L), kern, dim3((unsigned)n), dim3(XG_THREADS), XGemmSmem::TOTAL, st, S->wgate.mn, a, b);
 }
 
 // Column tiles over `cols` columns: how many, and how wide (a multiple of 16).
@@ -101,11 +104,11 @@ int launch_gate_sort(sh_layer* L, const void* x, float* zero, long n, cudaStream
   auto kern = small ? (ch == 512 ? sh_f32_gate_kernel<8, 512> : sh_f32_gate_kernel<8, 1024>)
                     : (ch == 512 ? sh_f32_gate_kernel<16, 512> : sh_f32_gate_kernel<16, 1024>);
   if (int rc = set_smem(kern, (int)smem)) return rc;
-  if (int rc = launch_k(true, kern, dim3((unsigned)((d.N + tok - 1) / tok)), dim3(512), smem, st, (const float*)x, (const float*)(ws + L->o.wgate32),
+  if (int rc = launch_k(chained(L), kern, dim3((unsigned)((d.N + tok - 1) / tok)), dim3(512), smem, st, (const float*)x, (const float*)(ws + L->o.wgate32),
                         (const float*)(ws + L->o.gbias), (int*)(ws + L->o.idx), (float*)(ws + L->o.gate), (float4*)zero, n / 4, d, (int)((uintptr_t)x % 16 == 0)))
     return rc;
   L->launches += 2;
-  return launch_k(true, sh_f32_sort_kernel, dim3(d.sides * d.H), dim3(1024), 0, st, (const int*)(ws + L->o.idx), (const float*)(ws + L->o.gate),
+  return launch_k(chained(L), sh_f32_sort_kernel, dim3(d.sides * d.H), dim3(1024), 0, st, (const int*)(ws + L->o.idx), (const float*)(ws + L->o.gate),
                   (int*)(ws + L->o.offsets), (int*)(ws + L->o.lists), (float*)(ws + L->o.lgate), (ShTile*)(ws + L->o.tiles), d, head_tiles(d));
 }
 
@@ -134,7 +137,7 @@ int launch_attn_t(sh_layer* L, float* zero, long n, cudaStream_t st) {
   char* ws = L->ws;
   if (int rc = set_smem(sh_f32_attn_kernel<D>, FAttnSmem<D>::TOTAL)) return rc;
   const int nq = (d.T - d.Tc + 31) / 32;
-  return launch_k(true, sh_f32_attn_kernel<D>, dim3((unsigned)nq * d.B * d.H), dim3(256), FAttnSmem<D>::TOTAL, st,
+  return launch_k(chained(L), sh_f32_attn_kernel<D>, dim3((unsigned)nq * d.B * d.H), dim3(256), FAttnSmem<D>::TOTAL, st,
                   (const float*)(ws + L->o.q), (const float*)(ws + L->o.k), (const float*)(ws + L->o.v), (float*)(ws + L->o.ahat),
                   (float*)(ws + L->o.f32stats), (float4*)zero, n / 4, d);
 }
@@ -175,7 +178,7 @@ int launch_attn_bw_t(sh_layer* L, const BwBuffers& w, cudaStream_t st) {
   const long units = (long)kt * d.B * d.H * qt / (d.causal ? 2 : 1);
   long run = units / (4l * sm_count(L));
   run = run < 2 ? 2 : run > qt ? qt : run;
-  return launch_k(true, sh_f32_attn_bw_kernel<D>, dim3((unsigned)kt * d.B * d.H, (unsigned)((qt + run - 1) / run)), dim3(256), FBwSmem<D>::TOTAL, st,
+  return launch_k(chained(L), sh_f32_attn_bw_kernel<D>, dim3((unsigned)kt * d.B * d.H, (unsigned)((qt + run - 1) / run)), dim3(256), FBwSmem<D>::TOTAL, st,
                   (const float*)(ws + L->o.q), (const float*)(ws + L->o.k), (const float*)(ws + L->o.v), (const float*)w.dahat,
                   (const float*)(ws + L->o.f32stats), (const float*)w.dsum, w.dq, w.dk, w.dv, d, (int)run);
 }
@@ -289,7 +292,7 @@ int sh_f32_backward(sh_layer* L, const void* x, const float* dout, float* dx, fl
   if ((rc = launch_x<X_DA>(L, st, part<X_DA>(L, g, d.H * ht, g.nsub, g.ksplit)))) return rc;
   // attention
   const int rows = d.N * d.H;
-  if ((rc = launch_k(true, sh_f32_rowdot_kernel, dim3((unsigned)((rows + 7) / 8)), dim3(256), 0, st, (const float*)w.dahat,
+  if ((rc = launch_k(chained(L), sh_f32_rowdot_kernel, dim3((unsigned)((rows + 7) / 8)), dim3(256), 0, st, (const float*)w.dahat,
                      (const float*)(ws + L->o.ahat), w.dsum, rows, d.D))) return rc;
   rc = d.D == 32 ? launch_attn_bw_t<32>(L, w, st) : d.D == 64 ? launch_attn_bw_t<64>(L, w, st)
      : d.D == 128 ? launch_attn_bw_t<128>(L, w, st) : launch_attn_bw_t<256>(L, w, st);
@@ -298,7 +301,7 @@ int sh_f32_backward(sh_layer* L, const void* x, const float* dout, float* dx, fl
   g = src;
   col_tiles(g, d.M);
   if ((rc = launch_x<X_DR>(L, st, part<X_DR>(L, g, d.H * ht, g.nsub)))) return rc;
-  if ((rc = launch_k(true, sh_f32_dz_kernel, dim3((unsigned)(((long)d.N * d.k + 255) / 256), 2 * d.H), dim3(256), 0, st, (const float*)w.ds,
+  if ((rc = launch_k(chained(L), sh_f32_dz_kernel, dim3((unsigned)(((long)d.N * d.k + 255) / 256), 2 * d.H), dim3(256), 0, st, (const float*)w.ds,
                      (const int*)(ws + L->o.lists), (const float*)(ws + L->o.lgate), (const int*)(ws + L->o.offsets), w.dz, src.ldz, d))) return rc;
   // queries, keys and gates: the rest of dx
   g = src;
@@ -332,7 +335,7 @@ int sh_f32_backward(sh_layer* L, const void* x, const float* dout, float* dx, fl
   }
   const XWPart pq = wpart(gq, mt, ct, gq.ksplit), pv = wpart(gv, d.H * d.E * gv.ksplit, gv.nsub, mt), po = wpart(go, d.H * d.E * go.ksplit, go.nsub, dt);
   if ((rc = set_smem(sh_f32_wgrad_kernel, XWgradSmem::TOTAL))) return rc;
-  if ((rc = launch_k(true, sh_f32_wgrad_kernel, dim3((unsigned)(pq.n + pv.n + po.n)), dim3(XW_THREADS), XWgradSmem::TOTAL, st, pq, pv, po))) return rc;
+  if ((rc = launch_k(chained(L), sh_f32_wgrad_kernel, dim3((unsigned)(pq.n + pv.n + po.n)), dim3(XW_THREADS), XWgradSmem::TOTAL, st, pq, pv, po))) return rc;
   SH_CUDA_CHECK(cudaGetLastError());
   L->launches += 4;
   return SH_OK;
