@@ -8,6 +8,7 @@
 #include "sh_f32_attn.cuh"
 #include "sh_f32_select.cuh"
 
+#include <cstdlib>
 #include <new>
 
 using namespace shtc;
@@ -17,8 +18,10 @@ namespace {
 // The split weights as [3 planes, rows, inner]: boxes of 64 rows x 32 positions where a row runs along the
 // contraction (k), of 32 rows x 64 columns where the contraction runs over rows (mn).
 struct PlaneMap { CUtensorMap k, mn; };
-struct F32State { PlaneMap wqk, wgate, wv, wo, wq_e, wk_e; };
-
+struct F32State {
+  PlaneMap wqk, wgate, wv, wo, wq_e, wk_e;
+  bool pdl = true;          // kernels chained by programmatic dependent launch (the debug library's SH_NO_PDL: ordinary launches)
+};
 
 int sm_count(sh_layer* L) {
   if (L->sm_count == 0) {
@@ -32,8 +35,8 @@ int sm_count(sh_layer* L) {
 // Row tiles of one head in a side's tile table (sh_f32_select_kernel).
 int head_tiles(const ShDims& d) { return (int)(((long long)d.N * d.k + 127ll * d.E) / 128); }
 
-// Kernels are chained by programmatic dependent launch, except in a stage-timed pass.
-bool chained(const sh_layer* L) { return !L->ev; }
+// Kernels are chained, except in a stage-timed pass.
+bool chained(const sh_layer* L) { return ((const F32State*)L->f32)->pdl && !L->ev; }
 
 // One mode's tiles as a part of a launch.
 template <int MODE>
@@ -200,6 +203,9 @@ int sh_f32_prepare(sh_layer* L) {
   F32State* S = new (std::nothrow) F32State();
   if (!S) { sh_set_error("out of host memory"); return SH_ERR_INVALID_ARG; }
   L->f32 = S;
+#ifdef SH_DEBUG
+  S->pdl = !getenv("SH_NO_PDL");
+#endif
   const ShDims& d = L->d;
   char* ws = L->ws;
   auto enc = [&](PlaneMap& m, size_t off, uint64_t inner, uint64_t rows) -> int {

@@ -171,6 +171,12 @@ __device__ __forceinline__ void store_row(float* dst, const float (&v)[N], int v
   }
 }
 
+// Token of a list entry (0 where the debug library finds that it is none).
+__device__ __forceinline__ int xg_token(const XGemmArgs& g, size_t li) {
+  const int t = g.lists[li];
+  return SH_INDEX_OK(t, g.d.N, g.status, SH_SITE_V_LIST) ? t : 0;
+}
+
 struct XTile { int x, y, z; };           // which tile of its mode a block works on
 
 // One tile.  mapW: planes of the mode's weights, rows [(which*H + h)*D + dd][m] (Q, K), [(h*E + e)*D + dd][m] (V),
@@ -209,6 +215,8 @@ __device__ __forceinline__ void xg_tile(const CUtensorMap& mapW, const CUtensorM
   if (LIST_ROWS) {
     const ShTile tl = g.tiles[blk.x];
     if (tl.nrows == 0) return;                             // (before any allocation)
+    if (!SH_INDEX_OK(tl.h, d.H, g.status, SH_SITE_V_TILE) || !SH_INDEX_OK(tl.e, d.E, g.status, SH_SITE_V_TILE) ||
+        !SH_INDEX_OK(tl.nrows - 1, SH_TILE_ROWS, g.status, SH_SITE_V_TILE) || !SH_INDEX_OK(tl.row0, (long long)d.N * d.k - tl.nrows + 1, g.status, SH_SITE_V_TILE)) return;
     h = tl.h; e = tl.e; row0 = tl.row0; nrows = tl.nrows;
     n0 = blk.y * g.sub_cols;
     ncols = min(g.sub_cols, ((MODE == X_O || MODE == X_DR) ? d.M : d.Dt) - n0);
@@ -328,7 +336,7 @@ __device__ __forceinline__ void xg_tile(const CUtensorMap& mapW, const CUtensorM
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
         const int r = row0 + min(8 * warp + (lane >> 3) + 4 * u + 64 * j, nrows - 1);
-        const size_t t = LIST_ROWS ? g.lists[lbase + r] : r;
+        const size_t t = LIST_ROWS ? xg_token(g, lbase + r) : r;
         arow[j][u] = (MODE == X_QK || MODE == X_V ? g.x + t * d.M
                     : MODE == X_O ? g.ahat + t * HD + h * d.D
                     : MODE == X_DA ? g.dy + t * d.M
@@ -414,7 +422,7 @@ __device__ __forceinline__ void xg_tile(const CUtensorMap& mapW, const CUtensorM
     if (r < nrows && valid > 0 && !dead) {
       if (LIST_ROWS) {
         const size_t li = lbase + row0 + r;
-        const int t = g.lists[li];
+        const int t = xg_token(g, li);
         const float gt = g.lgate[li];
         if (MODE == X_DA || MODE == X_DR) {
           // gate gradient: the ungated result against the forward operand of the same row
@@ -471,7 +479,7 @@ __device__ __forceinline__ void xg_tile(const CUtensorMap& mapW, const CUtensorM
         const int n = (ncols + 3) & ~3;
         float* o = nullptr;
         if (LIST_ROWS) {
-          const int t = g.lists[lbase + row0 + tid];
+          const int t = xg_token(g, lbase + row0 + tid);
           if (MODE == X_V) o = g.v + (((size_t)(t / d.T) * d.H + h) * d.T + t % d.T) * d.D + n0;
           if (MODE == X_O) { const int orow = sh_out_row(d, t); if (orow >= 0) o = g.y + (size_t)orow * d.M + n0; }   // (cache tokens have no output row)
           if (MODE == X_DA) o = g.dahat + (size_t)t * HD + h * d.D + n0;

@@ -133,7 +133,8 @@ sh_f32_sort_kernel(const int* __restrict__ idx, const float* __restrict__ gate, 
     unsigned sel = 0;
     if (t < d.N) {
       const size_t o = (((size_t)side * d.N + t) * d.H + h) * d.k;
-      for (int j = 0; j < d.k; ++j) sel |= 1u << idx[o + j];
+      for (int j = 0; j < d.k; ++j)
+        if (SH_INDEX_OK(idx[o + j], d.E, d.status, SH_SITE_SORT_EXPERT)) sel |= 1u << idx[o + j];
     }
     for (int e = 0; e < d.E; ++e) {
       const unsigned bal = __ballot_sync(0xffffffffu, (sel >> e) & 1u);
@@ -175,7 +176,8 @@ sh_f32_sort_kernel(const int* __restrict__ idx, const float* __restrict__ gate, 
     const size_t o = (((size_t)side * d.N + t) * d.H + h) * d.k;
     unsigned sel = 0;
     if (live)
-      for (int j = 0; j < d.k; ++j) sel |= 1u << idx[o + j];
+      for (int j = 0; j < d.k; ++j)
+        if (SH_INDEX_OK(idx[o + j], d.E, d.status, SH_SITE_SORT_EXPERT)) sel |= 1u << idx[o + j];
     unsigned mybal = 0;                                    // lane e: which lanes chose expert e
     for (int e = 0; e < d.E; ++e) {
       const unsigned bal = __ballot_sync(0xffffffffu, (sel >> e) & 1u);
@@ -198,10 +200,12 @@ sh_f32_sort_kernel(const int* __restrict__ idx, const float* __restrict__ gate, 
     for (int j = 0; j < d.k; ++j) {
       const int e = live ? idx[o + j] : 0;
       const unsigned bal = __shfl_sync(0xffffffffu, mybal, e);
-      if (live) {
+      if (live && SH_INDEX_OK(e, d.E, d.status, SH_SITE_SORT_EXPERT)) {
         const int pos = s_w[warp][e] + __popc(bal & ((1u << lane) - 1u));
-        ls[pos] = t;
-        lg[pos] = gate[o + j];
+        if (SH_INDEX_OK(pos, (long long)d.N * d.k, d.status, SH_SITE_SORT_SLOT)) {
+          ls[pos] = t;
+          lg[pos] = gate[o + j];
+        }
       }
     }
     __syncthreads();
@@ -224,5 +228,5 @@ sh_f32_dz_kernel(const float* __restrict__ ds, const int* __restrict__ lists, co
   while (e < d.E - 1 && off[e + 1] <= p) ++e;
   const size_t li = (size_t)grp * per + p;
   const float g = lgate[li];
-  dz[(size_t)lists[li] * ldz + grp * d.E + e] = ds[li] * g * (1.f - g);
+  if (SH_INDEX_OK(lists[li], d.N, d.status, SH_SITE_V_LIST)) dz[(size_t)lists[li] * ldz + grp * d.E + e] = ds[li] * g * (1.f - g);
 }

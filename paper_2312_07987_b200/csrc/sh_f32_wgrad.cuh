@@ -58,6 +58,7 @@ __device__ __forceinline__ void xw_tile(const XGemmArgs& g, XTile blk) {
     const int grp = blk.x / g.ksplit, part = blk.x % g.ksplit;
     h = grp / d.E; e = grp % d.E;
     const int o0 = g.offsets[h * (d.E + 1) + e], o1 = g.offsets[h * (d.E + 1) + e + 1];
+    if (!SH_INDEX_OK(o0, (long long)d.N * d.k + 1, g.status, SH_SITE_V_TILE) || !SH_INDEX_OK(o1, (long long)d.N * d.k + 1, g.status, SH_SITE_V_TILE)) return;
     const int per = (((o1 - o0 + XG_BK - 1) / XG_BK + g.ksplit - 1) / g.ksplit) * XG_BK;
     kbeg = min(o1, o0 + part * per); kend = min(o1, kbeg + per);
     n0 = blk.y * g.sub_cols; m0 = blk.z * 128;
@@ -143,7 +144,7 @@ __device__ __forceinline__ void xw_tile(const XGemmArgs& g, XTile blk) {
       for (int u = 0; u < 2; ++u) {
         const int pa = p0 + 2 * warp + u;
         if (!LIST) ta[u] = min(pa, d.N - 1);
-        else if (pa < kend) ta[u] = __ldg(g.lists + lbase + pa);
+        else if (pa < kend) ta[u] = xg_token(g, lbase + pa);
       }
       if (LIST && p0 + ar < kend) gnext = __ldg(g.lgate + lbase + p0 + ar);
     };

@@ -7,6 +7,7 @@ tests/test_gpu_debug_library.py starts this module as a child process with both 
     python -m tests.debug_driver CASE
 
 Prints DEBUG_DRIVER_OK as its last line when every check of the case passed."""
+import ctypes
 import os
 import sys
 
@@ -33,6 +34,34 @@ def main(case: str) -> None:
             tp.full_check(inputs.make_inputs(inputs.LayerConfig("edge_bf16_wide", inputs.DTYPE_BF16, B, T, M, H, D, E, k, seed=300 + T)))
         for cfg in tp._random_bf16_configs(4, 11):
             tp.full_check(inputs.make_inputs(cfg), check_stage_buffers=False)
+    elif case == "f32":
+        # both directions of the fp32 layer with index checks: silent on edge shapes, and a token that is none is
+        # recorded (the number right behind the last one, in memory with a row to spare)
+        from tests import test_gpu_f32_tiles as tt
+        for B, T, M, H, D, E, k in [(1, 1, 64, 1, 1, 1, 1), (2, 33, 128, 1, 64, 3, 3), (1, 129, 192, 2, 65, 4, 2), (2, 600, 128, 2, 76, 32, 4)]:
+            tt.run(B, T, M, H, D, E, k)
+        inp = inputs.make_inputs(inputs.LayerConfig("f32_dbg", inputs.DTYPE_F32, 1, 200, 128, 2, 64, 4, 2, seed=9))
+        layer = binding.layer_from_inputs(inp)
+        room = torch.zeros(2, 201, 128, device="cuda")
+        x, G = room[0, :200].view(1, 200, 128), room[1, :200].view(1, 200, 128)
+        x.copy_(binding.to_device(inp.x, 0))
+        G.fill_(1.0)
+        layer.sh_forward(x)
+        p, n = ctypes.c_void_p(), ctypes.c_size_t()
+        binding._check(binding.lib.sh_debug_buffer(layer.handle, binding.BUF["LISTS"], ctypes.byref(p), ctypes.byref(n)))
+        lists = layer.workspace[p.value - layer.workspace.data_ptr():][:n.value].view(torch.int32)
+        for entry in (0, lists.numel() - 1):              # a source-side and a destination-side list
+            was = int(lists[entry])
+            lists[entry] = 200
+            layer.sh_backward(x, G)
+            assert layer.sh_last_status() == -7, layer.sh_last_status()
+            w = layer.sh_status_block()
+            assert w[8:11] == [1, 200, 200], w
+            layer.sh_clear_status()
+            lists[entry] = was
+        layer.sh_backward(x, G)
+        assert layer.sh_last_status() == 0
+        layer.close()
     elif case == "sparse_o":
         # the shapes the 2:4-sparse output projection serves (or, with SH_O_MASKED, the masked kernel on them)
         for cfg in tp.SPARSE_O_CONFIGS:

@@ -52,3 +52,8 @@ def test_index_checks_stay_silent_on_edge_shapes():
 
 def test_index_check_records_a_bad_value_and_the_layer_recovers():
     run_case("index_selftest")
+
+
+@pytest.mark.parametrize("env", [{}, {"SH_NO_PDL": "1"}], ids=["default", "SH_NO_PDL"])
+def test_fp32_layer_with_index_checks(env):
+    run_case("f32", env)
