@@ -17,6 +17,8 @@ __device__ __forceinline__ void fa_cp16(float* dst, const float* src, bool ok) {
 __device__ __forceinline__ void fa_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N> __device__ __forceinline__ void fa_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
+template <bool B> struct fa_bool { static constexpr bool value = B; };
+
 // `rows` rows of W floats (row stride D in memory, LD in shared memory; rows at or past `live` zero), by 128 threads.
 template <int D>
 __device__ __forceinline__ void fa_tile(float* dst, const float* src, int rows, int live, long src_ld, int t) {
@@ -139,9 +141,12 @@ sh_f32_attn_kernel(const float* __restrict__ Q, const float* __restrict__ K, con
     group_sync(1 + grp, 128);                              // K read, P written, V there for every thread
     if (kt + 2 < ntile) fa_tile<D>(sK, Kb + (size_t)(kt + 2) * KT * D, KT, d.T - (kt + 2) * KT, D, t);
     fa_commit();
-    if (col_ok) {
+    // (a tile some row sees a part of: what a row does not see is left out of its sum, not multiplied by zero -
+    //  a value that is not finite stays with the rows that see it)
+    auto product = [&](auto part) {
+      const int kend = decltype(part)::value ? min(KT, nkeys - kt * KT) : KT;    // (past the last row's last key: nothing to add)
 #pragma unroll 2
-      for (int kk = 0; kk < KT; kk += 4) {
+      for (int kk = 0; kk < kend; kk += 4) {
         float4 pv[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) pv[i] = *reinterpret_cast<const float4*>(sP + (ty + 8 * i) * PLD + kk);
@@ -152,6 +157,7 @@ sh_f32_attn_kernel(const float* __restrict__ Q, const float* __restrict__ K, con
             const float4 vv = *reinterpret_cast<const float4*>(sV + (kk + u) * LD + 4 * tx + 64 * c);
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
+              if (decltype(part)::value && kt * KT + kk + u > q0 + ty + 8 * i) continue;
               const float p = u == 0 ? pv[i].x : u == 1 ? pv[i].y : u == 2 ? pv[i].z : pv[i].w;
               o[i][4 * c] = fmaf(p, vv.x, o[i][4 * c]);
               o[i][4 * c + 1] = fmaf(p, vv.y, o[i][4 * c + 1]);
@@ -161,6 +167,10 @@ sh_f32_attn_kernel(const float* __restrict__ Q, const float* __restrict__ K, con
           }
         }
       }
+    };
+    if (col_ok) {
+      if (d.causal && kt * KT + KT - 1 > q0) product(fa_bool<true>());
+      else product(fa_bool<false>());
     }
     group_sync(1 + grp, 128);                              // V and P read
     if (kt + 2 < ntile) fa_tile<D>(sV, Vb + (size_t)(kt + 2) * KT * D, KT, d.T - (kt + 2) * KT, D, t);
@@ -332,10 +342,13 @@ sh_f32_attn_bw_kernel(const float* __restrict__ Q, const float* __restrict__ K, 
       }
     }
     group_sync(1 + grp, 128);
-    if (col_ok) {
+    // (pairs of a partly visible tile that do not see one another are left out, as in the forward pass)
+    auto products = [&](auto part) {
+      constexpr bool PART = decltype(part)::value;
+      const int rlo = PART ? max(0, k0 - q0) : 0;            // the first row that sees a key of the block
       // dV, dK: keys 4 ty ... 4 ty + 3
 #pragma unroll 2
-      for (int r = 0; r < TQ; ++r) {
+      for (int r = rlo; r < TQ; ++r) {
         const float4 p4 = *reinterpret_cast<const float4*>(sP + r * PLD + 4 * ty);
         const float4 s4 = *reinterpret_cast<const float4*>(sS + r * PLD + 4 * ty);
         const float pp[4] = {p4.x, p4.y, p4.z, p4.w}, ss[4] = {s4.x, s4.y, s4.z, s4.w};
@@ -345,6 +358,7 @@ sh_f32_attn_bw_kernel(const float* __restrict__ Q, const float* __restrict__ K, 
           const float4 qv = *reinterpret_cast<const float4*>(sQ + r * LD + 4 * tx + 64 * c);
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
+            if (PART && k0 + 4 * ty + i > q0 + r) continue;
             gv[i][4 * c] = fmaf(pp[i], ov.x, gv[i][4 * c]); gv[i][4 * c + 1] = fmaf(pp[i], ov.y, gv[i][4 * c + 1]);
             gv[i][4 * c + 2] = fmaf(pp[i], ov.z, gv[i][4 * c + 2]); gv[i][4 * c + 3] = fmaf(pp[i], ov.w, gv[i][4 * c + 3]);
             gk[i][4 * c] = fmaf(ss[i], qv.x, gk[i][4 * c]); gk[i][4 * c + 1] = fmaf(ss[i], qv.y, gk[i][4 * c + 1]);
@@ -353,7 +367,7 @@ sh_f32_attn_bw_kernel(const float* __restrict__ Q, const float* __restrict__ K, 
         }
       }
       // dQ: rows r0 + ty + 8 i
-      for (int r0 = 0; r0 < TQ; r0 += 32) {
+      for (int r0 = rlo; r0 < TQ; r0 += 32) {
         float gq[4][4 * NC];
 #pragma unroll
         for (int i = 0; i < 4; ++i)
@@ -371,6 +385,7 @@ sh_f32_attn_bw_kernel(const float* __restrict__ Q, const float* __restrict__ K, 
               const float4 kv = *reinterpret_cast<const float4*>(sK + (kk + u) * LD + 4 * tx + 64 * c);
 #pragma unroll
               for (int i = 0; i < 4; ++i) {
+                if (PART && k0 + kk + u > q0 + r0 + ty + 8 * i) continue;
                 const float w = u == 0 ? sv[i].x : u == 1 ? sv[i].y : u == 2 ? sv[i].z : sv[i].w;
                 gq[i][4 * c] = fmaf(w, kv.x, gq[i][4 * c]); gq[i][4 * c + 1] = fmaf(w, kv.y, gq[i][4 * c + 1]);
                 gq[i][4 * c + 2] = fmaf(w, kv.z, gq[i][4 * c + 2]); gq[i][4 * c + 3] = fmaf(w, kv.w, gq[i][4 * c + 3]);
@@ -389,6 +404,10 @@ sh_f32_attn_bw_kernel(const float* __restrict__ Q, const float* __restrict__ K, 
               red_add_v4_f32(dst + 64 * c, gq[i][4 * c] * inv_sqrt_d, gq[i][4 * c + 1] * inv_sqrt_d, gq[i][4 * c + 2] * inv_sqrt_d, gq[i][4 * c + 3] * inv_sqrt_d);
         }
       }
+    };
+    if (col_ok) {
+      if (d.causal && k0 + 31 > q0) products(fa_bool<true>());
+      else products(fa_bool<false>());
     }
     group_sync(1 + grp, 128);                              // the tile's buffers are free
   }

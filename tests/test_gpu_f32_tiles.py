@@ -138,3 +138,27 @@ def test_f32_gate_kernel_sums_as_the_allocation_free_one(M, H, E, k, blocks):
     for a, b in zip(got, want):
         assert torch.equal(a, b)
     layer.close()
+
+
+@pytest.mark.parametrize("D", [32, 64, 128, 200])
+def test_f32_overflow_of_one_token_stays_behind_the_mask(D):
+    # finite inputs, but token 40's value row overflows (first column of x times that row of W_V): earlier rows of the
+    # output never see it; then token 40's dAhat overflows: later rows of dx never see that
+    B, T, M, H, E, k, t0 = 1, 100, 128, 2, 4, 2, 40
+    inp = inputs.make_inputs(inputs.LayerConfig("tiles", inputs.DTYPE_F32, B, T, M, H, D, E, k, seed=31 + D))
+    for W in (inp.Wq, inp.Wk, inp.Ws, inp.Wd):
+        W[:, 0] = 0.0
+    inp.Wv[:, :, 0] = 10.0
+    inp.Wo[:, :, :, 0] = 10.0
+    layer = binding.layer_from_inputs(inp)
+    x = binding.to_device(inp.x, inp.cfg.dtype)
+    G = torch.ones(B, T, M, device="cuda")
+    close = lambda a, b: float((a - b).abs().max() / b.abs().max()) < TOL
+    want_y, want_dx = layer.sh_forward(x), layer.sh_backward(x, G)["dx"]
+    G[0, t0, 0] = 1e38
+    dx = layer.sh_backward(x, G)["dx"]
+    assert close(dx[:, t0 + 1:], want_dx[:, t0 + 1:]) and not bool(torch.isfinite(dx[:, :t0 + 1]).all())
+    x[0, t0, 0] = 1e38
+    y = layer.sh_forward(x)
+    assert close(y[:, :t0], want_y[:, :t0]) and not bool(torch.isfinite(y[:, t0:]).all())
+    layer.close()
