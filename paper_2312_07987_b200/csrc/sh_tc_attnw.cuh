@@ -2,10 +2,12 @@
 //
 // The 512 tensor-memory columns hold O (up to 256), two S buffers of 64 keys and two P buffers, so one
 // query tile per CTA is all that fits; keys go in steps of 64 (K and V stages of 64 rows, two each,
-// beside the query tile: up to 192 KB).  The probabilities keep 22 bits: P = P_hi + P_lo, two fp16 values,
+// beside the query tile: up to 192 KB).  Probabilities are P_hi + P_lo, two fp16 values,
 // each multiplied with V (two UMMAs per 16 keys) - such a layer's probabilities were fp32 on the CUDA
 // cores before, and the second product costs nothing here: the softmax of a step, not the tensor pipe,
-// bounds the loop.  Measured at 16 x 512 tokens, 2 heads of 132: 18 us (one warp per query row on the CUDA
+// bounds the loop.  They are scaled by 2^7 (the sum they are divided by is as well): with the row maximum
+// behind by up to 2^8 that fills fp16's range, 22 bits for probabilities of 2^-9 of the largest and more, and
+// an error of at most 2^-32 of the largest below (unscaled: 2^-25).  Measured at 16 x 512 tokens, 2 heads of 132: 18 us (one warp per query row on the CUDA
 // cores: 4490); its floor is the softmax, one exponential per visible (query, key).
 //
 // S of step j + 1 is issued before the product of step j, so it runs under the softmax of step j.  Its
@@ -152,11 +154,12 @@ sh_tc_attention_wide_kernel(const __grid_constant__ CUtensorMap mapQ, const __gr
       float alpha = 1.f;
       bool raise = false;
       if (mx > m + 8.f) { alpha = fast_exp2(m - mx); m = mx; raise = j > 0; }
+      const float mp = m - 7.f;                              // (the probabilities' scale of 2^7)
       float sum4[4] = {0.f, 0.f, 0.f, 0.f};
       uint32_t hi[32], lo[32];
 #pragma unroll
       for (int c = 0; c < 32; ++c) {
-        const float p0 = fast_exp2(__uint_as_float(sv[2 * c]) - m), p1 = fast_exp2(__uint_as_float(sv[2 * c + 1]) - m);
+        const float p0 = fast_exp2(__uint_as_float(sv[2 * c]) - mp), p1 = fast_exp2(__uint_as_float(sv[2 * c + 1]) - mp);
         sum4[c & 3] += p0 + p1;
         const __half2 h = __floats2half2_rn(p0, p1);
         const float2 hf = __half22float2(h);

@@ -67,3 +67,34 @@ def test_selection_of_an_input_off_its_alignment():
     pu.check_selection(idx, gate, ref, 70, 2e-5)
     pu.check_lists(off, lists, ref)
     layer.close()
+
+
+def test_small_probabilities_keep_their_bits():
+    # token 0 takes all but 2^-24 of the attention and has no value; what a row reads is the sum over the others.  Two fp16
+    # parts of 2^7 p leave each of them an error of 2^-25 against 2^-17, 2^-8, which averages out over 100 keys and more;
+    # fp16 queries, keys and values add 2^-11 each
+    T, M, D = 256, 128, 132
+    g = torch.Generator(device="cuda").manual_seed(4)
+    x = torch.zeros(T, M, device="cuda")
+    x[1:, 0] = 1.0
+    x[0, 1] = 1.0
+    x[1:, 2:] = torch.randn(T - 1, M - 2, generator=g, device="cuda")
+    Wq, Wk = torch.zeros(1, M, D, device="cuda"), torch.zeros(1, M, D, device="cuda")
+    Wq[0, 0, 0] = 13.8
+    Wk[0, 1, 0] = 13.8
+    Wk[0, 2:, 0] = 0.05 * torch.randn(M - 2, generator=g, device="cuda")
+    Wv = torch.zeros(1, 1, M, D, device="cuda")
+    Wv[0, 0, 2:] = 4096 * torch.randn(M - 2, D, generator=g, device="cuda") / M ** 0.5     # (the sums are normal fp16 numbers)
+    Wo, Ws = torch.zeros(1, 1, D, M, device="cuda"), torch.zeros(1, M, 1, device="cuda")
+    x, Wq, Wk, Wv, Wo, Ws = (a.bfloat16() for a in (x, Wq, Wk, Wv, Wo, Ws))
+    layer = binding.Layer(M, 1, D, 1, 1)
+    layer.sh_configure(binding.SH_BF16, 1, T)
+    layer.sh_set_weights(Wq, Wk, Wv, Wo, Ws, Ws)
+    layer.sh_forward(x.view(1, T, M))
+    got = layer.sh_debug_buffer("AHAT")[100:, 0].double()
+    x, Wq, Wk, Wv = x.double(), Wq[0].double(), Wk[0].double(), Wv[0, 0].double()
+    s = (x @ Wq) @ (x @ Wk).T / D ** 0.5
+    p = torch.softmax(s.masked_fill(torch.ones(T, T, device="cuda").triu(1).bool(), -torch.inf), dim=1)
+    want = (p @ (0.5 * x @ Wv))[100:]
+    assert float((got - want).norm() / want.norm()) < 4e-3
+    layer.close()
