@@ -827,6 +827,7 @@ static int tc_forward_rest(sh_layer* L, const void* x, void* out, cudaStream_t s
     const bool halves = d.T <= 1024;
     if (d.D > 128) {
       const unsigned wgrid = (unsigned)((d.T + 127) / 128 * d.B * d.H);
+      a.q = (const __half*)(ws + L->o.q); a.k = (const __half*)(ws + L->o.k); a.v = (const __half*)(ws + L->o.v);
       if ((rc = set_smem(sh_tc_attention_wide_kernel, AttnWSmem::TOTAL))) return rc;
       if ((rc = launch_k(pdl, sh_tc_attention_wide_kernel, dim3(wgrid), dim3(192), AttnWSmem::TOTAL, st, S->map_q, S->map_k, S->map_v, a))) return rc;
     } else if (d.D == 128) {

@@ -27,6 +27,7 @@ struct TcAttnArgs {
   __half* ahat;          // [B*T, H, D]
   int* status;
   int balanced;          // pair query tile p with tile ntile-1-p (causal mask, grid fits the GPU in one wave)
+  const __half *q, *k, *v;   // [B, H, T, D]: the wide kernel's rows once more (attnw_row)
   const __half* bias;    // [B, H, T - Tc, T] added to the scores (Transformer-XL position and content-bias terms, log2 units), or nullptr
 };
 

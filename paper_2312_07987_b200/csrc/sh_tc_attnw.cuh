@@ -29,6 +29,29 @@ struct AttnWSmem {
   static constexpr int TOTAL = BAR_OFF + 256 + 1024;
 };
 
+// One row of Ahat by plain sums over the keys it sees.  The tensor pipe multiplies the masked probabilities of a step,
+// zeros, with value rows the query does not see; one of them past fp16's range makes the product NaN.  Rows
+// whose result is not finite although their scores are come here.
+static __device__ __noinline__ void attnw_row(const ShDims& d, const __half* q, const __half* k, const __half* v, int last, __half* dst) {
+  float o[256];
+  for (int c = 0; c < d.Dt; ++c) o[c] = 0.f;
+  float m = -INFINITY, l = 0.f;
+  for (int j = 0; j <= last; ++j) {
+    const __half *kr = k + (size_t)j * d.D, *vr = v + (size_t)j * d.D;
+    float s = 0.f;
+    for (int c = 0; c < d.Dt; ++c) s = fmaf(__half2float(q[c]), __half2float(kr[c]), s);
+    if (s > m) {
+      const float alpha = exp2f(m - s);
+      for (int c = 0; c < d.Dt; ++c) o[c] *= alpha;
+      l *= alpha; m = s;
+    }
+    const float p = exp2f(s - m);
+    l += p;
+    for (int c = 0; c < d.Dt; ++c) o[c] = fmaf(p, __half2float(vr[c]), o[c]);
+  }
+  for (int c = 0; c < d.Dt; ++c) dst[c] = __float2half_rn(o[c] / l);
+}
+
 static __global__ void __launch_bounds__(192, 1)
 sh_tc_attention_wide_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapK,
                             const __grid_constant__ CUtensorMap mapV, TcAttnArgs g) {
@@ -193,11 +216,15 @@ sh_tc_attention_wide_kernel(const __grid_constant__ CUtensorMap mapQ, const __gr
       const float inv = 1.f / l;
       const int bb = bh / d.H, hh = bh % d.H;
       __half* dst = g.ahat + (((size_t)bb * d.T + tq) * d.H + hh) * d.D;
+      float sum = 0.f;                                       // (not finite if a value of the row is not)
       for (int c = 0; c < db * 2; ++c) {                     // (up to the 64-column block the output projection loads: zeros behind d_head)
         uint32_t ov[32];
         tmem_ld32(tmem + lane_off + c * 32, ov);
         tmem_ld_wait();
         if (tq < d.T) {
+#pragma unroll
+          for (int i = 0; i < 32; ++i)
+            if (c * 32 + i < d.Dt) sum = fmaf(__uint_as_float(ov[i]), 0.f, sum);
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
             uint32_t w[4];
@@ -211,6 +238,10 @@ sh_tc_attention_wide_kernel(const __grid_constant__ CUtensorMap mapQ, const __gr
             *reinterpret_cast<uint4*>(dst + c * 32 + 8 * i) = make_uint4(w[0], w[1], w[2], w[3]);
           }
         }
+      }
+      if (tq < d.T && sum != sum && l < INFINITY) {          // (l: the scores' part, not NaN either)
+        const size_t row0 = (size_t)bh * d.T;
+        attnw_row(d, g.q + (row0 + tq) * d.D, g.k + row0 * d.D, g.v + row0 * d.D, d.causal ? tq : d.T - 1, dst);
       }
     }
   }

@@ -98,3 +98,22 @@ def test_small_probabilities_keep_their_bits():
     want = (p @ (0.5 * x @ Wv))[100:]
     assert float((got - want).norm() / want.norm()) < 4e-3
     layer.close()
+
+
+def test_overflow_of_one_token_stays_behind_the_mask():
+    # finite inputs, but token 70's value row passes fp16's range (first column of x times that row of W_V)
+    cfg = config(1, 200, 128, 2, 132, 4, 2)
+    inp = inputs.make_inputs(cfg)
+    for W in (inp.Wq, inp.Wk, inp.Ws, inp.Wd):
+        W[:, 0] = 0.0
+    inp.Wv[:, :, 0] = 128.0
+    inp.x[0, :, 0] = 0.0
+    layer = binding.layer_from_inputs(inp)
+    x = binding.to_device(inp.x, cfg.dtype)
+    want = layer.sh_forward(x)
+    x[0, 70, 0] = 8192.0
+    y = layer.sh_forward(x)
+    # (the rows of that token's tile are summed once more in another order: an fp16 unit, 2^-10, in what they read)
+    assert pu.rel_rms_err(y[:, :70].cpu().numpy(), want[:, :70].cpu().numpy()) < 1e-2 and not bool(torch.isfinite(y[:, 70:]).all())
+    assert layer.sh_last_status() == 0
+    layer.close()
