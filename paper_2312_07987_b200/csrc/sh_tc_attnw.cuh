@@ -216,7 +216,7 @@ sh_tc_attention_wide_kernel(const __grid_constant__ CUtensorMap mapQ, const __gr
       const float inv = 1.f / l;
       const int bb = bh / d.H, hh = bh % d.H;
       __half* dst = g.ahat + (((size_t)bb * d.T + tq) * d.H + hh) * d.D;
-      float sum = 0.f;                                       // (not finite if a value of the row is not)
+      float nan4[4] = {0.f, 0.f, 0.f, 0.f};                  // (NaN once a value of the row is not finite)
       for (int c = 0; c < db * 2; ++c) {                     // (up to the 64-column block the output projection loads: zeros behind d_head)
         uint32_t ov[32];
         tmem_ld32(tmem + lane_off + c * 32, ov);
@@ -224,7 +224,7 @@ sh_tc_attention_wide_kernel(const __grid_constant__ CUtensorMap mapQ, const __gr
         if (tq < d.T) {
 #pragma unroll
           for (int i = 0; i < 32; ++i)
-            if (c * 32 + i < d.Dt) sum = fmaf(__uint_as_float(ov[i]), 0.f, sum);
+            if (2 * c + (i >> 4) < kd) nan4[i & 3] = fmaf(__uint_as_float(ov[i]), 0.f, nan4[i & 3]);   // (the slices that were multiplied)
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
             uint32_t w[4];
@@ -239,7 +239,8 @@ sh_tc_attention_wide_kernel(const __grid_constant__ CUtensorMap mapQ, const __gr
           }
         }
       }
-      if (tq < d.T && sum != sum && l < INFINITY) {          // (l: the scores' part, not NaN either)
+      const float nan = (nan4[0] + nan4[1]) + (nan4[2] + nan4[3]);
+      if (tq < d.T && nan != nan && l < INFINITY) {          // (l: the scores' part, not NaN either)
         const size_t row0 = (size_t)bh * d.T;
         attnw_row(d, g.q + (row0 + tq) * d.D, g.k + row0 * d.D, g.v + row0 * d.D, d.causal ? tq : d.T - 1, dst);
       }
