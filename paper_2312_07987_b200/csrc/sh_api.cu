@@ -100,6 +100,7 @@ static void layout_workspace(sh_layer* L) {
   o.bw = take(f32 ? ((size_t)4 * d.N * HD + (size_t)2 * d.N * d.H * d.k + (size_t)d.N * (sh_f32_ldz(d) + d.H)) * 4 : 16);
   o.wgate32 = take(f32 ? (size_t)d.G * d.M * 4 : 16);
   o.f32stats = take(f32 ? (size_t)d.N * d.H * 8 : 16);
+  o.wo_overflow = take(16);                                  // d_head above 128, bf16 storage: a stored weight of W_O is not finite
   o.stamps = take(sizeof(ShStampBlock));
   o.total = off;
 }
@@ -235,10 +236,10 @@ extern "C" int sh_set_workspace(sh_layer* L, void* workspace, size_t bytes) {
 
 template <typename TI, typename TO, int PLANES = 1>
 static void repack(const void* in, void* out, int batch, int rows, int cols, long obs, long ors, long oes,
-                   cudaStream_t st, long plane = 0) {
+                   cudaStream_t st, long plane = 0, int* overflow = nullptr) {
   const unsigned gy = (unsigned)((rows + 31) / 32), gz = (unsigned)batch;
   dim3 grid((unsigned)((cols + 31) / 32), gy < 65535 ? gy : 65535, gz < 65535 ? gz : 65535);
-  sh_repack_kernel<TI, TO, PLANES><<<grid, 256, 0, st>>>((const TI*)in, (TO*)out, batch, rows, cols, obs, ors, oes, plane);
+  sh_repack_kernel<TI, TO, PLANES><<<grid, 256, 0, st>>>((const TI*)in, (TO*)out, batch, rows, cols, obs, ors, oes, plane, overflow);
 }
 
 template <typename TI, typename TM>
@@ -290,7 +291,8 @@ static int set_weights_t(sh_layer* L, const void* Wq, const void* Wk, const void
     }
     // Wv [H, E, M, D] -> [H, E, D, M];  Wo [H, E, D, M] -> [H, E, M, D]
     repack<TI, TI>(Wv, ws + L->o.wv, d.H * d.E, d.M, d.Dt, (long)d.D * d.M, d.M, 1, st);
-    repack<TI, TM>(Wo, ws + L->o.wo, d.H * d.E, d.Dt, d.M, (long)d.D * d.M, d.D, 1, st);
+    SH_CUDA_CHECK(cudaMemsetAsync(ws + L->o.wo_overflow, 0, 16, st));
+    repack<TI, TM>(Wo, ws + L->o.wo, d.H * d.E, d.Dt, d.M, (long)d.D * d.M, d.D, 1, st, 0, (int*)(ws + L->o.wo_overflow));
     if (sh_o_sparse_ok(L)) {
       // Wo [H, E, D, M] -> [H, M, D*E]: element (h, e, dd, m) at (h*M + m)*(D*E) + dd*E + e
       if (d.D != d.Dt) SH_CUDA_CHECK(cudaMemsetAsync(ws + L->o.wos, 0, (size_t)HD * d.E * d.M * sizeof(TM), st));

@@ -7,13 +7,13 @@
 // ---------------------------------------------------------------------------------------
 // Weight repack: out[b*obs + c*ors + r*oes] = in[b*rows*cols + r*cols + c]  (a batched transpose with free
 // output strides), with type conversion; PLANES = 3: into three bf16 planes, `plane` elements apart, whose
-// sum is the fp32 value (fp32 configuration).  32 x 32 tiles through shared memory, so that reads run along
-// c and writes along r (a thread per element in output order read a column of `in` at a time, a 32-byte
-// sector for every value).
+// sum is the fp32 value (fp32 configuration).  `overflow`, where given, is set if a stored value is not finite.
+// 32 x 32 tiles through shared memory, so that reads run along c and writes along r (a thread per element in
+// output order read a column of `in` at a time, a 32-byte sector for every value).
 // ---------------------------------------------------------------------------------------
 template <typename TI, typename TO, int PLANES = 1>
 __global__ void __launch_bounds__(256)
-sh_repack_kernel(const TI* __restrict__ in, TO* __restrict__ out, int batch, int rows, int cols, long obs, long ors, long oes, long plane) {
+sh_repack_kernel(const TI* __restrict__ in, TO* __restrict__ out, int batch, int rows, int cols, long obs, long ors, long oes, long plane, int* overflow) {
   __shared__ float tile[32][33];
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   const int c0 = blockIdx.x * 32;
@@ -35,6 +35,7 @@ sh_repack_kernel(const TI* __restrict__ in, TO* __restrict__ out, int batch, int
           // (the leading one of three saturates: see split_bf16x3)
           const TO w = sh_from_float<TO>(PLANES == 3 && p == 0 ? fminf(fmaxf(v, -3.3895313892515355e38f), 3.3895313892515355e38f) : v);
           o[p * plane] = w;
+          if (PLANES == 1 && overflow && !(fabsf(sh_to_float<TO>(w)) < INFINITY)) *overflow = 1;
           v -= sh_to_float<TO>(w);
         }
       }

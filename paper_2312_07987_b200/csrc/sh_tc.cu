@@ -914,6 +914,7 @@ static int tc_forward_rest(sh_layer* L, const void* x, void* out, cudaStream_t s
         }
         if (as < 2) { sh_set_error("output projection: n_heads*k = %d does not fit in shared memory", d.H * d.k); return SH_ERR_UNSUPPORTED; }
         a.a_slots = as; a.tail = S->o_tail;
+        a.ahat = (const __half*)(ws + L->o.ahat); a.wo = (const __half*)(ws + L->o.wo); a.wo_overflow = (const int*)(ws + L->o.wo_overflow);
         if (int r = set_smem(kern, smem)) return r;
         return launch_k(pdl, kern, dim3(grid), dim3(320), smem, st, S->map_ahat, S->map_wo256, S->map_ahat_tail, S->map_wo_tail, a);
       };

@@ -41,6 +41,8 @@ struct TcOprojArgs {
   int a_slots;           // 32 KB weight stages in the ring: 3 or 2
   int tail;              // single-CTA kernel: columns loaded of d_head's last 64-column block (64, 32 or 16)
   int sel_global;        // single-CTA kernel: selections read from global memory (their copy does not fit shared memory)
+  const __half *ahat, *wo;   // single-CTA kernel, d_head above 128: Ahat [N, H, D] and W_O [H, E, M, D] once more (oproj_element)
+  const int* wo_overflow;    // ... and whether a weight of W_O passed fp16's range when it was stored
   int nwork;             // nblk * ceil(M / 256)
   int* status;
 };
@@ -62,13 +64,31 @@ __device__ __forceinline__ void oproj_put4(float* out, size_t elem, float4 v, in
 template <int DB, int NB>
 struct OprojSmem {
   static constexpr int A_BYTES = 256 * 64 * 2;           // one weight stage: 256 features x 64 columns
-  static constexpr int B_BYTES = 128 * DB * 64 * 2;      // Ahat tile: 128 tokens x 64 DB
   static constexpr int STAGING = 8 * 32 * 32 * 4;        // per epilogue warp a 32 x 32 fp32 transpose tile
   __host__ __device__ static int b_bytes(int tail) { return (DB - 1) * 128 * 128 + 128 * tail * 2; }   // tail: columns loaded of the last block
   static int total(int a_slots, int H, int k, int tail) {
     return a_slots * A_BYTES + NB * b_bytes(tail) + STAGING + 128 * H * k * 8 + 512 + 1024;
   }
 };
+
+// One result by plain sums over the token's selected experts.  The kernel multiplies a token with every expert and the
+// results of those it did not select by zero; a weight of theirs past fp16's range makes the sum NaN.  (Where there is
+// one, the results that are not finite are put right behind the last unit: a check in the unit's own store cost 3 %.)
+static __device__ __forceinline__ float oproj_element(const TcOprojArgs& g, int tokn, int f) {
+  const ShDims& d = g.d;
+  float y = 0.f;
+  for (int h = 0; h < d.H; ++h)
+    for (int j = 0; j < d.k; ++j) {
+      const size_t sel = ((size_t)tokn * d.H + h) * d.k + j;
+      const int e = g.idx[sel];
+      if (!SH_INDEX_OK(e, d.E, g.status, SH_SITE_O_EXPERT)) continue;
+      const __half *a = g.ahat + ((size_t)tokn * d.H + h) * d.D, *w = g.wo + ((size_t)(h * d.E + e) * d.M + f) * d.D;
+      float v = 0.f;
+      for (int c = 0; c < d.Dt; ++c) v = fmaf(__half2float(a[c]), __half2float(w[c]), v);
+      y = fmaf(g.gate[sel], v, y);
+    }
+  return y;
+}
 
 template <int DB, int NB>
 __global__ void __launch_bounds__(320, 1)
@@ -271,6 +291,17 @@ sh_tc_oproj_kernel(const __grid_constant__ CUtensorMap mapAhat, const __grid_con
             if (r < rows_here)
               oproj_put4(g.out, obase + (size_t)r * d.M + c * 32 + 4 * ch, *reinterpret_cast<const float4*>(stg + r * 32 + ((ch ^ (r & 7)) << 2)), g.out_f16);
           }
+        }
+      }
+    }
+    if (DB > 2 && ok && *g.wo_overflow) {
+      __syncwarp();                                          // (a row was stored by other lanes of its warp)
+      for (int w = blockIdx.x; w < g.nwork; w += gridDim.x) {
+        const int row = (w / nfc) * 128 + tok, col0 = (w % nfc) * 256 + half * 128;
+        if (row >= sh_out_rows(d)) continue;
+        for (int f = col0; f < min(col0 + 128, d.M); ++f) {
+          float* o = g.out + (size_t)row * d.M + f;
+          if (!(fabsf(*o) < INFINITY)) *o = oproj_element(g, sh_ctx_tok(d, row), f);
         }
       }
     }

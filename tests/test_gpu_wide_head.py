@@ -117,3 +117,22 @@ def test_overflow_of_one_token_stays_behind_the_mask():
     assert pu.rel_rms_err(y[:, :70].cpu().numpy(), want[:, :70].cpu().numpy()) < 1e-2 and not bool(torch.isfinite(y[:, 70:]).all())
     assert layer.sh_last_status() == 0
     layer.close()
+
+
+def test_overflowing_weight_reaches_the_tokens_that_selected_its_expert():
+    # 1e5 is a finite bf16 weight, but past fp16's range: feature 3 of head 1's output expert 2
+    cfg = config(1, 150, 256, 2, 168, 4, 2)
+    inp = inputs.make_inputs(cfg)
+    layer = binding.layer_from_inputs(inp)
+    x = binding.to_device(inp.x, cfg.dtype)
+    want = layer.sh_forward(x)
+    hit = (layer.sh_gate_topk(x)[0][1, :, 1] == 2).any(dim=1)
+    assert 0 < int(hit.sum()) < 150
+    inp.Wo[1, 2, 0, 3] = 1e5
+    layer.sh_set_weights(*[binding.to_device(a, cfg.dtype) for a in (inp.Wq, inp.Wk, inp.Wv, inp.Wo, inp.Ws, inp.Wd)])
+    y = layer.sh_forward(x)
+    assert pu.rel_rms_err(y[:, ~hit].cpu().numpy(), want[:, ~hit].cpu().numpy()) < 1e-5      # (two fp32 orders)
+    assert not bool(torch.isfinite(y[0, hit, 3]).any())
+    keep = torch.arange(256, device="cuda") != 3
+    assert torch.equal(y[..., keep], want[..., keep])
+    layer.close()
