@@ -233,8 +233,8 @@ int sh_gate_topk(sh_layer* layer, const void* x, int32_t* idx, float* gate, int3
 /* (No counterpart in the paper: an addition for callers that cannot allocate device memory.)
  * Some callers run where cudaMalloc is not an option - inside a memory pool they do not own,
  * in a process whose allocations are fixed at start-up, or simply without a workspace to
- * hand over.  This entry point runs the gate + top-k + bucket-sort stage (the same kernels
- * as sh_gate_topk on the CUDA cores) without a layer handle and without any allocation:
+ * hand over.  This entry point runs the gate + top-k + bucket-sort stage (on the CUDA cores; bit
+ * for bit what sh_gate_topk gives for an fp32 layer, and for bf16 storage with d_head above 128) without a layer handle and without any allocation:
  * its scratch memory - the per-block selection histograms, the gate values in list order
  * and the row-tile table the sort kernel emits - lives in fixed arrays inside the library
  * (about 2.3 MB on every GPU that loads it, held until the process exits).  It calls no

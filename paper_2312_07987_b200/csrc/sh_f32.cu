@@ -229,6 +229,20 @@ void sh_f32_release(sh_layer* L) {
 
 int sh_f32_gate_sort(sh_layer* L, const void* x, cudaStream_t st) { return launch_gate_sort(L, x, nullptr, 0, st); }
 
+static size_t bf16_gate_smem(const ShDims& d) { return (size_t)(GB_TOK * (GB_XLD + d.G) + GB_NC * GB_WLD) * 4; }
+bool sh_bf16_gate_ok(const sh_layer* L) { return bf16_gate_smem(L->d) <= 227 * 1024; }
+
+int sh_bf16_gate(sh_layer* L, const void* x, int* blockcnt, bool pdl, cudaStream_t st) {
+  const ShDims& d = L->d;
+  char* ws = L->ws;
+  const size_t smem = bf16_gate_smem(d);
+  const int passes = (d.N + GB_TOK - 1) / GB_TOK, most = 2 * sm_count(L);    // (a block keeps its weights for all of its passes)
+  if (int rc = set_smem(sh_bf16_gate_kernel, (int)smem)) return rc;
+  L->launches += 1;
+  return launch_k(pdl, sh_bf16_gate_kernel, dim3((unsigned)(passes < most ? passes : most)), dim3(GB_THREADS), smem, st, (const __nv_bfloat16*)x,
+                  (const __nv_bfloat16*)(ws + L->o.wgate), (const float*)(ws + L->o.gbias), (int*)(ws + L->o.idx), (float*)(ws + L->o.gate), blockcnt, d, (int)((uintptr_t)x % 16 == 0));
+}
+
 int sh_f32_forward(sh_layer* L, const void* x, void* out, cudaStream_t st) {
   const ShDims& d = L->d;
   const F32State* S = (const F32State*)L->f32;

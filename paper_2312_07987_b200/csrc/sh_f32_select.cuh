@@ -1,6 +1,49 @@
-// Gates, selection and bucket sort of the fp32 configuration.
+// Gates, selection and bucket sort of the fp32 configuration; sh_gate_topk's gates of bf16 storage with d_head above 128.
 #pragma once
 #include "sh_internal.cuh"
+
+// Lane sums of TOK tokens (8 or 16): at each step a lane keeps half of its tokens and hands the others over; then lane
+// l holds token *tok, the same as a butterfly (xor 16, 8, ... 1) over each of them.
+template <int TOK>
+__device__ __forceinline__ float sh_lane_sums(float (&acc)[TOK], int lane, int* tok) {
+  int t = 0;
+#pragma unroll
+  for (int n = TOK / 2, o = 16; n >= 1; n >>= 1, o >>= 1) {
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int r = 0; r < n; ++r) {
+      const float give = up ? acc[r] : acc[r + n], keep = up ? acc[r + n] : acc[r];
+      acc[r] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+    }
+    t += up ? n : 0;
+  }
+#pragma unroll
+  for (int o = 32 / TOK / 2; o > 0; o >>= 1) acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], o);
+  *tok = t;
+  return acc[0];
+}
+
+// Bias, top-k and sigmoid of one (token, side, head) from its E logits in shared memory.  blockcnt, where given
+// (cleared before): how often each expert is selected, per 128 tokens.
+__device__ __forceinline__ void sh_select(float* z, const float* __restrict__ gbias, int* __restrict__ idx, float* __restrict__ gate,
+                                          int* __restrict__ blockcnt, const ShDims& d, int t, int grp) {
+  const int side = grp / d.H, h = grp % d.H;
+  for (int e = 0; e < d.E; ++e) z[e] += gbias[grp * d.E + e];
+  const size_t o = (((size_t)side * d.N + t) * d.H + h) * d.k;
+  unsigned sel = 0;
+  for (int j = 0; j < d.k; ++j) {
+    float best = 0.f;
+    int pick = -1;
+    for (int e = 0; e < d.E; ++e) {
+      const float v = z[e];
+      if (!((sel >> e) & 1u) && (pick < 0 || v > best)) { best = v; pick = e; }
+    }
+    sel |= 1u << pick;
+    idx[o + j] = pick;
+    gate[o + j] = 1.f / (1.f + expf(-best));
+    if (blockcnt) atomicAdd(blockcnt + (size_t)(t / SH_TILE_ROWS) * d.G + grp * d.E + pick, 1);
+  }
+}
 
 // Logits, top-k (a larger logit first, the lower index on a tie) and sigmoid of the chosen ones, on the
 // CUDA cores: TOK tokens per block with their rows in shared memory (CH columns at a time: 512, or 1024 where d_model is larger), a warp per
@@ -68,23 +111,11 @@ sh_f32_gate_kernel(const float* __restrict__ x, const float* __restrict__ wgate,
       }
     }
     if (one) {
-      // lane sums of TOK tokens: at each step a lane keeps half of its tokens and hands the others over
 #pragma unroll
       for (int q = 0; q < 2; ++q) {
-        int tokn = 0;
-#pragma unroll
-        for (int n = TOK / 2, o = 16; n >= 1; n >>= 1, o >>= 1) {
-          const bool up = (lane & o) != 0;
-#pragma unroll
-          for (int r = 0; r < n; ++r) {
-            const float give = up ? acc[q][r] : acc[q][r + n], keep = up ? acc[q][r + n] : acc[q][r];
-            acc[q][r] = keep + __shfl_xor_sync(0xffffffffu, give, o);
-          }
-          tokn += up ? n : 0;
-        }
-#pragma unroll
-        for (int o = 32 / TOK / 2; o > 0; o >>= 1) acc[q][0] += __shfl_xor_sync(0xffffffffu, acc[q][0], o);
-        if (lane % (32 / TOK) == 0 && (q == 0 || two)) s_z[tokn * d.G + g + 16 * q] = acc[q][0];
+        int tokn;
+        const float z = sh_lane_sums<TOK>(acc[q], lane, &tokn);
+        if (lane % (32 / TOK) == 0 && (q == 0 || two)) s_z[tokn * d.G + g + 16 * q] = z;
       }
     }
   }
@@ -92,22 +123,108 @@ sh_f32_gate_kernel(const float* __restrict__ x, const float* __restrict__ wgate,
   __syncthreads();
   const int groups = d.sides * d.H;
   for (int i = tid; i < TOK * groups; i += 512) {
-    const int r = i / groups, grp = i % groups, side = grp / d.H, h = grp % d.H, t = t0 + r;
-    if (t >= d.N) continue;
-    float* z = s_z + r * d.G + grp * d.E;
-    for (int e = 0; e < d.E; ++e) z[e] += gbias[grp * d.E + e];
-    const size_t o = (((size_t)side * d.N + t) * d.H + h) * d.k;
-    unsigned sel = 0;
-    for (int j = 0; j < d.k; ++j) {
-      float best = 0.f;
-      int pick = -1;
-      for (int e = 0; e < d.E; ++e) {
-        const float v = z[e];
-        if (!((sel >> e) & 1u) && (pick < 0 || v > best)) { best = v; pick = e; }
+    const int r = i / groups, grp = i % groups;
+    if (t0 + r < d.N) sh_select(s_z + r * d.G + grp * d.E, gbias, idx, gate, nullptr, d, t0 + r, grp);
+  }
+}
+
+// The same sums for bf16 storage (sh_gate_topk with d_head above 128): 16 tokens and 32 gate columns in shared memory, a
+// warp works on 8 x 8 of them.  A word holds two neighbouring columns of a row; half a warp covers 32 columns of
+// one token, lane j the sums of the columns 2 j and 2 j + 1 modulo 32 as one FFMA2 per word.  8192 tokens of 32
+// columns of 1024: 28 us, of which the FMA pipe's share is 7.4 (four warps a scheduler, 58 % of the issue slots).
+constexpr int GB_TOK = 16, GB_NC = 32, GB_CH = 1024, GB_THREADS = 256, GB_XLD = GB_CH / 2 + 16, GB_WLD = GB_CH / 2;
+static __global__ void __launch_bounds__(GB_THREADS, 2)
+sh_bf16_gate_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restrict__ wgate, const float* __restrict__ gbias, int* __restrict__ idx,
+                    float* __restrict__ gate, int* __restrict__ blockcnt, ShDims d, int vec) {
+  extern __shared__ __align__(16) uint32_t gsw[];
+  uint32_t* s_x = gsw;                                     // [GB_TOK][GB_XLD]: two tokens' words fall into different banks
+  uint32_t* s_w = s_x + GB_TOK * GB_XLD;                   // [GB_NC][GB_WLD]
+  float* s_z = reinterpret_cast<float*>(s_w + GB_NC * GB_WLD);   // [GB_TOK][G] logits
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tg = (warp >> 2) * 8, cg = (warp & 3) * 8;     // this warp's tokens and columns
+  const int half = lane >> 4, j = lane & 15;
+  auto copy16 = [](uint32_t* dst, const __nv_bfloat16* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+  };
+  const int passes = (d.N + GB_TOK - 1) / GB_TOK, groups = d.sides * d.H;
+  for (int pass = blockIdx.x; pass < passes; pass += gridDim.x) {
+    const int t0 = pass * GB_TOK;
+    for (int g0 = 0; g0 < d.G; g0 += GB_NC) {
+      float2 acc[8][4];                                    // [column][pair of tokens]
+#pragma unroll
+      for (int q = 0; q < 8; ++q)
+#pragma unroll
+        for (int p = 0; p < 4; ++p) acc[q][p] = make_float2(0.f, 0.f);
+      for (int m0 = 0; m0 < d.M; m0 += GB_CH) {
+        const int mw = min(GB_CH, d.M - m0), n16 = mw / 8; // a multiple of 128; its 16-byte pieces
+        __syncthreads();
+        if (g0 == 0 || d.M > GB_CH)                        // (a row that fits is read once)
+          for (int i = tid; i < GB_TOK * n16; i += GB_THREADS) {
+            const int r = i / n16, c = i % n16;
+            const __nv_bfloat16* p = x + (size_t)min(t0 + r, d.N - 1) * d.M + m0 + c * 8;
+            uint32_t* o = s_x + r * GB_XLD + c * 4;
+            if (vec) copy16(o, p);
+            else
+              for (int u = 0; u < 4; ++u)                  // (x off its alignment: sh_gate_topk takes it)
+                o[u] = (uint32_t)__bfloat16_as_ushort(p[2 * u]) | ((uint32_t)__bfloat16_as_ushort(p[2 * u + 1]) << 16);
+          }
+        if (pass == (int)blockIdx.x || d.G > GB_NC || d.M > GB_CH)
+          for (int i = tid; i < GB_NC * n16; i += GB_THREADS) {
+            const int r = i / n16, c = i % n16;
+            copy16(s_w + r * GB_WLD + c * 4, wgate + (size_t)min(g0 + r, d.G - 1) * d.M + m0 + c * 8);
+          }
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncthreads();
+        if (g0 + cg >= d.G) continue;                      // (whole warps)
+        const uint32_t* px = s_x + (tg + half) * GB_XLD + j;
+        const uint32_t* pw = s_w + cg * GB_WLD + j;
+        // (a sum runs over its columns of the whole row in order: the order of sh_gate_topk_kernel, bit for bit)
+#pragma unroll 2
+        for (int b = 0; b < mw / 2; b += 16) {
+          float2 xv[4], wv[8];
+#pragma unroll
+          for (int p = 0; p < 4; ++p) {
+            const uint32_t v = px[2 * p * GB_XLD + b];
+            xv[p] = make_float2(__uint_as_float(v << 16), __uint_as_float(v & 0xFFFF0000u));
+          }
+#pragma unroll
+          for (int q = 0; q < 8; ++q) {
+            const uint32_t v = pw[q * GB_WLD + b];
+            wv[q] = make_float2(__uint_as_float(v << 16), __uint_as_float(v & 0xFFFF0000u));
+          }
+#pragma unroll
+          for (int q = 0; q < 8; ++q)
+#pragma unroll
+            for (int p = 0; p < 4; ++p) acc[q][p] = __ffma2_rn(xv[p], wv[q], acc[q][p]);
+        }
       }
-      sel |= 1u << pick;
-      idx[o + j] = pick;
-      gate[o + j] = 1.f / (1.f + expf(-best));
+      if (g0 + cg < d.G) {
+        // sums over the 16 lanes: a lane keeps half of the 32 values at each step; value i is column i / 4, pair i % 4
+        float2* v = &acc[0][0];
+        int first = 0;
+#pragma unroll
+        for (int n = 16, o = 8; o >= 1; n >>= 1, o >>= 1) {
+          const bool up = (lane & o) != 0;
+#pragma unroll
+          for (int i = 0; i < n; ++i) {
+            const float2 give = up ? v[i] : v[i + n], keep = up ? v[i + n] : v[i];
+            v[i] = make_float2(keep.x + __shfl_xor_sync(0xffffffffu, give.x, o), keep.y + __shfl_xor_sync(0xffffffffu, give.y, o));
+          }
+          first += up ? n : 0;
+        }
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          const int col = g0 + cg + ((first + i) >> 2), r = tg + 2 * ((first + i) & 3) + half;
+          if (col < d.G) s_z[r * d.G + col] = v[i].x + v[i].y;
+        }
+      }
+    }
+    __syncthreads();
+    for (int i = tid; i < GB_TOK * groups; i += GB_THREADS) {
+      const int r = i / groups, grp = i % groups;
+      if (t0 + r < d.N) sh_select(s_z + r * d.G + grp * d.E, gbias, idx, gate, blockcnt, d, t0 + r, grp);
     }
   }
 }

@@ -197,6 +197,10 @@ int sh_f32_gate_sort(sh_layer* L, const void* x, cudaStream_t st);
 int sh_f32_forward(sh_layer* L, const void* x, void* out, cudaStream_t st);
 int sh_f32_backward(sh_layer* L, const void* x, const float* dout, float* dx, float* dWq, float* dWk, float* dWv,
                     float* dWo, float* dWs, float* dWd, cudaStream_t st);
+// Gate logits and selections on the CUDA cores for bf16 storage (sh_gate_topk with d_head above 128), with the
+// per-block counts the sort wants (cleared by the caller).
+int sh_bf16_gate(sh_layer* L, const void* x, int* blockcnt, bool pdl, cudaStream_t st);
+bool sh_bf16_gate_ok(const sh_layer* L);        // its logits fit shared memory (up to about 2000 gate columns)
 // The CUDA-core attention kernel on fp32 storage (the relative-position term of Transformer-XL).
 int sh_simt_attention_f32(sh_layer* L, cudaStream_t st);
 

@@ -324,9 +324,24 @@ static int tc_gate_sort(sh_layer* L, const void* x, void* out, bool zero_for_for
   const ShDims& d = L->d;
   char* ws = L->ws;
   int rc;
-  if (!S->gate_gp || (S->simt_mask & SH_STAGE_GATE) || (d.D > 128 && (uintptr_t)x % 16 != 0)) {
-    // more than 256 gate columns (or the debug library's switch): the CUDA-core gate kernel; also an x that no
-    // tensor map can describe, which sh_gate_topk has taken for such layers (sh_forward wants x aligned)
+  // The selections themselves, d_head above 128: fp32 FMA chains, bit for bit sh_noalloc_gate_topk's, from an x of any
+  // alignment.  (The tensor core's sums of bf16 products truncate: gate values 2.4e-7 and 3.8e-7 from double precision
+  // at d_model 1024 and 1536 against 4.4e-8.  A forward pass takes them all the same, its result is no further off.)
+  const bool exact = d.D > 128 && !zero_for_forward;
+  if (exact && !(S->simt_mask & SH_STAGE_GATE) && sh_bf16_gate_ok(L)) {
+    const bool pdl = S->pdl && !L->ev;
+    int* blockcnt = (int*)(ws + L->o.blockcnt);
+    SH_CUDA_CHECK(cudaMemsetAsync(blockcnt, 0, (size_t)d.nblk * d.G * 4, st));
+    if ((rc = sh_bf16_gate(L, x, blockcnt, pdl, st))) return rc;
+    const size_t ssm = sh_sort_smem_bytes(d);
+    if ((rc = set_smem(sh_sort_kernel, (int)ssm))) return rc;
+    L->launches += 1;
+    return launch_k(pdl, sh_sort_kernel, dim3(d.nblk), dim3(sh_sort_threads(d)), ssm, st, (const int*)(ws + L->o.idx), (const float*)(ws + L->o.gate),
+                    (const int*)blockcnt, (int*)(ws + L->o.offsets), (int*)(ws + L->o.lists), (float*)(ws + L->o.lgate),
+                    (ShTile*)(ws + L->o.tiles), (int*)(ws + L->o.ntiles), d);
+  }
+  if (!S->gate_gp || exact || (S->simt_mask & SH_STAGE_GATE)) {
+    // more gate columns than those kernels hold (256 here, about 2000 above), or the debug library's switch: a warp per token
     if ((rc = sh_simt_run_bf16(L, SH_STAGE_GATE, x, nullptr, st))) return rc;
     if (zero_for_forward) {
       SH_CUDA_CHECK(cudaMemsetAsync(ws + L->o.v, 0, (size_t)d.N * d.H * d.D * 2, st));

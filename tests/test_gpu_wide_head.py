@@ -136,3 +136,17 @@ def test_overflowing_weight_reaches_the_tokens_that_selected_its_expert():
     keep = torch.arange(256, device="cuda") != 3
     assert torch.equal(y[..., keep], want[..., keep])
     layer.close()
+
+
+@pytest.mark.parametrize("T,M,H,E,k", [(70, 128, 1, 2, 1), (300, 1152, 2, 9, 3), (5000, 1024, 2, 8, 4), (130, 1536, 4, 16, 4)])
+def test_gates_are_the_allocation_free_entry_points_bit_for_bit(T, M, H, E, k):
+    # fp32 FMA chains in both: one and several passes a block, rows in one and two pieces, up to 128 gate columns
+    inp = inputs.make_inputs(config(1, T, M, H, 132, E, k))
+    layer = binding.layer_from_inputs(inp)
+    x = binding.to_device(inp.x, inp.cfg.dtype)
+    wg = torch.from_numpy(np.concatenate([np.transpose(w, (0, 2, 1)).reshape(-1, M) for w in (inp.Ws, inp.Wd)])).to(x).contiguous()
+    layer.sh_forward(x)
+    for a, b in zip(layer.sh_gate_topk(x), binding.sh_noalloc_gate_topk(inp.cfg.dtype, x[0], wg, None, H, E, k)):
+        assert torch.equal(a, b)
+    assert layer.sh_last_status() == 0
+    layer.close()
