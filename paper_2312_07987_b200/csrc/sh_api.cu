@@ -276,7 +276,7 @@ static int set_weights_t(sh_layer* L, const void* Wq, const void* Wk, const void
     // Wv [H, 1, M, D] joins the fused projection; Wo [H, 1, D, M] -> Wo_t[m][h*D + dd]
     repack<TI, TI>(Wv, wqk + 2 * HD * d.M, d.H, d.M, d.Dt, (long)d.D * d.M, d.M, 1, st);
     repack<TI, TM>(Wo, ws + L->o.wo, d.H, d.Dt, d.M, d.D, HD, 1, st);
-  } else {
+  } else if constexpr (sizeof(TI) == 2) {                    // (the fp32 SwitchHead layer: set_weights_f32)
     // Ws, Wd [H, M, E] -> Wgate[(side*H + h)*E + e][m]
     TI* wg = (TI*)(ws + L->o.wgate);
     repack<TI, TI>(Ws, wg, d.H, d.M, d.E, (long)d.E * d.M, d.M, 1, st);
@@ -405,17 +405,22 @@ static int launch_gate_sort(sh_layer* L, const void* x, cudaStream_t st) {
   return SH_OK;
 }
 
+// (fp32: the dense comparator, and attention for the relative-position term - the fp32 SwitchHead layer's weights are
+//  stored as planes, which the other stages here would misread)
 template <typename TI, typename TM>
 static int forward_simt(sh_layer* L, int stages, const void* x, void* out, cudaStream_t st) {
+  constexpr bool F32 = sizeof(TI) == 4;
   const ShDims& d = L->d;
   char* ws = L->ws;
   const int HD = d.H * d.D;
   const float qscale = 1.4426950408889634f / sqrtf((float)d.Dt);
   const bool all = stages == SH_STAGE_ALL;
   if (all) sh_mark(L, 0, st);
-  if (!L->dense && (stages & SH_STAGE_GATE)) {
-    int rc = launch_gate_sort<TI>(L, x, st);
-    if (rc != SH_OK) return rc;
+  if constexpr (!F32) {
+    if (!L->dense && (stages & SH_STAGE_GATE)) {
+      int rc = launch_gate_sort<TI>(L, x, st);
+      if (rc != SH_OK) return rc;
+    }
   }
   if (all) sh_mark(L, 1, st);
   if (stages & SH_STAGE_QK) {
@@ -431,7 +436,7 @@ static int forward_simt(sh_layer* L, int stages, const void* x, void* out, cudaS
       dim3 grid_qk(d.nblk, (g.ncols + 63) / 64);
       sh_simt_gemm_kernel<TI, TI, TM, SH_EPI_QKV><<<grid_qk, 256, 0, st>>>(g);
       L->launches += 1;
-    } else {
+    } else if constexpr (!F32) {
       // query / key experts: whichever of the two is dense is one projection of HD columns; an expert
       // projection is the value experts' grouped GEMM with its own weights, side and output
       g.ncols = HD;
@@ -470,16 +475,18 @@ static int forward_simt(sh_layer* L, int stages, const void* x, void* out, cudaS
     }
   }
   if (all) sh_mark(L, 2, st);
-  if (!L->dense && (stages & SH_STAGE_V)) {
-    SH_CUDA_CHECK(cudaMemsetAsync(ws + L->o.v, 0, (size_t)d.N * HD * sizeof(TM), st));
-    ShGemmArgs v{};
-    v.d = d; v.A = x; v.lda = d.M; v.Bt = ws + L->o.wv; v.ldb = d.M; v.K = d.M; v.ncols = d.D;
-    v.lists = (const int*)(ws + L->o.lists); v.lgate = (const float*)(ws + L->o.lgate);
-    v.tiles = (const ShTile*)(ws + L->o.tiles); v.ntiles = (const int*)(ws + L->o.ntiles);
-    v.b_group_stride = (long)d.D * d.M; v.out0 = ws + L->o.v;
-    dim3 grid_v(d.max_tiles, (d.D + 63) / 64);
-    sh_simt_gemm_kernel<TI, TI, TM, SH_EPI_V><<<grid_v, 256, 0, st>>>(v);
-    L->launches += 2;
+  if constexpr (!F32) {
+    if (!L->dense && (stages & SH_STAGE_V)) {
+      SH_CUDA_CHECK(cudaMemsetAsync(ws + L->o.v, 0, (size_t)d.N * HD * sizeof(TM), st));
+      ShGemmArgs v{};
+      v.d = d; v.A = x; v.lda = d.M; v.Bt = ws + L->o.wv; v.ldb = d.M; v.K = d.M; v.ncols = d.D;
+      v.lists = (const int*)(ws + L->o.lists); v.lgate = (const float*)(ws + L->o.lgate);
+      v.tiles = (const ShTile*)(ws + L->o.tiles); v.ntiles = (const int*)(ws + L->o.ntiles);
+      v.b_group_stride = (long)d.D * d.M; v.out0 = ws + L->o.v;
+      dim3 grid_v(d.max_tiles, (d.D + 63) / 64);
+      sh_simt_gemm_kernel<TI, TI, TM, SH_EPI_V><<<grid_v, 256, 0, st>>>(v);
+      L->launches += 2;
+    }
   }
   if (all) sh_mark(L, 3, st);
   if (stages & SH_STAGE_ATTN) {
@@ -497,19 +504,21 @@ static int forward_simt(sh_layer* L, int stages, const void* x, void* out, cudaS
   if (all) sh_mark(L, 4, st);
   if (!(stages & SH_STAGE_O)) {
   } else if (!L->dense) {
-    SH_CUDA_CHECK(cudaMemsetAsync(out, 0, (size_t)sh_out_rows(d) * d.M * 4, st));
-    ShGemmArgs o{};
-    o.d = d; o.A = ws + L->o.ahat; o.lda = HD; o.a_head_stride = d.D; o.Bt = ws + L->o.wo; o.ldb = d.D;
-    o.K = d.D; o.ncols = d.M;
-    // destination-side lists and tiles (with a shared selection: the one side there is)
-    const size_t side1 = d.sides == 2 ? (size_t)d.H * d.N * d.k : 0;
-    o.lists = (const int*)(ws + L->o.lists) + side1; o.lgate = (const float*)(ws + L->o.lgate) + side1;
-    o.tiles = (const ShTile*)(ws + L->o.tiles) + (d.sides == 2 ? d.max_tiles : 0);
-    o.ntiles = (const int*)(ws + L->o.ntiles) + (d.sides == 2 ? 1 : 0);
-    o.b_group_stride = (long)d.M * d.D; o.out0 = out;
-    dim3 grid_o(d.max_tiles, (d.M + 63) / 64);
-    sh_simt_gemm_kernel<TM, TM, float, SH_EPI_O><<<grid_o, 256, 0, st>>>(o);
-    L->launches += 2;
+    if constexpr (!F32) {
+      SH_CUDA_CHECK(cudaMemsetAsync(out, 0, (size_t)sh_out_rows(d) * d.M * 4, st));
+      ShGemmArgs o{};
+      o.d = d; o.A = ws + L->o.ahat; o.lda = HD; o.a_head_stride = d.D; o.Bt = ws + L->o.wo; o.ldb = d.D;
+      o.K = d.D; o.ncols = d.M;
+      // destination-side lists and tiles (with a shared selection: the one side there is)
+      const size_t side1 = d.sides == 2 ? (size_t)d.H * d.N * d.k : 0;
+      o.lists = (const int*)(ws + L->o.lists) + side1; o.lgate = (const float*)(ws + L->o.lgate) + side1;
+      o.tiles = (const ShTile*)(ws + L->o.tiles) + (d.sides == 2 ? d.max_tiles : 0);
+      o.ntiles = (const int*)(ws + L->o.ntiles) + (d.sides == 2 ? 1 : 0);
+      o.b_group_stride = (long)d.M * d.D; o.out0 = out;
+      dim3 grid_o(d.max_tiles, (d.M + 63) / 64);
+      sh_simt_gemm_kernel<TM, TM, float, SH_EPI_O><<<grid_o, 256, 0, st>>>(o);
+      L->launches += 2;
+    }
   } else {
     ShGemmArgs o{};
     o.d = d; o.A = ws + L->o.ahat; o.lda = HD; o.Bt = ws + L->o.wo; o.ldb = HD; o.K = HD; o.ncols = d.M;

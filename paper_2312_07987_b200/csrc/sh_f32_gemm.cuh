@@ -50,7 +50,7 @@ enum { X_QK = 0,    // q, k = x [Wq | Wk]                     rows: tokens
 struct XGemmArgs {
   ShDims d;
   const float *x, *dy;                   // [N, M]; dy [N, M]
-  const float *ahat, *dahat_in;          // [N, H, D]
+  const float* ahat;                     // [N, H, D]
   const float *dq, *dk, *dv, *dz;        // [N, H, D]; dz [N, ldz] (columns (side*H + h)*E + e)
   int ldz;
   const int* lists; const float* lgate; const int* offsets; const ShTile* tiles;   // of the side the mode works on

@@ -98,7 +98,7 @@ sh_tc_attention_wide_kernel(const __grid_constant__ CUtensorMap mapQ, const __gr
   const uint32_t tmem = *tmem_slot;                        // O: columns 0..255; S: 256, 320; P (hi 32 columns, lo 32): 384, 448
   if (threadIdx.x == 0) sh_stamp_resident(d.stamps, SH_K_ATTN);
   pdl_wait();
-  pdl_trigger();                                           // (behind the wait: the output projection reads the selections ahead of its own)
+  pdl_trigger();                                           // (behind the wait: what the next kernel does ahead of its own then sees every earlier kernel complete)
   if (threadIdx.x == 0) sh_stamp_start(d.stamps, SH_K_ATTN);
 
   if (warp == 0) {
