@@ -162,3 +162,29 @@ def test_f32_overflow_of_one_token_stays_behind_the_mask(D):
     y = layer.sh_forward(x)
     assert close(y[:, :t0], want_y[:, :t0]) and not bool(torch.isfinite(y[:, t0:]).all())
     layer.close()
+
+
+def test_f32_forward_and_backward_in_a_captured_graph():
+    cfg = inputs.LayerConfig("tiles", inputs.DTYPE_F32, 2, 150, 128, 2, 76, 4, 2, seed=23)
+    inp = inputs.make_inputs(cfg)
+    layer = binding.layer_from_inputs(inp)
+    x = binding.to_device(inp.x, cfg.dtype)
+    other = x.flip(1).contiguous()
+    G = torch.ones_like(x)
+    layer.sh_forward(other)
+    want = dict(layer.sh_backward(other, G), y=layer.sh_forward(other))
+    layer.sh_forward(x)
+    layer.sh_backward(x, G)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        y = layer.sh_forward(x)
+        got = dict(layer.sh_backward(x, G), y=y)
+    x.copy_(other)
+    for _ in range(3):
+        graph.replay()
+    torch.cuda.synchronize()
+    for name, w in want.items():
+        assert float((got[name] - w).abs().max() / w.abs().max()) < TOL, name
+    assert layer.sh_last_status() == 0
+    layer.close()

@@ -150,3 +150,7 @@ def test_gates_are_the_allocation_free_entry_points_bit_for_bit(T, M, H, E, k):
         assert torch.equal(a, b)
     assert layer.sh_last_status() == 0
     layer.close()
+
+
+def test_shared_selection():
+    full_check(inputs.make_inputs(config(2, 150, 128, 2, 132, 5, 2)), shared_selection=True)
