@@ -108,7 +108,7 @@ sh_layer* sh_create_dense(int d_model, int n_heads, int d_head);
 
 /* Fix the storage type and the problem size.  dtype SH_F32: x and weights fp32;
  * projections on the tensor cores with every fp32 operand as the sum of three bf16 values (six products,
- * fp32 accumulation: fp32 accuracy), gates and attention in fp32 on the CUDA cores.  dtype SH_BF16: x and weights bf16, tensor-core products
+ * fp32 accumulation: fp32 accuracy, for operands of 2^-109 and more in magnitude), gates and attention in fp32 on the CUDA cores.  dtype SH_BF16: x and weights bf16, tensor-core products
  * with fp32 accumulation, fp16 intermediates (Q, K, V, P, A^h V^h); requires d_model a
  * multiple of 128.  `out` is fp32 in both cases.
  * batch*seq*n_heads*k must be below 2^31.  Invalidates workspace and weights. */
@@ -186,7 +186,7 @@ int sh_set_rope(sh_layer* layer, double base, void* stream);
 /* The whole forward pass (gates + top-k + bucket sort, Q/K projections, value experts,
  * causal attention, output experts with the gate-weighted sum) of x [B, T, d_model] into
  * out [B, T, d_model] fp32 (with a cache, sh_configure_xl: x [B, cache_len + T, d_model]).  Both are device pointers aligned to 16 bytes (else
- * SH_ERR_INVALID_ARG).  out is fully overwritten.  Enqueues kernels only. */
+ * SH_ERR_INVALID_ARG).  out is fully overwritten; in the fp32 configuration it may overlap x.  Enqueues kernels only. */
 int sh_forward(sh_layer* layer, const void* x, void* out, void* stream);
 
 /* Kernel slots of sh_forward_stamped. */

@@ -1,5 +1,6 @@
 // fp32 contractions on the tensor cores: every projection of the fp32 configuration, forward and
-// backward.
+// backward, but the weight gradients, which are in sh_f32_wgrad.cuh (their modes are numbered here: they share the
+// arguments).
 //
 // An fp32 value is the exact sum of three bf16 values, x = h + m + l (8 + 8 + 8 mantissa bits: h is x
 // rounded, m the rest rounded, l what is left), so a product of two is
@@ -25,13 +26,12 @@
 // activation is read as fp32 by the workers, two steps ahead, by asynchronous copies into shared memory
 // that only the copying warp uses (a prefetch that costs no registers and no block-wide barrier), split and
 // stored into the swizzled planes.  One thread issues the UMMAs; the workers read the accumulators and
-// write the result.  The weight gradients, whose operands are both activations, are in sh_f32_wgrad.cuh.
+// write the result.
 // Operands are addressed row by row (a gathered token list, a head's slice of a row), either as rows of
-// the contraction (K-major) or as rows of the other index (MN-major: the weight gradients contract over
-// tokens), so no transposed or gathered copy is made.  Results that are added to, and rows handed on
-// whole, go through a padded copy in shared memory and leave as one bulk operation per row: as vector
-// reductions from the accumulator layout (a lane per row, 16 bytes each) they were a third of the
-// short contractions' time.
+// the contraction (K-major) or as rows of the other index (MN-major: weights in the backward pass), so no
+// transposed or gathered copy is made.  Results that are added to, and rows handed on whole, go through a
+// padded copy in shared memory and leave as one bulk operation per row: as vector reductions from the
+// accumulator layout (a lane per row, 16 bytes each) they were a third of the short contractions' time.
 #pragma once
 #include "sh_tc_prims.cuh"
 

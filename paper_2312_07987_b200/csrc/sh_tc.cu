@@ -573,8 +573,9 @@ static int o_pairs(K kern, int smem) {
 }
 
 // Output features per work unit of those kernels.  A unit works off all experts of its tokens whatever its width -
-// the pipe's part of it shrinks with the width, the builders' does not -, so narrower units pay exactly as long as
-// the wide ones leave pairs without a unit.
+// the pipe's part of it shrinks with the width, the builders' does not -, so narrower units pay while the wide ones
+// leave pairs without a unit.  (449 shapes of 200 to 4500 tokens, every width forced: this choice is 1.5 % slower than
+// 256 at worst, 2.4 % faster on average; one step narrower than it, up to a third slower.)
 static int oproj_features(const TcState* S, const ShDims& d) {
   const int rows = (sh_out_rows(d) + 255) / 256;
   int fn = 256;
