@@ -3,6 +3,7 @@
 // (sh_f32_attn.cuh), selection and sort in one launch (sh_f32_select.cuh).
 #include "sh_internal.cuh"
 #include "sh_launch.cuh"
+#include "sh_simt.cuh"
 #include "sh_f32_gemm.cuh"
 #include "sh_f32_wgrad.cuh"
 #include "sh_f32_attn.cuh"
@@ -107,10 +108,22 @@ int launch_gate_sort(sh_layer* L, const void* x, float* zero, long n, cudaStream
   auto kern = small ? (ch == 512 ? sh_f32_gate_kernel<8, 512> : sh_f32_gate_kernel<8, 1024>)
                     : (ch == 512 ? sh_f32_gate_kernel<16, 512> : sh_f32_gate_kernel<16, 1024>);
   if (int rc = set_smem(kern, (int)smem)) return rc;
+  const size_t ssm = sh_sort_smem_bytes(d);
+  int* blockcnt = d.N > F32_SORT_MAX && ssm <= 227 * 1024 ? (int*)(ws + L->o.blockcnt) : nullptr;
+  if (blockcnt) {
+    SH_CUDA_CHECK(cudaMemsetAsync(blockcnt, 0, (size_t)d.nblk * d.G * 4, st));
+    SH_CUDA_CHECK(cudaMemsetAsync(ws + L->o.tiles, 0, (size_t)2 * d.max_tiles * sizeof(ShTile), st));
+  }
   if (int rc = launch_k(chained(L), kern, dim3((unsigned)((d.N + tok - 1) / tok)), dim3(512), smem, st, (const float*)x, (const float*)(ws + L->o.wgate32),
-                        (const float*)(ws + L->o.gbias), (int*)(ws + L->o.idx), (float*)(ws + L->o.gate), (float4*)zero, n / 4, d, (int)((uintptr_t)x % 16 == 0)))
+                        (const float*)(ws + L->o.gbias), (int*)(ws + L->o.idx), (float*)(ws + L->o.gate), blockcnt, (float4*)zero, n / 4, d, (int)((uintptr_t)x % 16 == 0)))
     return rc;
   L->launches += 2;
+  if (blockcnt) {
+    if (int rc = set_smem(sh_sort_kernel, (int)ssm)) return rc;
+    return launch_k(chained(L), sh_sort_kernel, dim3(d.nblk), dim3(sh_sort_threads(d)), ssm, st, (const int*)(ws + L->o.idx), (const float*)(ws + L->o.gate),
+                    (const int*)blockcnt, (int*)(ws + L->o.offsets), (int*)(ws + L->o.lists), (float*)(ws + L->o.lgate),
+                    (ShTile*)(ws + L->o.tiles), (int*)(ws + L->o.ntiles), d);
+  }
   return launch_k(chained(L), sh_f32_sort_kernel, dim3(d.sides * d.H), dim3(1024), 0, st, (const int*)(ws + L->o.idx), (const float*)(ws + L->o.gate),
                   (int*)(ws + L->o.offsets), (int*)(ws + L->o.lists), (float*)(ws + L->o.lgate), (ShTile*)(ws + L->o.tiles), d, head_tiles(d));
 }

@@ -53,7 +53,7 @@ __device__ __forceinline__ void sh_select(float* z, const float* __restrict__ gb
 template <int TOK, int CH>
 static __global__ void __launch_bounds__(512, 1)
 sh_f32_gate_kernel(const float* __restrict__ x, const float* __restrict__ wgate, const float* __restrict__ gbias, int* __restrict__ idx,
-                   float* __restrict__ gate, float4* __restrict__ zero, long nzero, ShDims d, int vec) {
+                   float* __restrict__ gate, int* __restrict__ blockcnt, float4* __restrict__ zero, long nzero, ShDims d, int vec) {
   extern __shared__ __align__(16) float gsm[];             // [TOK][CH] of x, then [TOK][G] logits
   float* s_z = gsm + TOK * CH;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -124,7 +124,7 @@ sh_f32_gate_kernel(const float* __restrict__ x, const float* __restrict__ wgate,
   const int groups = d.sides * d.H;
   for (int i = tid; i < TOK * groups; i += 512) {
     const int r = i / groups, grp = i % groups;
-    if (t0 + r < d.N) sh_select(s_z + r * d.G + grp * d.E, gbias, idx, gate, nullptr, d, t0 + r, grp);
+    if (t0 + r < d.N) sh_select(s_z + r * d.G + grp * d.E, gbias, idx, gate, blockcnt, d, t0 + r, grp);
   }
 }
 
@@ -229,9 +229,12 @@ sh_bf16_gate_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __
   }
 }
 
-// Bucket sort, one block per (side, head): the stable counting sort of the tokens by chosen expert, in
+// Bucket sort of up to F32_SORT_MAX tokens, one block per (side, head): the stable counting sort of the tokens by chosen expert, in
 // two sweeps of 1024 tokens at a time (totals, then placement).  No block needs another's counts: every
 // head owns a fixed range of the row-tile table (mt = (N k + 127 E) / 128 entries, the unused ones empty).
+// Above, sh_sort_kernel with a block per 128 tokens (it wants their counts and an empty tile table ahead of it): 53 us
+// here for 8192 tokens, and in proportion beyond.
+constexpr int F32_SORT_MAX = 4096;
 static __global__ void __launch_bounds__(1024)
 sh_f32_sort_kernel(const int* __restrict__ idx, const float* __restrict__ gate, int* __restrict__ offsets, int* __restrict__ lists,
                    float* __restrict__ lgate, ShTile* __restrict__ tiles, ShDims d, int mt) {

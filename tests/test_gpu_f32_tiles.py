@@ -55,6 +55,8 @@ def run(B, T, M, H, D, E, k, causal=True, offset=0, zipf=0.0, change=None):
     (3, 50, 128, 1, 256, 3, 1),
     (1, 2100, 64, 1, 40, 1, 1),      # three selection sweeps; contractions over tokens in parts
     (2, 600, 128, 2, 76, 32, 4),     # 32 experts, hardly a full tile among them
+    (64, 64, 64, 1, 16, 3, 2),       # the most tokens of the one-block sort
+    (41, 100, 64, 2, 16, 5, 2),      # ... and just past it: a block per 128 tokens
 ])
 def test_f32_tile_edges(B, T, M, H, D, E, k):
     run(B, T, M, H, D, E, k)
