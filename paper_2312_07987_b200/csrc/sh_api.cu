@@ -97,7 +97,7 @@ static void layout_workspace(sh_layer* L) {
   //  in list order, the gate gradients once more as a matrix [N, G], rowsum(dAhat o Ahat) [N, H]); the gate weights
   //  once more in fp32; per attention row the score maximum and 1 / normaliser)
   const bool f32 = L->dtype == SH_F32 && !L->dense;
-  o.bw = take(f32 ? ((size_t)4 * d.N * HD + (size_t)2 * d.N * d.H * d.k + (size_t)d.N * (sh_f32_ldz(d) + d.H)) * 4 : 16);
+  o.bw = take(f32 ? ((size_t)4 * d.N * HD + (size_t)d.N * (sh_f32_ldz(d) + d.H)) * 4 : 16);
   o.wgate32 = take(f32 ? (size_t)d.G * d.M * 4 : 16);
   o.f32stats = take(f32 ? (size_t)d.N * d.H * 8 : 16);
   o.wo_overflow = take(16);                                  // d_head above 128, bf16 storage: a stored weight of W_O is not finite

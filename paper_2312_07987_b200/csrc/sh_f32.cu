@@ -169,16 +169,15 @@ int launch_attn(sh_layer* L, float* zero, long n, cudaStream_t st) {
   }
 }
 
-struct BwBuffers { float *dq, *dk, *dv, *dahat, *ds, *dz, *dsum; size_t cleared; };
+struct BwBuffers { float *dq, *dk, *dv, *dahat, *dz, *dsum; size_t cleared; };
 BwBuffers bw_buffers(sh_layer* L) {
   const ShDims& d = L->d;
   const size_t nhd = (size_t)d.N * d.H * d.D;
   BwBuffers b;
   b.dq = (float*)(L->ws + L->o.bw); b.dk = b.dq + nhd; b.dv = b.dk + nhd; b.dahat = b.dv + nhd;
   b.dz = b.dahat + nhd;
-  b.ds = b.dz + (size_t)d.N * sh_f32_ldz(d);
-  b.dsum = b.ds + (size_t)2 * d.N * d.H * d.k;
-  b.cleared = (size_t)(b.dsum - b.dq);
+  b.dsum = b.dz + (size_t)d.N * sh_f32_ldz(d);
+  b.cleared = (size_t)(b.dsum - b.dq) + (size_t)d.N * d.H;
   return b;
 }
 
@@ -305,43 +304,15 @@ int sh_f32_backward(sh_layer* L, const void* x, const float* dout, float* dx, fl
   const int ht = head_tiles(d), mt = (d.M + 127) / 128, dt = (d.Dt + 127) / 128;
   int rc;
   L->launches = 0;
-  SH_CUDA_CHECK(cudaMemsetAsync(w.dq, 0, w.cleared * 4, st));
-  SH_CUDA_CHECK(cudaMemsetAsync(dx, 0, (size_t)d.N * d.M * 4, st));
   XGemmArgs src = base_args(L, x);                         // source side; dst: destination side
-  src.dy = dout; src.dq = w.dq; src.dk = w.dk; src.dv = w.dv; src.dz = w.dz; src.dahat = w.dahat; src.dx = dx;
+  src.dy = dout; src.dq = w.dq; src.dk = w.dk; src.dv = w.dv; src.dz = w.dz; src.dsum = w.dsum; src.dahat = w.dahat; src.dx = dx;
   src.dWq = dWq; src.dWk = dWk; src.dWv = dWv; src.dWo = dWo; src.dWs = dWs; src.dWd = dWd;
   auto aligned = [](const void* p) { return (uintptr_t)p % 16 == 0; };
   src.vec_dy = aligned(dout);
   src.vec_out = aligned(dx) && aligned(dWq) && aligned(dWk) && aligned(dWv) && aligned(dWo);
   XGemmArgs dst = src;
   use_side(src, L, 0); use_side(dst, L, 1);
-  src.ds = w.ds; dst.ds = w.ds + (size_t)d.H * d.N * d.k;
-  XGemmArgs g;
-  // output experts: dAhat and the destination gates' gradients
-  g = dst;
-  col_tiles(g, d.Dt);
-  // (about half of the experts' last tiles are worth counting; the rest of the table is empty)
-  g.ksplit = half_blocks(L, ((long)d.H * d.N * d.k / 128 + d.H * d.E / 2) * g.nsub, d.M / XG_BK);
-  if ((rc = launch_x<X_DA>(L, st, part<X_DA>(L, g, d.H * ht, g.nsub, g.ksplit)))) return rc;
-  // attention
-  const int rows = d.N * d.H;
-  if ((rc = launch_k(chained(L), sh_f32_rowdot_kernel, dim3((unsigned)((rows + 7) / 8)), dim3(256), 0, st, (const float*)w.dahat,
-                     (const float*)(ws + L->o.ahat), w.dsum, rows, d.D))) return rc;
-  rc = d.D == 32 ? launch_attn_bw_t<32>(L, w, st) : d.D == 64 ? launch_attn_bw_t<64>(L, w, st)
-     : d.D == 128 ? launch_attn_bw_t<128>(L, w, st) : launch_attn_bw_t<256>(L, w, st);
-  if (rc) return rc;
-  // value experts: their part of dx, and the source gates' gradients
-  g = src;
-  col_tiles(g, d.M);
-  if ((rc = launch_x<X_DR>(L, st, part<X_DR>(L, g, d.H * ht, g.nsub)))) return rc;
-  if ((rc = launch_k(chained(L), sh_f32_dz_kernel, dim3((unsigned)(((long)d.N * d.k + 255) / 256), 2 * d.H), dim3(256), 0, st, (const float*)w.ds,
-                     (const int*)(ws + L->o.lists), (const float*)(ws + L->o.lgate), (const int*)(ws + L->o.offsets), w.dz, src.ldz, d))) return rc;
-  // queries, keys and gates: the rest of dx
-  g = src;
-  col_tiles(g, d.M);
-  g.ksplit = half_blocks(L, (long)d.nblk * g.nsub, 2 * d.H * ((d.Dt + XG_BK - 1) / XG_BK));
-  if ((rc = launch_x<X_DX>(L, st, part<X_DX>(L, g, d.nblk, g.nsub, g.ksplit)))) return rc;
-  // weight gradients, one launch
+  // weight gradients: how the contractions are split
   auto wpart = [](const XGemmArgs& a, int gx, int gy, int gz) { XWPart p; p.g = a; p.gx = gx; p.gy = gy; p.n = gx * gy * gz; return p; };
   XGemmArgs gq = src, gv = src, go = dst;
   col_tiles(gq, d.Dt, XW_BN); col_tiles(gv, d.Dt, XW_BN); col_tiles(go, d.M, XW_BN);
@@ -356,20 +327,40 @@ int sh_f32_backward(sh_layer* L, const void* x, const float* dout, float* dx, fl
     if (nq * ((sq + l - 1) / l) + nl * ((sl + l - 1) / l) <= sm_count(L)) { len = l; break; }
   gq.ksplit = (int)((sq + len - 1) / len);
   gv.ksplit = go.ksplit = (int)((sl + len - 1) / len);
-  if (gq.ksplit > 1) {
-    SH_CUDA_CHECK(cudaMemsetAsync(dWq, 0, (size_t)d.H * d.M * d.Dt * 4, st));
-    SH_CUDA_CHECK(cudaMemsetAsync(dWk, 0, (size_t)d.H * d.M * d.Dt * 4, st));
-    SH_CUDA_CHECK(cudaMemsetAsync(dWs, 0, (size_t)d.H * d.M * d.E * 4, st));
-    SH_CUDA_CHECK(cudaMemsetAsync(dWd, 0, (size_t)d.H * d.M * d.E * 4, st));
-  }
-  if (gv.ksplit > 1) {
-    SH_CUDA_CHECK(cudaMemsetAsync(dWv, 0, (size_t)d.H * d.E * d.M * d.Dt * 4, st));
-    SH_CUDA_CHECK(cudaMemsetAsync(dWo, 0, (size_t)d.H * d.E * d.Dt * d.M * 4, st));
-  }
+  // what is added into
+  const long hmd = (long)d.H * d.M * d.Dt, hme = (long)d.H * d.M * d.E;
+  FClear c{};
+  int nc = 0;
+  auto clear = [&](float* p, long n) { c.p[nc] = p; c.n[nc++] = n; };
+  clear(w.dq, (long)w.cleared); clear(dx, (long)d.N * d.M);
+  if (gq.ksplit > 1) { clear(dWq, hmd); clear(dWk, hmd); clear(dWs, hme); clear(dWd, hme); }
+  if (gv.ksplit > 1) { clear(dWv, hmd * d.E); clear(dWo, hmd * d.E); }
+  if ((rc = launch_k(chained(L), sh_f32_clear_kernel, dim3(4u * (unsigned)sm_count(L)), dim3(256), 0, st, c))) return rc;
+  XGemmArgs g;
+  // output experts: dAhat and the destination gates' gradients
+  g = dst;
+  col_tiles(g, d.Dt);
+  // (about half of the experts' last tiles are worth counting; the rest of the table is empty)
+  g.ksplit = half_blocks(L, ((long)d.H * d.N * d.k / 128 + d.H * d.E / 2) * g.nsub, d.M / XG_BK);
+  if ((rc = launch_x<X_DA>(L, st, part<X_DA>(L, g, d.H * ht, g.nsub, g.ksplit)))) return rc;
+  // attention
+  rc = d.D == 32 ? launch_attn_bw_t<32>(L, w, st) : d.D == 64 ? launch_attn_bw_t<64>(L, w, st)
+     : d.D == 128 ? launch_attn_bw_t<128>(L, w, st) : launch_attn_bw_t<256>(L, w, st);
+  if (rc) return rc;
+  // value experts: their part of dx, and the source gates' gradients
+  g = src;
+  col_tiles(g, d.M);
+  if ((rc = launch_x<X_DR>(L, st, part<X_DR>(L, g, d.H * ht, g.nsub)))) return rc;
+  // queries, keys and gates: the rest of dx
+  g = src;
+  col_tiles(g, d.M);
+  g.ksplit = half_blocks(L, (long)d.nblk * g.nsub, 2 * d.H * ((d.Dt + XG_BK - 1) / XG_BK));
+  if ((rc = launch_x<X_DX>(L, st, part<X_DX>(L, g, d.nblk, g.nsub, g.ksplit)))) return rc;
+  // weight gradients, one launch
   const XWPart pq = wpart(gq, mt, ct, gq.ksplit), pv = wpart(gv, d.H * d.E * gv.ksplit, gv.nsub, mt), po = wpart(go, d.H * d.E * go.ksplit, go.nsub, dt);
   if ((rc = set_smem(sh_f32_wgrad_kernel, XWgradSmem::TOTAL))) return rc;
   if ((rc = launch_k(chained(L), sh_f32_wgrad_kernel, dim3((unsigned)(pq.n + pv.n + po.n)), dim3(XW_THREADS), XWgradSmem::TOTAL, st, pq, pv, po))) return rc;
   SH_CUDA_CHECK(cudaGetLastError());
-  L->launches += 4;
+  L->launches += 3;
   return SH_OK;
 }

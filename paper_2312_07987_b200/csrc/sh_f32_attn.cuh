@@ -226,18 +226,21 @@ sh_f32_attn_kernel(const float* __restrict__ Q, const float* __restrict__ K, con
 }
 
 // ---- backward --------------------------------------------------------------------------------------
-// rowsum(dAhat o Ahat) of every (token, head): dsum [N, H].  One warp per row.
+// What the backward pass adds into, cleared in one launch (as memsets, up to six of them, each with a gap in the chain
+// of launches in front and behind: 24 us of a 47M-scale step).  Pointers may be 4-byte aligned.
+struct FClear { float* p[8]; long n[8]; };
 static __global__ void __launch_bounds__(256)
-sh_f32_rowdot_kernel(const float* __restrict__ a, const float* __restrict__ b, float* __restrict__ out, int rows, int D) {
+sh_f32_clear_kernel(const __grid_constant__ FClear c) {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  if (row >= rows) return;
-  float s = 0.f;
-  for (int i = lane; i < D; i += 32) s = fmaf(a[(size_t)row * D + i], b[(size_t)row * D + i], s);
+  const long me = (long)blockIdx.x * 256 + threadIdx.x, all = (long)gridDim.x * 256;
 #pragma unroll
-  for (int x = 16; x > 0; x >>= 1) s += __shfl_xor_sync(0xffffffffu, s, x);
-  if (lane == 0) out[row] = s;
+  for (int r = 0; r < 8; ++r) {
+    float* const p = c.p[r];
+    const long n = c.n[r], n4 = (uintptr_t)p % 16 == 0 ? n / 4 : 0;
+    for (long i = me; i < n4; i += all) reinterpret_cast<float4*>(p)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (long i = 4 * n4 + me; i < n; i += all) p[i] = 0.f;
+  }
 }
 
 // Block: 32 keys of one (sequence, head) and a run of query tiles (TQ queries each; blockIdx.y), two

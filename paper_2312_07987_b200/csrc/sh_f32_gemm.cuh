@@ -51,7 +51,8 @@ struct XGemmArgs {
   ShDims d;
   const float *x, *dy;                   // [N, M]; dy [N, M]
   const float* ahat;                     // [N, H, D]
-  const float *dq, *dk, *dv, *dz;        // [N, H, D]; dz [N, ldz] (columns (side*H + h)*E + e)
+  const float *dq, *dk, *dv;             // [N, H, D]
+  float *dz, *dsum;                      // gate gradients [N, ldz], columns (side*H + h)*E + e; rowsum(dahat o ahat) [N, H]
   int ldz;
   const int* lists; const float* lgate; const int* offsets; const ShTile* tiles;   // of the side the mode works on
   int nsub, sub_cols;                    // column tiles per head (or of M), and columns per tile (a multiple of 16)
@@ -59,7 +60,7 @@ struct XGemmArgs {
   int ksplit;                            // parts of the contraction (weight gradients: with more than one the results are added)
   float *q, *k, *v;                      // X_QK: q, k [B, H, T, D]; X_V: v
   float *y;                              // X_O [rows of out, M]
-  float *dahat, *ds, *dx;                // ds: gate gradients in list order
+  float *dahat, *dx;
   float *dWq, *dWk, *dWv, *dWo, *dWs, *dWd;
   float qscale, vscale;
   const float2* rope;
@@ -438,7 +439,10 @@ __device__ __forceinline__ void xg_tile(const CUtensorMap& mapW, const CUtensorM
               for (int j = 0; j < 4; ++j) if (i + j < valid) dot += acc[i + j] * __ldg(other + i + j);
             }
           }
-          atomicAdd(g.ds + li, dot);
+          // ds s (1 - s) is linear in ds, and rowsum(dahat o ahat) = sum over the selected experts of s ds: both are
+          // added up here, part by part (kernels of their own for them: 5 us of a step)
+          atomicAdd(g.dz + (size_t)t * g.ldz + ((MODE == X_DA ? d.H : 0) + h) * d.E + e, dot * gt * (1.f - gt));
+          if (MODE == X_DA) atomicAdd(g.dsum + (size_t)t * d.H + h, gt * dot);
         }
         const float f = MODE == X_V && g.vscale != 0.f ? gt * g.vscale : gt;
 #pragma unroll

@@ -331,22 +331,3 @@ sh_f32_sort_kernel(const int* __restrict__ idx, const float* __restrict__ gate, 
     __syncthreads();
   }
 }
-
-// Gate gradients from list order into the matrix the projections' backward GEMMs contract with:
-// dz[t, (side, h, e)] = ds s (1 - s) at the selected entries (the matrix is zero elsewhere).
-static __global__ void __launch_bounds__(256)
-sh_f32_dz_kernel(const float* __restrict__ ds, const int* __restrict__ lists, const float* __restrict__ lgate, const int* __restrict__ offsets,
-                 float* __restrict__ dz, int ldz, ShDims d) {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  const long per = (long)d.N * d.k;
-  const int grp = blockIdx.y;                              // (side, head)
-  const long p = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= per) return;
-  const int* off = offsets + (size_t)grp * (d.E + 1);
-  int e = 0;
-  while (e < d.E - 1 && off[e + 1] <= p) ++e;
-  const size_t li = (size_t)grp * per + p;
-  const float g = lgate[li];
-  if (SH_INDEX_OK(lists[li], d.N, d.status, SH_SITE_V_LIST)) dz[(size_t)lists[li] * ldz + grp * d.E + e] = ds[li] * g * (1.f - g);
-}
