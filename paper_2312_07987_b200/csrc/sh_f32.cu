@@ -16,9 +16,9 @@ using namespace shtc;
 
 namespace {
 
-// The split weights as [3 planes, rows, inner]: boxes of 64 rows x 32 positions where a row runs along the
+// The split weights as [3 planes, rows, inner]: boxes of k_rows rows x 32 positions where a row runs along the
 // contraction (k), of 32 rows x 64 columns where the contraction runs over rows (mn).
-struct PlaneMap { CUtensorMap k, mn; };
+struct PlaneMap { CUtensorMap k, mn; int k_rows; };
 struct F32State {
   PlaneMap wqk, wgate, wv, wo, wq_e, wk_e;
   bool pdl = true;          // kernels chained by programmatic dependent launch (the debug library's SH_NO_PDL: ordinary launches)
@@ -46,7 +46,7 @@ XPart part(sh_layer* L, const XGemmArgs& g, int gx, int gy, int gz = 1, const Pl
   constexpr bool K_MAJOR = MODE == X_QK || MODE == X_V || MODE == X_O;
   if (!w) w = MODE == X_O || MODE == X_DA ? &S->wo : MODE == X_V || MODE == X_DR ? &S->wv : &S->wqk;
   XPart p;
-  p.w = K_MAJOR ? w->k : w->mn; p.g = g; p.gx = gx; p.gy = gy; p.n = gx * gy * gz;
+  p.w = K_MAJOR ? w->k : w->mn; p.g = g; p.g.b_rows = w->k_rows; p.gx = gx; p.gy = gy; p.n = gx * gy * gz;
   return p;
 }
 
@@ -62,9 +62,32 @@ int launch_x(sh_layer* L, cudaStream_t st, const XPart& a, const XPart& b = XPar
 }
 
 // Column tiles over `cols` columns: how many, and how wide (a multiple of 16).
-void col_tiles(XGemmArgs& g, int cols, int bn = XG_BN) {
-  g.nsub = (cols + bn - 1) / bn;
-  g.sub_cols = ((cols + g.nsub - 1) / g.nsub + 15) / 16 * 16;
+int col_width(int cols) { const int n = (cols + XG_BN - 1) / XG_BN; return ((cols + n - 1) / n + 15) / 16 * 16; }
+void col_tiles(XGemmArgs& g, int cols) {
+  g.nsub = (cols + XG_BN - 1) / XG_BN;
+  g.sub_cols = col_width(cols);
+}
+
+// A contraction over d_head of a side's lists: up to 128 positions on the kernel that keeps its rows in tensor memory,
+// the columns split among as many blocks per row tile as the device has SMs for.  (Half of the experts' last tiles are
+// worth counting; the rest of the table is empty.)
+template <int MODE>
+int launch_d(sh_layer* L, cudaStream_t st, XGemmArgs g) {
+  const F32State* S = (const F32State*)L->f32;
+  const ShDims& d = L->d;
+  const PlaneMap& w = MODE == X_O ? S->wo : S->wv;
+  if (d.Dt > 128) {
+    col_tiles(g, d.M);
+    return launch_x<MODE>(L, st, part<MODE>(L, g, d.H * head_tiles(d), g.nsub));
+  }
+  const int ntile = (d.M + XGemmDSmem::BN - 1) / XGemmDSmem::BN;
+  const long rows = (long)d.H * d.N * d.k / 128 + d.H * d.E / 2;
+  long split = sm_count(L) / (rows < 1 ? 1 : rows);
+  split = split < 1 ? 1 : split > ntile ? ntile : split;
+  auto kern = sh_f32_gemm_d_kernel<MODE>;
+  if (int rc = set_smem(kern, XGemmDSmem::TOTAL)) return rc;
+  L->launches += 1;
+  return launch_k(chained(L), kern, dim3((unsigned)(d.H * head_tiles(d)), (unsigned)split), dim3(XG_THREADS), XGemmDSmem::TOTAL, st, MODE == X_O ? w.k : w.mn, g);
 }
 
 XGemmArgs base_args(sh_layer* L, const void* x) {
@@ -198,11 +221,9 @@ int launch_attn_bw_t(sh_layer* L, const BwBuffers& w, cudaStream_t st) {
                   (const float*)(ws + L->o.f32stats), (const float*)w.dsum, w.dq, w.dk, w.dv, d, (int)run);
 }
 
-// Parts of a contraction on the half-SM blocks, where its result is added anyway: enough blocks for both
-// places of every SM, at least eight steps each (a block works off about one step a us whether it has the SM
-// to itself or shares it).
-int half_blocks(sh_layer* L, long blocks, long steps) {
-  long p = 2l * sm_count(L) / (blocks < 1 ? 1 : blocks);
+// Parts of a contraction whose result is added anyway: enough blocks for every SM, at least eight steps each.
+int k_parts(sh_layer* L, long blocks, long steps) {
+  long p = sm_count(L) / (blocks < 1 ? 1 : blocks);
   const long most = steps / 8;
   p = p > most ? most : p;
   return p < 1 ? 1 : p > 8 ? 8 : (int)p;
@@ -220,18 +241,20 @@ int sh_f32_prepare(sh_layer* L) {
 #endif
   const ShDims& d = L->d;
   char* ws = L->ws;
-  auto enc = [&](PlaneMap& m, size_t off, uint64_t inner, uint64_t rows) -> int {
-    if (int rc = sh_tc_encode_planes(&m.k, ws + off, inner, rows, XG_BK, XG_BN)) return rc;
-    return sh_tc_encode_planes(&m.mn, ws + off, inner, rows, XG_BN, XG_BK);
+  auto enc = [&](PlaneMap& m, size_t off, uint64_t inner, uint64_t rows, int k_rows) -> int {
+    m.k_rows = k_rows;
+    if (int rc = sh_tc_encode_planes(&m.k, ws + off, inner, rows, XG_BK, k_rows)) return rc;
+    return sh_tc_encode_planes(&m.mn, ws + off, inner, rows, 64, XG_BK);
   };
   const uint64_t HD = (uint64_t)d.H * d.D;
+  const int cw = col_width(d.Dt);
   int rc;
-  if ((rc = enc(S->wqk, L->o.wqk, d.M, 2 * HD))) return rc;
-  if ((rc = enc(S->wgate, L->o.wgate, d.M, d.G))) return rc;
-  if ((rc = enc(S->wv, L->o.wv, d.M, HD * d.E))) return rc;
-  if ((rc = enc(S->wo, L->o.wo, d.D, (uint64_t)d.H * d.E * d.M))) return rc;
-  if (L->moe_q && (rc = enc(S->wq_e, L->o.wq_e, d.M, HD * d.E))) return rc;
-  if (L->moe_k && (rc = enc(S->wk_e, L->o.wk_e, d.M, HD * d.E))) return rc;
+  if ((rc = enc(S->wqk, L->o.wqk, d.M, 2 * HD, cw))) return rc;
+  if ((rc = enc(S->wgate, L->o.wgate, d.M, d.G, 64))) return rc;
+  if ((rc = enc(S->wv, L->o.wv, d.M, HD * d.E, cw))) return rc;
+  if ((rc = enc(S->wo, L->o.wo, d.D, (uint64_t)d.H * d.E * d.M, d.Dt > 128 ? XG_BN : XGemmDSmem::BN))) return rc;
+  if (L->moe_q && (rc = enc(S->wq_e, L->o.wq_e, d.M, HD * d.E, cw))) return rc;
+  if (L->moe_k && (rc = enc(S->wk_e, L->o.wk_e, d.M, HD * d.E, cw))) return rc;
   return SH_OK;
 }
 
@@ -289,8 +312,7 @@ int sh_f32_forward(sh_layer* L, const void* x, void* out, cudaStream_t st) {
   XGemmArgs g = base_args(L, x);
   use_side(g, L, 1);
   g.y = (float*)out;
-  col_tiles(g, d.M);
-  if ((rc = launch_x<X_O>(L, st, part<X_O>(L, g, d.H * head_tiles(d), g.nsub)))) return rc;
+  if ((rc = launch_d<X_O>(L, st, g))) return rc;
   sh_mark(L, 5, st);
   SH_CUDA_CHECK(cudaGetLastError());
   return SH_OK;
@@ -315,7 +337,7 @@ int sh_f32_backward(sh_layer* L, const void* x, const float* dout, float* dx, fl
   // weight gradients: how the contractions are split
   auto wpart = [](const XGemmArgs& a, int gx, int gy, int gz) { XWPart p; p.g = a; p.gx = gx; p.gy = gy; p.n = gx * gy * gz; return p; };
   XGemmArgs gq = src, gv = src, go = dst;
-  col_tiles(gq, d.Dt, XW_BN); col_tiles(gv, d.Dt, XW_BN); col_tiles(go, d.M, XW_BN);
+  col_tiles(gq, d.Dt); col_tiles(gv, d.Dt); col_tiles(go, d.M);
   gq.qk_groups = 2 * d.H;
   const int ct = gq.qk_groups * gq.nsub + (d.G + XW_BN - 1) / XW_BN;
   // parts: the shortest ones (of eight steps at least) that still fit the SMs in one round; one part each where
@@ -341,20 +363,18 @@ int sh_f32_backward(sh_layer* L, const void* x, const float* dout, float* dx, fl
   g = dst;
   col_tiles(g, d.Dt);
   // (about half of the experts' last tiles are worth counting; the rest of the table is empty)
-  g.ksplit = half_blocks(L, ((long)d.H * d.N * d.k / 128 + d.H * d.E / 2) * g.nsub, d.M / XG_BK);
+  g.ksplit = k_parts(L, ((long)d.H * d.N * d.k / 128 + d.H * d.E / 2) * g.nsub, d.M / XG_BK);
   if ((rc = launch_x<X_DA>(L, st, part<X_DA>(L, g, d.H * ht, g.nsub, g.ksplit)))) return rc;
   // attention
   rc = d.D == 32 ? launch_attn_bw_t<32>(L, w, st) : d.D == 64 ? launch_attn_bw_t<64>(L, w, st)
      : d.D == 128 ? launch_attn_bw_t<128>(L, w, st) : launch_attn_bw_t<256>(L, w, st);
   if (rc) return rc;
   // value experts: their part of dx, and the source gates' gradients
-  g = src;
-  col_tiles(g, d.M);
-  if ((rc = launch_x<X_DR>(L, st, part<X_DR>(L, g, d.H * ht, g.nsub)))) return rc;
+  if ((rc = launch_d<X_DR>(L, st, src))) return rc;
   // queries, keys and gates: the rest of dx
   g = src;
   col_tiles(g, d.M);
-  g.ksplit = half_blocks(L, (long)d.nblk * g.nsub, 2 * d.H * ((d.Dt + XG_BK - 1) / XG_BK));
+  g.ksplit = k_parts(L, (long)d.nblk * g.nsub, 2 * d.H * ((d.Dt + XG_BK - 1) / XG_BK));
   if ((rc = launch_x<X_DX>(L, st, part<X_DX>(L, g, d.nblk, g.nsub, g.ksplit)))) return rc;
   // weight gradients, one launch
   const XWPart pq = wpart(gq, mt, ct, gq.ksplit), pv = wpart(gv, d.H * d.E * gv.ksplit, gv.nsub, mt), po = wpart(go, d.H * d.E * go.ksplit, go.nsub, dt);

@@ -57,8 +57,8 @@ sh_f32_attn_kernel(const float* __restrict__ Q, const float* __restrict__ K, con
   constexpr int LD = SM::LD, KT = SM::KT, PLD = SM::PLD, KJ = KT / 16;
   constexpr int NC = D >= 64 ? D / 64 : 1;
   extern __shared__ __align__(16) float fsm[];
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  pdl_wait();
+  pdl_trigger();                                           // (behind the wait: what the next kernel reads ahead of its own is complete)
   const int tid = threadIdx.x, grp = tid >> 7, t = tid & 127, ty = t >> 4, tx = t & 15;
   float* sQ = fsm;
   float* sK = fsm + 32 * LD + grp * SM::GROUP;
@@ -264,8 +264,8 @@ sh_f32_attn_bw_kernel(const float* __restrict__ Q, const float* __restrict__ K, 
   constexpr int LD = SM::LD, TQ = SM::TQ, PLD = SM::PLD, RI = TQ / 16;
   constexpr int NC = D >= 64 ? D / 64 : 1;
   extern __shared__ __align__(16) float fsm[];
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  pdl_wait();
+  pdl_trigger();                                           // (behind the wait: what the next kernel reads ahead of its own is complete)
   const int tid = threadIdx.x, grp = tid >> 7, t = tid & 127;
   const int sy = t >> 3, sx = t & 7;                       // scores: rows sy + 16 i, keys sx + 8 j
   const int ty = t >> 4, tx = t & 15;                      // products: rows, columns 4 tx + 64 c

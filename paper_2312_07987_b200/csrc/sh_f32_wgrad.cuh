@@ -17,6 +17,70 @@
 
 namespace shtc {
 
+// acc += 16 tensor-memory columns at a time (more in flight than that costs registers the operands need).
+template <int N>
+__device__ __forceinline__ void tmem_add16(uint32_t taddr, float (&acc)[N]) {
+#pragma unroll
+  for (int c = 0; c < N; c += 16) {
+    uint32_t u[16];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+        : "=r"(u[0]), "=r"(u[1]), "=r"(u[2]), "=r"(u[3]), "=r"(u[4]), "=r"(u[5]), "=r"(u[6]), "=r"(u[7]),
+          "=r"(u[8]), "=r"(u[9]), "=r"(u[10]), "=r"(u[11]), "=r"(u[12]), "=r"(u[13]), "=r"(u[14]), "=r"(u[15])
+        : "r"(taddr + c)
+        : "memory");
+    tmem_ld_wait();
+#pragma unroll
+    for (int i = 0; i < 16; ++i) acc[c + i] += __uint_as_float(u[i]);
+  }
+}
+
+// Eight values into the three planes at byte offset `off` of the operand's tile.
+__device__ __forceinline__ void store_planes(unsigned char* tile, uint32_t off, int plane, const float (&v)[8]) {
+  uint32_t h[4], m[4], l[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) split_bf16x3(v[2 * i], v[2 * i + 1], h[i], m[i], l[i]);
+  *reinterpret_cast<uint4*>(tile + off) = make_uint4(h[0], h[1], h[2], h[3]);
+  *reinterpret_cast<uint4*>(tile + off + plane) = make_uint4(m[0], m[1], m[2], m[3]);
+  *reinterpret_cast<uint4*>(tile + off + 2 * plane) = make_uint4(l[0], l[1], l[2], l[3]);
+}
+
+// A warp's fp32 pieces of a step pass through 1 KB (64 chunks of 16 bytes) of shared memory that only this
+// warp uses: copied chunk by chunk in the order of the rows, so that an instruction covers whole 128-byte
+// lines, read as two neighbouring chunks (8 values of a row) by each lane.  Chunk c sits at c ^ (c >> 3 & 1):
+// the eight lanes of a read phase then meet eight different 16-byte banks.
+__device__ __forceinline__ uint32_t raw_chunk(int c) { return (uint32_t)((c ^ ((c >> 3) & 1)) << 4); }
+__device__ __forceinline__ void read8(float (&v)[8], const unsigned char* kb, int c) {
+  const float4 a = *reinterpret_cast<const float4*>(kb + raw_chunk(c)), b = *reinterpret_cast<const float4*>(kb + raw_chunk(c + 1));
+  v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+}
+
+// acc += the row's gate times a value: four adjacent floats at a time when the row is 16-byte aligned.
+template <int N>
+__device__ __forceinline__ void red_row(float* dst, const float (&v)[N], int valid, bool vec) {
+#pragma unroll
+  for (int i = 0; i < N; i += 4) {
+    if (vec && i + 4 <= valid) red_add_v4_f32(dst + i, v[i], v[i + 1], v[i + 2], v[i + 3]);
+    else {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) if (i + j < valid) atomicAdd(dst + i + j, v[i + j]);
+    }
+  }
+}
+template <int N>
+__device__ __forceinline__ void store_row(float* dst, const float (&v)[N], int valid, bool vec) {
+#pragma unroll
+  for (int i = 0; i < N; i += 4) {
+    if (vec && i + 4 <= valid) *reinterpret_cast<float4*>(dst + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+    else {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) if (i + j < valid) dst[i + j] = v[i + j];
+    }
+  }
+}
+
+
 struct XWgradSmem {
   static constexpr int A_PLANE = 128 * XG_BK * 2, B_PLANE = 64 * XG_BK * 2, B_HALF = 3 * B_PLANE;
   static constexpr int STAGES = 2, STAGE = 3 * A_PLANE + 2 * B_HALF;
@@ -80,7 +144,7 @@ __device__ __forceinline__ void xw_tile(const XGemmArgs& g, XTile blk) {
   }
   if (g.ksplit > 1 && kbeg >= kend) return;                // (the results are added to zeros)
   const int steps = (kend - kbeg + XG_BK - 1) / XG_BK;
-  const int chunk = xg_chunk(steps);
+  const int chunk = steps <= 8 ? 2 : 4;
   if (warp == 16) { tmem_alloc(tmem_slot, 512); tmem_relinquish(); }
   tc_fence_before();
   __syncthreads();
@@ -174,9 +238,9 @@ __device__ __forceinline__ void xw_tile(const XGemmArgs& g, XTile blk) {
           float t[16];
 #pragma unroll
           for (int i = 0; i < 16; ++i) t[i] = 0.f;
-          tmem_add<16>(tb + 128 + c0, t);                    // (smallest first)
-          tmem_add<16>(tb + 64 + c0, t);
-          tmem_add<16>(tb + c0, t);
+          tmem_add16(tb + 128 + c0, t);                    // (smallest first)
+          tmem_add16(tb + 64 + c0, t);
+          tmem_add16(tb + c0, t);
 #pragma unroll
           for (int i = 0; i < 16; ++i) acc[c0 + i] += t[i];
         }
