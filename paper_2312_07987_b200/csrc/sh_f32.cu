@@ -323,7 +323,7 @@ int sh_f32_backward(sh_layer* L, const void* x, const float* dout, float* dx, fl
   const ShDims& d = L->d;
   char* ws = L->ws;
   const BwBuffers w = bw_buffers(L);
-  const int ht = head_tiles(d), mt = (d.M + 127) / 128, dt = (d.Dt + 127) / 128;
+  const int ht = head_tiles(d), mt = (d.M + 127) / 128;
   int rc;
   L->launches = 0;
   XGemmArgs src = base_args(L, x);                         // source side; dst: destination side
@@ -337,12 +337,12 @@ int sh_f32_backward(sh_layer* L, const void* x, const float* dout, float* dx, fl
   // weight gradients: how the contractions are split
   auto wpart = [](const XGemmArgs& a, int gx, int gy, int gz) { XWPart p; p.g = a; p.gx = gx; p.gy = gy; p.n = gx * gy * gz; return p; };
   XGemmArgs gq = src, gv = src, go = dst;
-  col_tiles(gq, d.Dt); col_tiles(gv, d.Dt); col_tiles(go, d.M);
+  col_tiles(gq, d.Dt); col_tiles(gv, d.Dt); col_tiles(go, d.Dt);
   gq.qk_groups = 2 * d.H;
   const int ct = gq.qk_groups * gq.nsub + (d.G + XW_BN - 1) / XW_BN;
   // parts: the shortest ones (of eight steps at least) that still fit the SMs in one round; one part each where
   // whole contractions already need more rounds
-  const long nq = (long)mt * ct, nl = (long)d.H * d.E * (mt * gv.nsub + dt * go.nsub);
+  const long nq = (long)mt * ct, nl = (long)d.H * d.E * mt * (gv.nsub + go.nsub);
   const long sq = (d.N + XG_BK - 1) / XG_BK, sl = ((long)d.N * d.k / d.E + XG_BK - 1) / XG_BK;
   long len = sq > sl ? sq : sl;
   for (long l = 8; l < len; ++l)
@@ -377,7 +377,7 @@ int sh_f32_backward(sh_layer* L, const void* x, const float* dout, float* dx, fl
   g.ksplit = k_parts(L, (long)d.nblk * g.nsub, 2 * d.H * ((d.Dt + XG_BK - 1) / XG_BK));
   if ((rc = launch_x<X_DX>(L, st, part<X_DX>(L, g, d.nblk, g.nsub, g.ksplit)))) return rc;
   // weight gradients, one launch
-  const XWPart pq = wpart(gq, mt, ct, gq.ksplit), pv = wpart(gv, d.H * d.E * gv.ksplit, gv.nsub, mt), po = wpart(go, d.H * d.E * go.ksplit, go.nsub, dt);
+  const XWPart pq = wpart(gq, mt, ct, gq.ksplit), pv = wpart(gv, d.H * d.E * gv.ksplit, gv.nsub, mt), po = wpart(go, d.H * d.E * go.ksplit, go.nsub, mt);
   if ((rc = set_smem(sh_f32_wgrad_kernel, XWgradSmem::TOTAL))) return rc;
   if ((rc = launch_k(chained(L), sh_f32_wgrad_kernel, dim3((unsigned)(pq.n + pv.n + po.n)), dim3(XW_THREADS), XWgradSmem::TOTAL, st, pq, pv, po))) return rc;
   SH_CUDA_CHECK(cudaGetLastError());
