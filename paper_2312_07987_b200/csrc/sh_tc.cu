@@ -817,7 +817,7 @@ static int tc_forward_rest(sh_layer* L, const void* x, void* out, cudaStream_t s
       // kernel adds it to its S tiles
       const float qscale = 1.4426950408889634f / sqrtf((float)d.Dt);
       const long nkeys = (long)d.B * d.H * d.T;
-      if ((rc = launch_k(false, sh_xl_uk_kernel, dim3((unsigned)((nkeys * 8 + 255) / 256)), dim3(256), 0, st, (const __half*)(ws + L->o.k),
+      if ((rc = launch_k(pdl, sh_xl_uk_kernel, dim3((unsigned)((nkeys * 8 + 255) / 256)), dim3(256), 0, st, (const __half*)(ws + L->o.k),
                          (const float*)(ws + L->o.xl_uv), (float*)(ws + L->o.xl_uk), d.H, d.T, d.D, nkeys, qscale)))
         return rc;
       TcXlBiasArgs bg{};
@@ -826,10 +826,10 @@ static int tc_forward_rest(sh_layer* L, const void* x, void* out, cudaStream_t s
       const unsigned bgrid = (unsigned)(d.B * d.H * ((d.T - d.Tc) / 128));
       if (d.D == 128) {
         if ((rc = set_smem(sh_tc_xlbias_kernel<128>, XlBiasSmem<128>::TOTAL))) return rc;
-        if ((rc = launch_k(pdl, sh_tc_xlbias_kernel<128>, dim3(bgrid), dim3(320), XlBiasSmem<128>::TOTAL, st, S->map_q2d, S->map_r16, bg))) return rc;
+        if ((rc = launch_k(pdl, sh_tc_xlbias_kernel<128>, dim3(bgrid), dim3(192), XlBiasSmem<128>::TOTAL, st, S->map_q2d, S->map_r16, bg))) return rc;
       } else {
         if ((rc = set_smem(sh_tc_xlbias_kernel<64>, XlBiasSmem<64>::TOTAL))) return rc;
-        if ((rc = launch_k(pdl, sh_tc_xlbias_kernel<64>, dim3(bgrid), dim3(320), XlBiasSmem<64>::TOTAL, st, S->map_q2d, S->map_r16, bg))) return rc;
+        if ((rc = launch_k(pdl, sh_tc_xlbias_kernel<64>, dim3(bgrid), dim3(192), XlBiasSmem<64>::TOTAL, st, S->map_q2d, S->map_r16, bg))) return rc;
       }
       L->launches += 2;
       a.bias = (const __half*)(ws + L->o.xl_bias);
@@ -847,12 +847,12 @@ static int tc_forward_rest(sh_layer* L, const void* x, void* out, cudaStream_t s
       if ((rc = set_smem(sh_tc_attention_wide_kernel, AttnWSmem::TOTAL))) return rc;
       if ((rc = launch_k(pdl, sh_tc_attention_wide_kernel, dim3(wgrid), dim3(192), AttnWSmem::TOTAL, st, S->map_q, S->map_k, S->map_v, a))) return rc;
     } else if (d.D == 128) {
-      auto kern = halves ? sh_tc_attention3_kernel<128> : sh_tc_attention2_kernel<128>;
+      auto kern = halves ? (a.bias ? sh_tc_attention3_kernel<128, true> : sh_tc_attention3_kernel<128, false>) : sh_tc_attention2_kernel<128>;
       const int smem = halves ? Attn3Smem<128>::TOTAL : Attn2Smem<128>::TOTAL;
       if ((rc = set_smem(kern, smem))) return rc;
       if ((rc = launch_k(pdl, kern, dim3(grid), dim3(320), smem, st, S->map_q, S->map_k, S->map_v, a))) return rc;
     } else {
-      auto kern = halves ? sh_tc_attention3_kernel<64> : sh_tc_attention2_kernel<64>;
+      auto kern = halves ? (a.bias ? sh_tc_attention3_kernel<64, true> : sh_tc_attention3_kernel<64, false>) : sh_tc_attention2_kernel<64>;
       const int smem = halves ? Attn3Smem<64>::TOTAL : Attn2Smem<64>::TOTAL;
       if ((rc = set_smem(kern, smem))) return rc;
       if ((rc = launch_k(pdl, kern, dim3(grid), dim3(320), smem, st, S->map_q, S->map_k, S->map_v, a))) return rc;

@@ -28,15 +28,20 @@ struct TcAttnArgs {
   int* status;
   int balanced;          // pair query tile p with tile ntile-1-p (causal mask, grid fits the GPU in one wave)
   const __half *q, *k, *v;   // [B, H, T, D]: the wide kernel's rows once more (attnw_row)
-  const __half* bias;    // [B, H, T - Tc, T] added to the scores (Transformer-XL position and content-bias terms, log2 units), or nullptr
+  const __half* bias;    // [B, H, (T - Tc) / 128, T / 8, 128, 8] added to the scores (Transformer-XL position and content-bias terms, log2 units), or nullptr
 };
 
-// Adds 64 or 128 consecutive bias values (fp16, 16-byte aligned run of this query row) to the scores in sv.
+// A query row's bias of 8 keys at a time: 16 bytes, 128 rows apart (a warp's are 512 contiguous bytes).
+__device__ __forceinline__ const uint4* score_bias_row(const TcAttnArgs& g, int bh, int tq) {
+  const int r = tq - g.d.Tc;
+  return reinterpret_cast<const uint4*>(g.bias) + ((size_t)bh * ((g.d.T - g.d.Tc) / 128) + r / 128) * (g.d.T / 8) * 128 + r % 128;
+}
+// Adds 8 N consecutive bias values to the scores in sv.
 template <int N>
-__device__ __forceinline__ void add_score_bias(uint32_t* sv, const __half* run) {
+__device__ __forceinline__ void add_score_bias(uint32_t* sv, const uint4 (&b)[N]) {
 #pragma unroll
-  for (int i = 0; i < N / 8; ++i) {
-    const uint4 b4 = __ldg(reinterpret_cast<const uint4*>(run) + i);
+  for (int i = 0; i < N; ++i) {
+    const uint4 b4 = b[i];
     const __half2* h2 = reinterpret_cast<const __half2*>(&b4);
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
@@ -209,8 +214,13 @@ sh_tc_attention2_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_c
 #pragma unroll
       for (int c = 0; c < 4; ++c) tmem_ld32(tmem_s + lane_off + c * 32, *reinterpret_cast<uint32_t(*)[32]>(&sv[c * 32]));
       tmem_ld_wait();
-      if (g.bias && qrow[t] + r < d.T)
-        add_score_bias<128>(sv, g.bias + ((size_t)bh * (d.T - d.Tc) + (qrow[t] - d.Tc + r)) * d.T + j * 128);
+      if (g.bias) {
+        const uint4* row = score_bias_row(g, bh, qrow[t] + r) + (size_t)j * 16 * 128;
+        uint4 b[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) b[i] = __ldg(row + i * 128);
+        add_score_bias(sv, b);
+      }
       if (j == n - 1) {
         // last tile: the diagonal one (key c visible iff c <= r), or without the causal mask the
         // tile that holds the end of the sequence (keys past it were zero-filled by the loads)

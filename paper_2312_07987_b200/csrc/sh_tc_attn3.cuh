@@ -21,6 +21,8 @@
 // at that moment (it is issued when its P arrives, which can be after this half's S completed), so a
 // warp that rescales first waits for the last product issued for its tile (pv_done counts them).
 //
+// BIAS: a score bias is added (sh_tc_xlbias_kernel); a half's is loaded under the half before.
+//
 // CTA = (batch, head, two query tiles); warp roles (320 threads): warp 0 = TMA producer, warp 1 =
 // TMEM owner + UMMA issuer, warps 2..5 / 6..9 = softmax of query tile 0 / 1 (thread = query row).
 // TMEM columns: tile t: S_a at t*128, S_b at t*128 + 64, O at 256 + t*128.
@@ -39,7 +41,7 @@ struct Attn3Smem {
   static constexpr int TOTAL = BAR_OFF + 256 + 1024;
 };
 
-template <int D>
+template <int D, bool BIAS>
 __global__ void __launch_bounds__(320, 1)
 sh_tc_attention3_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapK,
                         const __grid_constant__ CUtensorMap mapV, TcAttnArgs g) {
@@ -194,6 +196,15 @@ sh_tc_attention3_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_c
     const uint32_t tmem_o = tmem + 256 + t * 128;
     float m = -INFINITY, l = 0.f;
     bool ok = true;
+    uint4 bb[8];                                           // the next half's bias
+    const uint4* brow = BIAS ? score_bias_row(g, bh, qrow[t] + r) : nullptr;
+    auto fetch_bias = [&](int half) {
+      if (BIAS && half < 2 * n) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) bb[i] = __ldg(brow + (size_t)(half * 8 + i) * 128);
+      }
+    };
+    fetch_bias(0);
     int npv = 0;                                           // products issued for this tile before the half being processed
     for (int j = 0; j < n && ok; ++j) {
 #pragma unroll
@@ -205,8 +216,10 @@ sh_tc_attention3_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_c
         tmem_ld32(tmem_s + lane_off, *reinterpret_cast<uint32_t(*)[32]>(&sv[0]));
         tmem_ld32(tmem_s + lane_off + 32, *reinterpret_cast<uint32_t(*)[32]>(&sv[32]));
         tmem_ld_wait();
-        if (g.bias && qrow[t] + r < d.T)
-          add_score_bias<64>(sv, g.bias + ((size_t)bh * (d.T - d.Tc) + (qrow[t] - d.Tc + r)) * d.T + j * 128 + 64 * x);
+        if (BIAS) {
+          add_score_bias(sv, bb);
+          fetch_bias(2 * j + x + 1);
+        }
         if (j == n - 1) {
           // last tile: the diagonal one (key c visible iff c <= r), or without the causal mask the
           // tile that holds the end of the sequence (keys past it were zero-filled by the loads)

@@ -5,15 +5,19 @@
 // S tiles, which are in the same units).  The first term is a GEMM over DISTANCES - Q[b,h] (chunk rows)
 // times R16[h]^T - whose result must be shifted, row by row, from distance order to key order (the
 // "relative shift" of Transformer-XL).  A warp-uniform TMEM address cannot shift per row, so the shift
-// happens in the store: the 32 x 32 chunk of a warp goes through shared memory and every store
-// instruction writes 32 consecutive keys of one query row (2-byte elements, coalesced).
+// happens in shared memory: a lane holds one query row's 32 distances and puts them where its keys are, in a
+// window of 64 keys of its own; 32 distances complete 32 keys of every row, with the same boundaries for all rows.
+//
+// The result is laid out for its reader, a thread of the attention kernel per query row that takes 8 keys (16 bytes) at
+// a time: [b, h, 128-row tile, key / 8, row, 8 keys], so that a warp's 16-byte pieces are 512 contiguous bytes, here and
+// there.  (In row-major order the writer stored 2 bytes per lane, 32 keys of a row at a time: 41 us at 8192 chunk tokens
+// of 1024 keys, bound by issue; and the reader's lanes met 32 different lines per load.)
 //
 // CTA = (batch*head, 128-query tile of the chunk): Q tile loaded once, 64-distance tiles of R16[h]
 // streamed through a ring of 2 (only distances up to the tile's largest query position exist), UMMA
-// N = 64 into two alternating TMEM buffers, eight epilogue warps (two per TMEM lane quarter, one
-// 32-column chunk each).  The epilogue is a chain of short latencies, so what helps is warps: the
-// CTA is sized (100 KB of shared memory) for two per SM.
-// Warp roles (320 threads): warp 0 = TMA producer, warp 1 = TMEM owner + UMMA issuer, warps 2..9 = epilogue.
+// N = 64 into two alternating TMEM buffers, four epilogue warps (a TMEM lane quarter each).  Sized (100 KB of
+// shared memory) for two CTAs per SM, which fill each other's latencies.
+// Warp roles (192 threads): warp 0 = TMA producer, warp 1 = TMEM owner + UMMA issuer, warps 2..5 = epilogue.
 #pragma once
 #include "sh_tc_prims.cuh"
 
@@ -23,7 +27,7 @@ struct TcXlBiasArgs {
   ShDims d;
   const float* vr;       // [H, T]     c * v^h . r_dist
   const float* uk;       // [B, H, T]  c * u^h . k_s
-  __half* bias;          // [B, H, T - Tc, T]
+  __half* bias;          // [B, H, (T - Tc) / 128, T / 8, 128, 8]
   int* status;
 };
 
@@ -35,13 +39,14 @@ struct XlBiasSmem {
   static constexpr int Q_OFF = 0;
   static constexpr int R_OFF = T_BYTES;
   static constexpr int STG_OFF = R_OFF + RST * R_BYTES;
-  static constexpr int STG_WARP = (32 * 33 + 64) * 4;   // the 32 x 32 chunk (padded rows) + the 63 u.k values it meets
-  static constexpr int BAR_OFF = STG_OFF + 8 * STG_WARP;
+  static constexpr int WIN_LD = 68;                       // a row's window of 64 keys: lanes' 4-byte stores (bank 69 row - column) and 16-byte loads are conflict-free
+  static constexpr int STG_WARP = (32 * WIN_LD + 64 + 64) * 4;   // windows, v.r of 64 distances, u.k of 64 keys
+  static constexpr int BAR_OFF = STG_OFF + 4 * STG_WARP;
   static constexpr int TOTAL = BAR_OFF + 256 + 1024;
 };
 
 template <int D>
-__global__ void __launch_bounds__(320, 2)
+__global__ void __launch_bounds__(192, 2)
 sh_tc_xlbias_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapR, TcXlBiasArgs g) {
   using SM = XlBiasSmem<D>;
   constexpr int DB = D / 64, RST = SM::RST;
@@ -55,7 +60,7 @@ sh_tc_xlbias_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
   uint64_t* r_full = bars + 1;       // [RST]
   uint64_t* r_empty = bars + 5;      // [RST]
   uint64_t* acc_full = bars + 9;     // [2]
-  uint64_t* acc_empty = bars + 11;   // [2] eight arrivals (epilogue warps)
+  uint64_t* acc_empty = bars + 11;   // [2] four arrivals (epilogue warps)
   uint32_t* tmem_slot = (uint32_t*)(bars + 13);
 
   const ShDims& d = g.d;
@@ -69,7 +74,7 @@ sh_tc_xlbias_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
   if (threadIdx.x == 0) {
     mbar_init(q_full, 1);
     for (int s = 0; s < RST; ++s) { mbar_init(&r_full[s], 1); mbar_init(&r_empty[s], 1); }
-    for (int b = 0; b < 2; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], 8); }
+    for (int b = 0; b < 2; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], 4); }
     fence_barrier_init();
     tma_prefetch_desc(&mapQ); tma_prefetch_desc(&mapR);
   }
@@ -114,44 +119,73 @@ sh_tc_xlbias_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
       }
     }
   } else {
-    // ---- epilogue: warp = 32 query rows (TMEM lane quarter), thread = query row while reading TMEM ----
-    const int q = warp & 3, half = (warp - 2) >> 2;
+    // ---- epilogue: warp = 32 query rows (TMEM lane quarter), thread = query row ----
+    const int q = warp & 3;
     const uint32_t lane_off = (uint32_t)(q * 32) << 16;
-    float* stg = reinterpret_cast<float*>(sgen + SM::STG_OFF + (warp - 2) * SM::STG_WARP);
-    float* suk = stg + 32 * 33;
-    const int qi0 = it * 128 + q * 32;                     // first query row (inside the chunk) of this warp
-    __half* out_bh = g.bias + (size_t)bh * Tq * d.T;
+    float* win = reinterpret_cast<float*>(sgen + SM::STG_OFF + (warp - 2) * SM::STG_WARP);
+    float* svr = win + 32 * SM::WIN_LD;
+    float* suk = svr + 64;
+    float* wrow = win + lane * SM::WIN_LD;
+    const int p0 = d.Tc + it * 128 + q * 32;               // position of this warp's first row
+    uint4* out = reinterpret_cast<uint4*>(g.bias) + ((size_t)bh * tiles_q + it) * (d.T / 8) * 128 + q * 32 + lane;   // + 128 per 8 keys
     const float* vr = g.vr + (size_t)h * d.T;
     const float* ukr = g.uk + (size_t)bh * d.T;
     for (int ct = 0; ct < ncol; ++ct) {
       const int b = ct & 1;
+      // v.r of the tile's distances and u.k of the keys it completes: p0 - 64 ct - 32 ... + 63
+      const int kb = p0 - ct * 64 - 32;
+      reinterpret_cast<float2*>(svr)[lane] = __ldg(reinterpret_cast<const float2*>(vr + ct * 64) + lane);
+      suk[lane] = kb + lane >= 0 ? __ldg(ukr + kb + lane) : 0.f;
+      suk[32 + lane] = kb + 32 + lane >= 0 ? __ldg(ukr + kb + 32 + lane) : 0.f;
+      __syncwarp();
       if (!mbar_wait(&acc_full[b], (ct >> 1) & 1, g.status, dead)) break;
       tc_fence_after();
-      {
-        const int dist0 = ct * 64 + half * 32;             // this warp's 32 distances of the tile
-        const int s_lo = d.Tc + qi0 - dist0 - 31;          // keys this chunk meets: s_lo .. s_lo + 62
-        const float vrd = vr[dist0 + lane];
-        const float uk0 = (s_lo + lane >= 0) ? ukr[s_lo + lane] : 0.f;
-        const float uk1 = (s_lo + 32 + lane >= 0 && s_lo + 32 + lane < d.T) ? ukr[s_lo + 32 + lane] : 0.f;
-        uint32_t v[32];
-        tmem_ld32(tmem + lane_off + b * 64 + half * 32, v);
-        tmem_ld_wait();
-        tc_fence_before();                                 // this warp's share of the accumulator is in registers
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&acc_empty[b]);
 #pragma unroll
-        for (int i = 0; i < 32; ++i) stg[lane * 33 + i] = __uint_as_float(v[i]);
-        suk[lane] = uk0;
-        suk[32 + lane] = uk1;
-        __syncwarp();
-        __half* op = out_bh + ((long)qi0 * d.T + (s_lo + 31 - lane));   // row qi0 + rr, key s_lo + 31 + rr - lane: += T + 1 per row
-        const int s0 = s_lo + 31 - lane;
-#pragma unroll 8
-        for (int rr = 0; rr < 32; ++rr) {
-          if (s0 + rr >= 0) op[(long)rr * (d.T + 1)] = __float2half_rn(stg[rr * 33 + lane] + vrd + suk[31 + rr - lane]);
+      for (int hh = 0; hh < 2; ++hh) {
+        // 32 distances from dist0 on: keys base + lane - c.  Those from base on (c <= lane) complete the 32 keys from base
+        // on - the distances before left the rest -, those below start the 32 before; base is a multiple of 32
+        const int base = p0 - ct * 64 - hh * 32;
+        float* hi = wrow + (base & 32) + lane;
+        float* lo = wrow + ((base & 32) ^ 32) + 32 + lane;
+        uint32_t v[32];
+        tmem_ld32(tmem + lane_off + b * 64 + hh * 32, v);
+        tmem_ld_wait();
+        if (hh == 1) {
+          tc_fence_before();                               // this warp's share of the accumulator is in registers
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&acc_empty[b]);
         }
-        __syncwarp();
+#pragma unroll
+        for (int c = 0; c < 32; c += 4) {
+          const float4 r4 = *reinterpret_cast<const float4*>(svr + hh * 32 + c);
+          const float2 a = __fadd2_rn(make_float2(__uint_as_float(v[c]), __uint_as_float(v[c + 1])), make_float2(r4.x, r4.y));
+          const float2 e = __fadd2_rn(make_float2(__uint_as_float(v[c + 2]), __uint_as_float(v[c + 3])), make_float2(r4.z, r4.w));
+          (lane >= c ? hi : lo)[-c] = a.x;
+          (lane >= c + 1 ? hi : lo)[-c - 1] = a.y;
+          (lane >= c + 2 ? hi : lo)[-c - 2] = e.x;
+          (lane >= c + 3 ? hi : lo)[-c - 3] = e.y;
+        }
+        // (a row's own window: no other lane is involved)
+        if (base >= 0) {
+          const float* full = wrow + (base & 32);
+          const float* uk = suk + 32 - hh * 32;
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const float4 w0 = *reinterpret_cast<const float4*>(full + 8 * i), w1 = *reinterpret_cast<const float4*>(full + 8 * i + 4);
+            const float4 u0 = *reinterpret_cast<const float4*>(uk + 8 * i), u1 = *reinterpret_cast<const float4*>(uk + 8 * i + 4);
+            __half2 o[4];
+            o[0] = __float22half2_rn(__fadd2_rn(make_float2(w0.x, w0.y), make_float2(u0.x, u0.y)));
+            o[1] = __float22half2_rn(__fadd2_rn(make_float2(w0.z, w0.w), make_float2(u0.z, u0.w)));
+            o[2] = __float22half2_rn(__fadd2_rn(make_float2(w1.x, w1.y), make_float2(u1.x, u1.y)));
+            o[3] = __float22half2_rn(__fadd2_rn(make_float2(w1.z, w1.w), make_float2(u1.z, u1.w)));
+            uint4 w;
+            w.x = *reinterpret_cast<uint32_t*>(&o[0]); w.y = *reinterpret_cast<uint32_t*>(&o[1]);
+            w.z = *reinterpret_cast<uint32_t*>(&o[2]); w.w = *reinterpret_cast<uint32_t*>(&o[3]);
+            out[(size_t)(base / 8 + i) * 128] = w;
+          }
+        }
       }
+      __syncwarp();                                        // (v.r and u.k of the next tile)
     }
   }
   tc_fence_before();
