@@ -57,12 +57,13 @@ static void layout_workspace(sh_layer* L) {
   const size_t slots = (size_t)2 * d.N * d.H * d.k;
   o.idx = take(slots * 4);
   o.gate = take(slots * 4);
-  // (a layer whose value projection is tiled by expert pairs sorts H * E(E-1)/2 buckets in a forward pass)
-  const bool vp = sh_v_pairs_ok(L);
-  const size_t hist = vp && 2 * d.H * sh_pair_count(d.E) > d.G ? (size_t)2 * d.H * sh_pair_count(d.E) : (size_t)d.G;
+  // (a layer whose value projection is tiled by sets of experts sorts H * choose(E, k) buckets in a forward pass)
+  const bool vp = sh_v_sets_ok(L);
+  const size_t nset = vp ? sh_choose(d.E, d.k) : 0;
+  const size_t hist = 2 * d.H * nset > (size_t)d.G ? 2 * d.H * nset : (size_t)d.G;
   o.blockcnt = take((size_t)d.nblk * hist * 4);
   o.blockoff = take((size_t)d.nblk * hist * 4);
-  o.offsets = take(((size_t)2 * d.H * (d.E + 1) + (vp ? (size_t)2 * d.H * (sh_pair_count(d.E) + 1) : 0)) * 4);
+  o.offsets = take(((size_t)2 * d.H * (d.E + 1) + (vp ? (size_t)2 * d.H * (nset + 1) : 0)) * 4);
   o.lists = take(slots * 4);
   o.lgate = take(slots * 4);
   o.tiles = take((size_t)2 * d.max_tiles * sizeof(ShTile));
@@ -192,7 +193,7 @@ static int configure_common(sh_layer* L, int dtype, int batch, int seq, int cach
   L->dtype = dtype;
   L->d.B = batch; L->d.T = T; L->d.Tc = cache_len; L->d.N = batch * T;
   L->d.nblk = (L->d.N + SH_TILE_ROWS - 1) / SH_TILE_ROWS;
-  L->d.max_tiles = (int)((slots + SH_TILE_ROWS - 1) / SH_TILE_ROWS) + d0.H * d0.E + d0.H * sh_pair_count(d0.E > 8 ? 2 : d0.E);
+  L->d.max_tiles = (int)((slots + SH_TILE_ROWS - 1) / SH_TILE_ROWS) + d0.H * d0.E + d0.H * 35;   // (up to 35 sets of experts: sh_v_sets_ok)
   L->d.tile_rows_src = SH_TILE_ROWS;
   // (k >= 3: the fp16 reductions of a value row arrive in a different order from run to run - two
   //  passes have been seen 1e-2 of the output RMS apart; with the first rows, which reach the output

@@ -31,14 +31,33 @@ struct ShDims {
   int* status;             // the status block at the start of the workspace (nullptr: the allocation-free gate entry point)
 };
 
-// Unordered pairs {a < b} of E experts, numbered row by row: (0,1), (0,2), ..., (0,E-1), (1,2), ...
-// (the value projection of a k = 2 layer is tiled by (head, pair): sh_tc_vpair_kernel).
-__host__ __device__ __forceinline__ int sh_pair_count(int E) { return E * (E - 1) / 2; }
-__host__ __device__ __forceinline__ int sh_pair_id(int a, int b, int E) { return a * (2 * E - a - 1) / 2 + (b - a - 1); }
-__host__ __device__ __forceinline__ void sh_pair_decode(int id, int E, int& a, int& b) {
-  a = 0;
-  while (a < E - 2 && id >= E - 1 - a) { id -= E - 1 - a; ++a; }
-  b = a + 1 + id;
+// Sets of k <= 4 experts {e0 < e1 < ...} of E, numbered: pairs row by row, (0,1), (0,2), ..., (0,E-1), (1,2), ..., larger
+// sets by sum of choose(e_i, i + 1) (the value projection of such a layer is tiled by (head, set): sh_tc_vset_kernel).
+__host__ __device__ __forceinline__ int sh_choose(int n, int k) {
+  return k == 1 ? n : k == 2 ? n * (n - 1) / 2 : k == 3 ? n * (n - 1) * (n - 2) / 6 : k == 4 ? n * (n - 1) * (n - 2) * (n - 3) / 24 : 0;
+}
+#ifdef __CUDACC__
+__device__ __forceinline__ int sh_set_id(unsigned mask, int k, int E) {     // k >= 2 bits
+  const int lo = __ffs(mask) - 1, hi = 31 - __clz(mask);
+  if (k == 2) return lo * (2 * E - lo - 1) / 2 + (hi - lo - 1);
+  const unsigned rest = mask & ~(1u << lo) & ~(1u << hi);
+  int id = lo + sh_choose(hi, k) + sh_choose(__ffs(rest) - 1, 2);
+  if (k > 3) id += sh_choose(31 - __clz(rest), 3);
+  return id;
+}
+#endif
+__host__ __device__ __forceinline__ void sh_set_decode(int id, int k, int E, int* e) {
+  if (k == 2) {
+    e[0] = 0;
+    while (e[0] < E - 2 && id >= E - 1 - e[0]) { id -= E - 1 - e[0]; ++e[0]; }
+    e[1] = e[0] + 1 + id;
+    return;
+  }
+  for (int i = k, n = E - 1; i >= 1; --i) {
+    while (n > i - 1 && sh_choose(n, i) > id) --n;
+    e[i - 1] = n;
+    id -= sh_choose(n--, i);
+  }
 }
 
 // With a cache in front of every sequence (ShDims::Tc): the row of `out` that belongs to context token
@@ -138,11 +157,17 @@ inline bool sh_o_sparse_ok(const sh_layer* L) {
   return L->dtype == SH_BF16 && !L->dense && d.k <= 2 && (d.E == 4 || d.E == 8) && d.D == 128 && d.H <= 4;
 }
 
-// Shapes whose value projection is tiled by (head, pair of selected experts) instead of (head, expert):
-// k = 2, so every (token, head) belongs to exactly one pair; few enough pairs for the sort's 32-bit masks.
-inline bool sh_v_pairs_ok(const sh_layer* L) {
+// Shapes whose value projection is tiled by (head, set of selected experts) instead of (head, expert): the k experts of a
+// set side by side are at most 256 columns, and there are few enough sets for their partly filled tiles - half a tile of
+// 256 rows each, on two SMs, against half a tile of 128 per expert - not to cost more than the k - 1 further gathers of
+// every row.
+inline bool sh_v_sets_ok(const sh_layer* L) {
   const ShDims& d = L->d;
-  return L->dtype == SH_BF16 && !L->dense && d.k == 2 && d.E >= 2 && d.E <= 8 && d.D == 128;
+  if (L->dtype != SH_BF16 || L->dense || d.k < 2 || d.k > 4 || d.E < d.k) return false;
+  const int sets = d.E <= 16 ? sh_choose(d.E, d.k) : 1 << 20;
+  if (d.k == 2 && d.D == 128) return sets <= 28;
+  if (d.D != 64 || sets > 35 || L->moe_q || L->moe_k) return false;
+  return 128l * sets - 64l * d.E <= (long)d.N * (d.k - 1);
 }
 
 template <typename T> __device__ __forceinline__ float sh_to_float(T v);

@@ -15,7 +15,7 @@
 #include "sh_tc_qkpair.cuh"
 #include "sh_tc_xlbias.cuh"
 #include "sh_tc_oproj_sp.cuh"
-#include "sh_tc_vpair.cuh"
+#include "sh_tc_vset.cuh"
 #include "sh_tc_front.cuh"
 
 using namespace shtc;
@@ -104,7 +104,7 @@ static int encode_3d_f16_store32(CUtensorMap* map, const void* base, uint64_t in
 struct TcState {
   CUtensorMap map_q, map_k, map_v;
   CUtensorMap map_q_st, map_k_st;   // Q and K as the one-grid front's epilogue stores them
-  CUtensorMap map_wqk, map_wqk128, map_wv, map_wq_e, map_wk_e, map_wo, map_wo256, map_wo_tail, map_ahat_tail, map_wos, map_wo_n[2], map_wos_n[2], map_ahat, map_wgate;
+  CUtensorMap map_wqk, map_wqk128, map_wv, map_wv32, map_wq_e, map_wk_e, map_wo, map_wo256, map_wo_tail, map_ahat_tail, map_wos, map_wo_n[2], map_wos_n[2], map_ahat, map_wgate;
   CUtensorMap map_q2d, map_r16;  // score-bias GEMM of the Transformer-XL position term: Q as [B*H*T, D], R16 as [H*T, D]
   CUtensorMap map_x;             // tensor map of the last x pointer seen (x_cached)
   CUtensorMap map_x64;           // the same tensor in 64-token boxes (gate tile of the one-grid front, 64 tokens per CTA)
@@ -126,8 +126,8 @@ struct TcState {
   bool qk_two_grids = true; // ... as two grids around the gate kernel
   bool qk_pair = true;      // CTA-pair Q/K kernel (else single-CTA persistent)
   bool o_pair = true;       // CTA-pair output projection for k <= 3 (else single-CTA)
-  bool v_pairs = true;      // value projection tiled by (head, expert pair) on CTA pairs where the shape allows (sh_v_pairs_ok)
-  int v_pairs_max = 0;      // clusters of that kernel the device holds at once (0: not asked yet, -1: none)
+  bool v_sets = true;      // value projection tiled by (head, set of selected experts) on CTA pairs where the shape allows (sh_v_sets_ok)
+  int v_clusters_max = 0;      // clusters of that kernel the device holds at once (0: not asked yet, -1: none)
   bool o_sparse = true;     // sparse-A CTA-pair output projection where the shape allows (sh_o_sparse_ok)
   bool persistent = true;   // persistent Q/K and value-expert GEMMs (else one CTA per tile)
   bool fused_sort = true;   // sort fused into the gate kernel when it needs at most half of the SMs
@@ -199,7 +199,7 @@ int sh_tc_prepare(sh_layer* L) {
   S->qk_pair = !getenv("SH_QK_SINGLE");
   S->o_pair = !getenv("SH_O_SINGLE");
   S->o_sparse = !getenv("SH_O_MASKED");
-  S->v_pairs = !getenv("SH_V_BY_EXPERT");
+  S->v_sets = !getenv("SH_V_BY_EXPERT");
   S->persistent = !getenv("SH_NO_PERSISTENT");
   S->fused_sort = !getenv("SH_SORT_SEPARATE");
   S->one_grid_front = !getenv("SH_NO_FRONT");
@@ -241,6 +241,7 @@ int sh_tc_prepare(sh_layer* L) {
   if ((rc = sh_tc_encode_2d(&S->map_wqk128, 0, ws + L->o.wqk, d.M, (uint64_t)nproj * HD, (uint64_t)d.M * 2, 64, 128))) return rc;
   if (!L->dense) {
     if ((rc = sh_tc_encode_2d(&S->map_wv, 0, ws + L->o.wv, d.M, (uint64_t)d.H * d.E * d.D, (uint64_t)d.M * 2, 64, d.D > 128 ? (d.Dt + 15) / 16 * 16 : d.D))) return rc;
+    if (d.D == 64 && (rc = sh_tc_encode_2d(&S->map_wv32, 0, ws + L->o.wv, d.M, (uint64_t)d.H * d.E * d.D, (uint64_t)d.M * 2, 64, 32))) return rc;
     if (L->moe_q && (rc = sh_tc_encode_2d(&S->map_wq_e, 0, ws + L->o.wq_e, d.M, (uint64_t)d.H * d.E * d.D, (uint64_t)d.M * 2, 64, d.D))) return rc;
     if (L->moe_k && (rc = sh_tc_encode_2d(&S->map_wk_e, 0, ws + L->o.wk_e, d.M, (uint64_t)d.H * d.E * d.D, (uint64_t)d.M * 2, 64, d.D))) return rc;
     if ((rc = sh_tc_encode_2d(&S->map_wo, 1, ws + L->o.wo, d.D, (uint64_t)d.H * d.E * d.M, (uint64_t)d.D * 2, 64, 128))) return rc;
@@ -302,20 +303,22 @@ static int gate_smem_bytes(int Gp, int G, int stages) {   // G: histogram width 
   return bar_off + 256 + 3 * G * 4 + 1024;
 }
 
-using VPS = VPairSmem<6>;
-// Forward passes of a k = 2 layer tile the value projection by (head, pair of selected experts): the gate
-// kernel then buckets the source side by pair, and sh_tc_vpair_kernel replaces the expert-tiled kernel.
-static bool use_v_pairs(sh_layer* L) {
+using VPS = VSetSmem<6>;
+// The set-tiled value kernel of a layer: kern(kernel) for its k and stored d_head.
+template <typename F>
+static auto with_vset(const ShDims& d, F f) {
+  if (d.D == 128) return f(sh_tc_vset_kernel<6, 2, 128>);
+  return d.k == 2 ? f(sh_tc_vset_kernel<6, 2, 64>) : d.k == 3 ? f(sh_tc_vset_kernel<6, 3, 64>) : f(sh_tc_vset_kernel<6, 4, 64>);
+}
+// Forward passes of such a layer tile the value projection by (head, set of selected experts): the gate
+// kernel then buckets the source side by set, and sh_tc_vset_kernel replaces the expert-tiled kernel.
+static bool use_v_sets(sh_layer* L) {
   TcState* S = (TcState*)L->tc;
-  if (!S->v_pairs || !sh_v_pairs_ok(L) || !S->gate_gp || (S->simt_mask & (SH_STAGE_GATE | SH_STAGE_V))) return false;
-  if (S->v_pairs_max == 0) {
-    if (set_smem(sh_tc_vpair_kernel<6>, VPS::TOTAL) != SH_OK) S->v_pairs_max = -1;
-    else {
-      S->v_pairs_max = max_pairs(sh_tc_vpair_kernel<6>, 320, VPS::TOTAL);
-      if (S->v_pairs_max <= 0) S->v_pairs_max = -1;
-    }
-  }
-  return S->v_pairs_max > 0;
+  if (!S->v_sets || !sh_v_sets_ok(L) || !S->gate_gp || (S->simt_mask & (SH_STAGE_GATE | SH_STAGE_V))) return false;
+  if (S->v_clusters_max == 0)
+    S->v_clusters_max = with_vset(L->d, [&](auto kern) { return set_smem(kern, VPS::TOTAL) == SH_OK ? max_pairs(kern, 320, VPS::TOTAL) : 0; });
+  if (S->v_clusters_max <= 0) S->v_clusters_max = -1;
+  return S->v_clusters_max > 0;
 }
 
 // Gate + top-k + bucket sort.  With zero_for_forward the gate kernel also clears the value buffer.
@@ -356,10 +359,10 @@ static int tc_gate_sort(sh_layer* L, const void* x, void* out, bool zero_for_for
   g.d = d; g.Gp = S->gate_gp; g.gbias = (const float*)(ws + L->o.gbias);
   g.idx = (int*)(ws + L->o.idx); g.gate = (float*)(ws + L->o.gate);
   g.blockcnt = (int*)(ws + L->o.blockcnt);
-  const bool vp = zero_for_forward && use_v_pairs(L);
+  const bool vp = zero_for_forward && use_v_sets(L);
   // (query experts are tiled by the DESTINATION side's pairs: then both sides are bucketed by pair)
-  g.vpairs = vp ? ((L->moe_q && d.sides == 2) ? 2 : 1) : 0;
-  g.NP = sh_pair_count(d.E); g.GH = vp ? g.vpairs * d.H * g.NP : d.G; g.gid = (int*)(ws + L->o.gid);
+  g.vsets = vp ? ((L->moe_q && d.sides == 2) ? 2 : 1) : 0;
+  g.NS = sh_choose(d.E, d.k); g.GH = vp ? g.vsets * d.H * g.NS : d.G; g.gid = (int*)(ws + L->o.gid);
   const int GHmax = g.GH > d.G ? g.GH : d.G;
   g.zero_v = (zero_for_forward && !vp) ? (void*)(ws + L->o.v) : nullptr;    // (the pair-tiled kernel stores every value row once)
   g.zero_out = (zero_for_forward && (S->simt_mask & SH_STAGE_O) && d.Tc == 0) ? (float*)out : nullptr;
@@ -375,7 +378,7 @@ static int tc_gate_sort(sh_layer* L, const void* x, void* out, bool zero_for_for
   // sort's loops run over sides * H groups.
   ShDims ds = d;
   if (zero_for_forward && !(S->simt_mask & SH_STAGE_O)) ds.sides = 1;
-  if (vp) { ds.sides = g.vpairs; ds.E = g.NP; ds.k = 1; ds.G = g.GH; ds.tile_rows_src = 256; }   // buckets (side, head, pair), one entry per (token, head)
+  if (vp) { ds.sides = g.vsets; ds.E = g.NS; ds.k = 1; ds.G = g.GH; ds.tile_rows_src = 256; }   // buckets (side, head, pair), one entry per (token, head)
   // Fused sort: when every CTA of the gate kernel can be resident at once (cooperative launch) and the
   // sort's scratch fits behind the logits tile in the idle operand ring, the gate kernel places the
   // tokens itself and there is no sort kernel.  Used when the gate kernel needs at most half of the SMs:
@@ -463,10 +466,10 @@ static bool front_plan(sh_layer* L) {
   if (!S->one_grid_front || L->dense || L->moe_q || L->moe_k || S->simt_mask || !S->gate_gp || S->qk_bn != 256 ||
       !S->persistent || !S->qk_pair)
     return false;
-  const bool vp = use_v_pairs(L);
+  const bool vp = use_v_sets(L);
   ShDims ds = d;
   ds.sides = 1;
-  if (vp) { ds.sides = 1; ds.E = sh_pair_count(d.E); ds.k = 1; ds.G = d.H * ds.E; }
+  if (vp) { ds.sides = 1; ds.E = sh_choose(d.E, d.k); ds.k = 1; ds.G = d.H * ds.E; }
   const int GH = vp ? ds.G : d.G;
   S->front_sort_bytes = (int)(vp ? sh_sort_smem_bytes(ds) : sh_sort_smem_bytes(d));
   int dev = 0, coop = 0, optin = 0;
@@ -513,9 +516,9 @@ static int tc_front(sh_layer* L, const void* x, cudaStream_t st) {
   g.d = d; g.Gp = S->gate_gp; g.gbias = (const float*)(ws + L->o.gbias);
   g.idx = (int*)(ws + L->o.idx); g.gate = (float*)(ws + L->o.gate);
   g.blockcnt = (int*)(ws + L->o.blockcnt);
-  const bool vp = use_v_pairs(L);
-  g.vpairs = vp ? 1 : 0;
-  g.NP = sh_pair_count(d.E); g.GH = vp ? d.H * g.NP : d.G; g.gid = (int*)(ws + L->o.gid);
+  const bool vp = use_v_sets(L);
+  g.vsets = vp ? 1 : 0;
+  g.NS = sh_choose(d.E, d.k); g.GH = vp ? d.H * g.NS : d.G; g.gid = (int*)(ws + L->o.gid);
   g.zero_v = vp ? nullptr : (void*)(ws + L->o.v);          // (the pair-tiled kernel stores every value row once)
   g.zero_out = nullptr;
   g.status = status;
@@ -633,8 +636,8 @@ int sh_tc_forward(sh_layer* L, const void* x, void* out, cudaStream_t st) {
   if (L->moe_q || L->moe_k) {
     // expert projections of keys / queries run on the pair-tiled kernel (pair-bucketed lists), or - debug
     // library, SH_SIMT_STAGES - on the CUDA-core kernels together with gate and value stage (expert lists)
-    const bool bad = (simt & SH_STAGE_QK) ? use_v_pairs(L)
-                                          : (!use_v_pairs(L) || !S->persistent || !S->qk_pair || qk_pairs_max(S) <= 0);
+    const bool bad = (simt & SH_STAGE_QK) ? use_v_sets(L)
+                                          : (!use_v_sets(L) || !S->persistent || !S->qk_pair || qk_pairs_max(S) <= 0);
     if (bad) {
       sh_set_error("query / key experts need the CTA-pair projection kernels on this device and in this build");
       return SH_ERR_UNSUPPORTED;
@@ -743,25 +746,26 @@ static int tc_forward_rest(sh_layer* L, const void* x, void* out, cudaStream_t s
   if (!L->dense) {
     if (simt & SH_STAGE_V) {
       if ((rc = sh_simt_run_bf16(L, SH_STAGE_V, x, out, st))) return rc;
-    } else if (use_v_pairs(L)) {
-      TcVPairArgs g{};
+    } else if (use_v_sets(L)) {
+      TcVSetArgs g{};
       g.d = d; g.x = x; g.lists = (const int*)(ws + L->o.lists);
       g.tiles = (const ShTile*)(ws + L->o.tiles); g.ntiles = (const int*)(ws + L->o.ntiles);
       g.idx = (const int*)(ws + L->o.idx); g.gate = (const float*)(ws + L->o.gate);
       g.v = (__half*)(ws + L->o.v); g.status = status;
-      const int bound = (d.N * d.H + 255) / 256 + d.H * sh_pair_count(d.E);       // tiles: at most this many
-      const unsigned pgrid = 2u * (unsigned)(bound < S->v_pairs_max ? bound : S->v_pairs_max);
+      const int bound = (d.N * d.H + 255) / 256 + d.H * sh_choose(d.E, d.k);       // tiles: at most this many
+      const unsigned pgrid = 2u * (unsigned)(bound < S->v_clusters_max ? bound : S->v_clusters_max);
       g.scale = 0.f; g.stamp_id = SH_K_V;
-      // (behind the one-grid front: wait for the sort's counter, not for the grid - see sh_tc_vpair_kernel)
+      // (behind the one-grid front: wait for the sort's counter, not for the grid - see sh_tc_vset_kernel)
       if (front && pdl) { g.ready = status + SH_ST_SORTED; g.ready_count = d.nblk; }
-      if ((rc = launch_k_pairs(pdl, sh_tc_vpair_kernel<6>, dim3(pgrid), dim3(320), VPS::TOTAL, st, S->map_wv, g))) return rc;
+      const CUtensorMap& wmap = d.k == 3 ? S->map_wv32 : S->map_wv;
+      if ((rc = with_vset(d, [&](auto kern) { return launch_k_pairs(pdl, kern, dim3(pgrid), dim3(320), VPS::TOTAL, st, wmap, g); }))) return rc;
       g.ready = nullptr;
       L->launches += 1;
       // key / query experts: the same kernel with the key (query) experts' weights, the source
       // (destination) side's pair tiles and gates, into the K (Q) buffer; queries carry the score scale
       if (L->moe_k && !(simt & SH_STAGE_QK)) {
         g.v = (__half*)(ws + L->o.k); g.stamp_id = -1;
-        if ((rc = launch_k_pairs(pdl, sh_tc_vpair_kernel<6>, dim3(pgrid), dim3(320), VPS::TOTAL, st, S->map_wk_e, g))) return rc;
+        if ((rc = launch_k_pairs(pdl, sh_tc_vset_kernel<6, 2, 128>, dim3(pgrid), dim3(320), VPS::TOTAL, st, S->map_wk_e, g))) return rc;
         L->launches += 1;
       }
       if (L->moe_q && !(simt & SH_STAGE_QK)) {
@@ -771,7 +775,7 @@ static int tc_forward_rest(sh_layer* L, const void* x, void* out, cudaStream_t s
         g.ntiles = (const int*)(ws + L->o.ntiles) + s1;
         g.idx = (const int*)(ws + L->o.idx) + s1 * (size_t)d.N * d.H * d.k; g.gate = (const float*)(ws + L->o.gate) + s1 * (size_t)d.N * d.H * d.k;
         g.v = (__half*)(ws + L->o.q); g.scale = 1.4426950408889634f / sqrtf((float)d.Dt); g.stamp_id = -1;
-        if ((rc = launch_k_pairs(pdl, sh_tc_vpair_kernel<6>, dim3(pgrid), dim3(320), VPS::TOTAL, st, S->map_wq_e, g))) return rc;
+        if ((rc = launch_k_pairs(pdl, sh_tc_vset_kernel<6, 2, 128>, dim3(pgrid), dim3(320), VPS::TOTAL, st, S->map_wq_e, g))) return rc;
         L->launches += 1;
       }
     } else {

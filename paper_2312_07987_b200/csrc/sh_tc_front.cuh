@@ -394,7 +394,6 @@ sh_tc_front_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_consta
           const int side = grp / d.H, h = grp % d.H;
           const size_t o = (((size_t)side * d.N + t) * d.H + h) * d.k;
           unsigned taken = 0;
-          int first = 0;
           for (int j = 0; j < d.k; ++j) {
             int best = -1;
             float bz = 0.f;
@@ -407,13 +406,12 @@ sh_tc_front_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_consta
             const float gv = 1.f / (1.f + expf(-bz));
             gg.idx[o + j] = best;
             gg.gate[o + j] = gv;
-            if (gg.vpairs) {
-              if (j == 0) first = best;
-              else if (side < gg.vpairs) {
-                const int pid = sh_pair_id(min(first, best), max(first, best), d.E);
-                gg.gid[((size_t)side * d.N + t) * d.H + h] = pid;
-                s_idx[side * 128 * d.H + r * d.H + h] = pid;
-                atomicAdd(&s_hist[(side * d.H + h) * gg.NP + pid], 1);
+            if (gg.vsets) {
+              if (j == d.k - 1 && side < gg.vsets) {
+                const int sid = sh_set_id(taken, d.k, d.E);
+                gg.gid[((size_t)side * d.N + t) * d.H + h] = sid;
+                s_idx[side * 128 * d.H + r * d.H + h] = sid;
+                atomicAdd(&s_hist[(side * d.H + h) * gg.NS + sid], 1);
               }
               continue;
             }
@@ -449,7 +447,7 @@ sh_tc_front_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_consta
     if (*(volatile int*)s_flag) {
       ShDims ds = d;
       ds.sides = gg.sort_sides;
-      if (gg.vpairs) { ds.sides = gg.vpairs; ds.E = gg.NP; ds.k = 1; ds.G = gg.GH; }   // buckets (side, head, pair), one entry per (token, head)
+      if (gg.vsets) { ds.sides = gg.vsets; ds.E = gg.NS; ds.k = 1; ds.G = gg.GH; }   // buckets (side, head, set), one entry per (token, head)
       ds.tile_rows_src = gg.tile_rows_src;
       sh_sort_block(gg.idx, gg.gate, gg.blockcnt, gg.offsets, gg.lists, gg.lgate, gg.tiles, gg.ntiles, ds, s_sort, et, NSEL, blk, true, sel_sync);
     }

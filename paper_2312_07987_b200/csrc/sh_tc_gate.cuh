@@ -40,12 +40,12 @@ struct TcGateArgs {
   int* offsets; int* lists; float* lgate; ShTile* tiles; int* ntiles;
   int* gridbar;              // {arrived, departed}, both 0 between launches
   // value projection tiled by expert PAIRS (k = 2, forward pass only): the source side is bucketed by
-  // (head, pair number) - histogram, sort and tile table run over H * NP buckets with one entry per
+  // (head, set number) - histogram, sort and tile table run over H * NS buckets with one entry per
   // (token, head) - and the destination side is not bucketed at all
-  int vpairs;                // 0, or the number of sides bucketed by pair: 1 = the source side, 2 = both (query experts)
-  int NP;                    // pairs per head: E (E - 1) / 2
-  int GH;                    // histogram width: vpairs ? vpairs * H * NP : G
-  int* gid;                  // [vpairs, N, H] pair number of every (token, head)
+  int vsets;                // 0, or the number of sides bucketed by set of selected experts: 1 = the source side, 2 = both (query experts)
+  int NS;                    // sets per head: choose(E, k)
+  int GH;                    // histogram width: vsets ? vsets * H * NS : G
+  int* gid;                  // [vsets, N, H] set number of every (token, head)
 };
 
 constexpr int GATE_THREADS = 608;
@@ -198,7 +198,6 @@ sh_tc_gate_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constan
           const int side = grp / d.H, h = grp % d.H;
           const size_t o = (((size_t)side * d.N + t) * d.H + h) * d.k;
           unsigned taken = 0;
-          int first = 0;
           for (int j = 0; j < d.k; ++j) {
             int best = -1;
             float bz = 0.f;
@@ -211,13 +210,12 @@ sh_tc_gate_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constan
             const float gv = 1.f / (1.f + expf(-bz));
             g.idx[o + j] = best;
             g.gate[o + j] = gv;
-            if (g.vpairs) {
-              if (j == 0) first = best;
-              else if (side < g.vpairs) {
-                const int pid = sh_pair_id(min(first, best), max(first, best), d.E);
-                g.gid[((size_t)side * d.N + t) * d.H + h] = pid;
-                if (g.fused) s_idx[side * 128 * d.H + r * d.H + h] = pid;
-                atomicAdd(&s_hist[(side * d.H + h) * g.NP + pid], 1);
+            if (g.vsets) {
+              if (j == d.k - 1 && side < g.vsets) {
+                const int sid = sh_set_id(taken, d.k, d.E);
+                g.gid[((size_t)side * d.N + t) * d.H + h] = sid;
+                if (g.fused) s_idx[side * 128 * d.H + r * d.H + h] = sid;
+                atomicAdd(&s_hist[(side * d.H + h) * g.NS + sid], 1);
               }
               continue;
             }
@@ -257,7 +255,7 @@ sh_tc_gate_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constan
       if (*(volatile int*)s_flag) {
         ShDims ds = d;
         ds.sides = g.sort_sides;
-        if (g.vpairs) { ds.sides = g.vpairs; ds.E = g.NP; ds.k = 1; ds.G = g.GH; }   // buckets (side, head, pair), one entry per (token, head)
+        if (g.vsets) { ds.sides = g.vsets; ds.E = g.NS; ds.k = 1; ds.G = g.GH; }   // buckets (side, head, set), one entry per (token, head)
         sh_sort_block(g.idx, g.gate, g.blockcnt, g.offsets, g.lists, g.lgate, g.tiles, g.ntiles, ds, s_sort, et, NSEL, (int)blockIdx.x, true, sel_sync);
       }
     }

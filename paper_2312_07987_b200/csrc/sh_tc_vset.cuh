@@ -1,18 +1,18 @@
-// Value-expert projection of a k = 2 layer on CTA pairs, tiled by (head, PAIR of selected experts)
-// (Sec. 2.2, the value equation):  V^h[t] = s^h[t,a] * x[t] W_V^{h,a} + s^h[t,b] * x[t] W_V^{h,b},  {a, b} = E_S^h(t).
+// Value-expert projection of a layer with k = 2, 3 or 4 on CTA pairs, tiled by (head, SET of selected experts)
+// (Sec. 2.2, the value equation):  V^h[t] = sum over e in E_S^h(t) of s^h[t,e] * x[t] W_V^{h,e}.
 //
 // The expert-tiled kernel (sh_tc_pgemm_kernel<PG_V>) gathers every token row once per selected expert -
-// H*k times per token - and adds the k gate-scaled results with reductions in global memory.  With k = 2
-// every (token, head) has exactly one pair {a < b}; sorting the tokens of a head by their pair instead of
-// by expert gives tiles whose rows ALL want the same two experts:  one gather of the row (H times per
-// token), one UMMA of N = 256 against [W^{h,a} | W^{h,b}], and the gate-weighted sum of the two halves of
-// the accumulator row in the epilogue, stored once - no reductions, no cleared buffer, no dependence on
+// H*k times per token - and adds the k gate-scaled results with reductions in global memory.  Every (token, head) has
+// exactly one set {e0 < e1 < ...}; sorting the tokens of a head by their set instead of
+// by expert gives tiles whose rows ALL want the same experts:  one gather of the row (H times per
+// token), one UMMA of N = k d_head <= 256 against [W^{h,e0} | W^{h,e1} | ...], and the gate-weighted sum of the k parts of
+// the accumulator row in the epilogue, in fp32, stored once - no reductions, no cleared buffer, no dependence on
 // arrival order.  On a CTA pair (tcgen05 cta_group::2, M = 256) each CTA gathers its own 128 rows and
-// loads ONE of the two experts' 128 weight rows; the pair's tensor cores read both.  L2 -> shared memory
-// per (token, head): 2 rows' worth of x + 2 of weights per 128 rows... 4 KB at d_model 1024 against 6 KB.
+// loads half of the weight rows (k = 2: one expert); the pair's tensor cores read both.  L2 -> shared memory
+// per (token, head), k = 2, d_head 128: 4 KB at d_model 1024 against 6 KB.
 //
-// Tile table and lists come from the same bucket sort, run over (head, pair) buckets: lists[h][...] holds
-// the tokens of head h ordered by pair number, a tile = up to 256 consecutive entries of one pair.
+// Tile table and lists come from the same bucket sort, run over (head, set) buckets: lists[h][...] holds
+// the tokens of head h ordered by set number, a tile = up to 256 consecutive entries of one set.
 //
 // Warp roles per CTA (320 threads): warp 0 lane 0 = weight producer (TMA), warp 1 = TMEM allocation and,
 // in the leader, the UMMA issuer, warps 2..5 = epilogue (thread = accumulator row), warps 6..9 = row
@@ -25,18 +25,18 @@
 
 namespace shtc {
 
-#ifndef VPAIR_LAG
-#define VPAIR_LAG 2                                        // gather rounds in flight per thread before it waits for the oldest
+#ifndef VSET_LAG
+#define VSET_LAG 2                                        // gather rounds in flight per thread before it waits for the oldest
 #endif
 
-struct TcVPairArgs {
+struct TcVSetArgs {
   ShDims d;
   const void* x;             // [N, M] bf16
-  const int* lists;          // [H][N]: tokens of head h ordered by pair
-  const ShTile* tiles;       // (h, pair, row0, nrows <= 256)
+  const int* lists;          // [H][N]: tokens of head h ordered by set
+  const ShTile* tiles;       // (h, set, row0, nrows <= 256)
   const int* ntiles;
-  const int* idx;            // source side [N, H, 2]
-  const float* gate;         // source side [N, H, 2]
+  const int* idx;            // source side [N, H, k]
+  const float* gate;         // source side [N, H, k]
   __half* v;                 // [B, H, T, D]: the projection's result (V; K or Q of a layer with key / query experts)
   float scale;               // extra factor on the result (the queries' log2(e)/sqrt(d_head)); 0 = none
   int stamp_id;              // SH_K_V, or -1: no stamps (the key / query launches)
@@ -46,18 +46,33 @@ struct TcVPairArgs {
 };
 
 template <int STAGES>
-struct VPairSmem {
+struct VSetSmem {
   static constexpr int A_BYTES = 128 * 64 * 2;             // this CTA's 128 gathered rows, 64 columns
-  static constexpr int B_BYTES = 128 * 64 * 2;             // this CTA's expert: 128 feature rows, 64 columns
+  static constexpr int B_BYTES = 128 * 64 * 2;             // this CTA's half of the experts' feature rows (up to 128), 64 columns
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
   static constexpr int BAR_OFF = STAGES * STAGE_BYTES;
   static constexpr int TOTAL = BAR_OFF + 256 + 1024;
 };
 
-template <int STAGES>
+// 16 tensor-memory columns
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&u)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(u[0]), "=r"(u[1]), "=r"(u[2]), "=r"(u[3]), "=r"(u[4]), "=r"(u[5]), "=r"(u[6]), "=r"(u[7]),
+        "=r"(u[8]), "=r"(u[9]), "=r"(u[10]), "=r"(u[11]), "=r"(u[12]), "=r"(u[13]), "=r"(u[14]), "=r"(u[15])
+      : "r"(taddr)
+      : "memory");
+}
+
+// k experts of DH columns each
+template <int STAGES, int K, int DH>
 __global__ void __launch_bounds__(320, 1)
-sh_tc_vpair_kernel(const __grid_constant__ CUtensorMap mapW, TcVPairArgs g) {
-  using SM = VPairSmem<STAGES>;
+sh_tc_vset_kernel(const __grid_constant__ CUtensorMap mapW, TcVSetArgs g) {
+  using SM = VSetSmem<STAGES>;
+  constexpr int HALF = K * DH / 2;                         // weight rows of a CTA
+  constexpr int BOX = K == 3 ? 32 : DH;                    // rows of a weight box
+  static_assert(K * DH <= 256 && HALF % BOX == 0, "");
   extern __shared__ unsigned char smem_raw[];
   const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
   unsigned char* sgen = smem_raw + (sbase - smem_u32(smem_raw));
@@ -117,11 +132,11 @@ sh_tc_vpair_kernel(const __grid_constant__ CUtensorMap mapW, TcVPairArgs g) {
   //  costs this kernel's start 2-3 us while the Q/K projection's operand traffic keeps L2 busy)
   const ShTile tile_first = g.tiles[pair];                // (the table has room for every pair's index)
   const int ntiles = dead ? 0 : *g.ntiles;
-  const int NP = sh_pair_count(d.E);
+  const int NS = sh_choose(d.E, K);
   auto tile_of = [&](int t) -> ShTile {
     ShTile tl = t == pair ? tile_first : g.tiles[t];
 #ifdef SH_DEBUG
-    const bool ok = SH_INDEX_OK(tl.h, d.H, g.status, SH_SITE_V_TILE) && SH_INDEX_OK(tl.e, NP, g.status, SH_SITE_V_TILE) &&
+    const bool ok = SH_INDEX_OK(tl.h, d.H, g.status, SH_SITE_V_TILE) && SH_INDEX_OK(tl.e, NS, g.status, SH_SITE_V_TILE) &&
                     SH_INDEX_OK(tl.nrows, 257, g.status, SH_SITE_V_TILE) &&
                     SH_INDEX_OK((long long)tl.row0 + tl.nrows, (long long)d.N + 1, g.status, SH_SITE_V_TILE);
     if (!ok) { tl.h = 0; tl.e = 0; tl.row0 = 0; tl.nrows = 0; }
@@ -135,20 +150,29 @@ sh_tc_vpair_kernel(const __grid_constant__ CUtensorMap mapW, TcVPairArgs g) {
       uint32_t par = 1;
       for (int t = pair; t < ntiles && !dead; t += npairs) {
         const ShTile tl = tile_of(t);
-        int ea, eb;
-        sh_pair_decode(tl.e, d.E, ea, eb);
-        const int brow = (tl.h * d.E + (rank == 0 ? ea : eb)) * d.D;     // this CTA's expert: its D = 128 feature rows
+        int ex[K], brow[HALF / BOX];                       // the set's experts; this CTA's boxes of their feature rows
+        sh_set_decode(tl.e, K, d.E, ex);
+#pragma unroll
+        for (int i = 0; i < HALF / BOX; ++i) {
+          const int r0 = (int)rank * HALF + i * BOX, j = r0 / DH;
+          int e = ex[0];
+#pragma unroll
+          for (int u = 1; u < K; ++u) e = j == u ? ex[u] : e;
+          brow[i] = (tl.h * d.E + e) * DH + r0 % DH;
+        }
         for (int kb = 0; kb < KB; ++kb) {
           if (!mbar_wait(&empty_bar[s], par, g.status, dead)) break;
-          if (rank == 0) mbar_expect_tx(&full_bar[s], 2 * SM::B_BYTES);
-          tma_load_2d_pair(sbase + s * SM::STAGE_BYTES + SM::A_BYTES, &mapW, &full_bar[s], kb * 64, brow);
+          if (rank == 0) mbar_expect_tx(&full_bar[s], 2 * HALF * 128);
+#pragma unroll
+          for (int i = 0; i < HALF / BOX; ++i)
+            tma_load_2d_pair(sbase + s * SM::STAGE_BYTES + SM::A_BYTES + i * BOX * 128, &mapW, &full_bar[s], kb * 64, brow[i]);
           if (++s == STAGES) { s = 0; par ^= 1; }
         }
       }
     }
   } else if (warp == 1) {
     if (lane == 0 && rank == 0) {
-      constexpr uint32_t idesc = make_idesc_f16(256, 256, 1, 1, 0);
+      constexpr uint32_t idesc = make_idesc_f16(256, K * DH, 1, 1, 0);
       const uint32_t a_lo0 = desc_lo_k(sbase), b_lo0 = desc_lo_k(sbase + SM::A_BYTES);
       int s = 0, it = 0;
       uint32_t par = 0;
@@ -208,8 +232,8 @@ sh_tc_vpair_kernel(const __grid_constant__ CUtensorMap mapW, TcVPairArgs g) {
           cp_async_16(sa + (rb + 16 * i) * 128 + dsw, src[i] + (long)kb * 128, ok[i]);
         cp_async_commit();
         ++issued;
-        if (issued - n_arr > VPAIR_LAG) {                  // the copies of the stage issued VPAIR_LAG rounds ago have landed
-          cp_async_wait<VPAIR_LAG>();
+        if (issued - n_arr > VSET_LAG) {                  // the copies of the stage issued VSET_LAG rounds ago have landed
+          cp_async_wait<VSET_LAG>();
           landed();
         }
         if (++s == STAGES) { s = 0; par ^= 1; }
@@ -219,27 +243,41 @@ sh_tc_vpair_kernel(const __grid_constant__ CUtensorMap mapW, TcVPairArgs g) {
     if (!dead)
       while (n_arr < issued) landed();
   } else {
-    // ---- epilogue: thread = accumulator row = TMEM lane: gate-weighted sum of the two experts' halves ----
+    // ---- epilogue: thread = accumulator row = TMEM lane: gate-weighted sum of the experts' columns ----
     const int q = warp & 3;
     const uint32_t lane_off = (uint32_t)(q * 32) << 16;
+    constexpr int CW = K == 2 ? 32 : 16;                   // columns at a time
     int it = 0;
     for (int t = pair; t < ntiles; t += npairs, ++it) {
       const int b = it & 1;
       const ShTile tl = tile_of(t);
       const int r = (int)rank * 128 + q * 32 + lane;
       int tok = -1;
-      float ga = 0.f, gb = 0.f;
+      float gt[K];                                         // in the order of the experts' numbers
+#pragma unroll
+      for (int j = 0; j < K; ++j) gt[j] = 0.f;
       if (r < tl.nrows) {                                  // fetched before the wait: hides the list latency
         tok = g.lists[(size_t)tl.h * d.N + tl.row0 + r];
         if (!SH_INDEX_OK(tok, d.N, g.status, SH_SITE_V_TOKEN)) tok = -1;
       }
       if (tok >= 0) {
-        const size_t so = ((size_t)tok * d.H + tl.h) * 2;
-        const int i0 = g.idx[so], i1 = g.idx[so + 1];
-        const float g0 = g.gate[so], g1 = g.gate[so + 1];
-        ga = i0 < i1 ? g0 : g1;                            // a = the lower expert index of the pair
-        gb = i0 < i1 ? g1 : g0;
-        if (g.scale != 0.f) { ga *= g.scale; gb *= g.scale; }
+        const size_t so = ((size_t)tok * d.H + tl.h) * K;
+        int ix[K];
+        float gv[K];
+#pragma unroll
+        for (int j = 0; j < K; ++j) { ix[j] = g.idx[so + j]; gv[j] = g.gate[so + j]; }
+#pragma unroll
+        for (int j = 0; j < K; ++j) {
+          int pos = 0;
+#pragma unroll
+          for (int u = 0; u < K; ++u) pos += ix[u] < ix[j];
+#pragma unroll
+          for (int u = 0; u < K; ++u) gt[u] = pos == u ? gv[j] : gt[u];
+        }
+        if (g.scale != 0.f) {
+#pragma unroll
+          for (int j = 0; j < K; ++j) gt[j] *= g.scale;
+        }
       }
       if (!mbar_wait(&acc_full[b], (it >> 1) & 1, g.status, dead)) break;
       tc_fence_after();
@@ -247,27 +285,31 @@ sh_tc_vpair_kernel(const __grid_constant__ CUtensorMap mapW, TcVPairArgs g) {
       const int bb = tok >= 0 ? tok / d.T : 0, tt = tok >= 0 ? tok % d.T : 0;
       __half* dst = g.v + (((size_t)bb * d.H + tl.h) * d.T + tt) * d.D;
 #pragma unroll 1
-      for (int c0 = 0; c0 < 128; c0 += 32) {
-        uint32_t va[32], vb[32];
-        tmem_ld32(trow + c0, va);
-        tmem_ld32(trow + 128 + c0, vb);
+      for (int c0 = 0; c0 < DH; c0 += CW) {
+        uint32_t a[K][CW];
+#pragma unroll
+        for (int j = 0; j < K; ++j) {
+          if constexpr (CW == 32) tmem_ld32(trow + j * DH + c0, a[j]);
+          else tmem_ld16(trow + j * DH + c0, a[j]);
+        }
         tmem_ld_wait();
-        if (c0 == 96) {                                    // the accumulator is in registers: hand the buffer back
+        if (c0 == DH - CW) {                               // the accumulator is in registers: hand the buffer back
           tc_fence_before();
           __syncwarp();
           if (lane == 0) mbar_arrive_leader(&acc_empty[b]);
         }
         if (tok < 0) continue;
-        uint32_t p[16];
+        uint32_t p[CW / 2];
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          const float y0 = fmaf(ga, __uint_as_float(va[2 * i]), gb * __uint_as_float(vb[2 * i]));
-          const float y1 = fmaf(ga, __uint_as_float(va[2 * i + 1]), gb * __uint_as_float(vb[2 * i + 1]));
+        for (int i = 0; i < CW / 2; ++i) {
+          float y0 = gt[K - 1] * __uint_as_float(a[K - 1][2 * i]), y1 = gt[K - 1] * __uint_as_float(a[K - 1][2 * i + 1]);
+#pragma unroll
+          for (int j = K - 2; j >= 0; --j) { y0 = fmaf(gt[j], __uint_as_float(a[j][2 * i]), y0); y1 = fmaf(gt[j], __uint_as_float(a[j][2 * i + 1]), y1); }
           __half2 hv = __floats2half2_rn(y0, y1);
           p[i] = *reinterpret_cast<uint32_t*>(&hv);
         }
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+        for (int i = 0; i < CW / 8; ++i)
           *reinterpret_cast<uint4*>(dst + c0 + 8 * i) = make_uint4(p[4 * i], p[4 * i + 1], p[4 * i + 2], p[4 * i + 3]);
       }
     }
