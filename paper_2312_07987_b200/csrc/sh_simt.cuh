@@ -146,11 +146,12 @@ static __device__ __forceinline__ void sh_sort_block(const int* __restrict__ idx
   // loads do not depend on the selections copy below, so both are in flight together.
   int my_b = -1, my_tot = 0, my_pre = 0;
   {
-    const int parts = max(1, nthreads / nb);
+    const int used = d.sides * d.H * d.E;                  // (a forward pass sorts the first side only)
+    const int parts = max(1, nthreads / used);
     if (nb <= nthreads) {
-      if (tid / nb < parts) {
-        my_b = tid % nb;
-        const int part = tid / nb;
+      if (tid / used < parts) {
+        my_b = tid % used;
+        const int part = tid / used;
 #pragma unroll 8
         for (int bk = part; bk < d.nblk; bk += parts) {
           const int c = blockcnt[(size_t)bk * nb + my_b];
@@ -210,10 +211,12 @@ static __device__ __forceinline__ void sh_sort_block(const int* __restrict__ idx
         const int ev = s_idx[side * 128 * per_tok + (tl * d.H + h) * d.k + j];
         if (SH_INDEX_OK(ev, d.E, d.status, SH_SITE_SORT_EXPERT)) mask |= 1u << ev;
       }
+    unsigned mine = 0;                                     // lane e: which lanes chose expert e
     for (int e = 0; e < d.E; ++e) {
       const unsigned bal = __ballot_sync(0xffffffffu, (mask >> e) & 1u);
-      if (lane == 0) s_wcnt[(grp * d.E + e) * 4 + twarp] = __popc(bal);
+      if (lane == e) mine = bal;
     }
+    if (lane < d.E) s_wcnt[(grp * d.E + lane) * 4 + twarp] = __popc(mine);
   }
   sync();
   {
@@ -244,21 +247,23 @@ static __device__ __forceinline__ void sh_sort_block(const int* __restrict__ idx
           const int ev = s_idx[sel + j];
           if (SH_INDEX_OK(ev, d.E, d.status, SH_SITE_SORT_EXPERT)) mask |= 1u << ev;
         }
+      unsigned mine = 0;
       for (int e = 0; e < d.E; ++e) {
-        const bool mine = (mask >> e) & 1u;
-        const unsigned bal = __ballot_sync(0xffffffffu, mine);
-        if (mine) {
-          const int b = grp * d.E + e;
-          int pos = __popc(bal & ((1u << lane) - 1u));
-          for (int w = 0; w < twarp; ++w) pos += s_wcnt[b * 4 + w];
-          float gv = 0.f;
-          for (int j = 0; j < d.k; ++j)
-            if (s_idx[sel + j] == e) gv = s_gt[sel + j];
-          const size_t dst = (size_t)grp * d.N * d.k + s_off[b] + s_pre[b] + pos;
-          if (SH_INDEX_OK(s_off[b] + s_pre[b] + pos, (long long)d.N * d.k, d.status, SH_SITE_SORT_SLOT)) {
-            lists[dst] = t;
-            lgate[dst] = gv;
-          }
+        const unsigned bal = __ballot_sync(0xffffffffu, (mask >> e) & 1u);
+        if (lane == e) mine = bal;
+      }
+      // (selection by selection, not expert by expert: a chain of trips to shared memory each)
+      for (int j = 0; j < d.k; ++j) {
+        const int ev = tl < nrows ? s_idx[sel + j] : -1;
+        const unsigned bal = __shfl_sync(0xffffffffu, mine, ev & 31);
+        if ((unsigned)ev >= (unsigned)d.E) continue;
+        const int b = grp * d.E + ev;
+        int pos = __popc(bal & ((1u << lane) - 1u));
+        for (int w = 0; w < twarp; ++w) pos += s_wcnt[b * 4 + w];
+        const size_t dst = (size_t)grp * d.N * d.k + s_off[b] + s_pre[b] + pos;
+        if (SH_INDEX_OK(s_off[b] + s_pre[b] + pos, (long long)d.N * d.k, d.status, SH_SITE_SORT_SLOT)) {
+          lists[dst] = t;
+          lgate[dst] = s_gt[sel + j];
         }
       }
     }
