@@ -94,13 +94,14 @@ static void layout_workspace(sh_layer* L) {
   // query / key experts (sh_create_moe_qk): [H, E, D, M] like the value experts
   o.wq_e = take(L->moe_q ? HD * d.E * d.M * win : 16);
   o.wk_e = take(L->moe_k ? HD * d.E * d.M * win : 16);      // pair number of every (token, head), source side
-  // fp32 configuration: scratch of the backward pass (dQ, dK, dV, dAhat [N, H, D] and the gate gradients [2, N, H, k]
-  //  in list order, the gate gradients once more as a matrix [N, G], rowsum(dAhat o Ahat) [N, H]); the gate weights
+  // fp32 configuration: scratch of the backward pass (dQ, dK, dV, dAhat [N, H, D], the gate gradients as a matrix [N, G],
+  //  rowsum(dAhat o Ahat) [N, H]; the forward attention keeps partial results there); the gate weights
   //  once more in fp32; per attention row the score maximum and 1 / normaliser)
   const bool f32 = L->dtype == SH_F32 && !L->dense;
   o.bw = take(f32 ? ((size_t)4 * d.N * HD + (size_t)d.N * (sh_f32_ldz(d) + d.H)) * 4 : 16);
   o.wgate32 = take(f32 ? (size_t)d.G * d.M * 4 : 16);
   o.f32stats = take(f32 ? (size_t)d.N * d.H * 8 : 16);
+  o.f32arrived = take(f32 ? (size_t)((d.T + 127) / 128) * d.B * d.H * 4 : 16);   // forward attention: parts of a query tile that are done (zero between passes)
   o.wo_overflow = take(16);                                  // d_head above 128, bf16 storage: a stored weight of W_O is not finite
   o.stamps = take(sizeof(ShStampBlock));
   o.total = off;
@@ -311,6 +312,7 @@ static int set_weights_f32(sh_layer* L, const float* Wq, const float* Wk, const 
   const ShDims& d = L->d;
   char* ws = L->ws;
   const long HD = (long)d.H * d.D, nqk = 2 * HD * d.M, nexp = HD * d.E * d.M, ngate = (long)d.G * d.M;
+  SH_CUDA_CHECK(cudaMemsetAsync(ws + L->o.f32arrived, 0, (size_t)((d.T + 127) / 128) * d.B * d.H * 4, st));
   SH_CUDA_CHECK(cudaMemsetAsync(ws + L->o.status, 0, 256, st));
   for (int i = 0; i < L->n_guards; ++i) SH_CUDA_CHECK(cudaMemsetAsync(ws + L->guard_off[i], SH_GUARD_BYTE, SH_GUARD_BYTES, st));
   if (d.D != d.Dt) {

@@ -1,12 +1,14 @@
 // fp32 configuration of the SwitchHead layer: launch sequences of the forward and the backward pass.
-// Projections on the tensor cores in split bf16 (sh_f32_gemm.cuh), attention on the CUDA cores
-// (sh_f32_attn.cuh), selection and sort in one launch (sh_f32_select.cuh).
+// Projections on the tensor cores in split bf16 (sh_f32_gemm.cuh, sh_f32_wgrad.cuh), attention on the CUDA cores
+// (sh_f32_attn.cuh) or, for longer sequences forward, the tensor cores (sh_f32_attn_tc.cuh), selection and sort in
+// one launch (sh_f32_select.cuh).
 #include "sh_internal.cuh"
 #include "sh_launch.cuh"
 #include "sh_simt.cuh"
 #include "sh_f32_gemm.cuh"
 #include "sh_f32_wgrad.cuh"
 #include "sh_f32_attn.cuh"
+#include "sh_f32_attn_tc.cuh"
 #include "sh_f32_select.cuh"
 
 #include <cstdlib>
@@ -170,6 +172,34 @@ XPart part_v(sh_layer* L, const void* x, int side, const PlaneMap& w, float* dst
   return part<X_V>(L, g, d.H * head_tiles(d), g.nsub, ksplit, &w);
 }
 
+// Key tiles of a part of a query tile's keys: the fewest, two at least, that keep the units at or below F32_ATTN_UNITS and their
+// partial results in the backward pass's scratch; all of them (no parts, no scratch) where there are that many query tiles.
+int attn_part_tiles(const ShDims& d) {
+  const int nqt = (d.T - d.Tc + 127) / 128, most = (d.T + 63) / 64;
+  const long room = 4l * d.N * d.H * d.D / (128 * (d.D + 2)), cap = room < F32_ATTN_UNITS ? room : F32_ATTN_UNITS;
+  for (int per = 2; per < most; ++per) {
+    long units = 0;
+    for (int i = 0; i < nqt; ++i) units += (fattn_key_tiles(d, i) + per - 1) / per;
+    if (units * d.B * d.H <= cap) return per;
+  }
+  return most;
+}
+
+template <int D>
+int launch_attn_tc(sh_layer* L, float* zero, long n, cudaStream_t st) {
+  const ShDims& d = L->d;
+  char* ws = L->ws;
+  if (int rc = set_smem(sh_f32_attn_tc_kernel<D>, FAttnTcSmem<D>::TOTAL)) return rc;
+  FAttnTcArgs g{};
+  g.q = (const float*)(ws + L->o.q); g.k = (const float*)(ws + L->o.k); g.v = (const float*)(ws + L->o.v);
+  g.ahat = (float*)(ws + L->o.ahat); g.stats = (float*)(ws + L->o.f32stats);
+  g.part = (float*)(ws + L->o.bw); g.arrived = (unsigned*)(ws + L->o.f32arrived);
+  g.zero = (float4*)zero; g.nzero = n / 4; g.d = d; g.per = attn_part_tiles(d); g.status = (int*)(ws + L->o.status);
+  long units = 0;
+  for (int i = 0; i < (d.T - d.Tc + 127) / 128; ++i) units += (fattn_key_tiles(d, i) + g.per - 1) / g.per;
+  return launch_k(chained(L), sh_f32_attn_tc_kernel<D>, dim3((unsigned)(units * d.B * d.H)), dim3(288), FAttnTcSmem<D>::TOTAL, st, g);
+}
+
 template <int D>
 int launch_attn_t(sh_layer* L, float* zero, long n, cudaStream_t st) {
   const ShDims& d = L->d;
@@ -182,12 +212,18 @@ int launch_attn_t(sh_layer* L, float* zero, long n, cudaStream_t st) {
 }
 
 // Attention; beside it `zero` (n values), which the output projection adds into, is cleared.
+// On the tensor cores from 320 keys on, or from 129 on where the other kernel's blocks of 32 queries go one and a half
+// times round the SMs: its time is that of the longest chain of key tiles, theirs mostly that of a unit.  (Whole passes of
+// a small layer, CUDA cores / tensor cores, us: d_head 112, 8 heads, 256 keys 46 / 50, 320 55 / 53, 512 68 / 56, 800 102 / 77;
+// 64 heads, 128 keys 66 / 64, 256 keys 110 / 86; 32 heads, 192 keys 53 / 58, 256 keys 73 / 71.)
 int launch_attn(sh_layer* L, float* zero, long n, cudaStream_t st) {
   L->launches += 1;
-  switch (L->d.D) {
-    case 32: return launch_attn_t<32>(L, zero, n, st);
-    case 64: return launch_attn_t<64>(L, zero, n, st);
-    case 128: return launch_attn_t<128>(L, zero, n, st);
+  const ShDims& d = L->d;
+  const bool tc = d.T >= 320 || (d.T > 128 && 2l * ((d.T - d.Tc + 31) / 32) * d.B * d.H >= 3l * sm_count(L));
+  switch (d.D) {
+    case 32: return tc ? launch_attn_tc<32>(L, zero, n, st) : launch_attn_t<32>(L, zero, n, st);
+    case 64: return tc ? launch_attn_tc<64>(L, zero, n, st) : launch_attn_t<64>(L, zero, n, st);
+    case 128: return tc ? launch_attn_tc<128>(L, zero, n, st) : launch_attn_t<128>(L, zero, n, st);
     default: return launch_attn_t<256>(L, zero, n, st);
   }
 }

@@ -1,4 +1,5 @@
-// Attention of the fp32 configuration, forward and backward, on the CUDA cores (fp32 FMA).
+// Attention of the fp32 configuration, forward and backward, on the CUDA cores (fp32 FMA).  The forward pass of longer
+// sequences is in sh_f32_attn_tc.cuh.
 //
 // A layer's share of attention is small here (sequences of a few hundred tokens: 0.5 of the 7 GFLOP of
 // a 262M-scale forward pass), and what bounds it is the longest chain of key tiles one SM works off,
@@ -227,7 +228,7 @@ sh_f32_attn_kernel(const float* __restrict__ Q, const float* __restrict__ K, con
 
 // ---- backward --------------------------------------------------------------------------------------
 // What the backward pass adds into, cleared in one launch (as memsets, up to six of them, each with a gap in the chain
-// of launches in front and behind: 24 us of a 47M-scale step).  Pointers may be 4-byte aligned.
+// of launches in front and behind: 16 us of a step of 8 x 256 tokens with the two small kernels that went with them).  Pointers may be 4-byte aligned.
 struct FClear { float* p[8]; long n[8]; };
 static __global__ void __launch_bounds__(256)
 sh_f32_clear_kernel(const __grid_constant__ FClear c) {

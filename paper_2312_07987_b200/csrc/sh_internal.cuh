@@ -108,7 +108,7 @@ __device__ __forceinline__ void sh_stamp_end(unsigned long long* s, int k) { if 
 
 struct ShWorkspace {
   size_t status, wqk, wgate, gbias, wv, wo, q, k, v, ahat, idx, gate, blockcnt, blockoff,
-         offsets, lists, lgate, tiles, ntiles, rope, vearly, vearly_cnt, xl_emb, xl_r, xl_uv, xl_r16, xl_vr, xl_uk, xl_bias, wos, gid, wq_e, wk_e, bw, wgate32, f32stats, wo_overflow, stamps, total;
+         offsets, lists, lgate, tiles, ntiles, rope, vearly, vearly_cnt, xl_emb, xl_r, xl_uv, xl_r16, xl_vr, xl_uk, xl_bias, wos, gid, wq_e, wk_e, bw, wgate32, f32stats, f32arrived, wo_overflow, stamps, total;
 };
 
 // Words of the 256-byte status block at the start of the workspace.
@@ -160,7 +160,7 @@ inline bool sh_o_sparse_ok(const sh_layer* L) {
 // Shapes whose value projection is tiled by (head, set of selected experts) instead of (head, expert): the k experts of a
 // set side by side are at most 256 columns, and there are few enough sets for their partly filled tiles - half a tile of
 // 256 rows each, on two SMs, against half a tile of 128 per expert - not to cost more than the k - 1 further gathers of
-// every row.
+// every row.  (8192 tokens, 2 heads of 64, three of five experts: 59.1 -> 48.6 us a pass.)
 inline bool sh_v_sets_ok(const sh_layer* L) {
   const ShDims& d = L->d;
   if (L->dtype != SH_BF16 || L->dense || d.k < 2 || d.k > 4 || d.E < d.k) return false;
