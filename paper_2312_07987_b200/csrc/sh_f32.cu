@@ -72,7 +72,7 @@ void col_tiles(XGemmArgs& g, int cols) {
 
 // A contraction over d_head of a side's lists: up to 128 positions on the kernel that keeps its rows in tensor memory,
 // the columns split among as many blocks per row tile as the device has SMs for.  (Half of the experts' last tiles are
-// worth counting; the rest of the table is empty.)
+// worth counting, the rest of the table is empty; with k = E every list is as long as the batch.)
 template <int MODE>
 int launch_d(sh_layer* L, cudaStream_t st, XGemmArgs g) {
   const F32State* S = (const F32State*)L->f32;
@@ -83,7 +83,7 @@ int launch_d(sh_layer* L, cudaStream_t st, XGemmArgs g) {
     return launch_x<MODE>(L, st, part<MODE>(L, g, d.H * head_tiles(d), g.nsub));
   }
   const int ntile = (d.M + XGemmDSmem::BN - 1) / XGemmDSmem::BN;
-  const long rows = (long)d.H * d.N * d.k / 128 + d.H * d.E / 2;
+  const long rows = d.k == d.E ? (long)d.H * d.E * ((d.N + 127) / 128) : (long)d.H * d.N * d.k / 128 + d.H * d.E / 2;
   long split = sm_count(L) / (rows < 1 ? 1 : rows);
   split = split < 1 ? 1 : split > ntile ? ntile : split;
   auto kern = sh_f32_gemm_d_kernel<MODE>;
