@@ -1,0 +1,65 @@
+"""fp32 attention of long sequences, forward on the tensor cores: the shortest sequence that takes it and its neighbours,
+query tiles of 128 and key tiles of 64 with one row more or less, keys in parts (one query tile's up to as many as its
+pairs of tiles) and in one, stored widths of 32, 64 and 128 columns, no mask, a cache; values that are not finite."""
+import numpy as np
+import pytest
+import torch
+
+from oracle.switchhead_backward import switchhead_backward
+from oracle.switchhead_oracle import switchhead_forward
+from paper_2312_07987_b200 import binding, inputs
+
+pytestmark = pytest.mark.gpu
+# max-abs error / largest value: fp32 sums of up to K terms, sqrt(K) 2^-24 of their size, times 5 for the largest of
+# ~1e5 values: K <= 1100, 1e-5
+TOL = 1e-5
+
+
+@pytest.mark.parametrize("B,T,H,D,causal", [
+    (1, 320, 1, 32, True),           # the first length; three query tiles of five parts in all
+    (1, 321, 2, 64, False),          # one key into the sixth key tile, no mask
+    (2, 385, 1, 112, True),          # one row into the fourth query tile
+    (1, 383, 3, 76, True),           # one row less than three
+    (1, 1025, 1, 20, True),          # nine query tiles; nine parts for the last one
+    (40, 130, 2, 128, True),         # many heads: parts of the whole row, nothing to join
+])
+def test_f32_attention_parts(B, T, H, D, causal):
+    M, E, k = 64, 2, 1
+    cfg = inputs.LayerConfig("parts", inputs.DTYPE_F32, B, T, M, H, D, E, k, seed=T + D)
+    inp = inputs.make_inputs(cfg)
+    layer = binding.layer_from_inputs(inp)
+    layer.sh_set_causal(causal)
+    x = binding.to_device(inp.x, cfg.dtype)
+    ones = np.ones(inp.x.shape, dtype=np.float32)
+    y = [layer.sh_forward(x).cpu().numpy() for _ in range(3)]
+    dx = layer.sh_backward(x, torch.from_numpy(ones).cuda())["dx"].cpu().numpy()      # (with the pass's maxima and normalisers)
+    assert layer.sh_last_status() == 0
+    layer.sh_check_guards()
+    args = (inp.x, inp.Wq, inp.Wk, inp.Wv, inp.Wo, inp.Ws, inp.Wd, k)
+    want = switchhead_forward(*args, inp.bias_s, inp.bias_d, causal=causal, return_stages=False)["y"]
+    for got in y:
+        assert np.abs(got - want).max() / np.abs(want).max() < TOL
+    want = switchhead_backward(*args, ones, inp.bias_s, inp.bias_d, causal=causal)["dx"]
+    assert np.abs(dx - want.reshape(dx.shape)).max() / np.abs(want).max() < TOL
+    layer.close()
+
+
+@pytest.mark.parametrize("D", [32, 64, 128])
+@pytest.mark.parametrize("t0", [40, 300])
+def test_f32_overflow_of_one_value_row_stays_behind_the_mask(D, t0):
+    # finite inputs, but token t0's value row overflows (first column of x times that row of W_V): earlier rows never see it
+    B, T, M, H, E, k = 1, 400, 128, 2, 4, 2
+    inp = inputs.make_inputs(inputs.LayerConfig("parts", inputs.DTYPE_F32, B, T, M, H, D, E, k, seed=31 + D))
+    for W in (inp.Wq, inp.Wk, inp.Ws, inp.Wd):
+        W[:, 0] = 0.0
+    inp.Wv[:, :, 0] = 10.0
+    layer = binding.layer_from_inputs(inp)
+    x = binding.to_device(inp.x, inp.cfg.dtype)
+    want = layer.sh_forward(x)
+    x[0, t0, 0] = 1e38
+    y = layer.sh_forward(x)
+    close = lambda a, b: float((a - b).abs().max() / b.abs().max()) < TOL
+    assert close(y[:, :t0], want[:, :t0]) and not bool(torch.isfinite(y[:, t0:]).all())
+    x.copy_(binding.to_device(inp.x, inp.cfg.dtype))
+    assert close(layer.sh_forward(x), want)                 # and nothing of it is left behind
+    layer.close()
