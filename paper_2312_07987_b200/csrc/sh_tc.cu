@@ -851,12 +851,14 @@ static int tc_forward_rest(sh_layer* L, const void* x, void* out, cudaStream_t s
       if ((rc = set_smem(sh_tc_attention_wide_kernel, AttnWSmem::TOTAL))) return rc;
       if ((rc = launch_k(pdl, sh_tc_attention_wide_kernel, dim3(wgrid), dim3(192), AttnWSmem::TOTAL, st, S->map_q, S->map_k, S->map_v, a))) return rc;
     } else if (d.D == 128) {
-      auto kern = halves ? (a.bias ? sh_tc_attention3_kernel<128, true> : sh_tc_attention3_kernel<128, false>) : sh_tc_attention2_kernel<128>;
+      auto kern = halves ? (a.bias ? sh_tc_attention3_kernel<128, true> : sh_tc_attention3_kernel<128, false>)
+                         : a.bias ? sh_tc_attention2_kernel<128, true> : sh_tc_attention2_kernel<128, false>;
       const int smem = halves ? Attn3Smem<128>::TOTAL : Attn2Smem<128>::TOTAL;
       if ((rc = set_smem(kern, smem))) return rc;
       if ((rc = launch_k(pdl, kern, dim3(grid), dim3(320), smem, st, S->map_q, S->map_k, S->map_v, a))) return rc;
     } else {
-      auto kern = halves ? (a.bias ? sh_tc_attention3_kernel<64, true> : sh_tc_attention3_kernel<64, false>) : sh_tc_attention2_kernel<64>;
+      auto kern = halves ? (a.bias ? sh_tc_attention3_kernel<64, true> : sh_tc_attention3_kernel<64, false>)
+                         : a.bias ? sh_tc_attention2_kernel<64, true> : sh_tc_attention2_kernel<64, false>;
       const int smem = halves ? Attn3Smem<64>::TOTAL : Attn2Smem<64>::TOTAL;
       if ((rc = set_smem(kern, smem))) return rc;
       if ((rc = launch_k(pdl, kern, dim3(grid), dim3(320), smem, st, S->map_q, S->map_k, S->map_v, a))) return rc;

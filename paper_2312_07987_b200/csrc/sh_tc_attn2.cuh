@@ -62,7 +62,7 @@ struct Attn2Smem {
   static constexpr int TOTAL = BAR_OFF + 256 + 1024;
 };
 
-template <int D>
+template <int D, bool BIAS>                             // BIAS: a score bias is added (sh_tc_xlbias_kernel)
 __global__ void __launch_bounds__(320, 1)
 sh_tc_attention2_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapK,
                         const __grid_constant__ CUtensorMap mapV, TcAttnArgs g) {
@@ -214,12 +214,13 @@ sh_tc_attention2_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_c
 #pragma unroll
       for (int c = 0; c < 4; ++c) tmem_ld32(tmem_s + lane_off + c * 32, *reinterpret_cast<uint32_t(*)[32]>(&sv[c * 32]));
       tmem_ld_wait();
-      if (g.bias) {
+      if (BIAS) {
         const uint4* row = score_bias_row(g, bh, qrow[t] + r) + (size_t)j * 16 * 128;
-        uint4 b[16];
 #pragma unroll
-        for (int i = 0; i < 16; ++i) b[i] = __ldg(row + i * 128);
-        add_score_bias(sv, b);
+        for (int i = 0; i < 16; i += 4) {
+          const uint4 b[4] = {__ldg(row + i * 128), __ldg(row + (i + 1) * 128), __ldg(row + (i + 2) * 128), __ldg(row + (i + 3) * 128)};
+          add_score_bias(sv + 8 * i, b);
+        }
       }
       if (j == n - 1) {
         // last tile: the diagonal one (key c visible iff c <= r), or without the causal mask the
