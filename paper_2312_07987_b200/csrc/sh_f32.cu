@@ -379,7 +379,8 @@ int sh_f32_backward(sh_layer* L, const void* x, const float* dout, float* dx, fl
   // parts: the shortest ones (of eight steps at least) that still fit the SMs in one round; one part each where
   // whole contractions already need more rounds
   const long nq = (long)mt * ct, nl = (long)d.H * d.E * mt * (gv.nsub + go.nsub);
-  const long sq = (d.N + XG_BK - 1) / XG_BK, sl = ((long)d.N * d.k / d.E + XG_BK - 1) / XG_BK;
+  // (of a list, a step at least: with fewer selections than experts most are empty, and their gradients are still stored)
+  const long sel = (long)d.N * d.k / d.E, sq = (d.N + XG_BK - 1) / XG_BK, sl = sel < 1 ? 1 : (sel + XG_BK - 1) / XG_BK;
   long len = sq > sl ? sq : sl;
   for (long l = 8; l < len; ++l)
     if (nq * ((sq + l - 1) / l) + nl * ((sl + l - 1) / l) <= sm_count(L)) { len = l; break; }

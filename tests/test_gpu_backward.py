@@ -44,6 +44,14 @@ def test_backward_shapes(T, B, M, H, D, E, k, causal):
     check(inputs.LayerConfig("bw", inputs.DTYPE_F32, B, T, M, H, D, E, k, seed=900 + T, zipf_bias=1.2 if E == 5 else 0.0), causal=causal)
 
 
+@pytest.mark.parametrize("T,E,k", [(27, 32, 1), (5, 16, 3), (2, 16, 3)])
+def test_backward_with_fewer_selections_than_experts(T, E, k):
+    # (most experts' lists are empty: their gradients are zeros, which nothing but the kernel writes)
+    cfg = inputs.LayerConfig("bw", inputs.DTYPE_F32, 1, T, 128, 3, 40, E, k, seed=930 + T)
+    torch.full((1 << 24,), float("nan"), device="cuda")     # what the gradients' memory holds before
+    check(cfg)
+
+
 @pytest.mark.parametrize("causal", [True, False])
 def test_backward_takes_the_mask_of_the_forward_pass(causal):
     # (sh_set_causal takes effect with the next forward pass)
