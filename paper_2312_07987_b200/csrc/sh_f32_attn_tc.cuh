@@ -13,12 +13,14 @@
 // take 32 keys each, P's planes go over S in tensor memory, O_part = P V (V's rows as MN-major planes), which the workers
 // read back and add to the running sum in registers.  The next K is split under P V, V under S.
 //
-// A value that is not finite stays with the rows that see it: a tile with such a V is added up on the CUDA cores, key by
-// key, leaving out what a row does not see (0 times infinity).
+// What is not finite: a tile with such a V is added up on the CUDA cores, key by key, leaving out what a row does not see
+// (0 times infinity), so that it stays with the rows that see it.  A row whose scores of a tile are not all finite takes them again there:
+// a score of minus infinity is one (a key of weight zero), not the NaN that its split products add up to.
 //
 // Warp roles (288 threads): warps 0..7 workers (rows 32 (w & 3) ..., keys / columns of half w >> 2), warp 8 UMMAs.
 #pragma once
 #include "sh_f32_gemm.cuh"
+#include "sh_f32_attn.cuh"
 
 namespace shtc {
 
@@ -245,6 +247,23 @@ sh_f32_attn_tc_kernel(const __grid_constant__ FAttnTcArgs g) {
       if (k16s > 4) tmem_add16(sa + 192, s);
       tmem_add16(sa, s);
       const int left = seen - key0 - half * 32;            // this thread's keys 0 .. left are visible
+      float2 fin = make_float2(0.f, 0.f);                  // NaN where a score is not finite
+#pragma unroll
+      for (int i = 0; i < 32; i += 2) fin = __ffma2_rn(make_float2(s[i], s[i + 1]), make_float2(0.f, 0.f), fin);
+      if (fin.x + fin.y != 0.f && r < nq) {
+        // (the planes of a value that is not finite are no sum, and products that overflow may do so with either sign)
+        const float* qr = g.q + ((size_t)bh * d.T + q0 + r) * D;
+#pragma unroll 1
+        for (int key = 0; key < min(32, left + 1); ++key) {
+          const float* kr = Kb + (size_t)(key0 + half * 32 + key) * D;
+          float v = 0.f;
+#pragma unroll 1
+          for (int c = 0; c < d.Dt; c += 4) v = dot4(__ldg(reinterpret_cast<const float4*>(qr + c)), __ldg(reinterpret_cast<const float4*>(kr + c)), v);
+#pragma unroll
+          for (int i = 0; i < 32; ++i) s[i] = i == key ? v : s[i];
+        }
+      }
+      __syncwarp();
       float mx = -INFINITY;
 #pragma unroll
       for (int i = 0; i < 32; ++i) {

@@ -63,3 +63,28 @@ def test_f32_overflow_of_one_value_row_stays_behind_the_mask(D, t0):
     x.copy_(binding.to_device(inp.x, inp.cfg.dtype))
     assert close(layer.sh_forward(x), want)                 # and nothing of it is left behind
     layer.close()
+
+
+@pytest.mark.parametrize("wk,wq", [(10.0, -5.0),                        # the key is infinite
+                                   (1.0046875, -1.3e6)])                # it is finite, its products with the queries are not
+@pytest.mark.parametrize("D", [32, 64, 128])
+@pytest.mark.parametrize("T", [100, 400, 700])
+def test_f32_score_of_minus_infinity_weighs_nothing(T, D, wk, wq):
+    # one key's score overflows to minus infinity for every query that sees it: its weight is zero and the row stays finite
+    M, H, E, k, t0 = 128, 2, 4, 2, 40
+    inp = inputs.make_inputs(inputs.LayerConfig("parts", inputs.DTYPE_F32, 1, T, M, H, D, E, k, seed=57 + D + T))
+    inp.x[0, :, 0] = 0.0
+    inp.x[0, t0, 0] = 2.0 ** 126
+    inp.x[0, :, 1] = 1.0
+    for W in (inp.Wq, inp.Wk, inp.Ws, inp.Wd, inp.Wv):
+        W[..., :2, :] = 0.0
+    inp.Wq[:, :, 0] = inp.Wk[:, :, 0] = 0.0                 # the first position of q and k is made of x's first two columns alone
+    inp.Wq[:, 1, 0] = wq
+    inp.Wk[:, 0, 0] = wk
+    layer = binding.layer_from_inputs(inp)
+    y = layer.sh_forward(binding.to_device(inp.x, inp.cfg.dtype)).cpu().numpy()
+    assert layer.sh_last_status() == 0
+    layer.close()
+    want = switchhead_forward(inp.x, inp.Wq, inp.Wk, inp.Wv, inp.Wo, inp.Ws, inp.Wd, k, inp.bias_s, inp.bias_d, return_stages=False)["y"]
+    assert np.isfinite(want).all()
+    assert np.abs(y - want).max() / np.abs(want).max() < TOL
