@@ -14,7 +14,7 @@
 // read back and add to the running sum in registers.  The next K is split under P V, V under S.
 //
 // What is not finite: a tile with such a V is added up on the CUDA cores, key by key, leaving out what a row does not see
-// (0 times infinity), so that it stays with the rows that see it.  A row whose scores of a tile are not all finite takes them again there:
+// (0 times infinity), so that it stays with the rows that see it.  A row that finds a NaN among a tile's scores takes them again there:
 // a score of minus infinity is one (a key of weight zero), not the NaN that its split products add up to.
 //
 // Warp roles (288 threads): warps 0..7 workers (rows 32 (w & 3) ..., keys / columns of half w >> 2), warp 8 UMMAs.
@@ -65,6 +65,13 @@ __device__ __forceinline__ FAttnUnit fattn_unit(const ShDims& d, int per, int u)
   }
   r.part = u - r.first;
   return r;
+}
+
+// The larger one, NaN where one of them is.
+__device__ __forceinline__ float fmax_nan(float a, float b) {
+  float m;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(m) : "f"(a), "f"(b));
+  return m;
 }
 
 // acc += 16 tensor-memory columns at a time (the running sums leave no registers for more).
@@ -247,29 +254,28 @@ sh_f32_attn_tc_kernel(const __grid_constant__ FAttnTcArgs g) {
       if (k16s > 4) tmem_add16(sa + 192, s);
       tmem_add16(sa, s);
       const int left = seen - key0 - half * 32;            // this thread's keys 0 .. left are visible
-      float2 fin = make_float2(0.f, 0.f);                  // NaN where a score is not finite
+      float mx = -INFINITY;                                // NaN where a score is
 #pragma unroll
-      for (int i = 0; i < 32; i += 2) fin = __ffma2_rn(make_float2(s[i], s[i + 1]), make_float2(0.f, 0.f), fin);
-      if (fin.x + fin.y != 0.f && r < nq) {
+      for (int i = 0; i < 32; ++i) {
+        if (i > left) s[i] = -INFINITY;
+        mx = fmax_nan(mx, s[i]);
+      }
+      if (mx != mx) {
         // (the planes of a value that is not finite are no sum, and products that overflow may do so with either sign)
-        const float* qr = g.q + ((size_t)bh * d.T + q0 + r) * D;
+        const float* qr = g.q + ((size_t)bh * d.T + q0 + min(r, nq - 1)) * D;
+        mx = -INFINITY;
 #pragma unroll 1
-        for (int key = 0; key < min(32, left + 1); ++key) {
+        for (int key = 0; key < min(32, min(left, d.T - 1 - key0 - half * 32) + 1); ++key) {
           const float* kr = Kb + (size_t)(key0 + half * 32 + key) * D;
           float v = 0.f;
 #pragma unroll 1
           for (int c = 0; c < d.Dt; c += 4) v = dot4(__ldg(reinterpret_cast<const float4*>(qr + c)), __ldg(reinterpret_cast<const float4*>(kr + c)), v);
+          mx = fmaxf(mx, v);
 #pragma unroll
           for (int i = 0; i < 32; ++i) s[i] = i == key ? v : s[i];
         }
       }
       __syncwarp();
-      float mx = -INFINITY;
-#pragma unroll
-      for (int i = 0; i < 32; ++i) {
-        if (i > left) s[i] = -INFINITY;
-        mx = fmaxf(mx, s[i]);
-      }
       sx[half * 128 + r] = mx;
       asm volatile("bar.sync %0, 64;" ::"r"(1 + q) : "memory");
       mx = fmaxf(m, fmaxf(mx, sx[(half ^ 1) * 128 + r]));
