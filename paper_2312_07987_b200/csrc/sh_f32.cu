@@ -211,15 +211,28 @@ int launch_attn_t(sh_layer* L, float* zero, long n, cudaStream_t st) {
                   (float*)(ws + L->o.f32stats), (float4*)zero, n / 4, d);
 }
 
-// Attention; beside it `zero` (n values), which the output projection adds into, is cleared.
-// On the tensor cores from 320 keys on, or from 129 on where the other kernel's blocks of 32 queries go one and a half
+// Attention is on the tensor cores from 320 keys on, or from 129 on where the other kernel's blocks of 32 queries go one and a half
 // times round the SMs: its time is that of the longest chain of key tiles, theirs mostly that of a unit.  (Whole passes of
 // a small layer, CUDA cores / tensor cores, us: d_head 112, 8 heads, 256 keys 46 / 50, 320 55 / 53, 512 68 / 56, 800 102 / 77;
-// 64 heads, 128 keys 66 / 64, 256 keys 110 / 86; 32 heads, 192 keys 53 / 58, 256 keys 73 / 71.)
+// 64 heads, 128 keys 66 / 64, 256 keys 110 / 86; 32 heads, 192 keys 53 / 58, 256 keys 73 / 71; d_head 32 and 64, 4 heads, 256 keys 36.8 / 38.1
+// and 40.0 / 41.7, 320 39.5 / 39.3 and 44.2 / 43.0, 512 45.6 / 39.7 and 51.0 / 43.4.)
+// But not up to 32 queries behind a cache - a block of the other kernel's, and a quarter of a unit, which takes a key tile in about 1.5
+// times the time of a block - where the heads go round the SMs as often either way: above one round, and below it with 128 columns
+// and the keys in one part.  (Whole passes, one query, d_head 32, 64 and 112: 160 heads, 330 keys 107 / 122, 116 / 134, 168 / 188;
+// 128 heads, 330 keys 95 / 93, 105 / 101, 129 / 139, 1000 keys 238 / 230, 279 / 264, 313 / 342; 64 heads, 1000 keys
+// 136 / 130, 151 / 144, 211 / 198; 64 queries, 160 heads, 400 keys 159 / 165, 181 / 185, 256 / 252.)
+bool attn_on_tensor_cores(sh_layer* L) {
+  const ShDims& d = L->d;
+  const long sms = sm_count(L), heads = (long)d.B * d.H, nq = d.T - d.Tc;
+  if (nq <= 32 && (heads > sms || (d.D == 128 && 2 * heads > sms))) return false;
+  return d.T >= 320 || (d.T > 128 && 2 * ((nq + 31) / 32) * heads >= 3 * sms);
+}
+
+// Attention; beside it `zero` (n values), which the output projection adds into, is cleared.
 int launch_attn(sh_layer* L, float* zero, long n, cudaStream_t st) {
   L->launches += 1;
   const ShDims& d = L->d;
-  const bool tc = d.T >= 320 || (d.T > 128 && 2l * ((d.T - d.Tc + 31) / 32) * d.B * d.H >= 3l * sm_count(L));
+  const bool tc = attn_on_tensor_cores(L);
   switch (d.D) {
     case 32: return tc ? launch_attn_tc<32>(L, zero, n, st) : launch_attn_t<32>(L, zero, n, st);
     case 64: return tc ? launch_attn_tc<64>(L, zero, n, st) : launch_attn_t<64>(L, zero, n, st);

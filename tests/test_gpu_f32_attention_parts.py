@@ -1,12 +1,12 @@
 """fp32 attention of long sequences, forward on the tensor cores: the shortest sequence that takes it and its neighbours,
-query tiles of 128 and key tiles of 64 with one row more or less, keys in parts (one query tile's up to as many as its
-pairs of tiles) and in one, stored widths of 32, 64 and 128 columns, no mask, a cache; values that are not finite."""
+query tiles of 128 and key tiles of 64 with one row more or less, keys in parts (one query tile's up to as many as there are
+SMs) and in one, stored widths of 32, 64 and 128 columns, no mask, a cache; scores and values that are not finite."""
 import numpy as np
 import pytest
 import torch
 
 from oracle.switchhead_backward import switchhead_backward
-from oracle.switchhead_oracle import switchhead_forward
+from oracle.switchhead_oracle import switchhead_forward, switchhead_xl_forward
 from paper_2312_07987_b200 import binding, inputs
 
 pytestmark = pytest.mark.gpu
@@ -16,11 +16,11 @@ TOL = 1e-5
 
 
 @pytest.mark.parametrize("B,T,H,D,causal", [
-    (1, 320, 1, 32, True),           # the first length; three query tiles of five parts in all
+    (1, 320, 1, 32, True),           # the first length; three query tiles of six parts in all
     (1, 321, 2, 64, False),          # one key into the sixth key tile, no mask
     (2, 385, 1, 112, True),          # one row into the fourth query tile
     (1, 383, 3, 76, True),           # one row less than three
-    (1, 1025, 1, 20, True),          # nine query tiles; nine parts for the last one
+    (1, 1025, 1, 20, True),          # nine query tiles; five parts for the last one (the scratch holds no more)
     (40, 130, 2, 128, True),         # many heads: parts of the whole row, nothing to join
 ])
 def test_f32_attention_parts(B, T, H, D, causal):
@@ -88,3 +88,45 @@ def test_f32_score_of_minus_infinity_weighs_nothing(T, D, wk, wq):
     want = switchhead_forward(inp.x, inp.Wq, inp.Wk, inp.Wv, inp.Wo, inp.Ws, inp.Wd, k, inp.bias_s, inp.bias_d, return_stages=False)["y"]
     assert np.isfinite(want).all()
     assert np.abs(y - want).max() / np.abs(want).max() < TOL
+
+
+def parts_of(B, T, Tc, H, D):
+    """Parts of the last query tile's keys: two key tiles of 64 each or as many as keep the units at or below the number of SMs and their
+    partial results (128 rows of the stored width and two values) in the backward pass's scratch, four rows of it a token and head."""
+    Dp = 32 if D <= 32 else 64 if D <= 64 else 128
+    tiles = [-(-min(T, Tc + 128 * (i + 1)) // 64) for i in range(-(-(T - Tc) // 128))]
+    cap = min(torch.cuda.get_device_properties(0).multi_processor_count, 4 * B * T * H * Dp // (128 * (Dp + 2)))
+    for per in range(2, -(-T // 64)):
+        if sum(-(-n // per) for n in tiles) * B * H <= cap:
+            return -(-tiles[-1] // per)
+    return 1
+
+
+@pytest.mark.parametrize("T,Tc,B,H,D,parts", [
+    (330, 70, 1, 2, 76, 4),          # the cache ends inside a key tile, the chunk inside a query tile
+    (129, 200, 2, 1, 32, 3),         # one row into the second query tile
+    (1, 400, 1, 1, 112, 4),          # one query
+    (33, 399, 10, 8, 64, 1),         # whole rows: nothing to join
+    (100, 9000, 1, 1, 32, 72),       # the weights of many parts
+    (100, 18840, 1, 1, 20, 148),     # as many as there are SMs
+    (1, 400, 10, 8, 112, 0),         # one query for each of many heads: on the CUDA cores
+    (32, 400, 19, 8, 32, 0),         # ... and 32 for more of them than there are SMs
+])
+def test_f32_attention_behind_a_cache(T, Tc, B, H, D, parts):
+    M, E, k = 64, 2, 1
+    if parts:
+        assert parts_of(B, T + Tc, Tc, H, D) == parts
+    cfg = inputs.LayerConfig("parts", inputs.DTYPE_F32, B, Tc + T, M, H, D, E, k, seed=T + Tc)
+    inp = inputs.make_inputs(cfg)
+    layer = binding.layer_from_inputs(inp, cache_len=Tc)
+    x = binding.to_device(inp.x, cfg.dtype)
+    y = [layer.sh_forward(x).cpu().numpy() for _ in range(2)]
+    assert layer.sh_last_status() == 0
+    layer.sh_check_guards()
+    A = layer.sh_debug_buffer("AHAT").cpu().numpy().reshape(B, Tc + T, H, D)[:, Tc:]
+    layer.close()
+    # (the longest chain of additions is a thread's keys of a part, then the parts: shorter than the K of the bound)
+    want = switchhead_xl_forward(inp.x[:, Tc:], inp.x[:, :Tc], inp.Wq, inp.Wk, inp.Wv, inp.Wo, inp.Ws, inp.Wd, k, inp.bias_s, inp.bias_d)
+    assert np.abs(A - want["Ahat"]).max() / np.abs(want["Ahat"]).max() < TOL
+    for got in y:
+        assert np.abs(got - want["y"]).max() / np.abs(want["y"]).max() < TOL
