@@ -172,15 +172,21 @@ XPart part_v(sh_layer* L, const void* x, int side, const PlaneMap& w, float* dst
   return part<X_V>(L, g, d.H * head_tiles(d), g.nsub, ksplit, &w);
 }
 
-// Key tiles of a part of a query tile's keys: the fewest, two at least, that keep the units at or below F32_ATTN_UNITS and their
-// partial results in the backward pass's scratch; all of them (no parts, no scratch) where there are that many query tiles.
-int attn_part_tiles(const ShDims& d) {
+// Key tiles of a part of a query tile's keys: the fewest, two at least, that keep the units at or below the number of SMs and their
+// partial results in the backward pass's scratch (which decides for few heads of few columns); all of them (no parts, no scratch)
+// where there are that many query tiles.
+int attn_part_tiles(sh_layer* L) {
+  const ShDims& d = L->d;
   const int nqt = (d.T - d.Tc + 127) / 128, most = (d.T + 63) / 64;
-  const long room = 4l * d.N * d.H * d.D / (128 * (d.D + 2)), cap = room < F32_ATTN_UNITS ? room : F32_ATTN_UNITS;
-  for (int per = 2; per < most; ++per) {
+  const long heads = (long)d.B * d.H, room = 4l * d.N * d.H * d.D / (128 * (d.D + 2)), cap = room < sm_count(L) ? room : sm_count(L);
+  if (nqt * heads > cap) return most;
+  long all = 0;
+  for (int i = 0; i < nqt; ++i) all += fattn_key_tiles(d, i);
+  const long least = all * heads / cap;                    // (shorter parts are more units than that)
+  for (int per = least < 2 ? 2 : (int)least; per < most; ++per) {
     long units = 0;
     for (int i = 0; i < nqt; ++i) units += (fattn_key_tiles(d, i) + per - 1) / per;
-    if (units * d.B * d.H <= cap) return per;
+    if (units * heads <= cap) return per;
   }
   return most;
 }
@@ -194,7 +200,7 @@ int launch_attn_tc(sh_layer* L, float* zero, long n, cudaStream_t st) {
   g.q = (const float*)(ws + L->o.q); g.k = (const float*)(ws + L->o.k); g.v = (const float*)(ws + L->o.v);
   g.ahat = (float*)(ws + L->o.ahat); g.stats = (float*)(ws + L->o.f32stats);
   g.part = (float*)(ws + L->o.bw); g.arrived = (unsigned*)(ws + L->o.f32arrived);
-  g.zero = (float4*)zero; g.nzero = n / 4; g.d = d; g.per = attn_part_tiles(d); g.status = (int*)(ws + L->o.status);
+  g.zero = (float4*)zero; g.nzero = n / 4; g.d = d; g.per = attn_part_tiles(L); g.status = (int*)(ws + L->o.status);
   long units = 0;
   for (int i = 0; i < (d.T - d.Tc + 127) / 128; ++i) units += (fattn_key_tiles(d, i) + g.per - 1) / g.per;
   return launch_k(chained(L), sh_f32_attn_tc_kernel<D>, dim3((unsigned)(units * d.B * d.H)), dim3(288), FAttnTcSmem<D>::TOTAL, st, g);

@@ -4,9 +4,9 @@
 // fp32 as on the CUDA cores.  A layer's share of attention is small (0.5 of the 7 GFLOP of a 262M-scale forward pass) and
 // sequences are a few hundred tokens, so what counts is the longest chain of key tiles, not the work: on the CUDA cores
 // a block of 32 queries worked off 512 keys in 38 us with most SMs done long before (2 x 4 heads of 112; here 25).  Here a unit is 128 queries of one
-// (sequence, head) and a PART of their keys - as few 64-key tiles, two at least, as keep the number of units at or below F32_ATTN_UNITS,
-// one per SM -, and whoever ends last among a query tile's parts joins them (partial sums, maxima and normalisers in
-// scratch; the backward pass's, which holds nothing then).
+// (sequence, head) and a PART of their keys - as few 64-key tiles, two at least, as keep the number of units at or below that of
+// the SMs and their partial results in the scratch -, and whoever ends last among a query tile's parts joins them (partial sums, maxima and
+// normalisers; the scratch is the backward pass's, which holds nothing then).
 //
 // Per key tile: workers split K's rows into planes (shared memory, 128-byte swizzle; rows past the sequence are zeros),
 // S = Q K^T into P0 P1 P2 (and P3 for the positions from 64 on: as in sh_f32_gemm_d_kernel), two threads per query row
@@ -23,8 +23,6 @@
 #include "sh_f32_attn.cuh"
 
 namespace shtc {
-
-constexpr int F32_ATTN_UNITS = 148;      // parts are as short as this many units allow
 
 struct FAttnTcArgs {
   const float *q, *k, *v;                // [B, H, T, D]
