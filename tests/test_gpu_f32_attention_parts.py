@@ -130,3 +130,38 @@ def test_f32_attention_behind_a_cache(T, Tc, B, H, D, parts):
     assert np.abs(A - want["Ahat"]).max() / np.abs(want["Ahat"]).max() < TOL
     for got in y:
         assert np.abs(got - want["y"]).max() / np.abs(want["y"]).max() < TOL
+
+
+@pytest.mark.parametrize("cache", [0, 70])
+def test_f32_long_output_in_place_of_the_input(cache):
+    cfg = inputs.LayerConfig("parts", inputs.DTYPE_F32, 2, 400 + cache, 128, 2, 76, 4, 2, seed=19)
+    inp = inputs.make_inputs(cfg)
+    layer = binding.layer_from_inputs(inp, cache_len=cache)
+    x = binding.to_device(inp.x, cfg.dtype)
+    want = layer.sh_forward(x)
+    out = x.view(-1)[:want.numel()].view(want.shape)
+    layer.sh_forward(x, out=out)
+    assert float((out - want).abs().max() / want.abs().max()) < TOL
+    layer.close()
+
+
+def test_f32_long_sequence_with_rotary_positions_in_a_captured_graph():
+    cfg = inputs.LayerConfig("parts", inputs.DTYPE_F32, 2, 400, 128, 2, 64, 4, 2, seed=23)
+    inp = inputs.make_inputs(cfg)
+    layer = binding.layer_from_inputs(inp)
+    layer.sh_set_rope(10000.0)
+    x = torch.zeros(inp.x.shape, device="cuda")
+    layer.sh_forward(x)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        y = layer.sh_forward(x)
+    x.copy_(binding.to_device(inp.x, cfg.dtype))
+    want = switchhead_forward(inp.x, inp.Wq, inp.Wk, inp.Wv, inp.Wo, inp.Ws, inp.Wd, cfg.k, inp.bias_s, inp.bias_d, rope_base=10000.0,
+                              return_stages=False)["y"]
+    for _ in range(3):                                      # (the counters of a tile's parts go back to zero by themselves)
+        y.fill_(7.0)
+        graph.replay()
+        assert np.abs(y.cpu().numpy() - want).max() / np.abs(want).max() < TOL
+    del graph
+    layer.close()
