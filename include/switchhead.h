@@ -93,7 +93,7 @@ sh_layer* sh_create_shared(int d_model, int n_heads, int d_head, int n_experts, 
  * d_head] (moe_q) and Wk as [H, E, d_model, d_head] (moe_k) instead of [H, d_model, d_head].
  * shared_selection != 0: one gate for both sides, as sh_create_shared (keys and queries then use the
  * same selection).  SH_F32 takes every shape.  SH_BF16 (tensor-core path): an expert projection of
- * keys / queries runs on the pair-tiled value-expert kernel, so sh_configure wants k = 2, 2..8
+ * keys / queries runs on the value-expert kernel tiled by pairs of experts, so sh_configure wants k = 2, 2..8
  * experts, d_head in 65..128 and, when only one of the two is an expert projection, an even number
  * of heads; it refuses other shapes.  sh_set_rope refuses such a layer.  Other arguments and limits
  * as sh_create. */
@@ -276,8 +276,8 @@ int sh_backward(sh_layer* layer, const void* x, const float* dout, float* dx, fl
  * fp32 for SH_F32, fp16 for SH_BF16 (Q, K, V, AHAT); int32 / fp32 for the gate buffers.
  * The offsets and lists buffers hold what the last call left there: after sh_gate_topk the
  * per-(side, head, expert) lists that call returns; after an sh_forward with bf16 storage only
- * what that pass's kernels needed - the source side alone, and for a k = 2 layer the tokens
- * of a head bucketed by their PAIR of selected experts instead of by expert.
+ * what that pass's kernels needed - the source side alone, and where the value projection is tiled by
+ * sets (k = 2 to 4) the tokens of a head bucketed by their SET of selected experts instead of by expert.
  * Testing aid: lets a failing output be traced to the stage that produced it. */
 int sh_debug_buffer(sh_layer* layer, int which, void** dev_ptr, size_t* bytes);
 

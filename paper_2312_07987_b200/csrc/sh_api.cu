@@ -90,10 +90,10 @@ static void layout_workspace(sh_layer* L) {
   o.xl_bias = take(xlb ? (size_t)d.B * d.H * (d.T - d.Tc) * d.T * 2 : 16);
   // W_O once more with the experts innermost on the contraction axis: [H, M, D*E] (sparse output projection)
   o.wos = take(sh_o_sparse_ok(L) ? HD * d.E * d.M * mid : 16);
-  o.gid = take(vp ? (size_t)2 * d.N * d.H * 4 : 16);  // (both sides: query experts are tiled by the destination side's pairs)
+  o.gid = take(vp ? (size_t)2 * d.N * d.H * 4 : 16);  // set number of every (token, head) (both sides: query experts are tiled by the destination side's)
   // query / key experts (sh_create_moe_qk): [H, E, D, M] like the value experts
   o.wq_e = take(L->moe_q ? HD * d.E * d.M * win : 16);
-  o.wk_e = take(L->moe_k ? HD * d.E * d.M * win : 16);      // pair number of every (token, head), source side
+  o.wk_e = take(L->moe_k ? HD * d.E * d.M * win : 16);
   // fp32 configuration: scratch of the backward pass (dQ, dK, dV, dAhat [N, H, D], the gate gradients as a matrix [N, G],
   //  rowsum(dAhat o Ahat) [N, H]; the forward attention keeps partial results there); the gate weights
   //  once more in fp32; per attention row the score maximum and 1 / normaliser)
@@ -166,7 +166,7 @@ static int configure_common(sh_layer* L, int dtype, int batch, int seq, int cach
   }
   if (cache_len > 0 && L->dense) { sh_set_error("the dense comparator has no cache"); return SH_ERR_UNSUPPORTED; }
   if ((L->moe_q || L->moe_k) && dtype != SH_F32) {
-    // on the tensor-core path an expert projection of keys or queries is the pair-tiled value kernel with
+    // on the tensor-core path an expert projection of keys or queries is the value kernel tiled by pairs of experts with
     // other weights: the shapes that kernel serves, and a dense half (if any) the CTA-pair GEMM can tile
     const bool ok = d0.k == 2 && d0.E >= 2 && d0.E <= 8 && d0.Dt > 64 && d0.Dt <= 128 &&
                     ((L->moe_q && L->moe_k) || (d0.H * 128) % 256 == 0);
@@ -196,7 +196,8 @@ static int configure_common(sh_layer* L, int dtype, int batch, int seq, int cach
   L->d.nblk = (L->d.N + SH_TILE_ROWS - 1) / SH_TILE_ROWS;
   L->d.max_tiles = (int)((slots + SH_TILE_ROWS - 1) / SH_TILE_ROWS) + d0.H * d0.E + d0.H * 35;   // (up to 35 sets of experts: sh_v_sets_ok)
   L->d.tile_rows_src = SH_TILE_ROWS;
-  // (k >= 3: the fp16 reductions of a value row arrive in a different order from run to run - two
+  // (Of the expert-tiled value kernel, which also serves a layer tiled by sets where the device holds no cluster of its kernel.
+  //  k >= 3: the fp16 reductions of a value row arrive in a different order from run to run - two
   //  passes have been seen 1e-2 of the output RMS apart; with the first rows, which reach the output
   //  unaveraged, summed in fp32 they stay within 4e-3)
   L->d.early_rows = (dtype == SH_BF16 && (T >= SH_EARLY_MIN_SEQ || d0.k >= 3)) ? SH_EARLY_ROWS : 0;

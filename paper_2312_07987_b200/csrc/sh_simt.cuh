@@ -192,7 +192,7 @@ static __device__ __forceinline__ void sh_sort_block(const int* __restrict__ idx
       run += s_tot[g * d.E + e];
     }
   }
-  // One entry per (token, group) (k = 1: also the (head, expert pair) buckets of the pair-tiled value
+  // One entry per (token, group) (k = 1: also the (head, set of experts) buckets of the set-tiled value
   // projection, which can be many): the lanes of a warp that share a bucket find each other with
   // match.any instead of one ballot per bucket.
   const bool one_sel = d.k == 1;

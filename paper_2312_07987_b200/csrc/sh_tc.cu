@@ -126,8 +126,8 @@ struct TcState {
   bool qk_two_grids = true; // ... as two grids around the gate kernel
   bool qk_pair = true;      // CTA-pair Q/K kernel (else single-CTA persistent)
   bool o_pair = true;       // CTA-pair output projection for k <= 3 (else single-CTA)
-  bool v_sets = true;      // value projection tiled by (head, set of selected experts) on CTA pairs where the shape allows (sh_v_sets_ok)
-  int v_clusters_max = 0;      // clusters of that kernel the device holds at once (0: not asked yet, -1: none)
+  bool v_sets = true;       // value projection tiled by (head, set of selected experts) on CTA pairs where the shape allows (sh_v_sets_ok)
+  int v_clusters_max = 0;   // clusters of that kernel the device holds at once (0: not asked yet, -1: none)
   bool o_sparse = true;     // sparse-A CTA-pair output projection where the shape allows (sh_o_sparse_ok)
   bool persistent = true;   // persistent Q/K and value-expert GEMMs (else one CTA per tile)
   bool fused_sort = true;   // sort fused into the gate kernel when it needs at most half of the SMs
@@ -296,7 +296,7 @@ static int x_map(sh_layer* L, const void* x, const CUtensorMap** out) {
 
 // The gate kernel's x stream comes cold from HBM (~1.2 us per box round trip), so what bounds its
 // main loop is the bytes in flight per CTA: 8 stages when they fit, else 4.
-static int gate_smem_bytes(int Gp, int G, int stages) {   // G: histogram width (gate columns, or (head, pair) buckets if more)
+static int gate_smem_bytes(int Gp, int G, int stages) {   // G: histogram width (gate columns, or (head, set) buckets if more)
   const int stage = 128 * 64 * 2 + ((Gp * 128 + 1023) & ~1023);
   const int pipe = stages * stage, stag = 128 * (Gp + 1) * 4;
   const int bar_off = ((pipe > stag ? pipe : stag) + 1023) & ~1023;
@@ -360,11 +360,11 @@ static int tc_gate_sort(sh_layer* L, const void* x, void* out, bool zero_for_for
   g.idx = (int*)(ws + L->o.idx); g.gate = (float*)(ws + L->o.gate);
   g.blockcnt = (int*)(ws + L->o.blockcnt);
   const bool vp = zero_for_forward && use_v_sets(L);
-  // (query experts are tiled by the DESTINATION side's pairs: then both sides are bucketed by pair)
+  // (query experts are tiled by the DESTINATION side's sets: then both sides are bucketed by set)
   g.vsets = vp ? ((L->moe_q && d.sides == 2) ? 2 : 1) : 0;
   g.NS = sh_choose(d.E, d.k); g.GH = vp ? g.vsets * d.H * g.NS : d.G; g.gid = (int*)(ws + L->o.gid);
   const int GHmax = g.GH > d.G ? g.GH : d.G;
-  g.zero_v = (zero_for_forward && !vp) ? (void*)(ws + L->o.v) : nullptr;    // (the pair-tiled kernel stores every value row once)
+  g.zero_v = (zero_for_forward && !vp) ? (void*)(ws + L->o.v) : nullptr;    // (the set-tiled kernel stores every value row once)
   g.zero_out = (zero_for_forward && (S->simt_mask & SH_STAGE_O) && d.Tc == 0) ? (float*)out : nullptr;
   if (zero_for_forward && (S->simt_mask & SH_STAGE_O) && d.Tc > 0)          // (out has fewer rows than there are tokens)
     SH_CUDA_CHECK(cudaMemsetAsync(out, 0, (size_t)sh_out_rows(d) * d.M * 4, st));
@@ -378,7 +378,7 @@ static int tc_gate_sort(sh_layer* L, const void* x, void* out, bool zero_for_for
   // sort's loops run over sides * H groups.
   ShDims ds = d;
   if (zero_for_forward && !(S->simt_mask & SH_STAGE_O)) ds.sides = 1;
-  if (vp) { ds.sides = g.vsets; ds.E = g.NS; ds.k = 1; ds.G = g.GH; ds.tile_rows_src = 256; }   // buckets (side, head, pair), one entry per (token, head)
+  if (vp) { ds.sides = g.vsets; ds.E = g.NS; ds.k = 1; ds.G = g.GH; ds.tile_rows_src = 256; }   // buckets (side, head, set), one entry per (token, head)
   // Fused sort: when every CTA of the gate kernel can be resident at once (cooperative launch) and the
   // sort's scratch fits behind the logits tile in the idle operand ring, the gate kernel places the
   // tokens itself and there is no sort kernel.  Used when the gate kernel needs at most half of the SMs:
@@ -519,7 +519,7 @@ static int tc_front(sh_layer* L, const void* x, cudaStream_t st) {
   const bool vp = use_v_sets(L);
   g.vsets = vp ? 1 : 0;
   g.NS = sh_choose(d.E, d.k); g.GH = vp ? d.H * g.NS : d.G; g.gid = (int*)(ws + L->o.gid);
-  g.zero_v = vp ? nullptr : (void*)(ws + L->o.v);          // (the pair-tiled kernel stores every value row once)
+  g.zero_v = vp ? nullptr : (void*)(ws + L->o.v);          // (the set-tiled kernel stores every value row once)
   g.zero_out = nullptr;
   g.status = status;
   g.fused = 1;
@@ -634,7 +634,7 @@ int sh_tc_forward(sh_layer* L, const void* x, void* out, cudaStream_t st) {
   int qkA = 0, qkB = 0;                                    // CTA pairs of the two grids
   TcGemmArgs qg{};
   if (L->moe_q || L->moe_k) {
-    // expert projections of keys / queries run on the pair-tiled kernel (pair-bucketed lists), or - debug
+    // expert projections of keys / queries run on the set-tiled kernel (lists bucketed by pair of experts), or - debug
     // library, SH_SIMT_STAGES - on the CUDA-core kernels together with gate and value stage (expert lists)
     const bool bad = (simt & SH_STAGE_QK) ? use_v_sets(L)
                                           : (!use_v_sets(L) || !S->persistent || !S->qk_pair || qk_pairs_max(S) <= 0);

@@ -376,7 +376,7 @@ sh_tc_front_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_consta
     }
     const int per_tok = d.H * d.k;
     int* s_idx = s_sort + 8 * gg.GH;                      // [2][128 * per_tok], as sh_sort_block lays it out
-    float* s_gt = reinterpret_cast<float*>(s_idx + 2 * 128 * per_tok);     // (pair mode: [128 * H] pair numbers; gates unused)
+    float* s_gt = reinterpret_cast<float*>(s_idx + 2 * 128 * per_tok);     // (by sets: [128 * H] set numbers; gates unused)
     for (int i = et; i < d.G; i += NSEL) s_bias[i] = gg.gbias[i];
     sel_sync();
     // (one polling lane per warp: the acquire is the lane's, the warp barrier hands it on)

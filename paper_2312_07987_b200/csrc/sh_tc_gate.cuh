@@ -39,10 +39,10 @@ struct TcGateArgs {
   int max_tiles;
   int* offsets; int* lists; float* lgate; ShTile* tiles; int* ntiles;
   int* gridbar;              // {arrived, departed}, both 0 between launches
-  // value projection tiled by expert PAIRS (k = 2, forward pass only): the source side is bucketed by
+  // value projection tiled by SETS of selected experts (forward pass only): the source side is bucketed by
   // (head, set number) - histogram, sort and tile table run over H * NS buckets with one entry per
-  // (token, head) - and the destination side is not bucketed at all
-  int vsets;                // 0, or the number of sides bucketed by set of selected experts: 1 = the source side, 2 = both (query experts)
+  // (token, head) - and so is the destination side of a layer with query experts; else it is not bucketed at all
+  int vsets;                 // 0, or the number of sides bucketed by set of selected experts: 1 = the source side, 2 = both (query experts)
   int NS;                    // sets per head: choose(E, k)
   int GH;                    // histogram width: vsets ? vsets * H * NS : G
   int* gid;                  // [vsets, N, H] set number of every (token, head)
@@ -186,7 +186,7 @@ sh_tc_gate_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constan
     int* s_sort = reinterpret_cast<int*>(sgen + ((stag_bytes + 15) & ~15));
     const int per_tok = d.H * d.k;
     int* s_idx = s_sort + 8 * g.GH;                       // [2][128 * per_tok], as sh_sort_block lays it out
-    float* s_gt = reinterpret_cast<float*>(s_idx + 2 * 128 * per_tok);     // (pair mode: [128 * H] pair numbers; gates unused)
+    float* s_gt = reinterpret_cast<float*>(s_idx + 2 * 128 * per_tok);     // (by sets: [128 * H] set numbers; gates unused)
     const bool sel_ok = mbar_wait(logits_ready, 0, g.status, dead);
     if (sel_ok) {
       const int r = et & 127, sub = et >> 7;
