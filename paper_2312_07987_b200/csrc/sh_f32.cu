@@ -49,6 +49,8 @@ XPart part(sh_layer* L, const XGemmArgs& g, int gx, int gy, int gz = 1, const Pl
   if (!w) w = MODE == X_O || MODE == X_DA ? &S->wo : MODE == X_V || MODE == X_DR ? &S->wv : &S->wqk;
   XPart p;
   p.w = K_MAJOR ? w->k : w->mn; p.g = g; p.g.b_rows = w->k_rows; p.gx = gx; p.gy = gy; p.n = gx * gy * gz;
+  // (about half of the experts' last tiles are worth counting; the rest of a side's table is empty)
+  p.busy = MODE == X_QK || MODE == X_DX ? p.n : p.n - L->d.H * L->d.E / 2 * gy * gz;
   return p;
 }
 
@@ -57,10 +59,15 @@ int launch_x(sh_layer* L, cudaStream_t st, const XPart& a, const XPart& b = XPar
   const F32State* S = (const F32State*)L->f32;
   const int n = a.n + (B >= 0 ? b.n : 0);
   if (n == 0) return SH_OK;
-  auto kern = sh_f32_gemm_kernel<A, B>;
-  if (int rc = set_smem(kern, XGemmSmem::TOTAL)) return rc;
   L->launches += 1;
-  return launch_k(chained(L), kern, dim3((unsigned)n), dim3(XG_THREADS), XGemmSmem::TOTAL, st, S->wgate.mn, a, b);
+  auto go = [&](auto kern, int smem) {
+    if (int rc = set_smem(kern, smem)) return rc;
+    return launch_k(chained(L), kern, dim3((unsigned)n), dim3(XG_THREADS), smem, st, S->wgate.mn, a, b);
+  };
+  if constexpr (A != X_DX && A != X_O && A != X_DR)
+    if (a.g.sub_cols <= 64 && (B < 0 || b.g.sub_cols <= 64) && a.busy + (B >= 0 ? b.busy : 0) > sm_count(L))
+      return go(sh_f32_gemm_kernel<A, B, true>, XGemmSmem<XG_HALF>::TOTAL);
+  return go(sh_f32_gemm_kernel<A, B, false>, XGemmSmem<XG_WIDE>::TOTAL);
 }
 
 // Column tiles over `cols` columns: how many, and how wide (a multiple of 16).

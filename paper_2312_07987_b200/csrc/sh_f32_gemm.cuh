@@ -169,25 +169,34 @@ __device__ __forceinline__ XTile xg_unpack(int i, int gx, int gy) { return {i % 
 // six products - the planes of B lie one behind the other, one operand of three times the columns -
 //   h x [h' m' l'] -> P0 P1 P2,   m x [h' m'] -> P1 P2,   l x h' -> P2,
 // all of them twice in tensor memory and read every chunk.  (336 tokens, 8 heads of 32: 63 us a pass with six, 58 with three.)
+// As many narrow tiles as go more than once round the SMs run two blocks to an SM (XG_HALF), each with one accumulator, the A planes of
+// one step and weights of two: its hand-overs stand one behind the other, and the other block's fill them, as they do a tile's set-up and
+// drain.  (Whole passes, one block / two, us: 8 heads of 64, d_model 256, 168 tiles 52.5 / 48.6, 2024 tiles 337 / 294; 4 heads of 64, d_model 1024,
+// 112 tiles 68.2 / 70.5, 160 tiles 108.8 / 98.8; 2 heads of 64, d_model 512, 130 tiles 62.1 / 62.9, 192 tiles 82.9 / 75.9.)
+enum { XG_WIDE = 0, XG_NARROW = 1, XG_HALF = 2 };
+template <int KIND>
 struct XGemmSmem {
-  static constexpr int NB = 4, NR = 4;
-  static constexpr int B_STEP = 3 * XG_BN * XG_BK * 2, RAW = 128 * XG_BK * 4;
+  static constexpr int NB = KIND == XG_HALF ? 2 : 4, NR = 4, BN = KIND == XG_HALF ? 64 : XG_BN;
+  static constexpr int B_STEP = 3 * BN * XG_BK * 2, RAW = 128 * XG_BK * 4;
   static constexpr int RAW_OFF = NB * B_STEP, BAR_OFF = RAW_OFF + NR * RAW;
-  static constexpr int LD = XG_BN + 4;                     // result rows (they take the weights' place)
+  static constexpr int LD = BN + 4;                        // result rows (they take the weights' place, and that of the pieces)
   static constexpr int TOTAL = BAR_OFF + 256 + 1024;
-  static_assert(128 * LD * 4 <= RAW_OFF, "result rows take the weights' ring only");
+  static_assert(128 * LD * 4 <= BAR_OFF, "");
 };
 
 // One tile.  mapW: planes of the mode's weights, rows [(which*H + h)*D + dd][m] (Q, K), [(h*E + e)*D + dd][m] (V),
 // [(h*E + e)*M + m][dd] (O); mapG: of the gates' weights, rows [(side*H + h)*E + e][m].
-template <int MODE, bool NARROW>
+template <int MODE, int KIND>
 __device__ __forceinline__ void xg_tile(const CUtensorMap& mapW, const CUtensorMap& mapG, const XGemmArgs& g, XTile blk) {
-  using SM = XGemmSmem;
+  using SM = XGemmSmem<KIND>;
+  constexpr bool NARROW = KIND != XG_WIDE, HALF = KIND == XG_HALF;
+  constexpr int NB = SM::NB, NB_LOG = NB == 4 ? 2 : 1;     // (powers of two: a division costs the issuing thread as much as two UMMAs)
+  constexpr int NA = HALF ? 1 : 2, A_LOG = HALF ? 0 : 1;   // accumulators, and steps of A planes
   constexpr bool B_MN = MODE >= X_DA;
   constexpr bool LIST_ROWS = MODE == X_V || MODE == X_O || MODE == X_DA || MODE == X_DR;
   constexpr bool ADDED = MODE != X_QK;                     // results that are added to (as one bulk operation per row; stored by X_QK)
   constexpr int COLS = NARROW ? 32 : XG_BN / 2;            // columns of a worker thread
-  constexpr uint32_t P0 = 0, P0S = NARROW ? 192 : 128, P1 = 256, TA = 384;   // tensor-memory columns
+  constexpr uint32_t P0 = 0, P0S = NARROW ? 192 : 128, P1 = 256, TA = HALF ? 192 : 384;   // tensor-memory columns
   extern __shared__ unsigned char smem_raw[];
   const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
   unsigned char* sgen = smem_raw + (sbase - smem_u32(smem_raw));
@@ -210,7 +219,9 @@ __device__ __forceinline__ void xg_tile(const CUtensorMap& mapW, const CUtensorM
     fence_barrier_init();
   }
   pdl_wait();
-  pdl_trigger();                                           // (behind the wait: what runs ahead of the next kernel's wait sees all kernels up to the one ahead of this)
+  // (behind the wait: what runs ahead of the next kernel's wait sees all kernels up to the one ahead of this.  With room on the SM for a
+  //  block of the next kernel, behind the allocation too: that one may want all of the tensor memory and wait for this kernel's end)
+  if (!HALF) pdl_trigger();
   // ---- which tile ------------------------------------------------------------------------------
   int h = 0, e = 0, which = 0, row0 = 0, nrows = 0, n0 = 0, ncols = 0, steps = 0;
   const int sps = (d.Dt + XG_BK - 1) / XG_BK;                        // steps over one head's d_head
@@ -241,11 +252,12 @@ __device__ __forceinline__ void xg_tile(const CUtensorMap& mapW, const CUtensorM
     if (steps <= 0) return;
   }
   const int nchunk = (steps + XG_CHUNK - 1) / XG_CHUNK;
-  if (warp == 8) { tmem_alloc(tmem_slot, 512); tmem_relinquish(); }
+  if (warp == 8) { tmem_alloc(tmem_slot, HALF ? 256 : 512); tmem_relinquish(); }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  if (HALF) pdl_trigger();
 
   if (warp == 8) {
     if (lane == 0) {
@@ -267,22 +279,22 @@ __device__ __forceinline__ void xg_tile(const CUtensorMap& mapW, const CUtensorM
       const uint32_t w = B_MN ? 64 : g.b_rows;             // NARROW: columns of a plane
       const uint32_t id3 = xg_idesc(3 * w, B_MN), id2 = xg_idesc(2 * w, B_MN), id1 = xg_idesc(w, B_MN);
       for (int i = 0; i < steps && !dead; ++i) {
-        const int c = i / XG_CHUNK;                          // (powers of two: a division costs this thread as much as two UMMAs)
+        const int c = i / XG_CHUNK;
         if (i % XG_CHUNK == 0) {
-          if (!mbar_wait(&acc_empty[c & 1], ((c >> 1) & 1) ^ 1, g.status, dead)) break;
+          if (!mbar_wait(&acc_empty[c & (NA - 1)], ((c >> A_LOG) & 1) ^ 1, g.status, dead)) break;
           if (!NARROW && c > 0 && c % XG_P1_CHUNKS == 0 && !mbar_wait(p1_empty, (c / XG_P1_CHUNKS - 1) & 1, g.status, dead)) break;
         }
-        if (!mbar_wait(&b_full[i & 3], (i >> 2) & 1, g.status, dead)) break;
-        if (!mbar_wait(&a_full[i & 1], (i >> 1) & 1, g.status, dead)) break;
+        if (!mbar_wait(&b_full[i & (NB - 1)], (i >> NB_LOG) & 1, g.status, dead)) break;
+        if (!mbar_wait(&a_full[i & (NA - 1)], (i >> A_LOG) & 1, g.status, dead)) break;
         tc_fence_after();
         const int kn = (kvalid() + 15) / 16;
-        const uint32_t p0 = tmem + P0 + (c & 1) * P0S, p1 = tmem + P1;
+        const uint32_t p0 = tmem + P0 + (c & (NA - 1)) * P0S, p1 = tmem + P1;
         const uint32_t first0 = i % XG_CHUNK == 0, first1 = first0 && c % XG_P1_CHUNKS == 0;
 #pragma unroll
         for (int k = 0; k < XG_BK / 16; ++k) {
           if (k >= kn) break;
-          const uint32_t a = tmem + TA + (i & 1) * XG_A_STEP + k * 24;
-          const uint32_t b = b0 + (i & 3) * (SM::B_STEP >> 4) + BK * k;
+          const uint32_t a = tmem + TA + (i & (NA - 1)) * XG_A_STEP + k * 24;
+          const uint32_t b = b0 + (i & (NB - 1)) * (SM::B_STEP >> 4) + BK * k;
           if (NARROW) {
             umma_f16_tmem_a(p0, a, xg_desc(b, B_MN), id3, !(first0 && k == 0));
             umma_f16_tmem_a(p0 + w, a + 8, xg_desc(b, B_MN), id2, 1);
@@ -297,18 +309,18 @@ __device__ __forceinline__ void xg_tile(const CUtensorMap& mapW, const CUtensorM
           umma_f16_tmem_a(p1, a + 8, bh, id, 1);
           umma_f16_tmem_a(p0, a, bh, id, !(first0 && k == 0));
         }
-        umma_commit(&done[i & 3]);
-        if (i % XG_CHUNK == XG_CHUNK - 1 || i == steps - 1) umma_commit(&acc_full[c & 1]);
+        umma_commit(&done[i & (NB - 1)]);
+        if (i % XG_CHUNK == XG_CHUNK - 1 || i == steps - 1) umma_commit(&acc_full[c & (NA - 1)]);
       }
     }
     __syncwarp();
   } else if (warp == 9) {
     if (lane == 0) {
-      const int chunks64 = B_MN && ncols > 64 ? 2 : 1;
+      const int chunks64 = B_MN && !NARROW && ncols > 64 ? 2 : 1;
       const uint32_t bytes = B_MN ? chunks64 * 3 * 64 * XG_BK * 2 : 3 * g.b_rows * XG_BK * 2;
       for (int i = 0; i < steps && !dead; ++i) {
-        if (i >= SM::NB && !mbar_wait(&done[i & 3], ((i >> 2) - 1) & 1, g.status, dead)) break;
-        mbar_expect_tx(&b_full[i & 3], bytes);
+        if (i >= NB && !mbar_wait(&done[i & (NB - 1)], ((i >> NB_LOG) - 1) & 1, g.status, dead)) break;
+        mbar_expect_tx(&b_full[i & (NB - 1)], bytes);
         const int ii = s0 + i;
         int x = ii * XG_BK, y = 0;
         bool gm = false;
@@ -323,9 +335,9 @@ __device__ __forceinline__ void xg_tile(const CUtensorMap& mapW, const CUtensorM
           gm = seg >= 2 * d.H;
           y = gm ? (ii - 2 * d.H * sps) * XG_BK : seg * d.D + (ii - seg * sps) * XG_BK;
         }
-        const uint32_t dst = sbase + (i & 3) * SM::B_STEP;
-        tma_load_3d(dst, gm ? &mapG : &mapW, &b_full[i & 3], x, y, 0);
-        if (chunks64 == 2) tma_load_3d(dst + 3 * 64 * XG_BK * 2, gm ? &mapG : &mapW, &b_full[i & 3], x + 64, y, 0);
+        const uint32_t dst = sbase + (i & (NB - 1)) * SM::B_STEP;
+        tma_load_3d(dst, gm ? &mapG : &mapW, &b_full[i & (NB - 1)], x, y, 0);
+        if (chunks64 == 2) tma_load_3d(dst + 3 * 64 * XG_BK * 2, gm ? &mapG : &mapW, &b_full[i & (NB - 1)], x + 64, y, 0);
       }
     }
     __syncwarp();
@@ -372,11 +384,11 @@ __device__ __forceinline__ void xg_tile(const CUtensorMap& mapW, const CUtensorM
     for (int i = 0; i < COLS; ++i) acc[i] = 0.f;
     const bool mine = half * COLS < ncols;                 // (whole warps)
     auto promote = [&](int c) {
-      if (!mbar_wait(&acc_full[c & 1], (c >> 1) & 1, g.status, dead)) return;
+      if (!mbar_wait(&acc_full[c & (NA - 1)], (c >> A_LOG) & 1, g.status, dead)) return;
       tc_fence_after();
       const bool p1 = (c + 1) % XG_P1_CHUNKS == 0 || c == nchunk - 1;
       if (mine) {
-        const uint32_t a0 = tmem + tlane + P0 + (c & 1) * P0S + half * COLS, w = B_MN ? 64 : g.b_rows;
+        const uint32_t a0 = tmem + tlane + P0 + (c & (NA - 1)) * P0S + half * COLS, w = B_MN ? 64 : g.b_rows;
         if (NARROW) {
           tmem_add(a0 + 2 * w, acc);
           tmem_add(a0 + w, acc);
@@ -387,7 +399,7 @@ __device__ __forceinline__ void xg_tile(const CUtensorMap& mapW, const CUtensorM
       tc_fence_before();
       __syncwarp();
       if (lane == 0) {
-        mbar_arrive(&acc_empty[c & 1]);
+        mbar_arrive(&acc_empty[c & (NA - 1)]);
         if (!NARROW && p1) mbar_arrive(p1_empty);
       }
     };
@@ -405,18 +417,18 @@ __device__ __forceinline__ void xg_tile(const CUtensorMap& mapW, const CUtensorM
       __syncwarp();
       if (i + SM::NR < steps) load(i + SM::NR);
       cp_async_commit();
-      if (i >= 2 && !mbar_wait(&done[(i - 2) & 3], ((i - 2) >> 2) & 1, g.status, dead)) break;
+      if (i >= NA && !mbar_wait(&done[(i - NA) & (NB - 1)], ((i - NA) >> NB_LOG) & 1, g.status, dead)) break;
       tc_fence_after();
-      const uint32_t ta = tmem + tlane + TA + (i & 1) * XG_A_STEP + half * 24;
+      const uint32_t ta = tmem + tlane + TA + (i & (NA - 1)) * XG_A_STEP + half * 24;
       tmem_st8(ta, ph);
       tmem_st8(ta + 8, pm);
       tmem_st8(ta + 16, pl);
       tmem_st_wait();
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(&a_full[i & 1]);
-      // a chunk is read once two steps of the next one are in tensor memory
-      if (i % XG_CHUNK == 1 && i > XG_CHUNK) promote(promoted++);
+      if (lane == 0) mbar_arrive(&a_full[i & (NA - 1)]);
+      // a chunk is read once two steps of the next one are in tensor memory, or, with one accumulator, the first of them
+      if (HALF ? i % XG_CHUNK == 0 && i > 0 : i % XG_CHUNK == 1 && i > XG_CHUNK) promote(promoted++);
     }
     cp_async_wait<0>();
     for (; promoted < nchunk && !dead; ++promoted) promote(promoted);
@@ -466,7 +478,7 @@ __device__ __forceinline__ void xg_tile(const CUtensorMap& mapW, const CUtensorM
       }
     }
     {
-      // rows through shared memory (the weights' ring is free: every UMMA has been waited for), 16 bytes of
+      // rows through shared memory (the weights' ring and the pieces are free: every UMMA has been waited for), 16 bytes of
       // padding a row so that eight lanes' 16-byte stores meet different banks
       float* stg = reinterpret_cast<float*>(sgen);
       if (r < nrows && valid > 0 && !dead) {
@@ -508,24 +520,26 @@ __device__ __forceinline__ void xg_tile(const CUtensorMap& mapW, const CUtensorM
   __syncthreads();
   if (warp == 8) {
     tc_fence_after();
-    tmem_dealloc(tmem, 512);
+    tmem_dealloc(tmem, HALF ? 256 : 512);
   }
 }
 
 // A launch of one or two modes whose tiles do not depend on one another: the first blocks work on tiles
 // of mode A, the rest on mode B.  (One launch each leaves SMs idle in its last round,
 // and pays its set-up and drain by itself.)
-struct XPart { CUtensorMap w; XGemmArgs g; int gx, gy, n; };
+struct XPart { CUtensorMap w; XGemmArgs g; int gx, gy, n, busy; };   // busy: tiles that hold rows, about
 template <int M> struct xg_mode { static constexpr int value = M; };
-template <int A, int B>
-__global__ void __launch_bounds__(XG_THREADS, 1)
+template <int A, int B, bool HALF>                         // HALF: all tiles are narrow, two blocks to an SM
+__global__ void __launch_bounds__(XG_THREADS, HALF ? 2 : 1)
 sh_f32_gemm_kernel(const __grid_constant__ CUtensorMap mapG, const __grid_constant__ XPart pa, const __grid_constant__ XPart pb) {
   const int i = blockIdx.x;
   auto run = [&](auto mode, const XPart& p, int j) {
     constexpr int MODE = decltype(mode)::value;
     // (the columns of d_model are at least 64 a tile, and as many as 128 where there are more)
-    if (MODE != X_DX && MODE != X_O && MODE != X_DR && p.g.sub_cols <= 64) xg_tile<MODE, (MODE != X_DX && MODE != X_O && MODE != X_DR)>(p.w, mapG, p.g, xg_unpack(j, p.gx, p.gy));
-    else xg_tile<MODE, false>(p.w, mapG, p.g, xg_unpack(j, p.gx, p.gy));
+    constexpr bool D_MODEL = MODE == X_DX || MODE == X_O || MODE == X_DR;
+    if (HALF) xg_tile<MODE, XG_HALF>(p.w, mapG, p.g, xg_unpack(j, p.gx, p.gy));
+    else if (!D_MODEL && p.g.sub_cols <= 64) xg_tile<MODE, D_MODEL ? XG_WIDE : XG_NARROW>(p.w, mapG, p.g, xg_unpack(j, p.gx, p.gy));
+    else xg_tile<MODE, XG_WIDE>(p.w, mapG, p.g, xg_unpack(j, p.gx, p.gy));
   };
   if (B < 0 || i < pa.n) run(xg_mode<A>(), pa, i);
   else run(xg_mode<(B >= 0 ? B : A)>(), pb, i - pa.n);
