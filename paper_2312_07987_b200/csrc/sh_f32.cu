@@ -64,17 +64,35 @@ int launch_x(sh_layer* L, cudaStream_t st, const XPart& a, const XPart& b = XPar
     if (int rc = set_smem(kern, smem)) return rc;
     return launch_k(chained(L), kern, dim3((unsigned)n), dim3(XG_THREADS), smem, st, S->wgate.mn, a, b);
   };
-  if constexpr (A != X_DX && A != X_O && A != X_DR)
-    if (a.g.sub_cols <= 64 && (B < 0 || b.g.sub_cols <= 64) && a.busy + (B >= 0 ? b.busy : 0) > sm_count(L))
+  if constexpr (A != X_DX && A != X_DR)
+    if (a.g.sub_cols <= 64 && a.g.b_rows <= 64 && (B < 0 || (b.g.sub_cols <= 64 && b.g.b_rows <= 64)) && a.busy + (B >= 0 ? b.busy : 0) > sm_count(L))
       return go(sh_f32_gemm_kernel<A, B, true>, XGemmSmem<XG_HALF>::TOTAL);
   return go(sh_f32_gemm_kernel<A, B, false>, XGemmSmem<XG_WIDE>::TOTAL);
 }
 
 // Column tiles over `cols` columns: how many, and how wide (a multiple of 16).
 int col_width(int cols) { const int n = (cols + XG_BN - 1) / XG_BN; return ((cols + n - 1) / n + 15) / 16 * 16; }
-void col_tiles(XGemmArgs& g, int cols) {
-  g.nsub = (cols + XG_BN - 1) / XG_BN;
-  g.sub_cols = col_width(cols);
+void col_tiles(XGemmArgs& g, int cols, int width = 0) {
+  g.sub_cols = width ? width : col_width(cols);
+  g.nsub = (cols + g.sub_cols - 1) / g.sub_cols;
+}
+// Row tiles of a side's lists, about.
+long list_tiles(const ShDims& d) { return (long)d.H * d.N * d.k / 128 + d.H * d.E / 2; }
+// A head's columns of d_head 129 to 192 are three tiles of up to 64 (one operand for three products, two blocks to an SM) and not two,
+// except where two go once round the SMs and three do not.  (Two / three, a pass in us: 1 head of 160, d_model 960, 300 tokens 69.0 / 61.9, 2400
+// tokens - 116 tiles or 173 - 88.2 / 92.0; 2 heads of 168, d_model 448, 900 tokens - 128 or 192 - 60.5 / 65.2, 2400 tokens 124 / 103.)
+int proj_width(sh_layer* L) {
+  const ShDims& d = L->d;
+  const long two = 2 * (2l * d.H * d.nblk + list_tiles(d)), sms = sm_count(L);
+  const bool three = d.Dt > 128 && d.Dt <= 192 && (two > sms || 3 * two <= 2 * sms);
+  return three ? ((d.Dt + 2) / 3 + 15) / 16 * 16 : col_width(d.Dt);
+}
+// The output's columns, d_head above 128, are tiles of 64 instead of up to 128 where those leave more than a quarter of their rounds empty
+// (2 heads, 2 of 4 experts: 150, d_model 192, 2400 tokens, 158 tiles 24 / 17 us; 168, d_model 448, 316 tiles 36 / 30; but 132, d_model 1024, 300 tokens
+// of 4 of 8, 214 tiles, a pass 87.5 / 89.8).
+bool out_narrow(sh_layer* L) {
+  const long tiles = list_tiles(L->d) * ((L->d.M + XG_BN - 1) / XG_BN), sms = sm_count(L);
+  return L->d.Dt > 128 && tiles > sms && 5 * ((tiles + sms - 1) / sms * sms) >= 7 * tiles;
 }
 
 // A contraction over d_head of a side's lists: up to 128 positions on the kernel that keeps its rows in tensor memory,
@@ -86,11 +104,11 @@ int launch_d(sh_layer* L, cudaStream_t st, XGemmArgs g) {
   const ShDims& d = L->d;
   const PlaneMap& w = MODE == X_O ? S->wo : S->wv;
   if (d.Dt > 128) {
-    col_tiles(g, d.M);
+    col_tiles(g, d.M, MODE == X_O && out_narrow(L) ? 64 : 0);
     return launch_x<MODE>(L, st, part<MODE>(L, g, d.H * head_tiles(d), g.nsub));
   }
   const int ntile = (d.M + XGemmDSmem::BN - 1) / XGemmDSmem::BN;
-  const long rows = d.k == d.E ? (long)d.H * d.E * ((d.N + 127) / 128) : (long)d.H * d.N * d.k / 128 + d.H * d.E / 2;
+  const long rows = d.k == d.E ? (long)d.H * d.E * ((d.N + 127) / 128) : list_tiles(d);
   long split = sm_count(L) / (rows < 1 ? 1 : rows);
   split = split < 1 ? 1 : split > ntile ? ntile : split;
   auto kern = sh_f32_gemm_d_kernel<MODE>;
@@ -164,7 +182,7 @@ int launch_gate_sort(sh_layer* L, const void* x, float* zero, long n, cudaStream
 XPart part_qk(sh_layer* L, const void* x, int first, int groups) {
   XGemmArgs g = base_args(L, x);
   g.qk_first = first; g.qk_groups = groups;
-  col_tiles(g, L->d.Dt);
+  col_tiles(g, L->d.Dt, proj_width(L));
   return part<X_QK>(L, g, L->d.nblk, groups * g.nsub);
 }
 
@@ -174,7 +192,7 @@ XPart part_v(sh_layer* L, const void* x, int side, const PlaneMap& w, float* dst
   XGemmArgs g = base_args(L, x);
   use_side(g, L, side);
   g.v = dst; g.vscale = scale;
-  col_tiles(g, d.Dt);
+  col_tiles(g, d.Dt, proj_width(L));
   g.ksplit = ksplit;
   return part<X_V>(L, g, d.H * head_tiles(d), g.nsub, ksplit, &w);
 }
@@ -309,12 +327,12 @@ int sh_f32_prepare(sh_layer* L) {
     return sh_tc_encode_planes(&m.mn, ws + off, inner, rows, 64, XG_BK);
   };
   const uint64_t HD = (uint64_t)d.H * d.D;
-  const int cw = col_width(d.Dt);
+  const int cw = proj_width(L);
   int rc;
   if ((rc = enc(S->wqk, L->o.wqk, d.M, 2 * HD, cw))) return rc;
   if ((rc = enc(S->wgate, L->o.wgate, d.M, d.G, 64))) return rc;
   if ((rc = enc(S->wv, L->o.wv, d.M, HD * d.E, cw))) return rc;
-  if ((rc = enc(S->wo, L->o.wo, d.D, (uint64_t)d.H * d.E * d.M, d.Dt > 128 ? XG_BN : XGemmDSmem::BN))) return rc;
+  if ((rc = enc(S->wo, L->o.wo, d.D, (uint64_t)d.H * d.E * d.M, d.Dt > 128 && !out_narrow(L) ? XG_BN : 64))) return rc;
   if (L->moe_q && (rc = enc(S->wq_e, L->o.wq_e, d.M, HD * d.E, cw))) return rc;
   if (L->moe_k && (rc = enc(S->wk_e, L->o.wk_e, d.M, HD * d.E, cw))) return rc;
   return SH_OK;
@@ -426,7 +444,7 @@ int sh_f32_backward(sh_layer* L, const void* x, const float* dout, float* dx, fl
   g = dst;
   col_tiles(g, d.Dt);
   // (about half of the experts' last tiles are worth counting; the rest of the table is empty)
-  g.ksplit = k_parts(L, ((long)d.H * d.N * d.k / 128 + d.H * d.E / 2) * g.nsub, d.M / XG_BK);
+  g.ksplit = k_parts(L, list_tiles(d) * g.nsub, d.M / XG_BK);
   if ((rc = launch_x<X_DA>(L, st, part<X_DA>(L, g, d.H * ht, g.nsub, g.ksplit)))) return rc;
   // attention
   rc = d.D == 32 ? launch_attn_bw_t<32>(L, w, st) : d.D == 64 ? launch_attn_bw_t<64>(L, w, st)

@@ -1,6 +1,7 @@
-"""fp32 projections of up to 64 columns with more tiles than SMs (two blocks to an SM): d_head 20, 40 and 64 (weight boxes of 32,
-48 and 64 rows), contractions of one chunk of two steps, of three and of seventeen, lists whose last tiles are short; dAhat over as
-many tiles."""
+"""fp32 projections in tiles of up to 64 columns, more of them than SMs (two blocks to an SM): d_head 20, 40 and 64 (weight boxes of
+32, 48 and 64 rows), contractions of one chunk of two steps, of three and of seventeen, lists whose last tiles are short, dAhat over as
+many tiles; d_head 132, 150 and 192 in three tiles (boxes of 48 and 64 rows, the last tile 4 columns past a box of 16, 22, and whole),
+output and dx of the values in tiles of 64 columns over five and six steps, the last one 4 positions long, 22, and whole."""
 import numpy as np
 import pytest
 import torch
@@ -19,10 +20,16 @@ TOL = 1.5e-5
     (16, 130, 64, 8, 20, 3, 2),
     (13, 97, 1088, 6, 64, 4, 1),
     (8, 300, 192, 3, 40, 5, 3),
+    (24, 100, 192, 2, 132, 4, 2),
+    (10, 130, 448, 3, 150, 5, 3),
+    (30, 81, 256, 2, 192, 3, 2),
 ])
 def test_f32_narrow_tiles(B, T, M, H, D, E, k):
     cfg = inputs.LayerConfig("narrow", inputs.DTYPE_F32, B, T, M, H, D, E, k, seed=T + M)
-    tiles = -(-B * T // 128) * 2 * H + H * (B * T * k // 128 + E // 2)
+    lists = H * (B * T * k // 128 + E // 2)
+    tiles = -(-B * T // 128) * 2 * H + lists
+    if D > 128:
+        tiles = min(2 * tiles, lists * -(-M // 128))
     assert tiles > torch.cuda.get_device_properties(0).multi_processor_count
     inp = inputs.make_inputs(cfg)
     G = np.random.default_rng(5).standard_normal(inp.x.shape).astype(np.float32)
