@@ -17,7 +17,8 @@
 // (0 times infinity), so that it stays with the rows that see it.  A row that finds a NaN among a tile's scores takes them again there:
 // a score of minus infinity is one (a key of weight zero), not the NaN that its split products add up to.
 //
-// Warp roles (288 threads): warps 0..7 workers (rows 32 (w & 3) ..., keys / columns of half w >> 2), warp 8 UMMAs.
+// Warp roles (288 threads): warps 0..7 workers (rows 32 (w & 3) ..., keys / columns of half w >> 2), warp 8 UMMAs.  Nine
+// warps leave 168 registers a thread; with 128 columns the running sums and a piece of K or V in flight spill (212 bytes stored, 332 loaded).
 #pragma once
 #include "sh_f32_gemm.cuh"
 #include "sh_f32_attn.cuh"

@@ -10,7 +10,8 @@
 // Shared-memory traffic per step 136 KB, 1060 cycles, against 768 of tensor time (with A's planes there as well: 208 KB,
 // 1600 cycles).  One block per SM, 512 workers.  2 x 512 tokens, d_model 1024, 4 heads of 112: 328 tiles, 92 -> 84 us behind dx;
 // 8 x 256 tokens, d_model 448, 2 heads of 76: 60 -> 51 us.  What bounds it: 2.2 rounds of tiles, each with its set-up and drain, and
-// the hand-overs of a step, as in sh_f32_gemm.cuh.
+// the hand-overs of a step, as in sh_f32_gemm.cuh.  The warp that issues UMMAs is a seventeenth, which leaves 96 registers a thread (128
+// with 16 warps): 72 bytes of spills stored and 220 loaded.
 #pragma once
 #include "sh_f32_gemm.cuh"
 

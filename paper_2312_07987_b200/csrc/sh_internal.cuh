@@ -160,7 +160,12 @@ inline bool sh_o_sparse_ok(const sh_layer* L) {
 // Shapes whose value projection is tiled by (head, set of selected experts) instead of (head, expert): the k experts of a
 // set side by side are at most 256 columns, and there are few enough sets for their partly filled tiles - half a tile of
 // 256 rows each, on two SMs, against half a tile of 128 per expert - not to cost more than the k - 1 further gathers of
-// every row.  (8192 tokens, 2 heads of 64, three of five experts: 59.1 -> 48.6 us a pass.)
+// every row.  A row is the fp32 sum of its experts, rounded once, where the other kernel adds fp16 results in memory.
+// Passes back to back in us, by experts / by sets: 8192 tokens, 2 heads of 64, d_model 512, 3 of 5 experts 56.9 / 49.0.  At the line, 2 heads
+// and d_model 512, 4 and 1024: 1200 tokens, 3 of 6: 47.2 / 45.3, 65.6 / 67.6; 2400 tokens, 3 of 7: 49.2 / 49.2, 75.8 / 77.8; 1600 tokens, 4 of 7: 49.7 / 51.2,
+// 78.6 / 79.7; 3200 tokens, 2 of 8: 46.7 / 49.2, 74.8 / 75.9; 16000 tokens, 2 of 8: 80.3 / 74.9, 194.5 / 171.8; below it: 400 tokens, 4 of 6: 47.4 / 45.2,
+// 69.6 / 64.1.  With two experts and an odd number of heads, whose Q/K projection is a kernel of its own beside this one, the sets cost 2 to 15 % up
+// to 7000 tokens (800 tokens, 3 heads, d_model 2048, 2 of 3: 59.4 / 70.1): they stay for their rounding.
 inline bool sh_v_sets_ok(const sh_layer* L) {
   const ShDims& d = L->d;
   if (L->dtype != SH_BF16 || L->dense || d.k < 2 || d.k > 4 || d.E < d.k) return false;
